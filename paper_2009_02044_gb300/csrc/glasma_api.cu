@@ -129,8 +129,9 @@ static int check_params(const glasma_params* p) {
 }
 
 // The automatic choice, from CUDA-event timings on GB300: in FP64 the
-// plaquette kernel (24% fewer FMAs, and the FP64 pipe bounds the step:
-// 12.8 against 15.3 ms per SU(3) 512 x 64^2 step); in FP32 SU(3) with rows
+// two-pass plaquette form on every lattice whose scratch was allocated (the
+// fewest multiply-adds, and the FP64 pipe bounds the step; figures in
+// k_step_plaq64.cu); in FP32 SU(3) with rows
 // of 64 sites the staged staple kernel (0.446-0.449 ms against 0.472-0.475
 // for the one-site staple kernel, bitwise the same result), else the staple
 // kernel (0.469 ms, against 0.521 for the plaquette kernel and 0.572 for
@@ -139,9 +140,13 @@ static int check_params(const glasma_params* p) {
 // 1024 x 128^2 step, once a link's alpha and beta became one 16-byte load:
 // the pairs' 32-bit loads then stride 16 bytes).
 bool use_plaq_kernel(const glasma_ctx* c) {
+  if (c->rs == 8) return false;
   if (c->step_kernel == GLASMA_KERNEL_PLAQUETTE || c->step_kernel == GLASMA_KERNEL_PLAQUETTE_256) return plaq_fits(c);
-  return c->step_kernel == GLASMA_KERNEL_AUTO && c->rs == 8 && plaq_fits(c);
+  return false;
 }
+
+// both plaquette choices name this form in FP64
+bool use_parts_kernel(const glasma_ctx* c) { return c->part && c->step_kernel != GLASMA_KERNEL_STAPLE; }
 
 bool use_pair_kernel(const glasma_ctx* c) {
   if (c->rs != 4 || c->slab) return false;  // the pairs span the whole z range
@@ -153,7 +158,9 @@ bool use_staged_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_AUTO && staged_fits(c) && c->g.nx == 64;
 }
 
-int launch_step_chosen(glasma_ctx* c, bool hop) {
+int launch_step_chosen(glasma_ctx* c, bool hop, int* launches) {
+  if (use_parts_kernel(c)) return launch_step_parts(c, hop, c->step_zlen, launches);
+  *launches += 1;
   if (use_plaq_kernel(c)) return launch_step_plaq(c, hop, c->step_zlen);
   if (use_pair_kernel(c)) return launch_step_pair(c, hop);
   if (use_staged_kernel(c)) return launch_step_staged(c, hop);
@@ -275,6 +282,9 @@ static int create_ctx(const glasma_params* p, const double* rho_host, void* stre
       return st;
     }
   }
+  // scratch of the FP64 step: without it (too large a plane, or no memory
+  // left) the context steps with the staple kernel
+  if (parts_ring(c) > 0) c->part = (double*)ctx_alloc(c, parts_bytes(c));
   st = run_init(c, rho_host);
   if (st) {
     std::string keep = g_last_error;
@@ -334,8 +344,7 @@ int glasma_step(glasma_ctx* c, int n_steps) {
       c->last_iters = iters;
       launches += iters + 1;
     } else {
-      st = launch_step_chosen(c, hop);
-      launches += 1;
+      st = launch_step_chosen(c, hop, &launches);
     }
     // a step that did not converge has still been taken (last iterate kept)
     if (st && st != GLASMA_ERR_NOT_CONVERGED) return st;

@@ -43,6 +43,7 @@ struct glasma_ctx {
   int step_kernel = 0;        // GLASMA_KERNEL_* of the leapfrog step
   int step_zlen = 0;          // z slices per block of the plaquette kernel (0 = automatic)
   bool plaq_ready = false;    // the plaquette kernel's attributes are set on this device
+  double* part = nullptr;     // FP64 leapfrog: plaquette contributions (k_step_plaq64.cu)
   // staged step kernel (k_step_staged.cu): spin budget of one wait on its
   // copies (SM cycles), the timeout test's stall, and whether it has run
   // since its status word (dflag[1]) was last read
@@ -94,8 +95,15 @@ int launch_step_leapfrog(glasma_ctx* c, bool hop);
 // plaquette-centric leapfrog step (k_step_plaq.cu): zlen z slices per block
 int launch_step_plaq(glasma_ctx* c, bool hop, int zlen);
 bool plaq_fits(const glasma_ctx* c);
-// the step kernel glasma_step launches for this context: plaquette, staple
-// on site pairs (FP32), staged staple (FP32 SU(3)) or staple
+// the same form in FP64, in two passes through a scratch array
+// (k_step_plaq64.cu): its ring's slices (0: none) and bytes
+int parts_ring(const glasma_ctx* c);
+size_t parts_bytes(const glasma_ctx* c);
+int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches);
+// the step kernel glasma_step launches for this context: plaquette (FP64 in
+// two passes), staple on site pairs (FP32), staged staple (FP32 SU(3)) or
+// staple
+bool use_parts_kernel(const glasma_ctx* c);
 bool use_plaq_kernel(const glasma_ctx* c);
 bool use_pair_kernel(const glasma_ctx* c);
 bool use_staged_kernel(const glasma_ctx* c);
@@ -105,7 +113,7 @@ bool staged_fits(const glasma_ctx* c);
 int launch_step_staged(glasma_ctx* c, bool hop);
 // TIMEOUT if a staged launch recorded a wait that ran out (synchronises)
 int staged_status(glasma_ctx* c);
-int launch_step_chosen(glasma_ctx* c, bool hop);
+int launch_step_chosen(glasma_ctx* c, bool hop, int* launches);  // adds its launches
 // staple kernel on pairs of sites (t, iz), (t, iz + ceil(nz/2)), FP32 only
 int launch_step_pair(glasma_ctx* c, bool hop);
 int plaq_default_zlen(const glasma_ctx* c);

@@ -465,19 +465,19 @@ static int per_event_run(glasma_batch* b, int steps) {
   if (steps == 0) return GLASMA_OK;
   const size_t ne = b->ev.size();
   EventCursor cs(b);
-  int st = GLASMA_OK;
+  int st = GLASMA_OK, launches = 0;
   for (int k = 0; k < steps && !st; ++k) {
     for (size_t e = 0; e < ne && !st; ++e) {
       glasma_ctx* c = b->ev[e];
       c->cur = cs.cur[e];
       c->zA0 = cs.zA0[e];
       c->zB0 = cs.zB0[e];
-      st = launch_step_chosen(c, hop_at(cs.n[e], c->hop_p, c->hop_q));
+      st = launch_step_chosen(c, hop_at(cs.n[e], c->hop_p, c->hop_q), &launches);
     }
     cs.advance(b);
   }
   if (st) return st;
-  cs.store(b, steps * (int)ne);
+  cs.store(b, launches);
   return GLASMA_OK;
 }
 

@@ -166,8 +166,7 @@ __global__ void __launch_bounds__(192) k_implicit_prev(ImplArgs<R> a) {
   R e[NA];
 #pragma unroll
   for (int c = 0; c < NA; ++c) e[c] = a.E[(int64_t)(i * NA + c) * a.g.V + s];
-  typename G::M u = G::mul(G::expi_series(e, -a.dt), LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s));
-  if (sizeof(R) == 4) u = G::reunit(u);
+  const typename G::M u = G::evolve_series(e, -a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s));
   LinkIO<NC, R>::template store<R>(a.Uout, i, a.g.V, s, u);
 }
 
@@ -226,9 +225,7 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
       for (int c = 0; c < NA; ++c) ew[c] += dj[c];
     }
     // X^(0) = exp(i dt E(t_{n-1/2})) U_n
-    M u = G::mul(G::expi_series(e, a.dt), Ui);
-    if (sizeof(R) == 4) u = G::reunit(u);
-    LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, u);
+    LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, G::evolve_series(e, a.dt, Ui));
   }
   R F[NA];
   force_implicit<NC, R>(a, site_nbr_tz(a.g, t, iz), i, F, 1, 3);
@@ -284,9 +281,8 @@ __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t
     emax = fmax(emax, fabs(e[c]));
     a.E[idx] = e[c];
   }
-  M u = G::mul(G::expi_series(e, a.dt), LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s));
-  if (sizeof(R) == 4) u = G::reunit(u);
-  LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, u);
+  LinkIO<NC, R>::template store<R>(
+      a.Xn, i, a.g.V, s, G::evolve_series(e, a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s)));
 }
 
 // One fixed-point sweep: E = Ework + dt F_0(X), Xn = exp(i dt E) U_n, where

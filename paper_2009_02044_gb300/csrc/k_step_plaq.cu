@@ -1,5 +1,6 @@
-// Leapfrog step with the CPIC hop, plaquette-centric form (Sec. 3,
-// Eqs. lattice_1, plaquette, lattice_2, continuity).
+// FP32 leapfrog step with the CPIC hop, plaquette-centric form (Sec. 3,
+// Eqs. lattice_1, plaquette, lattice_2, continuity); k_step_plaq64.cu has the
+// FP64 form.
 //
 // The staple form (step_link) rebuilds every plaquette once for each of
 // its four links.  Here each site x forms the three plaquettes based at it,
@@ -76,9 +77,9 @@ struct PlaqWork {
 };
 
 // Block shapes: V = 0 up to 320 threads (96 registers at 2 FP32 blocks per
-// SM), V = 1 up to 256 threads (128 registers).  FP64 runs one block per SM.
+// SM), V = 1 up to 256 threads (128 registers).
 template <typename R, int V> struct PlaqOcc {
-  static constexpr int threads = V == 0 ? 320 : 256, blocks = sizeof(R) == 8 ? 1 : 2;
+  static constexpr int threads = V == 0 ? 320 : 256, blocks = 2;
 };
 
 template <int NC, typename R, int V>
@@ -293,9 +294,9 @@ static int plaq_attrs() {
 int plaq_prepare(glasma_ctx* c) {
   int st;
   if (c->p.nc == 2)
-    st = c->rs == 8 ? plaq_attrs<2, double>() : plaq_attrs<2, float>();
+    st = plaq_attrs<2, float>();
   else
-    st = c->rs == 8 ? plaq_attrs<3, double>() : plaq_attrs<3, float>();
+    st = plaq_attrs<3, float>();
   if (!st) c->plaq_ready = true;
   return st;
 }
@@ -312,7 +313,7 @@ int plaq_default_zlen(const glasma_ctx* c) {
   const int T = plaq_variant(c) ? 256 : 320;
   if (!plaq_shape(c->g.nx, c->g.ny, T, &rows, &halo)) return 16;
   const long long tiles = (c->g.ny + rows - 1) / rows;
-  const long long slots = 152LL * (c->rs == 8 ? 1 : 2);
+  const long long slots = 152LL * 2;
   long long z = tiles * (c->hi - c->lo) / (8 * slots);
   if (z < 4) z = 4;
   if (z > 64) z = 64;
@@ -322,11 +323,8 @@ int plaq_default_zlen(const glasma_ctx* c) {
 int launch_step_plaq(glasma_ctx* c, bool hop, int zlen) {
   if (zlen <= 0) zlen = plaq_default_zlen(c);
   const int v = plaq_variant(c);
-  if (c->p.nc == 2) {
-    if (c->rs == 8) return v ? launch_plaq_t<2, double, 1>(c, hop, zlen) : launch_plaq_t<2, double, 0>(c, hop, zlen);
-    return v ? launch_plaq_t<2, float, 1>(c, hop, zlen) : launch_plaq_t<2, float, 0>(c, hop, zlen);
-  }
-  if (c->rs == 8) return v ? launch_plaq_t<3, double, 1>(c, hop, zlen) : launch_plaq_t<3, double, 0>(c, hop, zlen);
+  if (c->rs != 4) return set_error(GLASMA_ERR_INTERNAL, "the marching plaquette kernel is FP32 only");
+  if (c->p.nc == 2) return v ? launch_plaq_t<2, float, 1>(c, hop, zlen) : launch_plaq_t<2, float, 0>(c, hop, zlen);
   return v ? launch_plaq_t<3, float, 1>(c, hop, zlen) : launch_plaq_t<3, float, 0>(c, hop, zlen);
 }
 

@@ -1,0 +1,223 @@
+// FP64 leapfrog step with the CPIC hop, plaquette-centric form in two passes
+// (Sec. 3, Eqs. lattice_1, plaquette, lattice_2, continuity).
+//
+// GB300 does two FP64 multiply-adds per SM and clock, so the FP64 step is
+// bound by their number, and device memory has time to spare (SU(3): some 2400
+// multiply-adds against 1.9 KB per site, 4.5 us against 0.3 us per 1000 sites).
+// Hence every plaquette is formed once, by a thread of its own, and what it
+// contributes to its four links goes through a scratch array:
+//   k_step_plaq_parts  one thread per (site, plane): A = U_b(x+a) U_a^dag(x+b),
+//                      B = U_b^dag(x) U_a(x); the projections of the loop at
+//                      its corners, pAB (corner x+a, link b), pBA (corner x+b,
+//                      link a) and p0 = U_a pAB U_a^dag (corner x);
+//   k_step_plaq_links  one thread per link: F_a(x) = sum over the other
+//                      directions of -+ w p0 and +- w pAB or pBA of the
+//                      plaquette below, then update_link.
+// Two products, two projections and one transport of an algebra vector are
+// 534 multiply-adds per SU(3) plaquette (594 with p0 from a third product)
+// and 68 per SU(2) plaquette, whose pAB and pBA differ in a cross product's
+// sign only.  Against a block that marches through z with a halo row and a
+// warm-up slice in shared memory, no work is done twice, and threads of both
+// passes are numbered straight through the sites, so a small lattice spreads
+// over all SMs and a plane of any size fills its warps.
+// Measured, whole events in FP64 against the marching form: SU(2) 128 x 16^2,
+// 100 steps, 19.7 -> 4.56 ms; SU(3) 160 x 24^2, 40 steps, 61.6 -> 21.0 ms (both
+// with the series exponentials of su_n.cuh, which came with it).
+//
+// The scratch holds a ring of slices (nine vectors per site).  A lattice whose
+// vectors pass kPartsBytes is stepped in chunks of slices; chunk k's parts
+// pass overwrites neither the parts its links pass reads from the slice below
+// nor any other, as the ring has one slice more than a chunk.  Every value is
+// formed by the same instructions whatever the chunk, so results do not
+// depend on it.
+#include "step_link.cuh"
+
+namespace glasma {
+
+// the scratch aims at this size (it then stays in the L2 cache between the
+// two passes); a ring of two slices may take kPartsMost, above which the
+// context steps with the staple kernel
+constexpr size_t kPartsBytes = (size_t)64 << 20;
+constexpr size_t kPartsMost = (size_t)512 << 20;
+constexpr int kPartsThreads = 128;
+
+// vectors per site: p0 of the planes xy, xz, yz, then their pAB, then pBA
+enum { kP0 = 0, kPAB = 3, kPBA = 6, kPartVecs = 9 };
+
+struct PartsArgs {
+  const double2* U;
+  double* part;
+  Geom g;
+  int zfirst, z0;  // slices zfirst..: one before z0 where a slab's halo has to be added
+  int ring;        // slices of the scratch
+  uint32_t sites;  // sites of the launch
+};
+
+template <int NC>
+struct PlaqCorners;
+
+template <>
+struct PlaqCorners<3> {
+  typedef Group<3, double> G;
+  __device__ __forceinline__ static void both(const G::M& A, const G::M& B, double* ab, double* ba) {
+    G::proj_mul(A, B, ab);
+    G::proj_mul(B, A, ba);
+  }
+};
+
+template <>
+struct PlaqCorners<2> {
+  typedef Group<2, double> G;
+  // A = p + i a.sigma, B = q + i b.sigma: AB and BA have the vector parts
+  // p b + q a -+ a x b
+  __device__ __forceinline__ static void both(const G::M& A, const G::M& B, double* ab, double* ba) {
+    const double p = A.a.re, q = B.a.re;
+    const double a[3] = {A.b.im, A.b.re, A.a.im}, b[3] = {B.b.im, B.b.re, B.a.im};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+      const double s = fma(p, b[k], q * a[k]), c = fma(a[k1], b[k2], -(a[k2] * b[k1]));
+      ab[k] = s - c;
+      ba[k] = s + c;
+    }
+  }
+};
+
+template <int NC>
+__global__ void __launch_bounds__(kPartsThreads, 2) k_step_plaq_parts(PartsArgs a) {
+  typedef Group<NC, double> G;
+  typedef LinkIO<NC, double> IO;
+  typedef typename G::M M;
+  constexpr int NA = G::NA;
+  const uint32_t idx = blockIdx.x * kPartsThreads + threadIdx.x;
+  if (idx >= a.sites) return;
+  const Geom& g = a.g;
+  const uint32_t nxy = (uint32_t)g.nxy, dz = idx / nxy, t = idx - dz * nxy;
+  const int z = a.zfirst + (int)dz, pl = (int)blockIdx.y;
+  const bool below = z < a.z0;  // only what reaches the slice above is wanted
+  if (pl == 0 ? below : z >= g.nz - 1) return;
+  const int da = pl == 2 ? 1 : 0, db = pl == 0 ? 1 : 2;
+  const SiteNbr n = site_nbr_tz(g, t, z);
+  const int64_t S = (int64_t)a.ring * nxy;
+  double* out = a.part + (int64_t)(z % a.ring) * nxy + t;
+  const M ua = IO::template load<double>(a.U, da, g.V, n.s);
+  const M A = G::mul_d(IO::template load<double>(a.U, db, g.V, n.p[da]),
+                       IO::template load<double>(a.U, da, g.V, n.p[db]));
+  const M B = G::d_mul(IO::template load<double>(a.U, db, g.V, n.s), ua);
+  double ab[NA], ba[NA];
+  PlaqCorners<NC>::both(A, B, ab, ba);
+#pragma unroll
+  for (int c = 0; c < NA; ++c) out[((kPBA + pl) * NA + c) * S] = ba[c];
+  if (below) return;
+#pragma unroll
+  for (int c = 0; c < NA; ++c) out[((kPAB + pl) * NA + c) * S] = ab[c];
+  G::adj(ua, ab);
+#pragma unroll
+  for (int c = 0; c < NA; ++c) out[((kP0 + pl) * NA + c) * S] = ab[c];
+}
+
+struct PartLinksArgs {
+  StepArgs<double> s;
+  const double* part;
+  int z0;
+  int ring;
+  uint32_t sites;
+};
+
+template <int NC>
+__global__ void __launch_bounds__(kPartsThreads, 2) k_step_plaq_links(PartLinksArgs pa) {
+  constexpr int NA = Group<NC, double>::NA;
+  const uint32_t idx = blockIdx.x * kPartsThreads + threadIdx.x;
+  if (idx >= pa.sites) return;
+  const StepArgs<double>& a = pa.s;
+  const Geom& g = a.g;
+  const uint32_t nxy = (uint32_t)g.nxy, dz = idx / nxy, t = idx - dz * nxy;
+  const int z = pa.z0 + (int)dz, i = (int)blockIdx.y;
+  if (i == 2 && z == g.nz - 1) return;  // no z link on the last slice
+  const SiteNbr n = site_nbr_tz(g, t, z);
+  const int64_t S = (int64_t)pa.ring * nxy, here = (int64_t)(z % pa.ring) * nxy;
+  double F[NA];
+#pragma unroll
+  for (int c = 0; c < NA; ++c) F[c] = 0.0;
+#pragma unroll 1
+  for (int j = 0; j < 3; ++j) {
+    if (j == i) continue;
+    const int pl = i + j - 1;
+    const double w = a.w[j], sgn = i < j ? -w : w;
+    if (j != 2 || z < g.nz - 1) {
+      const double* p = pa.part + (int64_t)(kP0 + pl) * NA * S + here + t;
+#pragma unroll
+      for (int c = 0; c < NA; ++c) F[c] = fma(sgn, p[c * S], F[c]);
+    }
+    if (j != 2 || z > 0) {
+      const int64_t at = j == 2 ? (int64_t)((z - 1) % pa.ring) * nxy + t : here + (n.m[j] - (n.s - t));
+      const double* p = pa.part + (int64_t)((i < j ? kPBA : kPAB) + pl) * NA * S + at;
+#pragma unroll
+      for (int c = 0; c < NA; ++c) F[c] = fma(-sgn, p[c * S], F[c]);
+    }
+  }
+  update_link<NC, double>(a, i, t, z, n.s, F);
+}
+
+// Slices of the ring a context's scratch has, 0 if it takes none.
+int parts_ring(const glasma_ctx* c) {
+  if (c->rs != 8 || c->p.scheme != GLASMA_LEAPFROG) return 0;
+  const size_t slice = sizeof(double) * kPartVecs * (size_t)c->na * (size_t)c->g.nxy;
+  if (2 * slice > kPartsMost) return 0;
+  size_t r = kPartsBytes / slice;
+  if (r < 2) r = 2;
+  if (r > (size_t)(c->hi - c->lo) + 1) r = (size_t)(c->hi - c->lo) + 1;
+  return (int)r;
+}
+
+size_t parts_bytes(const glasma_ctx* c) {
+  return sizeof(double) * kPartVecs * (size_t)c->na * (size_t)c->g.nxy * (size_t)parts_ring(c);
+}
+
+template <int NC>
+static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
+  PartsArgs p;
+  p.U = (const double2*)c->U[c->cur];
+  p.part = c->part;
+  p.g = c->g;
+  PartLinksArgs l;
+  StepArgs<double>& a = l.s;
+  a.U = p.U;
+  a.Un = (double2*)c->U[1 - c->cur];
+  a.E = (double*)c->E;
+  a.QA = (double*)c->QA;
+  a.QB = (double*)c->QB;
+  a.g = c->g;
+  a.dt = c->p.dt;
+  a.w[0] = 2.0 / (c->p.a_t * c->p.a_t);
+  a.w[1] = a.w[0];
+  a.w[2] = 2.0 / (c->p.a_z * c->p.a_z);
+  a.az2 = c->p.a_z * c->p.a_z;
+  a.hop = hop ? 1 : 0;
+  a.zA0 = c->zA0;
+  a.WA = c->WA;
+  a.zB0 = c->zB0;
+  a.WB = c->WB;
+  a.zlo = c->lo;
+  l.part = c->part;
+  p.ring = l.ring = parts_ring(c);
+  if (zlen <= 0 || zlen > p.ring - 1) zlen = p.ring - 1;
+  for (int z0 = c->lo; z0 < c->hi; z0 += zlen) {
+    const int z1 = z0 + zlen < c->hi ? z0 + zlen : c->hi;
+    p.z0 = l.z0 = z0;
+    p.zfirst = z0 == c->lo && z0 > 0 ? z0 - 1 : z0;
+    p.sites = (uint32_t)((z1 - p.zfirst) * c->g.nxy);
+    l.sites = (uint32_t)((z1 - z0) * c->g.nxy);
+    k_step_plaq_parts<NC><<<dim3((p.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream>>>(p);
+    k_step_plaq_links<NC><<<dim3((l.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream>>>(l);
+    *launches += 2;
+  }
+  return cuda_check(cudaGetLastError(), "k_step_plaq_parts / _links launch");
+}
+
+// zlen: slices per chunk (0: as many as the scratch holds)
+int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches) {
+  return c->p.nc == 2 ? launch_parts_t<2>(c, hop, zlen, launches) : launch_parts_t<3>(c, hop, zlen, launches);
+}
+
+}  // namespace glasma

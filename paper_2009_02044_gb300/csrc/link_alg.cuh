@@ -15,6 +15,8 @@
 //   proj_prod(x, y), proj_prod_d(x, y)              Im tr t^a (x y), (x y^+)
 //                                                   of two stored-form links
 //   expi(v, c)                                      exp(i c v^a t^a)
+//   evolve(v, c, u)                                 exp(i c v^a t^a) u,
+//                                                   re-unitarised in FP32
 //   reunit, adj (U q U^+), adj_dag (U^+ q U)
 //
 // The FP32 forms are templates over the lane type T: float (one site per
@@ -68,6 +70,8 @@ struct LinkAlg<NC, double> : Group<NC, double> {
   GL_HD static M expi_series(const double* v, double c) { return G::expi(v, c); }
   typedef M Sum;
   GL_HD static M full(const M& u) { return u; }
+  GL_HD static M evolve(const double* v, double c, const M& u) { return G::evolve(v, c, u); }
+  GL_HD static M evolve_series(const double* v, double c, const M& u) { return G::evolve(v, c, u); }
   GL_HD static Sum zero_sum() { return G::zero(); }
   GL_HD static void sum_add(Sum& s, double w, const M& t) { G::scale_add(s, w, t); }
   GL_HD static void proj_mul_sum(const M& u, const Sum& s, double* out) { G::proj_mul(u, s, out); }
@@ -401,6 +405,9 @@ struct LinkAlgDev3 {
   // link is used).
   GL_HD static void adj(const M& u, R* q) { G::adj(full(u), q); }
   GL_HD static void adj_dag(const M& u, R* q) { G::adj_dag(full(u), q); }
+  // the re-unitarised exp(i c v^a t^a) u
+  GL_HD static M evolve(const R* v, R c, const M& u) { return reunit(mul(expi(v, c), u)); }
+  GL_HD static M evolve_series(const R* v, R c, const M& u) { return reunit(mul(expi_series(v, c), u)); }
 };
 
 template <>
@@ -478,6 +485,9 @@ struct LinkAlgDev2 {
   }
   GL_HD static void adj(const M& u, R* q) { G::adj(full(u), q); }
   GL_HD static void adj_dag(const M& u, R* q) { G::adj_dag(full(u), q); }
+  // the re-unitarised exp(i c v^a t^a) u
+  GL_HD static M evolve(const R* v, R c, const M& u) { return reunit(mul(expi(v, c), u)); }
+  GL_HD static M evolve_series(const R* v, R c, const M& u) { return reunit(mul(expi_series(v, c), u)); }
 };
 
 template <>

@@ -76,9 +76,7 @@ __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint
   }
 #pragma unroll
   for (int c = 0; c < NA; ++c) a.E[(int64_t)(i * NA + c) * a.g.V + s] = e[c];
-  M un = G::mul(G::expi(e, a.dt), Ui);
-  if (sizeof(R) == 4) un = G::reunit(un);
-  LinkIO<NC, R>::template store<R>(a.Un, i, a.g.V, s, un);
+  LinkIO<NC, R>::template store<R>(a.Un, i, a.g.V, s, G::evolve(e, a.dt, Ui));
 }
 
 template <int NC, typename R>

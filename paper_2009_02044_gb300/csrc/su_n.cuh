@@ -93,35 +93,70 @@ struct Group<2, R> {
     acc.b = acc.b + w * x.b;
   }
   GL_HD static M zero() { return M{{R(0), R(0)}, {R(0), R(0)}}; }
-  // exp(i c sum_a v^a sigma^a/2) = cos(th) + i sin(th) n.sigma, th = c|v|/2
-  GL_HD static M expi(const R* v, R c) {
-    R n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    if (n2 == R(0)) return ident();
-    R nrm = gl_sqrt(n2);
-    R s, co;
-    gl_sincos(R(0.5) * c * nrm, &s, &co);
-    R f = s / nrm;
+  // exp(i c sum_a v^a sigma^a/2) - 1 = (cos(th) - 1) + i sin(th) n.sigma,
+  // th = c|v|/2.  For th <= 1/2 (every link of a time step and most of the
+  // initial state) cos(th) - 1 and sin(th)/th are their Taylor series in
+  // th^2, to th^16/16! (remainder below 1e-21): 15 multiply-adds in place of
+  // a square root, a sine, a cosine and a division, several times as many
+  // operations on the narrow FP64 pipe that bounds the FP64 kernels.
+  GL_HD static M expi_m1(const R* v, R c) {
+    const R n2 = fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+    const R x = R(0.25) * c * c * n2;  // th^2
+    R co, f;                           // cos(th) - 1, sin(th) / |v|
+    if (x <= R(0.25)) {
+      co = R(1.0 / 20922789888000.0);
+      co = fma(co, -x, R(1.0 / 87178291200.0));
+      co = fma(co, -x, R(1.0 / 479001600.0));
+      co = fma(co, -x, R(1.0 / 3628800.0));
+      co = fma(co, -x, R(1.0 / 40320.0));
+      co = fma(co, -x, R(1.0 / 720.0));
+      co = fma(co, -x, R(1.0 / 24.0));
+      co = fma(co, -x, R(0.5));
+      co = -x * co;
+      f = R(1.0 / 355687428096000.0);
+      f = fma(f, -x, R(1.0 / 1307674368000.0));
+      f = fma(f, -x, R(1.0 / 6227020800.0));
+      f = fma(f, -x, R(1.0 / 39916800.0));
+      f = fma(f, -x, R(1.0 / 362880.0));
+      f = fma(f, -x, R(1.0 / 5040.0));
+      f = fma(f, -x, R(1.0 / 120.0));
+      f = fma(f, -x, R(1.0 / 6.0));
+      f = R(0.5) * c * fma(f, -x, R(1));
+    } else {
+      const R nrm = gl_sqrt(n2);
+      R s, sh, ch;
+      gl_sincos(R(0.25) * c * nrm, &sh, &ch);
+      s = R(2) * sh * ch;
+      co = R(-2) * sh * sh;
+      f = s / nrm;
+    }
     return M{{co, f * v[2]}, {f * v[1], f * v[0]}};
   }
-  // i * (q^a sigma^a / 2) in (alpha, beta) form
-  GL_HD static M alg_i(const R* q) {
-    return M{{R(0), R(0.5) * q[2]}, {R(0.5) * q[1], R(0.5) * q[0]}};
+  GL_HD static M expi(const R* v, R c) {
+    M e = expi_m1(v, c);
+    e.a.re += R(1);
+    return e;
   }
-  GL_HD static void from_alg_i(const M& x, R* q) {
-    q[0] = R(2) * x.b.im;
-    q[1] = R(2) * x.b.re;
-    q[2] = R(2) * x.a.im;
+  // exp(i c v.sigma/2) u
+  GL_HD static M evolve(const R* v, R c, const M& u) {
+    const M e = expi_m1(v, c);
+    return M{fma_c(e.a, u.a, fma_cj(-e.b, u.b, u.a)), fma_c(e.a, u.b, fma_cj(e.b, u.a, u.b))};
+  }
+  // U = w + i (x, y, z).sigma with alpha = w + i z, beta = y + i x rotates
+  // the algebra vector: with c = (x, y, z) x q,
+  // U q U^+ = q + 2 [(x, y, z) x c - w c], and U^+ q U has w -> -w: 18
+  // multiply-adds, where the two matrix products take 32.
+  GL_HD static void rotate(R w, const M& u, R* q) {
+    const R x = u.b.im, y = u.b.re, z = u.a.im;
+    const R c0 = fma(y, q[2], -(z * q[1])), c1 = fma(z, q[0], -(x * q[2])), c2 = fma(x, q[1], -(y * q[0]));
+    q[0] = fma(R(2), fma(y, c2, fma(-z, c1, -(w * c0))), q[0]);
+    q[1] = fma(R(2), fma(z, c0, fma(-x, c2, -(w * c1))), q[1]);
+    q[2] = fma(R(2), fma(x, c1, fma(-y, c0, -(w * c2))), q[2]);
   }
   // q <- U^dagger q U
-  GL_HD static void adj_dag(const M& u, R* q) {
-    M t = mul(d_mul(u, alg_i(q)), u);
-    from_alg_i(t, q);
-  }
+  GL_HD static void adj_dag(const M& u, R* q) { rotate(-u.a.re, u, q); }
   // q <- U q U^dagger
-  GL_HD static void adj(const M& u, R* q) {
-    M t = mul_d(mul(u, alg_i(q)), u);
-    from_alg_i(t, q);
-  }
+  GL_HD static void adj(const M& u, R* q) { rotate(u.a.re, u, q); }
   GL_HD static M reunit(const M& x) {
     R n2 = x.a.re * x.a.re + x.a.im * x.a.im + x.b.re * x.b.re + x.b.im * x.b.im;
     R f = R(1) / gl_sqrt(n2);
@@ -297,13 +332,170 @@ struct Group<3, R> {
     v[6] = h.m[7].im - h.m[5].im;
     v[7] = r3 * (h.m[0].re + h.m[4].re - R(2) * h.m[8].re);
   }
-  GL_HD static void adj_dag(const M& u, R* q) {
-    M t = mul(d_mul(u, herm(q)), u);
-    from_herm(t, q);
+  // q <- V q V^+ (V = U, or V = U^+ for DAG) through the hermitian matrix H
+  // of q: M = V H with H's real diagonal (10 multiply-adds per entry), then
+  // the upper triangle of the hermitian M V^+ (its trace is that of H, 0):
+  // 138 multiply-adds, where two full products take 216.
+  template <bool DAG>
+  GL_HD static void conj_alg(const M& u, R* q) {
+    const M h = herm(q);
+    cplx<R> m[9], v[9];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) v[3 * i + j] = DAG ? cj(u.m[3 * j + i]) : u.m[3 * i + j];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const cplx<R> d = v[3 * i + j];
+        cplx<R> acc{h.m[4 * j].re * d.re, h.m[4 * j].re * d.im};
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          if (k != j) acc = fma_c(v[3 * i + k], h.m[3 * k + j], acc);
+        m[3 * i + j] = acc;
+      }
+    cplx<R> t01{R(0), R(0)}, t02{R(0), R(0)}, t12{R(0), R(0)};
+    R t0 = R(0), t1 = R(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      t01 = fma_cj(m[k], v[3 + k], t01);
+      t02 = fma_cj(m[k], v[6 + k], t02);
+      t12 = fma_cj(m[3 + k], v[6 + k], t12);
+      t0 = fma(m[k].re, v[k].re, fma(m[k].im, v[k].im, t0));
+      t1 = fma(m[3 + k].re, v[3 + k].re, fma(m[3 + k].im, v[3 + k].im, t1));
+    }
+    q[0] = R(2) * t01.re;
+    q[1] = R(-2) * t01.im;
+    q[2] = t0 - t1;
+    q[3] = R(2) * t02.re;
+    q[4] = R(-2) * t02.im;
+    q[5] = R(2) * t12.re;
+    q[6] = R(-2) * t12.im;
+    q[7] = R(1.73205080756887729353) * (t0 + t1);  // (t0 + t1 - 2 t2) / sqrt 3, t2 = -t0 - t1
   }
-  GL_HD static void adj(const M& u, R* q) {
-    M t = mul_d(mul(u, herm(q)), u);
-    from_herm(t, q);
+  GL_HD static void adj_dag(const M& u, R* q) { conj_alg<true>(u, q); }
+  GL_HD static void adj(const M& u, R* q) { conj_alg<false>(u, q); }
+
+  // exp(i c v^a t^a) - 1 by Cayley-Hamilton for ||Q||_F <= 1/2, Q = c v^a t^a:
+  // Q^3 = c1 Q + c0 with c1 = tr(Q^2)/2 and c0 = det Q, so every power is
+  // Q^n = al_n + be_n Q + ga_n Q^2 with al_{n+1} = c0 ga_n, be_{n+1} = al_n +
+  // c1 ga_n, ga_{n+1} = be_n, and the series sum_{n>=1} (i^n/n!) Q^n = f0 + f1 Q
+  // + f2 Q^2 is summed to n = N: its remainder is below ||Q||^(N+1)/(N+1)!.
+  template <int N>
+  GL_HD static M expi_series_m1(const M& Q) {
+    R d2[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      R acc = Q.m[4 * i].re * Q.m[4 * i].re;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (k != i) acc = fma(Q.m[3 * i + k].re, Q.m[3 * i + k].re, fma(Q.m[3 * i + k].im, Q.m[3 * i + k].im, acc));
+      d2[i] = acc;
+    }
+    // the upper triangle of Q^2: Q_ik Q_kj, with the traceless diagonal
+    const cplx<R> q01 = fma_c(Q.m[2], Q.m[7], (-Q.m[8].re) * Q.m[1]);
+    const cplx<R> q02 = fma_c(Q.m[1], Q.m[5], (-Q.m[4].re) * Q.m[2]);
+    const cplx<R> q12 = fma_c(Q.m[3], Q.m[2], (-Q.m[0].re) * Q.m[5]);
+    const R c1 = R(0.5) * (d2[0] + d2[1] + d2[2]);
+    // det Q = q00 q11 q22 + 2 Re(Q01 Q12 Q20) - q00 |Q12|^2 - q11 |Q02|^2 - q22 |Q01|^2
+    const cplx<R> t = Q.m[1] * Q.m[5];
+    R c0 = Q.m[0].re * Q.m[4].re * Q.m[8].re;
+    c0 = fma(R(2) * t.re, Q.m[2].re, c0);
+    c0 = fma(R(2) * t.im, Q.m[2].im, c0);
+    c0 = fma(-Q.m[0].re, fma(Q.m[5].re, Q.m[5].re, Q.m[5].im * Q.m[5].im), c0);
+    c0 = fma(-Q.m[4].re, fma(Q.m[2].re, Q.m[2].re, Q.m[2].im * Q.m[2].im), c0);
+    c0 = fma(-Q.m[8].re, fma(Q.m[1].re, Q.m[1].re, Q.m[1].im * Q.m[1].im), c0);
+    R al = R(0), be = R(1), ga = R(0), k = R(1);
+    cplx<R> f0{R(0), R(0)}, f1{R(0), R(1)}, f2{R(0), R(0)};
+#pragma unroll
+    for (int n = 2; n <= N; ++n) {
+      const R nal = c0 * ga, nbe = fma(c1, ga, al);
+      ga = be;
+      al = nal;
+      be = nbe;
+      k = k / R(n);
+      const R sk = (n & 2) ? -k : k;  // i^n: n mod 4 = 0: +1, 1: +i, 2: -1, 3: -i
+      if ((n & 1) == 0) {
+        f0.re = fma(sk, al, f0.re);
+        f1.re = fma(sk, be, f1.re);
+        f2.re = fma(sk, ga, f2.re);
+      } else {
+        f0.im = fma(sk, al, f0.im);
+        f1.im = fma(sk, be, f1.im);
+        f2.im = fma(sk, ga, f2.im);
+      }
+    }
+    M e;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const R qd = Q.m[4 * i].re;
+      e.m[4 * i] = cplx<R>{fma(f2.re, d2[i], fma(f1.re, qd, f0.re)), fma(f2.im, d2[i], fma(f1.im, qd, f0.im))};
+    }
+    e.m[1] = fma_c(f2, q01, f1 * Q.m[1]);
+    e.m[2] = fma_c(f2, q02, f1 * Q.m[2]);
+    e.m[5] = fma_c(f2, q12, f1 * Q.m[5]);
+    e.m[3] = fma_c(f2, cj(q01), f1 * Q.m[3]);
+    e.m[6] = fma_c(f2, cj(q02), f1 * Q.m[6]);
+    e.m[7] = fma_c(f2, cj(q12), f1 * Q.m[7]);
+    return e;
+  }
+
+  // exp(i c v^a t^a) - 1.  ||Q||_F <= 1/16 (a time step's links, dt E ~ 0.05)
+  // takes 9 terms (remainder below 4e-19 ||Q||), ||Q||_F <= 1/2 takes 15
+  // (below 2e-18 ||Q||), about 170 and 200 multiply-adds; larger arguments
+  // take the eigenvalue form below, whose inverse cosine, square roots,
+  // divisions and four sine and cosine pairs are some 600 operations of the
+  // FP64 pipe.
+  GL_HD static M expi_m1(const R* v, R c) {
+    R cv[8];
+    R nn = R(0);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      cv[a] = c * v[a];
+      nn = fma(cv[a], cv[a], nn);
+    }
+    nn *= R(0.5);  // ||Q||_F^2
+    if (nn <= R(1.0 / 256.0)) return expi_series_m1<9>(herm(cv));
+    if (nn <= R(0.25)) return expi_series_m1<15>(herm(cv));
+    M e;
+    expi_eigen(cv, &e);
+    e.m[0].re -= R(1);
+    e.m[4].re -= R(1);
+    e.m[8].re -= R(1);
+    return e;
+  }
+  GL_HD static M expi(const R* v, R c) {
+    R nn = R(0);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) nn = fma(c * v[a], c * v[a], nn);
+    M e;
+    if (R(0.5) * nn <= R(0.25)) {
+      e = expi_m1(v, c);
+      e.m[0].re += R(1);
+      e.m[4].re += R(1);
+      e.m[8].re += R(1);
+      return e;
+    }
+    R cv[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) cv[a] = c * v[a];
+    expi_eigen(cv, &e);
+    return e;
+  }
+  // exp(i c v^a t^a) u
+  GL_HD static M evolve(const R* v, R c, const M& u) {
+    const M e = expi_m1(v, c);
+    M r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        cplx<R> acc = fma_c(e.m[3 * i], u.m[j], u.m[3 * i + j]);
+        acc = fma_c(e.m[3 * i + 1], u.m[3 + j], acc);
+        r.m[3 * i + j] = fma_c(e.m[3 * i + 2], u.m[6 + j], acc);
+      }
+    return r;
   }
 
   // exp(i c H) for H = sum v^a t^a by the Cayley-Hamilton form
@@ -312,28 +504,12 @@ struct Group<3, R> {
   // Phys. Rev. D 69 (2004) 054501, Sec. III: c0 = det Q, c1 = tr(Q^2)/2,
   // theta = acos(c0 / c0max), u = sqrt(c1/3) cos(theta/3),
   // w = sqrt(c1) sin(theta/3); negative c0 by f_j(-c0) = (-1)^j conj f_j(c0).
-  GL_HD static M expi(const R* v, R c) {
-    R cv[8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) cv[a] = c * v[a];
+  // cv = c v.  Not inlined: no link of a time step comes here, and its
+  // registers stay out of the step kernels.
+  static __host__ __device__ __noinline__ void expi_eigen(const R* cv, M* out) {
     M Q = herm(cv);
     M Q2 = mul(Q, Q);
     R c1 = R(0.5) * (Q2.m[0].re + Q2.m[4].re + Q2.m[8].re);
-    if (c1 == R(0)) return ident();
-    // Small arguments: the series 1 + iQ - Q^2/2 is exact to rounding (its
-    // truncation |Q|^3/6 is below the unit roundoff), and the eigenvalue
-    // parametrisation below would underflow (c0max = 2 (c1/3)^{3/2} -> 0).
-    const R small = sizeof(R) == 4 ? R(1e-8) : R(1e-20);
-    if (c1 < small) {
-      M r;
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        cplx<R> acc{-R(0.5) * Q2.m[k].re - Q.m[k].im, -R(0.5) * Q2.m[k].im + Q.m[k].re};
-        if (k % 4 == 0) acc.re += R(1);
-        r.m[k] = acc;
-      }
-      return r;
-    }
     // det of the hermitian Q (real)
     cplx<R> d = Q.m[0] * (Q.m[4] * Q.m[8] - Q.m[5] * Q.m[7]) -
                 Q.m[1] * (Q.m[3] * Q.m[8] - Q.m[5] * Q.m[6]) +
@@ -385,7 +561,7 @@ struct Group<3, R> {
       if (k % 4 == 0) acc = acc + f0;
       r.m[k] = acc;
     }
-    return r;
+    *out = r;
   }
 
   // Rows 0, 1 Gram-Schmidt normalised, row 2 = conj(row0 x row1).
