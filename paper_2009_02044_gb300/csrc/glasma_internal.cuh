@@ -138,6 +138,7 @@ int slab_halo_hop(glasma_ctx* c);
 int launch_tmunu(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab = nullptr);
 int run_init(glasma_ctx* c, const double* rho_host);
 int device_philox_rho(const glasma_params& p, int na, double* rho, cudaStream_t s);
+int64_t poisson_elems(const glasma_params& p, int F);  // complex values of each work array
 int device_poisson(const glasma_params& p, const double* in, double* out, int F, double2* w0, double2* w1,
                    cudaStream_t s);
 int device_profile(const glasma_params& p, double* lam, cudaStream_t s);

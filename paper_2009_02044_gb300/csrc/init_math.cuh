@@ -75,43 +75,59 @@ GL_HD void jacobi_herm3(cplx<double>* A, cplx<double>* V) {
 // the arcsine series of S instead, arcsin x = sum_k c_k x^(2k+1) with
 // c_k / c_(k-1) = (2k-1)^2 / (2k (2k+1)), summed until a term is below
 // 1e-18 |S|: the link changes of one time step at the initial state are
-// of this kind, and the series costs a few matrix products where the
-// Jacobi sweeps cost many.
+// of this kind.  By Cayley-Hamilton, S^3 = t S^2 - e S + d (t = tr S,
+// e = (t^2 - tr S^2) / 2, d = det S), every power is al + be S + ga S^2 with
+// three scalars, so a term costs 12 multiply-adds, not two matrix products.
 GL_HD bool log_su3(const Group<3, double>::M& W, double* h) {
-  cplx<double> S[9], C[9], Vm[9];
+  typedef Group<3, double> G;
+  G::M S;
   double sn2 = 0.0;
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
-      cplx<double> w = W.m[3 * i + j], wt = cj(W.m[3 * j + i]);
-      cplx<double> d = w - wt, s = w + wt;
-      S[3 * i + j] = cplx<double>{0.5 * d.im, -0.5 * d.re};  // d / (2i)
-      C[3 * i + j] = 0.5 * s;
-      sn2 += S[3 * i + j].re * S[3 * i + j].re + S[3 * i + j].im * S[3 * i + j].im;
+      const cplx<double> d = W.m[3 * i + j] - cj(W.m[3 * j + i]);
+      S.m[3 * i + j] = cplx<double>{0.5 * d.im, -0.5 * d.re};  // d / (2i)
+      sn2 = fma(S.m[3 * i + j].re, S.m[3 * i + j].re, fma(S.m[3 * i + j].im, S.m[3 * i + j].im, sn2));
     }
   if (sn2 < 0.0625) {
-    typedef Group<3, double> G;
-    G::M Sm, S2, T, H;
-    for (int m = 0; m < 9; ++m) Sm.m[m] = S[m];
-    S2 = G::mul(Sm, Sm);
-    T = Sm;
-    H = Sm;
-    const double stop = 1e-36 * sn2;
-    for (int k = 1; k < 40; ++k) {
-      const double r = (double)((2 * k - 1) * (2 * k - 1)) / (double)(2 * k * (2 * k + 1));
-      T = G::mul(T, S2);
-      double t2 = 0.0;
-      for (int m = 0; m < 9; ++m) {
-        T.m[m] = r * T.m[m];
-        H.m[m] = H.m[m] + T.m[m];
-        t2 += T.m[m].re * T.m[m].re + T.m[m].im * T.m[m].im;
+    const G::M S2 = G::mul(S, S);
+    const double t = S.m[0].re + S.m[4].re + S.m[8].re, e = 0.5 * fma(t, t, -sn2);
+    const cplx<double> q = S.m[1] * S.m[5];
+    double d = S.m[0].re * S.m[4].re * S.m[8].re;
+    d = fma(2.0, fma(q.re, S.m[2].re, q.im * S.m[2].im), d);
+    d = fma(-S.m[0].re, fma(S.m[5].re, S.m[5].re, S.m[5].im * S.m[5].im), d);
+    d = fma(-S.m[4].re, fma(S.m[2].re, S.m[2].re, S.m[2].im * S.m[2].im), d);
+    d = fma(-S.m[8].re, fma(S.m[1].re, S.m[1].re, S.m[1].im * S.m[1].im), d);
+    double al = 0.0, be = 1.0, ga = 0.0, fb = 1.0, fg = 0.0, ck = 1.0, x = 1.0;
+#pragma unroll
+    for (int k = 1; k < 15; ++k) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const double na = d * ga, nb = fma(-e, ga, al), ng = fma(t, ga, be);
+        al = na;
+        be = nb;
+        ga = ng;
       }
-      if (t2 <= stop) break;
+      ck = ck * (2 * k - 1) / (2 * k);
+      const double c = ck / (2 * k + 1);
+      fb = fma(c, be, fb);
+      fg = fma(c, ga, fg);
+      x *= sn2;
+      if (x * c < 1e-18) break;
     }
-    G::from_herm(H, h);
+    G::M H;
+#pragma unroll
+    for (int m = 0; m < 9; ++m)
+      H.m[m] = cplx<double>{fma(fb, S.m[m].re, fg * S2.m[m].re), fma(fb, S.m[m].im, fg * S2.m[m].im)};
+    G::from_herm(H, h);  // drops the part proportional to 1
     return true;
   }
+  cplx<double> C[9], Vm[9];
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) C[3 * i + j] = 0.5 * (W.m[3 * i + j] + cj(W.m[3 * j + i]));
   cplx<double> A[9];
-  for (int m = 0; m < 9; ++m) A[m] = S[m];
+  for (int m = 0; m < 9; ++m) A[m] = S.m[m];
   jacobi_herm3(A, Vm);
   double th[3];
   bool ok = true;
@@ -120,7 +136,7 @@ GL_HD bool log_su3(const Group<3, double>::M& W, double* h) {
     for (int i = 0; i < 3; ++i)
       for (int j = 0; j < 3; ++j) {
         cplx<double> vi = cj(Vm[3 * i + k]), vj = Vm[3 * j + k];
-        sv = sv + vi * S[3 * i + j] * vj;
+        sv = sv + vi * S.m[3 * i + j] * vj;
         cv = cv + vi * C[3 * i + j] * vj;
       }
     if (!(cv.re > 0.0)) ok = false;
@@ -138,15 +154,26 @@ GL_HD bool log_su3(const Group<3, double>::M& W, double* h) {
 }
 
 // SU(2): W = cos(phi) + i sin(phi) n.sigma, H = phi n.sigma, h^a = 2 phi n^a.
+// For sin^2(phi) < 1/64 and cos(phi) > 0, phi / sin(phi) is the arcsine series
+// (to the 11th power of sin^2: remainder below 1e-22).
 GL_HD bool log_su2(const Group<2, double>::M& W, double* h) {
-  double v[3] = {W.b.im, W.b.re, W.a.im};  // sin(phi) n
-  double sn = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-  if (sn == 0.0) {
-    h[0] = h[1] = h[2] = 0.0;
-    return W.a.re > 0.0;
+  const double v[3] = {W.b.im, W.b.re, W.a.im};  // sin(phi) n
+  const double x = fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+  double f;  // 2 phi / sin(phi)
+  if (x < 0.015625 && W.a.re > 0.0) {
+    f = 1.0;
+#pragma unroll
+    for (int k = 11; k >= 1; --k) f = fma(((2 * k - 1) * (2 * k - 1) / (double)(2 * k * (2 * k + 1))) * x, f, 1.0);
+    f *= 2.0;
+  } else {
+    const double sn = sqrt(x);
+    if (sn == 0.0) {
+      h[0] = h[1] = h[2] = 0.0;
+      return W.a.re > 0.0;
+    }
+    f = 2.0 * atan2(sn, W.a.re) / sn;
   }
-  double phi = atan2(sn, W.a.re);
-  for (int a = 0; a < 3; ++a) h[a] = 2.0 * phi * v[a] / sn;
+  for (int a = 0; a < 3; ++a) h[a] = f * v[a];
   return W.a.re > 0.0;
 }
 

@@ -322,8 +322,8 @@ int adjoint_run(glasma_ctx* c, const double* rho_host, int n_steps, double half_
   double* rho = sc.get<double>(F * nxy);
   double* phi = sc.get<double>(F * nxy);
   double* lam = sc.get<double>(4 * (size_t)g.nz);
-  double2* w0 = sc.get<double2>(F * nxy);
-  double2* w1 = sc.get<double2>(F * nxy);
+  double2* w0 = sc.get<double2>(poisson_elems(p, (int)F));
+  double2* w1 = sc.get<double2>(poisson_elems(p, (int)F));
   double* Umb = sc.get<double>(8 * (size_t)g.V);
   double* phib_z = sc.get<double>(F * (size_t)g.V);
   double* phib = sc.get<double>(F * nxy);

@@ -32,54 +32,91 @@ __global__ void k_philox_rho(double* rho, int na, int nx, int ny, int S, unsigne
   }
 }
 
-// One DFT pass along x (axis 0) or y (axis 1) of F complex [ny][nx] fields:
-// out_k = sum_m in_m exp(sign 2 pi i k m / n).
-__global__ void k_dft(const double2* in, double2* out, int F, int ny, int nx, int axis, int sign) {
-  const int64_t total = (int64_t)F * nx * ny;
-  const int n = axis == 0 ? nx : ny;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % nx);
-    int64_t r = i / nx;
-    const int y = (int)(r % ny);
-    const int64_t f = r / ny;
-    const int k = axis == 0 ? x : y;
+// The transverse Poisson solve phi = ifft(fft(rho) / (k^2 + m^2)) of F real
+// [ny][nx] fields by separable DFTs.  The fields are real and the kernel even,
+// so only the columns kx = 0..nx/2 are transformed, the first pass takes real
+// input and the last gives real output: (1 + 2 + 2 + 1) n multiply-adds per
+// site where four full complex passes take 16 n.  The factors exp(2 pi i j / n)
+// come from a table: evaluating sincospi in the inner loop cost 30 times as
+// much (0.45 ms per pass of the SU(3) 64^2 fields, 1.29 ms of the SU(2) 128^2
+// ones).
+__global__ void k_twiddle(double2* tw, int nx, int ny) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nx + ny; i += gridDim.x * blockDim.x) {
+    const int n = i < nx ? nx : ny, j = i < nx ? i : i - nx;
+    double s, c;
+    sincospi(2.0 * (double)j / (double)n, &s, &c);
+    tw[i] = make_double2(c, s);
+  }
+}
+
+// out[f][y][kx] = sum_x in[f][y][x] exp(-2 pi i kx x / nx), kx < nh
+__global__ void k_dft_x(const double* in, double2* out, const double2* tw, int64_t rows, int nx, int nh) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows * nh; i += (int64_t)gridDim.x * blockDim.x) {
+    const int k = (int)(i % nh);
+    const double* row = in + (i / nh) * nx;
     double re = 0.0, im = 0.0;
-    for (int m = 0; m < n; ++m) {
-      const int64_t src = axis == 0 ? (f * ny + y) * nx + m : (f * ny + m) * nx + x;
-      const double2 v = in[src];
-      const int km = (int)(((int64_t)k * m) % n);
-      double s, c;
-      sincospi(2.0 * (double)km / (double)n, &s, &c);
-      s *= sign;
-      re += v.x * c - v.y * s;
-      im += v.x * s + v.y * c;
+    for (int m = 0, km = 0; m < nx; ++m) {
+      const double v = row[m];
+      const double2 w = tw[km];
+      re = fma(v, w.x, re);
+      im = fma(-v, w.y, im);
+      km += k;
+      if (km >= nx) km -= nx;
     }
     out[i] = make_double2(re, im);
   }
 }
 
-__global__ void k_real_to_cplx(const double* in, double2* out, int64_t total) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = make_double2(in[i], 0.0);
-}
-
-// multiply by 1 / (k^2 + m^2), k^2 = 4/a^2 [sin^2(pi kx/nx) + sin^2(pi ky/ny)]
-__global__ void k_poisson_kernel(double2* f, int F, int ny, int nx, double a_t, double m2, double uv2) {
-  const int64_t total = (int64_t)F * nx * ny;
+// out[f][k][kx] = sum_y in[f][y][kx] exp(sign 2 pi i k y / ny), times the
+// Poisson kernel 1 / (k^2 + m^2), k^2 = 4/a^2 [sin^2(pi kx/nx) + sin^2(pi ky/ny)]
+// in the forward pass (sign = -1)
+__global__ void k_dft_y(const double2* in, double2* out, const double2* tw, int F, int ny, int nx, int nh, int sign,
+                        double a_t, double m2, double uv2) {
+  const int64_t total = (int64_t)F * ny * nh;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int kx = (int)(i % nx);
-    const int ky = (int)((i / nx) % ny);
-    const double sx = sinpi((double)kx / nx), sy = sinpi((double)ky / ny);
-    const double k2 = 4.0 / (a_t * a_t) * (sy * sy) + 4.0 / (a_t * a_t) * (sx * sx);
-    double kern = 1.0 / (k2 + m2);
-    if (uv2 > 0.0 && k2 > uv2) kern = 0.0;
-    f[i] = make_double2(f[i].x * kern, f[i].y * kern);
+    const int kx = (int)(i % nh);
+    const int64_t r = i / nh;
+    const int k = (int)(r % ny);
+    const double2* col = in + (r / ny) * ny * nh + kx;
+    double re = 0.0, im = 0.0;
+    for (int m = 0, km = 0; m < ny; ++m) {
+      const double2 v = col[(int64_t)m * nh], w = tw[km];
+      const double s = sign * w.y;
+      re = fma(v.x, w.x, fma(-v.y, s, re));
+      im = fma(v.x, s, fma(v.y, w.x, im));
+      km += k;
+      if (km >= ny) km -= ny;
+    }
+    if (sign < 0) {
+      const double sx = sinpi((double)kx / nx), sy = sinpi((double)k / ny);
+      const double k2 = 4.0 / (a_t * a_t) * (sy * sy) + 4.0 / (a_t * a_t) * (sx * sx);
+      double kern = 1.0 / (k2 + m2);
+      if (uv2 > 0.0 && k2 > uv2) kern = 0.0;
+      re *= kern;
+      im *= kern;
+    }
+    out[i] = make_double2(re, im);
   }
 }
 
-__global__ void k_cplx_real_scaled(const double2* in, double* out, int64_t total, double scale) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = in[i].x * scale;
+// out[f][y][x] = scale Re sum_kx in[f][y][kx] exp(2 pi i kx x / nx) over all
+// nx columns, those above nx/2 the conjugates of the kept ones
+__global__ void k_dft_x_real(const double2* in, double* out, const double2* tw, int64_t rows, int nx, int nh,
+                             double scale) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows * nx; i += (int64_t)gridDim.x * blockDim.x) {
+    const int x = (int)(i % nx);
+    const double2* row = in + (i / nx) * nh;
+    double acc = 0.0;
+    for (int k = 1, kx = x; 2 * k < nx; ++k) {
+      const double2 v = row[k], w = tw[kx];
+      acc = fma(v.x, w.x, fma(-v.y, w.y, acc));
+      kx += x;
+      if (kx >= nx) kx -= nx;
+    }
+    acc = fma(2.0, acc, row[0].x);
+    if (nx % 2 == 0) acc += (x & 1) ? -row[nx / 2].x : row[nx / 2].x;
+    out[i] = acc * scale;
+  }
 }
 
 // lam[(t*2 + N)*nz + iz], t = 0: t0, 1: t0 - dt; N = 0: A, 1: B
@@ -113,28 +150,20 @@ __global__ void k_profile(double* lam, int nz, int zoff, double a_z, double sigm
 // path-ordered exp(i L_{S-1} phi_{S-1,N}) ... exp(i L_0 phi_{0,N}) with
 // L_s = clip(S lam - s, 0, 1), sheet 0 (the leading slab) acting first.
 template <int NC>
-GL_HD typename Group<NC, double>::M wilson_dag(const double* phi, int N, int na, int64_t nxy, int64_t t, double lam,
-                                               int S = 1, const typename Group<NC, double>::M* full = nullptr) {
+GL_HD typename Group<NC, double>::M wilson_dag(const double* phi, int N, int64_t nxy, int64_t t, double lam, int S) {
   typedef Group<NC, double> G;
   double v[G::NA];
-  if (S <= 1) {
-    if (lam == 0.0) return G::ident();
-    if (lam == 1.0 && full) return full[(int64_t)N * nxy + t];  // behind the nucleus: exp(i phi), tabulated
-    for (int a = 0; a < G::NA; ++a) v[a] = phi[((int64_t)N * na + a) * nxy + t];
-    return G::expi(v, lam);
-  }
   typename G::M m = G::ident();
   bool first = true;
   for (int s = 0; s < S; ++s) {
-    double ls = (double)S * lam - (double)s;
-    ls = ls < 0.0 ? 0.0 : (ls > 1.0 ? 1.0 : ls);
-    typename G::M f;
-    if (ls == 0.0) {
-      f = G::ident();
-    } else {
-      for (int a = 0; a < G::NA; ++a) v[a] = phi[((int64_t)(s * 2 + N) * na + a) * nxy + t];
-      f = G::expi(v, ls);
+    double ls = lam;
+    if (S > 1) {
+      ls = (double)S * lam - (double)s;
+      ls = ls < 0.0 ? 0.0 : (ls > 1.0 ? 1.0 : ls);
     }
+    if (ls == 0.0) continue;
+    for (int a = 0; a < G::NA; ++a) v[a] = phi[((int64_t)(s * 2 + N) * G::NA + a) * nxy + t];
+    const typename G::M f = G::expi(v, ls);
     m = first ? f : G::mul(f, m);
     first = false;
   }
@@ -157,84 +186,116 @@ GL_HD bool same(const typename Group<NC, double>::M& a, const typename Group<NC,
   return true;
 }
 
-// exp(i phi_N(x_T)) for every transverse site, the Wilson line of all the
-// slices a single-sheet nucleus has fully passed (Lambda = 1), computed once.
+// Behind a nucleus (Lambda = 1) the Wilson line and with it the links depend
+// on the transverse site alone: full[N][t] = V_N^dag(x_T), then
+// tail[N][i][t] = V_N(x) V_N^dag(x+i), formed once and copied to all slices.
 template <int NC>
-__global__ void k_wilson_full(const double* phi, typename Group<NC, double>::M* full, int64_t nxy) {
-  typedef Group<NC, double> G;
+__global__ void k_wilson_full(const double* phi, typename Group<NC, double>::M* full, int64_t nxy, int S) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * nxy; i += (int64_t)gridDim.x * blockDim.x) {
     const int N = (int)(i / nxy);
-    const int64_t t = i - (int64_t)N * nxy;
-    double v[G::NA];
-    for (int a = 0; a < G::NA; ++a) v[a] = phi[((int64_t)N * G::NA + a) * nxy + t];
-    full[i] = G::expi(v, 1.0);
+    full[i] = wilson_dag<NC>(phi, N, nxy, i - (int64_t)N * nxy, 1.0, S);
   }
 }
 
+template <int NC>
+__global__ void k_tail_links(const typename Group<NC, double>::M* full, typename Group<NC, double>::M* tail, Geom g) {
+  const int64_t nxy = g.nxy;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 4 * nxy; i += (int64_t)gridDim.x * blockDim.x) {
+    const int N = (int)(i / (2 * nxy)), d = (int)(i / nxy) & 1;
+    const uint32_t t = (uint32_t)(i % nxy);
+    const SiteNbr n = site_nbr_tz(g, t, 0);
+    tail[i] = Group<NC, double>::d_mul(full[N * nxy + t], full[N * nxy + n.p[d]]);
+  }
+}
+
+// Links at t0 (and at t0 - dt where asked for) and E of one slice and one tile
+// of kTileX x kTileY transverse sites.  The two profiles are disjoint (the
+// centres lie more than 4 sigma from the box centre), so at most one nucleus
+// has Lambda > 0 on a slice.  A slice ahead of both has unit links; a slice
+// whose Lambda is 1 at both times copies the tail links; both have E = 0.  On
+// the slices in between the Wilson lines of the tile and of its +x and +y
+// neighbours at both times are formed once each in shared memory (2.4
+// exponentials per site instead of the 6 that a thread by itself takes).
+// FP64-pipe bound there, bound by the stores elsewhere.  The whole initial
+// state, with the DFTs, the series logarithm and the split divergence: SU(3)
+// 512 x 64^2, sigma_L = 4, 7.5 -> 3.0 ms, SU(2) 1024 x 128^2 13.5 -> 6.1 ms.
+// U1, the buffer the first step writes, only needs the absent z links of the
+// last slice (all of it on a slab, whose halo slices are not stepped).
+constexpr int kTileX = 16, kTileY = 8;
+
 template <int NC, typename R>
-__global__ void k_init_links(const double* phi, const double* lam, typename V2T<R>::T* U0,
-                             typename V2T<R>::T* U1, typename V2T<R>::T* Uprev, R* E, Geom g, double dt,
-                             int* flag, int S, const typename Group<NC, double>::M* full) {
+__global__ void __launch_bounds__(kTileX * kTileY) k_init_links(
+    const double* phi, const double* lam, const typename Group<NC, double>::M* full,
+    const typename Group<NC, double>::M* tail, typename V2T<R>::T* U0, typename V2T<R>::T* U1,
+    typename V2T<R>::T* Uprev, R* E, Geom g, double dt, int* flag, int S, int whole) {
   typedef Group<NC, double> G;
   typedef typename G::M M;
-  constexpr int NA = G::NA;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < g.V; s += (int64_t)gridDim.x * blockDim.x) {
-    SiteNbr n = site_nbr(g, s);
-    const int64_t t0 = s % g.nxy;
-    const int64_t tx = n.p[0] % g.nxy, ty = n.p[1] % g.nxy;
-    M u[2][2];  // [time][direction]
-    // A nucleus whose Lambda is 0 on this slice (ahead of it) contributes
-    // the identity, and a slice whose Lambdas are the same at t0 and
-    // t0 - dt has the same links at both times (E = 0 there).  Before the
-    // collision at most one nucleus has Lambda > 0 on a slice, so most
-    // slices need one product per link.
-    const double lt[2][2] = {{lam[0 * g.nz + n.iz], lam[1 * g.nz + n.iz]},
-                             {lam[2 * g.nz + n.iz], lam[3 * g.nz + n.iz]}};
-    const bool moving = lt[0][0] != lt[1][0] || lt[0][1] != lt[1][1];
-    for (int t = 0; t < (moving ? 2 : 1); ++t) {
-      const double la = lt[t][0], lb = lt[t][1];
-      const bool ha = la != 0.0, hb = lb != 0.0;
-      M vda = G::ident(), vdb = G::ident();
-      if (ha) vda = wilson_dag<NC>(phi, 0, NA, g.nxy, t0, la, S, full);
-      if (hb) vdb = wilson_dag<NC>(phi, 1, NA, g.nxy, t0, lb, S, full);
-      for (int i = 0; i < 2; ++i) {
-        const int64_t tn = i == 0 ? tx : ty;
-        M m = G::ident();
-        if (ha) m = G::d_mul(vda, wilson_dag<NC>(phi, 0, NA, g.nxy, tn, la, S, full));  // V_A(x) V_A^dag(x+i)
-        if (hb) {
-          const M ub = G::d_mul(vdb, wilson_dag<NC>(phi, 1, NA, g.nxy, tn, lb, S, full));
-          m = ha ? G::mul(m, ub) : ub;
-        }
-        u[t][i] = m;
-      }
+  typedef LinkIO<NC, R> IO;
+  constexpr int NA = G::NA, PX = kTileX + 1, PN = PX * (kTileY + 1);
+  __shared__ __align__(16) unsigned char raw[2 * PN * sizeof(M)];
+  M* v = (M*)raw;  // [time][tile site]
+  const int iz = blockIdx.y;
+  const int ntx = (g.nx + kTileX - 1) / kTileX;
+  const int x0 = ((int)blockIdx.x % ntx) * kTileX, y0 = ((int)blockIdx.x / ntx) * kTileY;
+  const int lx = threadIdx.x % kTileX, ly = threadIdx.x / kTileX;
+  const int ix = x0 + lx, iy = y0 + ly;
+  const bool inside = ix < g.nx && iy < g.ny;
+  const int64_t t = (int64_t)iy * g.nx + ix, s = (int64_t)iz * g.nxy + t;
+  const bool copy1 = !whole || iz == g.nz - 1;
+  const int N = lam[0 * g.nz + iz] != 0.0 || lam[2 * g.nz + iz] != 0.0 ? 0 : 1;
+  const double l0 = lam[N * g.nz + iz], l1 = lam[(2 + N) * g.nz + iz];
+  const bool moving = l0 != l1;
+  if (moving) {
+    for (int q = threadIdx.x; q < 2 * PN; q += kTileX * kTileY) {
+      const int tm = q / PN, p = q - tm * PN;
+      const int64_t tt = (int64_t)((y0 + p / PX) % g.ny) * g.nx + (x0 + p % PX) % g.nx;
+      const double l = tm ? l1 : l0;
+      v[q] = l == 1.0 ? full[N * g.nxy + tt] : wilson_dag<NC>(phi, N, g.nxy, tt, l, S);
     }
-    if (!moving) {
-      u[1][0] = u[0][0];
-      u[1][1] = u[0][1];
-    }
-    for (int i = 0; i < 2; ++i) {
-      double h[NA];
-      if (same<NC>(u[0][i], u[1][i])) {
-        for (int a = 0; a < NA; ++a) h[a] = 0.0;
-      } else {
-        M w = G::mul_d(u[0][i], u[1][i]);
-        if (!group_log<NC>(w, h)) atomicOr(flag, 1);
-      }
-      for (int a = 0; a < NA; ++a) E[(int64_t)(i * NA + a) * g.V + s] = (R)(h[a] / dt);
-      LinkIO<NC, R>::template store<double>(U0, i, g.V, s, u[0][i]);
-      LinkIO<NC, R>::template store<double>(U1, i, g.V, s, u[0][i]);
-      if (Uprev) LinkIO<NC, R>::template store<double>(Uprev, i, g.V, s, u[1][i]);
-    }
-    for (int a = 0; a < NA; ++a) E[(int64_t)(2 * NA + a) * g.V + s] = (R)0;
-    M one = G::ident();
-    LinkIO<NC, R>::template store<double>(U0, 2, g.V, s, one);
-    LinkIO<NC, R>::template store<double>(U1, 2, g.V, s, one);
-    if (Uprev) LinkIO<NC, R>::template store<double>(Uprev, 2, g.V, s, one);
+    __syncthreads();
   }
+  if (!inside) return;
+  const M one = G::ident();
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    M u0 = one, u1 = one;
+    double h[NA];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) h[a] = 0.0;
+    if (moving) {
+      const int p = ly * PX + lx, pn = p + (i == 0 ? 1 : PX);
+      u0 = G::d_mul(v[p], v[pn]);
+      u1 = G::d_mul(v[PN + p], v[PN + pn]);
+      if (!same<NC>(u0, u1) && !group_log<NC>(G::mul_d(u0, u1), h)) atomicOr(flag, 1);
+    } else if (l0 != 0.0) {
+      u0 = l0 == 1.0 ? tail[(N * 2 + i) * g.nxy + t]
+                     : G::d_mul(wilson_dag<NC>(phi, N, g.nxy, t, l0, S),
+                                wilson_dag<NC>(phi, N, g.nxy,
+                                               i == 0 ? t - ix + (ix + 1) % g.nx
+                                                      : (int64_t)((iy + 1) % g.ny) * g.nx + ix, l0, S));
+      u1 = u0;
+    }
+#pragma unroll
+    for (int a = 0; a < NA; ++a) E[(int64_t)(i * NA + a) * g.V + s] = (R)(h[a] / dt);
+    IO::template store<double>(U0, i, g.V, s, u0);
+    if (copy1) IO::template store<double>(U1, i, g.V, s, u0);
+    if (Uprev) IO::template store<double>(Uprev, i, g.V, s, u1);
+  }
+#pragma unroll
+  for (int a = 0; a < NA; ++a) E[(int64_t)(2 * NA + a) * g.V + s] = (R)0;
+  IO::template store<double>(U0, 2, g.V, s, one);
+  if (copy1) IO::template store<double>(U1, 2, g.V, s, one);
+  if (Uprev) IO::template store<double>(Uprev, 2, g.V, s, one);
 }
 
 // rho(x) = sum_i [E_i(x) - U_i^dag(x-i) E_i(x-i) U_i(x-i)] / a_i^2 of the
-// stored state, in FP64; one block per z slice also records max |rho|.
+// stored state, in FP64, and max |rho| of every slice (slice_max begins as
+// zeros; the bits of non-negative doubles order as the doubles do).  Only the
+// slices inside the nuclei have fields, so kDivSplit blocks share a slice: with
+// one block each, those slices' FP64 work lay on 130 of 152 SMs, 8 warps each
+// (SU(3) 512 x 64^2: 1.38 ms).
+constexpr int kDivSplit = 8;
+
 template <int NC, typename R>
 __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U, const R* E, Geom g, double ia2t,
                                                     double ia2z, double* rho3, double* slice_max) {
@@ -243,9 +304,9 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
   __shared__ double sh[256];
   const int iz = blockIdx.x;
   double mx = 0.0;
-  for (int t = threadIdx.x; t < g.nxy; t += blockDim.x) {
+  for (uint32_t t = blockIdx.y * blockDim.x + threadIdx.x; t < g.nxy; t += gridDim.y * blockDim.x) {
     const int64_t s = (int64_t)iz * g.nxy + t;
-    SiteNbr n = site_nbr(g, s);
+    const SiteNbr n = site_nbr_tz(g, t, iz);
     double dv[NA];
     for (int c = 0; c < NA; ++c) dv[c] = 0.0;
     for (int i = 0; i < 3; ++i) {
@@ -274,7 +335,8 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
     if ((int)threadIdx.x < w) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) slice_max[iz] = sh[0];
+  if (threadIdx.x == 0)
+    atomicMax((unsigned long long*)&slice_max[iz], (unsigned long long)__double_as_longlong(sh[0]));
 }
 
 template <typename R>
@@ -304,14 +366,18 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
   const int S = p.n_sheets > 1 ? p.n_sheets : 1;
   const int F = 2 * S * na;
   int st;
-  // scratch: rho/phi (real), two complex work arrays, lambda table, rho3, slice max, flag
+  // scratch: rho/phi (real), two complex work arrays and the DFT factors,
+  // lambda table, Wilson lines and links behind the nuclei, rho3, slice max
   double* rho = (double*)ctx_alloc(c, sizeof(double) * F * nxy);
-  double2* w0 = (double2*)ctx_alloc(c, sizeof(double2) * F * nxy);
-  double2* w1 = (double2*)ctx_alloc(c, sizeof(double2) * F * nxy);
+  double2* w0 = (double2*)ctx_alloc(c, sizeof(double2) * poisson_elems(p, F));
+  double2* w1 = (double2*)ctx_alloc(c, sizeof(double2) * poisson_elems(p, F));
   double* lam = (double*)ctx_alloc(c, sizeof(double) * 4 * p.nz);
   double* rho3 = (double*)ctx_alloc(c, sizeof(double) * na * V);
   double* smax = (double*)ctx_alloc(c, sizeof(double) * p.nz);
-  if (!rho || !w0 || !w1 || !lam || !rho3 || !smax) return set_error(GLASMA_ERR_OOM, "init scratch allocation failed");
+  typedef typename Group<NC, double>::M MD;
+  MD* full = (MD*)ctx_alloc(c, sizeof(MD) * 2 * nxy);
+  MD* tail = (MD*)ctx_alloc(c, sizeof(MD) * 4 * nxy);
+  if (!rho || !w0 || !w1 || !lam || !rho3 || !smax || !full || !tail) return set_error(GLASMA_ERR_OOM, "init scratch allocation failed");
   if (rho_host) {
     st = cuda_check(cudaMemcpyAsync(rho, rho_host, sizeof(double) * F * nxy, cudaMemcpyHostToDevice, c->stream),
                     "rho upload");
@@ -320,33 +386,25 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
     k_philox_rho<<<grid_for(F * nxy), 256, 0, c->stream>>>(rho, na, p.nx, p.ny, S, p.seed,
                                                             S > 1 ? p.g2mu / sqrt((double)S) : p.g2mu);
   }
-  // Poisson: forward DFT x, y; kernel; inverse y, x; real part / (nx ny)
-  k_real_to_cplx<<<grid_for(F * nxy), 256, 0, c->stream>>>(rho, w0, F * nxy);
-  k_dft<<<grid_for(F * nxy), 256, 0, c->stream>>>(w0, w1, F, p.ny, p.nx, 0, -1);
-  k_dft<<<grid_for(F * nxy), 256, 0, c->stream>>>(w1, w0, F, p.ny, p.nx, 1, -1);
-  k_poisson_kernel<<<grid_for(F * nxy), 256, 0, c->stream>>>(w0, F, p.ny, p.nx, p.a_t, p.m_ir * p.m_ir,
-                                                               p.uv_cutoff > 0 ? p.uv_cutoff * p.uv_cutoff : 0.0);
-  k_dft<<<grid_for(F * nxy), 256, 0, c->stream>>>(w0, w1, F, p.ny, p.nx, 1, +1);
-  k_dft<<<grid_for(F * nxy), 256, 0, c->stream>>>(w1, w0, F, p.ny, p.nx, 0, +1);
-  k_cplx_real_scaled<<<grid_for(F * nxy), 256, 0, c->stream>>>(w0, rho, F * nxy, 1.0 / (double)nxy);  // rho <- phi
+  st = device_poisson(p, rho, rho, F, w0, w1, c->stream);  // rho <- phi
+  if (st) return st;
   // nucleus centres at t0 (box centre +- d) in global z (a slab's local
   // slice 0 is global slice zoff)
   const double zc = c->nz_glob * p.a_z / 2.0;
   const double d = p.z_offset > 0 ? p.z_offset : (ceil(4.0 * p.sigma_l / p.a_z) + 2.0) * p.a_z;
   k_profile<<<grid_for(4 * p.nz), 256, 0, c->stream>>>(lam, p.nz, c->zoff, p.a_z, p.sigma_l, zc + d, zc - d, p.dt);
   cudaMemsetAsync(c->dflag, 0, sizeof(int) * 8, c->stream);
-  typedef typename Group<NC, double>::M MD;
-  MD* full = nullptr;
-  if (S <= 1) {
-    full = (MD*)ctx_alloc(c, sizeof(MD) * 2 * nxy);
-    if (!full) return set_error(GLASMA_ERR_OOM, "init scratch allocation failed");
-    k_wilson_full<NC><<<grid_for(2 * nxy), 256, 0, c->stream>>>(rho, full, nxy);
-  }
-  k_init_links<NC, R><<<grid_for(V, 128), 128, 0, c->stream>>>(
-      rho, lam, (typename V2T<R>::T*)c->U[0], (typename V2T<R>::T*)c->U[1], (typename V2T<R>::T*)c->Uprev,
-      (R*)c->E, c->g, p.dt, c->dflag, S, full);
-  k_divergence<NC, R><<<p.nz, 256, 0, c->stream>>>((const typename V2T<R>::T*)c->U[0], (const R*)c->E, c->g,
-                                                  1.0 / (p.a_t * p.a_t), 1.0 / (p.a_z * p.a_z), rho3, smax);
+  cudaMemsetAsync(smax, 0, sizeof(double) * p.nz, c->stream);
+  k_wilson_full<NC><<<grid_for(2 * nxy, 64), 64, 0, c->stream>>>(rho, full, nxy, S);
+  k_tail_links<NC><<<grid_for(4 * nxy, 64), 64, 0, c->stream>>>(full, tail, c->g);
+  const unsigned tiles = (unsigned)(((p.nx + kTileX - 1) / kTileX) * ((p.ny + kTileY - 1) / kTileY));
+  k_init_links<NC, R><<<dim3(tiles, (unsigned)p.nz), kTileX * kTileY, 0, c->stream>>>(
+      rho, lam, full, tail, (typename V2T<R>::T*)c->U[0], (typename V2T<R>::T*)c->U[1],
+      (typename V2T<R>::T*)c->Uprev, (R*)c->E, c->g, p.dt, c->dflag, S, c->slab ? 0 : 1);
+  const int64_t per_slice = (nxy + 255) / 256;
+  k_divergence<NC, R><<<dim3(p.nz, (unsigned)(per_slice < kDivSplit ? per_slice : kDivSplit)), 256, 0, c->stream>>>(
+      (const typename V2T<R>::T*)c->U[0], (const R*)c->E, c->g, 1.0 / (p.a_t * p.a_t), 1.0 / (p.a_z * p.a_z), rho3,
+      smax);
   st = cuda_check(cudaGetLastError(), "init kernels");
   if (st) return st;
   std::vector<double> hmax(p.nz);
@@ -402,6 +460,7 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
     c->uprev_valid = true;
   }
   st = cuda_check(cudaStreamSynchronize(c->stream), "init sync 2");
+  ctx_free(c, tail);
   ctx_free(c, full);
   ctx_free(c, rho);
   ctx_free(c, w0);
@@ -414,24 +473,28 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
 
 // Device helpers shared with the adjoint: the MV draw, the transverse
 // Poisson solve of F real [ny][nx] fields (in and out may alias; w0, w1 hold
-// F*nx*ny complex values each) and the profile table lam[(t*2 + N)*nz + iz].
+// poisson_elems complex values each) and the profile table lam[(t*2 + N)*nz + iz].
 int device_philox_rho(const glasma_params& p, int na, double* rho, cudaStream_t s) {
   const int64_t n = (int64_t)2 * na * p.nx * p.ny;
   k_philox_rho<<<grid_for(n), 256, 0, s>>>(rho, na, p.nx, p.ny, 1, p.seed, p.g2mu);
   return cuda_check(cudaGetLastError(), "philox rho");
 }
 
+int64_t poisson_elems(const glasma_params& p, int F) {
+  return (int64_t)F * p.ny * (p.nx / 2 + 1) + p.nx + p.ny;
+}
+
 int device_poisson(const glasma_params& p, const double* in, double* out, int F, double2* w0, double2* w1,
                    cudaStream_t s) {
-  const int64_t nxy = (int64_t)p.nx * p.ny, n = F * nxy;
-  k_real_to_cplx<<<grid_for(n), 256, 0, s>>>(in, w0, n);
-  k_dft<<<grid_for(n), 256, 0, s>>>(w0, w1, F, p.ny, p.nx, 0, -1);
-  k_dft<<<grid_for(n), 256, 0, s>>>(w1, w0, F, p.ny, p.nx, 1, -1);
-  k_poisson_kernel<<<grid_for(n), 256, 0, s>>>(w0, F, p.ny, p.nx, p.a_t, p.m_ir * p.m_ir,
-                                                p.uv_cutoff > 0 ? p.uv_cutoff * p.uv_cutoff : 0.0);
-  k_dft<<<grid_for(n), 256, 0, s>>>(w0, w1, F, p.ny, p.nx, 1, +1);
-  k_dft<<<grid_for(n), 256, 0, s>>>(w1, w0, F, p.ny, p.nx, 0, +1);
-  k_cplx_real_scaled<<<grid_for(n), 256, 0, s>>>(w0, out, n, 1.0 / (double)nxy);
+  const int nx = p.nx, ny = p.ny, nh = nx / 2 + 1;
+  const int64_t rows = (int64_t)F * ny, nk = rows * nh, n = rows * nx;
+  double2* tw = w1 + nk;  // the factors of x, then of y
+  const double m2 = p.m_ir * p.m_ir, uv2 = p.uv_cutoff > 0 ? p.uv_cutoff * p.uv_cutoff : 0.0;
+  k_twiddle<<<grid_for(nx + ny, 128), 128, 0, s>>>(tw, nx, ny);
+  k_dft_x<<<grid_for(nk, 64), 64, 0, s>>>(in, w0, tw, rows, nx, nh);
+  k_dft_y<<<grid_for(nk, 64), 64, 0, s>>>(w0, w1, tw + nx, F, ny, nx, nh, -1, p.a_t, m2, uv2);
+  k_dft_y<<<grid_for(nk, 64), 64, 0, s>>>(w1, w0, tw + nx, F, ny, nx, nh, +1, p.a_t, m2, uv2);
+  k_dft_x_real<<<grid_for(n, 64), 64, 0, s>>>(w0, out, tw, rows, nx, nh, 1.0 / ((double)nx * ny));
   return cuda_check(cudaGetLastError(), "poisson");
 }
 
