@@ -250,9 +250,8 @@ static int create_ctx(const glasma_params* p, const double* rho_host, void* stre
     c->Ework = ctx_alloc(c, eb);
     c->conv = (double*)ctx_alloc(c, sizeof(double) * 2 * (p->implicit_max_iter + 1));
   }
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  c->red_cap = (size_t)sms * 4 * 8 + 64;
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
+  c->red_cap = (size_t)c->sms * 4 * 8 + 64;
   c->red = (double*)ctx_alloc(c, sizeof(double) * c->red_cap);
   c->tab = (double*)ctx_alloc(c, sizeof(double) * 4 * p->nz);
   c->tpart = (double*)ctx_alloc(c, sizeof(double) * 5 * kTmunuSplit * p->nz);

@@ -13,6 +13,7 @@
 struct glasma_ctx {
   glasma_params p;
   int device = 0;
+  int sms = 152;              // SMs of the device
   cudaStream_t stream = nullptr;
   glasma_allocator alloc{};
   bool has_alloc = false;

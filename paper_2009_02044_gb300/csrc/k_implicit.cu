@@ -95,6 +95,7 @@ struct ImplArgs {
   int zA0, WA, zB0, WB;
   int zlo, zhi;   // slices of the prepare and sweep kernels: the owned ones
   R omega, omc;   // relaxation of this sweep and 1 - omega (exact)
+  int zlen;       // slices per block of the prepare and sweep kernels
   int check;      // sweeps return at once after convergence (device test)
 };
 
@@ -233,11 +234,15 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
   for (int c = 0; c < NA; ++c) a.Ework[(int64_t)(i * NA + c) * a.g.V + s] = ew[c] + a.dt * F[c];
 }
 
-// Slices per block of the prepare and sweep kernels.  A block marches
-// through kImplZ consecutive z slices of its transverse tile, so the links
-// of slice z+1 that it reads as neighbours are in L1 when they become its
-// own links (the sweep reads two link arrays in the planes containing z):
-// 87 -> 70 ms per step of the SU(3) 2048 x 128^2 workload.
+// Slices per block of the prepare and sweep kernels, at most.  A block marches
+// through consecutive z slices of its transverse tile, so the links of slice
+// z+1 that it reads as neighbours are in L1 when they become its own links
+// (the sweep reads two link arrays in the planes containing z): 87 -> 70 ms per
+// step of the SU(3) 2048 x 128^2 workload with 16.  A lattice of fewer than four
+// waves of such blocks marches through fewer slices instead: SU(3) 160 x 32^2
+// had 160 blocks of 16 slices for 608 places, one block of serial load latency
+// on each SM (a step there, fields of the size of a collision: 0.86 -> 0.34 ms,
+// with the fewer queued sweeps below).
 constexpr int kImplZ = 16;
 
 // SLAB: the owned slices start at zlo (a whole lattice's at 0, fixed at
@@ -245,9 +250,9 @@ constexpr int kImplZ = 16;
 template <int NC, typename R, bool SLAB>
 __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_prep(ImplArgs<R> a) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * kImplZ;
+  const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * a.zlen;
 #pragma unroll 1
-  for (int k = 0; k < kImplZ && z0 + k < a.zhi; ++k) prep_link<NC, R>(a, (int)threadIdx.y, t, z0 + k);
+  for (int k = 0; k < a.zlen && z0 + k < a.zhi; ++k) prep_link<NC, R>(a, (int)threadIdx.y, t, z0 + k);
 }
 
 // The z links of a slab's lower halo slice (zlo - 1), as its owner prepares
@@ -301,9 +306,9 @@ __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_iter(ImplA
   const int i = (int)threadIdx.y;
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   R dmax = R(0), emax = R(0);
-  const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * kImplZ;
+  const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * a.zlen;
 #pragma unroll 1
-  for (int kz = 0; kz < kImplZ && z0 + kz < a.zhi; ++kz) {
+  for (int kz = 0; kz < a.zlen && z0 + kz < a.zhi; ++kz) {
     const int iz = z0 + kz;
     if (t >= (uint32_t)a.g.nxy || (i == 2 && iz == a.g.nz - 1)) continue;
     sweep_link<NC, R>(a, i, t, iz, dmax, emax);
@@ -341,6 +346,12 @@ __global__ void __launch_bounds__(64) k_implicit_iter_halo(ImplArgs<R> a) {
   sweep_link<NC, R>(a, 2, t, a.zlo - 1, dmax, emax);
 }
 
+static int impl_zlen(const glasma_ctx* c) {
+  const int64_t tiles = (c->g.nxy + 63) / 64, slots = (int64_t)c->sms * (c->rs == 4 ? 4 : 1);
+  const int64_t z = tiles * (c->hi - c->lo) / (4 * slots);
+  return (int)(z < 1 ? 1 : z > kImplZ ? kImplZ : z);
+}
+
 // Arguments of the prepare and sweep kernels (the iterate buffers and the
 // sweep index are set by the caller).
 template <typename R>
@@ -374,6 +385,7 @@ static ImplArgs<R> impl_args(glasma_ctx* c, bool hop) {
   a.zlo = c->lo;
   a.zhi = c->hi;
   a.check = 1;
+  a.zlen = impl_zlen(c);
   a.omega = R(1);
   a.omc = R(0);
   return a;
@@ -393,9 +405,9 @@ static void set_relaxation(const glasma_ctx* c, int k, ImplArgs<R>& a) {
 }
 
 // 64 transverse sites x the three directions per block; a row of blocks
-// per kImplZ owned slices
+// per impl_zlen owned slices
 static dim3 impl_grid(const glasma_ctx* c) {
-  return dim3((unsigned)((c->g.nxy + 63) / 64), (unsigned)((c->hi - c->lo + kImplZ - 1) / kImplZ));
+  return dim3((unsigned)((c->g.nxy + 63) / 64), (unsigned)((c->hi - c->lo + impl_zlen(c) - 1) / impl_zlen(c)));
 }
 
 // U(t_{n-1}) if unknown, the cleared maxima, and the prepare kernel (hop,
@@ -473,25 +485,30 @@ static int implicit_t(glasma_ctx* c, bool hop, int* iters) {
   int st = implicit_prepare<NC, R>(c, hop);
   if (st) return st;
   const int maxit = c->p.implicit_max_iter;
-  for (int k = 0; k < maxit; ++k) {
-    st = implicit_launch_sweep<NC, R>(c, hop, k, true);
-    if (st) return st;
-  }
   std::vector<double> conv(2 * (maxit + 1));
-  st = cuda_check(cudaMemcpyAsync(conv.data(), c->conv, sizeof(double) * conv.size(), cudaMemcpyDeviceToHost,
-                                  c->stream),
-                  "conv readback");
-  if (st) return st;
-  st = cuda_check(cudaStreamSynchronize(c->stream), "implicit sync");
-  if (st) return st;
-  int done = 0;
+  // Sweeps are queued without waiting, one more than the last step took, then
+  // in fours until the iteration has converged: a sweep queued beyond that
+  // returns at once but still costs a launch, and queueing all maxit of them
+  // cost 0.1 ms per step.
+  int queued = 0, done = 0;
   bool converged = false;
-  for (int k = 0; k < maxit; ++k) {
-    done = k + 1;
-    if (!isfinite(conv[k])) return set_error(GLASMA_ERR_NONFINITE, "implicit iteration met a non-finite value");
-    if (implicit_converged(conv.data(), maxit, k, c->p.implicit_tol, sizeof(R) == 4)) {
-      converged = true;
-      break;
+  while (queued < maxit && !converged) {
+    int upto = queued == 0 ? (c->last_iters > 0 ? c->last_iters + 1 : 8) : queued + 4;
+    if (upto > maxit) upto = maxit;
+    for (; queued < upto; ++queued) {
+      st = implicit_launch_sweep<NC, R>(c, hop, queued, true);
+      if (st) return st;
+    }
+    st = cuda_check(cudaMemcpyAsync(conv.data(), c->conv, sizeof(double) * conv.size(), cudaMemcpyDeviceToHost,
+                                    c->stream),
+                    "conv readback");
+    if (st) return st;
+    st = cuda_check(cudaStreamSynchronize(c->stream), "implicit sync");
+    if (st) return st;
+    for (; done < queued && !converged; ++done) {
+      if (!isfinite(conv[done]))
+        return set_error(GLASMA_ERR_NONFINITE, "implicit iteration met a non-finite value");
+      converged = implicit_converged(conv.data(), maxit, done, c->p.implicit_tol, sizeof(R) == 4);
     }
   }
   *iters = done;
