@@ -13,6 +13,15 @@
 // Adjoint convention: for a real quantity v, vbar = dO/dv; a quaternion's
 // adjoint is the 4-vector of partial derivatives of O with respect to its
 // components.
+//
+// Through the time steps a link's adjoint is kept in its tangent space: the
+// three derivatives g = dO/d eta of O under U -> (1 + i eta.sigma) U.  A step
+// keeps links on the group, so the fourth (radial) component never matters, and
+// every step of the map turns into rotations and cross products of 3-vectors:
+// about 510 multiply-adds per site for the plaquettes and 75 per link on the
+// FP64 pipe that bounds the reverse pass, against 2350 and 180 for reverse-mode
+// products of quaternions.  q_mul(q_pure(g), U) is the quaternion adjoint with
+// zero radial part, which the initial state's reverse works on.
 #pragma once
 #include "glasma_internal.cuh"
 
@@ -86,17 +95,8 @@ GL_HD void qb_store(double* B, int d, int64_t V, int64_t s, const Q4& q) {
   B[(int64_t)(d * 4 + 3) * V + s] = q.z;
 }
 
-// X = exp(i th.sigma/2) = (cos(r/2), sin(r/2) th / r), r = |th|
-GL_HD Q4 q_expi(const double* th) {
-  const double r2 = th[0] * th[0] + th[1] * th[1] + th[2] * th[2];
-  if (r2 == 0.0) return q_one();
-  const double r = sqrt(r2);
-  const double s = sin(0.5 * r), c = cos(0.5 * r);
-  const double f = s / r;
-  return Q4{c, f * th[0], f * th[1], f * th[2]};
-}
-
-// thbar += dX/dth^T Xbar for X = q_expi(th):
+// X = exp(i th.sigma/2) = (cos(r/2), sin(r/2) th / r), r = |th|; thbar +=
+// dX/dth^T Xbar:
 //   dX0/dth = -(sin(r/2) / (2 r)) th,
 //   dXv/dth = g I + (g'(r) / r) th th^T,  g(r) = sin(r/2) / r;
 // near r = 0 the Taylor series of the three coefficients is used.
@@ -170,19 +170,6 @@ GL_HD void transport_rev(const Q4& U, bool dagger_first, const double* q, const 
   qb[2] = pb.z;
 }
 
-// Reverse of e . Vec(X1 X2 X3 X4) (coefficient folded into e): the
-// adjoints of the four factors.
-GL_HD void chain4_rev(const Q4& x1, const Q4& x2, const Q4& x3, const Q4& x4, const double* e, Q4& b1, Q4& b2,
-                      Q4& b3, Q4& b4) {
-  const Q4 p1 = q_mul(x1, x2);
-  const Q4 p2 = q_mul(p1, x3);
-  const Q4 mb = Q4{0.0, e[0], e[1], e[2]};
-  Q4 p2b = q_zero(), p1b = q_zero();
-  q_mul_rev(p2, x4, mb, p2b, b4);
-  q_mul_rev(p1, x3, p2b, p1b, b3);
-  q_mul_rev(x1, x2, p1b, b1, b2);
-}
-
 // ---------------------------------------------------------------------------
 // Per-element bodies of the adjoint kernels (host and device, so that the
 // same code can be run on the CPU).
@@ -192,120 +179,125 @@ GL_HD void chain4_rev(const Q4& x1, const Q4& x2, const Q4& x3, const Q4& x4, co
 __host__ __device__ __forceinline__ int plane_i(int pl) { return pl == 2 ? 1 : 0; }
 __host__ __device__ __forceinline__ int plane_j(int pl) { return pl == 0 ? 1 : 2; }
 
+GL_HD void cross(const double* a, const double* b, double* c) {
+  c[0] = fma(a[1], b[2], -(a[2] * b[1]));
+  c[1] = fma(a[2], b[0], -(a[0] * b[2]));
+  c[2] = fma(a[0], b[1], -(a[1] * b[0]));
+}
+// v <- Vec(U (0, v) U^+), v <- Vec(U^+ (0, v) U)
+GL_HD void rotate(const Q4& u, double* v) {
+  typedef Group<2, double> G;
+  G::rotate(u.w, G::M{{0.0, u.z}, {u.y, u.x}}, v);
+}
+GL_HD void rotate_back(const Q4& u, double* v) { rotate(Q4{-u.w, u.x, u.y, u.z}, v); }
+
 // Per base site x and plane (i, j), i < j, with a = U_i(x), b = U_j(x+i),
-// c = U_i(x+j), d = U_j(x), the plaquette's share of
+// c = U_i(x+j), d = U_j(x) and P = a b c^+ d^+ = p0 + i p.sigma, the
+// plaquette's share of
 //   phi = fs * sum_links Ebar . F   (F of Sec. 3 Eq. lattice_1)
-//       + wsl(iz) * |a b - d c|_F^2 / (a_i a_j)^2   (its energy term)
-// where the force terms are -w_j Ebar_i(x).Vec(a b c^+ d^+),
-// -w_j Ebar_i(x+j).Vec(c b^+ a^+ d), -w_i Ebar_j(x).Vec(d c b^+ a^+) and
-// -w_i Ebar_j(x+i).Vec(b c^+ d^+ a).  Writes d phi / d{a,b,c,d} to
-// G[((plane*4 + role)*4 + component)*V + s] (zero for absent plaquettes).
+//       + wsl(iz) * |a b - d c|_F^2 / (a_i a_j)^2   (its energy term).
+// The loops at the four corners are P (link a), P^+ (link d), a^+ P a (link b)
+// and (d^+ P d)^+ (link c), so with s = -fs [w_j Ebar_i(x) - w_i Ebar_j(x)],
+// t4 = Ad_a(-fs w_i Ebar_j(x+i)), t2 = Ad_d(-fs w_j Ebar_i(x+j)) the force part
+// is (s + t4 - t2).p, and the energy part is 4 f (1 - p0).  Varying a link
+// multiplies P from one side: e.p changes by L(e).eta = (p0 e - p x e).eta from
+// the left and by R(e).eta = (p0 e + p x e).eta from the right, which gives
+//   g_a = L(s - t2) + R(t4) + 4 f p     g_b = Ad_a^+ [L(s + t4 - t2) + 4 f p]
+//   g_d = L(t2) - R(s + t4) - 4 f p     g_c = -Ad_d^+ [R(s + t4 - t2) + 4 f p].
+// Writes them to G[((plane*4 + role)*3 + component)*V + s] (zero for absent
+// plaquettes).
 GL_HD void plaq_rev_at(const double2* U, const double* Eb, double fs, const double* wsl, double* G, const Geom& g,
-                       double wt, double wz, double ia2t, double ia2z, int64_t s) {
-  {
-    const SiteNbr n = site_nbr(g, s);
-    for (int pl = 0; pl < 3; ++pl) {
-      const int i = plane_i(pl), j = plane_j(pl);
-      Q4 ab = q_zero(), bb = q_zero(), cb = q_zero(), db = q_zero();
-      const bool exists = (j != 2) || (n.iz <= g.nz - 2);
-      if (exists) {
-        const Q4 a = q_load(U, i, g.V, s), b = q_load(U, j, g.V, n.p[i]);
-        const Q4 c = q_load(U, i, g.V, n.p[j]), d = q_load(U, j, g.V, s);
-        const double wi = i == 2 ? wz : wt, wj = j == 2 ? wz : wt;
-        if (fs != 0.0) {
-          double e[3];
-          Q4 t1 = q_zero(), t2 = q_zero(), t3 = q_zero(), t4 = q_zero();
-          // link a: a b c^+ d^+
-          for (int k = 0; k < 3; ++k) e[k] = -fs * wj * Eb[(int64_t)(i * 3 + k) * g.V + s];
-          t1 = t2 = t3 = t4 = q_zero();
-          chain4_rev(a, b, q_dag(c), q_dag(d), e, t1, t2, t3, t4);
-          q_acc(ab, t1);
-          q_acc(bb, t2);
-          q_dag_rev(t3, cb);
-          q_dag_rev(t4, db);
-          // link c: c b^+ a^+ d
-          for (int k = 0; k < 3; ++k) e[k] = -fs * wj * Eb[(int64_t)(i * 3 + k) * g.V + n.p[j]];
-          t1 = t2 = t3 = t4 = q_zero();
-          chain4_rev(c, q_dag(b), q_dag(a), d, e, t1, t2, t3, t4);
-          q_acc(cb, t1);
-          q_dag_rev(t2, bb);
-          q_dag_rev(t3, ab);
-          q_acc(db, t4);
-          // link d: d c b^+ a^+
-          for (int k = 0; k < 3; ++k) e[k] = -fs * wi * Eb[(int64_t)(j * 3 + k) * g.V + s];
-          t1 = t2 = t3 = t4 = q_zero();
-          chain4_rev(d, c, q_dag(b), q_dag(a), e, t1, t2, t3, t4);
-          q_acc(db, t1);
-          q_acc(cb, t2);
-          q_dag_rev(t3, bb);
-          q_dag_rev(t4, ab);
-          // link b: b c^+ d^+ a
-          for (int k = 0; k < 3; ++k) e[k] = -fs * wi * Eb[(int64_t)(j * 3 + k) * g.V + n.p[i]];
-          t1 = t2 = t3 = t4 = q_zero();
-          chain4_rev(b, q_dag(c), q_dag(d), a, e, t1, t2, t3, t4);
-          q_acc(bb, t1);
-          q_dag_rev(t2, cb);
-          q_dag_rev(t3, db);
-          q_acc(ab, t4);
-        }
-        const double ws = wsl ? wsl[n.iz] : 0.0;
-        if (ws != 0.0) {
-          // |A - B|_F^2 = 2 |A - B|^2 (quaternion norm), A = a b, B = d c
-          const double f = ws * (i == 2 || j == 2 ? ia2t * ia2z : ia2t * ia2t);
-          const Q4 A = q_mul(a, b), B = q_mul(d, c);
-          const Q4 D = q_scale(q_sub(A, B), 4.0 * f);
-          q_mul_rev(a, b, D, ab, bb);
-          q_mul_rev(d, c, q_scale(D, -1.0), db, cb);
-        }
-      }
-      const Q4 r[4] = {ab, bb, cb, db};
-      for (int k = 0; k < 4; ++k) {
-        double* gp = G + (int64_t)((pl * 4 + k) * 4) * g.V + s;
-        gp[0] = r[k].w;
-        gp[g.V] = r[k].x;
-        gp[2 * g.V] = r[k].y;
-        gp[3 * g.V] = r[k].z;
-      }
+                       double wt, double wz, double ia2t, double ia2z, int64_t s, int pl) {
+  const SiteNbr n = site_nbr(g, s);
+  const int i = plane_i(pl), j = plane_j(pl);
+  double r[4][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  if ((j != 2) || (n.iz <= g.nz - 2)) {
+    const Q4 a = q_load(U, i, g.V, s), d = q_load(U, j, g.V, s);
+    const Q4 P = q_mul(q_mul(a, q_load(U, j, g.V, n.p[i])), q_dag(q_mul(d, q_load(U, i, g.V, n.p[j]))));
+    const double p[3] = {P.x, P.y, P.z};
+    const double wi = i == 2 ? wz : wt, wj = j == 2 ? wz : wt;
+    double e[3], t4[3], t2[3], pe[3], p4[3], p2[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      e[k] = -fs * (wj * Eb[(int64_t)(i * 3 + k) * g.V + s] - wi * Eb[(int64_t)(j * 3 + k) * g.V + s]);
+      t4[k] = -fs * wi * Eb[(int64_t)(j * 3 + k) * g.V + n.p[i]];
+      t2[k] = -fs * wj * Eb[(int64_t)(i * 3 + k) * g.V + n.p[j]];
+    }
+    rotate(a, t4);
+    rotate(d, t2);
+    cross(p, e, pe);
+    cross(p, t4, p4);
+    cross(p, t2, p2);
+    const double ws = wsl ? wsl[n.iz] : 0.0;
+    const double f = 4.0 * ws * (i == 2 || j == 2 ? ia2t * ia2z : ia2t * ia2t);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double fp = f * p[k], se = e[k] - t2[k], ce = pe[k] - p2[k];
+      r[0][k] = fma(P.w, se + t4[k], fp) - (ce - p4[k]);
+      r[1][k] = fma(P.w, se + t4[k], fp) - (ce + p4[k]);
+      r[2][k] = -(fma(P.w, se + t4[k], fp) + (ce + p4[k]));
+      r[3][k] = -(fma(P.w, se + t4[k], fp) + (pe[k] + p4[k] + p2[k]));
+    }
+    rotate_back(a, r[1]);
+    rotate_back(d, r[2]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) G[(int64_t)((pl * 4 + q) * 3 + k) * g.V + s] = r[q][k];
+}
+
+GL_HD void g_add(const double* G, int pl, int role, int64_t V, int64_t s, double* acc) {
+  const double* gp = G + (int64_t)((pl * 4 + role) * 3) * V + s;
+  acc[0] += gp[0];
+  acc[1] += gp[V];
+  acc[2] += gp[2 * V];
+}
+
+// acc += the parts of the four plaquettes that hold link (x, d): as a (base
+// x) and c (base x - j) when d is the plane's first direction, as d (base x)
+// and b (base x - i) when it is the second.
+GL_HD void gather_at(const double* G, const Geom& g, int d, const SiteNbr& n, double* acc) {
+  for (int pl = 0; pl < 3; ++pl) {
+    const int i = plane_i(pl), j = plane_j(pl);
+    if (d == i) {
+      g_add(G, pl, 0, g.V, n.s, acc);
+      if (j != 2 || n.iz >= 1) g_add(G, pl, 2, g.V, n.m[j], acc);
+    } else if (d == j) {
+      g_add(G, pl, 3, g.V, n.s, acc);
+      g_add(G, pl, 1, g.V, n.m[i], acc);
     }
   }
 }
 
-GL_HD void g_add(const double* G, int pl, int role, int64_t V, int64_t s, Q4& acc) {
-  const double* gp = G + (int64_t)((pl * 4 + role) * 4) * V + s;
-  acc.w += gp[0];
-  acc.x += gp[V];
-  acc.y += gp[2 * V];
-  acc.z += gp[3 * V];
+// g[(d*3 + k)*V + s]: tangent adjoints of the links
+GL_HD void tan_load(const double* T, int d, int64_t V, int64_t s, double* v) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = T[(int64_t)(d * 3 + k) * V + s];
+}
+GL_HD void tan_store(double* T, int d, int64_t V, int64_t s, const double* v) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) T[(int64_t)(d * 3 + k) * V + s] = v[k];
 }
 
-// Ubar_d(x) += the parts of the four plaquettes that hold link (x, d):
-// as a (base x) and c (base x - j) when d is the plane's first direction,
-// as d (base x) and b (base x - i) when it is the second.
-GL_HD void gather_at(const double* G, double* Ub, const Geom& g, int64_t s) {
-  {
-    const SiteNbr n = site_nbr(g, s);
-    for (int d = 0; d < 3; ++d) {
-      if (d == 2 && n.iz == g.nz - 1) continue;
-      Q4 acc = qb_load(Ub, d, g.V, s);
-      for (int pl = 0; pl < 3; ++pl) {
-        const int i = plane_i(pl), j = plane_j(pl);
-        if (d == i) {
-          g_add(G, pl, 0, g.V, s, acc);
-          if (j != 2 || n.iz >= 1) g_add(G, pl, 2, g.V, n.m[j], acc);
-        } else if (d == j) {
-          g_add(G, pl, 3, g.V, s, acc);
-          g_add(G, pl, 1, g.V, n.m[i], acc);
-        }
-      }
-      qb_store(Ub, d, g.V, s, acc);
-    }
+// The tangent adjoints T plus the plaquettes' parts G as quaternion adjoints
+// of the links (radial part zero).
+GL_HD void tangent_to_quat_at(const double2* U, const double* T, const double* G, double* Ub, const Geom& g, int d,
+                              int64_t s) {
+  const SiteNbr n = site_nbr(g, s);
+  double v[3] = {0.0, 0.0, 0.0};
+  if (d != 2 || n.iz != g.nz - 1) {
+    tan_load(T, d, g.V, s, v);
+    gather_at(G, g, d, n, v);
   }
+  qb_store(Ub, d, g.V, s, q_mul(q_pure(v), q_load(U, d, g.V, s)));
 }
 
 struct LinkRevArgs {
   const double2* U;   // U_n
   const double* En;   // E_{n+1/2}
-  double* Ub;         // in: adjoint of U_{n+1}; out: of U_n (before the force part)
+  const double* G;    // plaquettes' parts of the adjoint of U_{n+1}
+  double* T;          // in: the rest of it; out: adjoint of U_n before the force part
   double* Eb;         // adjoint of E_{n+1/2} (in and out)
   const double* QA;   // charges at step n (before the hop)
   const double* QB;
@@ -316,86 +308,129 @@ struct LinkRevArgs {
   double dt, az2;
 };
 
-// Reverse of U_{n+1} = exp(i dt E_{n+1/2}) U_n per link and, on hop steps,
-// of the charge transport and the current on the z links:
+// For X = exp(i th.sigma/2), r = |th|, x = r^2: A = sin(r) / (2 r),
+// B = (1 - cos r) / (2 x), C = (1 - sin(r) / r) / (2 x), by their series for
+// r <= 1 (remainders below 1e-18).
+GL_HD void expi_coeffs(double x, double& A, double& B, double& C) {
+  if (x <= 1.0) {
+    double a = 0.0, b = 0.0;
+    // 1 / (2 (2k+1)!) and 1 / (2 (2k+2)!): A from k = 0, C from k = 1
+    const double fa[10] = {0.5, 1.0 / 12.0, 1.0 / 240.0, 1.0 / 10080.0, 1.0 / 725760.0, 1.0 / 79833600.0,
+                           1.0 / 12454041600.0, 1.0 / 2615348736000.0, 1.0 / 711374856192000.0,
+                           1.0 / 243290200817664000.0};
+    const double fb[9] = {0.25, 1.0 / 48.0, 1.0 / 1440.0, 1.0 / 80640.0, 1.0 / 7257600.0, 1.0 / 958003200.0,
+                          1.0 / 174356582400.0, 1.0 / 41845579776000.0, 1.0 / 12804747411456000.0};
+#pragma unroll
+    for (int k = 9; k >= 1; --k) a = fma(-x, a, fa[k]);
+#pragma unroll
+    for (int k = 8; k >= 0; --k) b = fma(-x, b, fb[k]);
+    C = a;
+    A = fma(-x, a, 0.5);
+    B = b;
+  } else {
+    const double r = sqrt(x), sh = sin(0.5 * r);
+    A = sin(r) / (2.0 * r);
+    B = sh * sh / x;
+    C = (0.5 - A) / x;
+  }
+}
+
+// Reverse of U_{n+1} = X U_n, X = exp(i th.sigma/2), th = dt E_{n+1/2}: a
+// change of U_n turns with X, and of E enters through the derivative of the
+// exponential, delta X = i xi.sigma X with xi = A dth + B dth x th +
+// C (th.dth) th.  On hop steps the charge transport and the current on the z
+// links:
 //   B: Q'_B = Vec(U^+ (0, Q_B) U) at the slot of x, E_z(x) -= a_z^2 Q_B;
 //   A: Q'_A = Vec(U (0, Q_A) U^+) at the slot of x + z, E_z(x) += a_z^2 Q'_A.
-GL_HD void link_rev_at(const LinkRevArgs& a, int64_t idx) {
+GL_HD void link_rev_at(const LinkRevArgs& a, int d, int64_t s) {
   const Geom& g = a.g;
-  do {
-    const int d = (int)(idx / g.V);
-    const int64_t s = idx - (int64_t)d * g.V;
-    const int iz = (int)(s / g.nxy);
-    if (d == 2 && iz == g.nz - 1) {  // absent link: unchanged, no field
-      for (int k = 0; k < 3; ++k) a.Eb[(int64_t)(6 + k) * g.V + s] = 0.0;
-      break;
-    }
-    const Q4 u = q_load(a.U, d, g.V, s);
-    double th[3], thb[3] = {0.0, 0.0, 0.0};
-    for (int k = 0; k < 3; ++k) th[k] = a.dt * a.En[(int64_t)(d * 3 + k) * g.V + s];
-    const Q4 X = q_expi(th);
-    const Q4 ub1 = qb_load(a.Ub, d, g.V, s);
-    Q4 xb = q_zero(), ub = q_zero();
-    q_mul_rev(X, u, ub1, xb, ub);
-    q_expi_rev(th, xb, thb);
-    double eb[3];
-    for (int k = 0; k < 3; ++k) {
-      eb[k] = a.Eb[(int64_t)(d * 3 + k) * g.V + s] + a.dt * thb[k];
-      a.Eb[(int64_t)(d * 3 + k) * g.V + s] = eb[k];
-    }
-    if (d == 2 && a.hop) {
-      const int64_t t = s - (int64_t)iz * g.nxy;
-      const int kb = iz - a.zB0;
-      if (kb >= 0 && kb < a.WB) {
-        double q[3], qpb[3], qb[3];
+  const SiteNbr n = site_nbr(g, s);
+  const int iz = n.iz;
+  if (d == 2 && iz == g.nz - 1) {  // absent link: no field, no adjoint
+    for (int k = 0; k < 3; ++k) a.Eb[(int64_t)(6 + k) * g.V + s] = 0.0;
+    return;
+  }
+  double th[3], t[3], tx[3], u[3], eb[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) th[k] = a.dt * a.En[(int64_t)(d * 3 + k) * g.V + s];
+  tan_load(a.T, d, g.V, s, t);
+  gather_at(a.G, g, d, n, t);
+  const double x = fma(th[0], th[0], fma(th[1], th[1], th[2] * th[2]));
+  const double tt = fma(th[0], t[0], fma(th[1], t[1], th[2] * t[2]));
+  double A, B, C;
+  expi_coeffs(x, A, B, C);
+  cross(th, t, tx);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    u[k] = fma(2.0, fma(A, tx[k], B * fma(tt, th[k], -(x * t[k]))), t[k]);
+    eb[k] = fma(a.dt, fma(A, t[k], fma(B, tx[k], C * tt * th[k])), a.Eb[(int64_t)(d * 3 + k) * g.V + s]);
+    a.Eb[(int64_t)(d * 3 + k) * g.V + s] = eb[k];
+  }
+  if (d == 2 && a.hop) {
+    const int64_t tr = s - (int64_t)iz * g.nxy;
+    const int kb = iz - a.zB0, ka = iz + 1 - a.zA0;
+    const bool inb = kb >= 0 && kb < a.WB, ina = ka >= 0 && ka < a.WA;
+    if (inb || ina) {
+      const Q4 q4 = q_load(a.U, 2, g.V, s);
+      double q[3], qb[3], c[3];
+      if (inb) {
         for (int k = 0; k < 3; ++k) {
-          q[k] = a.QB[((int64_t)k * a.WB + kb) * g.nxy + t];
-          qpb[k] = a.QBb[((int64_t)k * a.WB + kb) * g.nxy + t];
+          q[k] = a.QB[((int64_t)k * a.WB + kb) * g.nxy + tr];
+          qb[k] = a.QBb[((int64_t)k * a.WB + kb) * g.nxy + tr];
         }
-        transport_rev(u, true, q, qpb, qb, ub);
-        for (int k = 0; k < 3; ++k) a.QBb[((int64_t)k * a.WB + kb) * g.nxy + t] = qb[k] - a.az2 * eb[k];
-      }
-      const int ka = iz + 1 - a.zA0;
-      if (ka >= 0 && ka < a.WA) {
-        double q[3], qpb[3], qb[3];
+        rotate(q4, qb);
+        cross(q, qb, c);
         for (int k = 0; k < 3; ++k) {
-          q[k] = a.QA[((int64_t)k * a.WA + ka) * g.nxy + t];
-          qpb[k] = a.QAb[((int64_t)k * a.WA + ka) * g.nxy + t] + a.az2 * eb[k];
+          u[k] = fma(2.0, c[k], u[k]);
+          a.QBb[((int64_t)k * a.WB + kb) * g.nxy + tr] = qb[k] - a.az2 * eb[k];
         }
-        transport_rev(u, false, q, qpb, qb, ub);
-        for (int k = 0; k < 3; ++k) a.QAb[((int64_t)k * a.WA + ka) * g.nxy + t] = qb[k];
+      }
+      if (ina) {
+        for (int k = 0; k < 3; ++k) {
+          q[k] = a.QA[((int64_t)k * a.WA + ka) * g.nxy + tr];
+          qb[k] = a.QAb[((int64_t)k * a.WA + ka) * g.nxy + tr] + a.az2 * eb[k];
+        }
+        rotate(q4, q);
+        cross(q, qb, c);
+        rotate_back(q4, qb);
+        for (int k = 0; k < 3; ++k) {
+          u[k] = fma(-2.0, c[k], u[k]);
+          a.QAb[((int64_t)k * a.WA + ka) * g.nxy + tr] = qb[k];
+        }
       }
     }
-    qb_store(a.Ub, d, g.V, s, ub);
-  } while (false);
+  }
+  tan_store(a.T, d, g.V, s, u);
 }
 
 // The current part of the observable's own E update (no transported-charge
-// adjoint): E'_z(x) += a_z^2 (Q'_A - Q_B) with adjoint Ebp_z(x).
+// adjoint): E'_z(x) += a_z^2 (Q'_A - Q_B) with adjoint Ebp_z(x); T holds the
+// tangent adjoints of the links.
 GL_HD void hop_current_rev_at(const double2* U, const double* Ebp, const double* QA, const double* QB, double* QAb,
-                              double* QBb, double* Ub, int zA0, int WA, int zB0, int WB, const Geom& g, double az2,
+                              double* QBb, double* T, int zA0, int WA, int zB0, int WB, const Geom& g, double az2,
                               int64_t s) {
-  {
-    const int iz = (int)(s / g.nxy);
-    const int64_t t = s - (int64_t)iz * g.nxy;
-    double eb[3];
-    for (int k = 0; k < 3; ++k) eb[k] = Ebp[(int64_t)(6 + k) * g.V + s];
-    const int kb = iz - zB0;
-    if (kb >= 0 && kb < WB)
-      for (int k = 0; k < 3; ++k) QBb[((int64_t)k * WB + kb) * g.nxy + t] -= az2 * eb[k];
-    const int ka = iz + 1 - zA0;
-    if (ka >= 0 && ka < WA) {
-      const Q4 u = q_load(U, 2, g.V, s);
-      double q[3], qpb[3], qb[3];
-      for (int k = 0; k < 3; ++k) {
-        q[k] = QA[((int64_t)k * WA + ka) * g.nxy + t];
-        qpb[k] = az2 * eb[k];
-      }
-      Q4 ub = qb_load(Ub, 2, g.V, s);
-      transport_rev(u, false, q, qpb, qb, ub);
-      qb_store(Ub, 2, g.V, s, ub);
-      for (int k = 0; k < 3; ++k) QAb[((int64_t)k * WA + ka) * g.nxy + t] += qb[k];
+  const int iz = (int)(s / g.nxy);
+  const int64_t t = s - (int64_t)iz * g.nxy;
+  double eb[3];
+  for (int k = 0; k < 3; ++k) eb[k] = Ebp[(int64_t)(6 + k) * g.V + s];
+  const int kb = iz - zB0;
+  if (kb >= 0 && kb < WB)
+    for (int k = 0; k < 3; ++k) QBb[((int64_t)k * WB + kb) * g.nxy + t] -= az2 * eb[k];
+  const int ka = iz + 1 - zA0;
+  if (ka >= 0 && ka < WA) {
+    const Q4 u = q_load(U, 2, g.V, s);
+    double q[3], qb[3], c[3], v[3];
+    for (int k = 0; k < 3; ++k) {
+      q[k] = QA[((int64_t)k * WA + ka) * g.nxy + t];
+      qb[k] = az2 * eb[k];
     }
+    rotate(u, q);
+    cross(q, qb, c);
+    rotate_back(u, qb);
+    tan_load(T, 2, g.V, s, v);
+    for (int k = 0; k < 3; ++k) v[k] = fma(-2.0, c[k], v[k]);
+    tan_store(T, 2, g.V, s, v);
+    for (int k = 0; k < 3; ++k) QAb[((int64_t)k * WA + ka) * g.nxy + t] += qb[k];
   }
 }
 
