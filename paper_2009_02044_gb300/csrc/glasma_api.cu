@@ -136,9 +136,9 @@ static int check_params(const glasma_params* p) {
 // for the one-site staple kernel, bitwise the same result), else the staple
 // kernel (0.469 ms, against 0.521 for the plaquette kernel and 0.572 for
 // site pairs, whose 168 registers leave too few warps to hide latency); in
-// FP32 SU(2) the staple kernel too (1.10 against 1.39 ms for site pairs per
-// 1024 x 128^2 step, once a link's alpha and beta became one 16-byte load:
-// the pairs' 32-bit loads then stride 16 bytes).
+// FP32 SU(2) one thread per site on large lattices (0.79 against 1.10 ms for
+// the staple kernel and 1.39 for site pairs per 1024 x 128^2 step), the staple
+// kernel on small ones.
 bool use_plaq_kernel(const glasma_ctx* c) {
   if (c->rs == 8) return false;
   if (c->step_kernel == GLASMA_KERNEL_PLAQUETTE || c->step_kernel == GLASMA_KERNEL_PLAQUETTE_256) return plaq_fits(c);
@@ -153,6 +153,15 @@ bool use_pair_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_STAPLE_PAIRS;
 }
 
+// One thread per site from 2^17 sites of the whole lattice on (a slab decides as
+// the lattice does): below that, three times fewer threads than links no longer
+// fill the GPU (200 x 30 x 20, 0.0129 against 0.0125 ms per step; 768 x 64^2,
+// 0.158 against 0.209).
+bool use_site_kernel(const glasma_ctx* c) {
+  return c->step_kernel == GLASMA_KERNEL_AUTO && c->rs == 4 && c->p.nc == 2 &&
+         (long long)c->nz_glob * c->g.nxy >= (1 << 17);
+}
+
 bool use_staged_kernel(const glasma_ctx* c) {
   if (c->step_kernel == GLASMA_KERNEL_STAPLE_STAGED) return staged_fits(c);
   return c->step_kernel == GLASMA_KERNEL_AUTO && staged_fits(c) && c->g.nx == 64;
@@ -163,6 +172,7 @@ int launch_step_chosen(glasma_ctx* c, bool hop, int* launches) {
   *launches += 1;
   if (use_plaq_kernel(c)) return launch_step_plaq(c, hop, c->step_zlen);
   if (use_pair_kernel(c)) return launch_step_pair(c, hop);
+  if (use_site_kernel(c)) return launch_step_site(c, hop);
   if (use_staged_kernel(c)) return launch_step_staged(c, hop);
   return launch_step_leapfrog(c, hop);
 }

@@ -107,6 +107,8 @@ int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches);
 bool use_parts_kernel(const glasma_ctx* c);
 bool use_plaq_kernel(const glasma_ctx* c);
 bool use_pair_kernel(const glasma_ctx* c);
+bool use_site_kernel(const glasma_ctx* c);
+int launch_step_site(glasma_ctx* c, bool hop);  // one thread per site, FP32 SU(2) (k_step_su2.cu)
 bool use_staged_kernel(const glasma_ctx* c);
 // staple kernel with the links staged in shared memory by bulk copies
 // (FP32 SU(3), rows of 32 or 64 sites, whole lattices)
