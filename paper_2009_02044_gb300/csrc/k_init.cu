@@ -187,8 +187,9 @@ GL_HD bool same(const typename Group<NC, double>::M& a, const typename Group<NC,
 }
 
 // Behind a nucleus (Lambda = 1) the Wilson line and with it the links depend
-// on the transverse site alone: full[N][t] = V_N^dag(x_T), then
-// tail[N][i][t] = V_N(x) V_N^dag(x+i), formed once and copied to all slices.
+// on the transverse site alone: full[N][t] = V_N^dag(x_T), then the links
+// V_N(x) V_N^dag(x+i) in their stored form, "direction" 2 N + i of a lattice of
+// one slice, formed once and copied to all slices.
 template <int NC>
 __global__ void k_wilson_full(const double* phi, typename Group<NC, double>::M* full, int64_t nxy, int S) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * nxy; i += (int64_t)gridDim.x * blockDim.x) {
@@ -197,14 +198,15 @@ __global__ void k_wilson_full(const double* phi, typename Group<NC, double>::M* 
   }
 }
 
-template <int NC>
-__global__ void k_tail_links(const typename Group<NC, double>::M* full, typename Group<NC, double>::M* tail, Geom g) {
+template <int NC, typename R>
+__global__ void k_tail_links(const typename Group<NC, double>::M* full, typename V2T<R>::T* tail, Geom g) {
   const int64_t nxy = g.nxy;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 4 * nxy; i += (int64_t)gridDim.x * blockDim.x) {
     const int N = (int)(i / (2 * nxy)), d = (int)(i / nxy) & 1;
     const uint32_t t = (uint32_t)(i % nxy);
     const SiteNbr n = site_nbr_tz(g, t, 0);
-    tail[i] = Group<NC, double>::d_mul(full[N * nxy + t], full[N * nxy + n.p[d]]);
+    LinkIO<NC, R>::template store<double>(tail, 2 * N + d, nxy, t,
+                                          Group<NC, double>::d_mul(full[N * nxy + t], full[N * nxy + n.p[d]]));
   }
 }
 
@@ -212,13 +214,14 @@ __global__ void k_tail_links(const typename Group<NC, double>::M* full, typename
 // of kTileX x kTileY transverse sites.  The two profiles are disjoint (the
 // centres lie more than 4 sigma from the box centre), so at most one nucleus
 // has Lambda > 0 on a slice.  A slice ahead of both has unit links; a slice
-// whose Lambda is 1 at both times copies the tail links; both have E = 0.  On
-// the slices in between the Wilson lines of the tile and of its +x and +y
-// neighbours at both times are formed once each in shared memory (2.4
-// exponentials per site instead of the 6 that a thread by itself takes).
-// FP64-pipe bound there, bound by the stores elsewhere.  The whole initial
-// state, with the DFTs, the series logarithm and the split divergence: SU(3)
-// 512 x 64^2, sigma_L = 4, 7.5 -> 3.0 ms, SU(2) 1024 x 128^2 13.5 -> 6.1 ms.
+// whose Lambda is 1 at both times copies the tail links; both have E = 0, and
+// no FP64 work (the conversions and the division by dt of every site took 3 ms
+// of an SU(2) 1024 x 128^2 event).  On the slices in between the Wilson lines of
+// the tile and of its +x and +y neighbours at both times are formed once each in
+// shared memory (2.4 exponentials per site instead of the 6 that a thread by
+// itself takes): FP64-pipe bound there, bound by the stores elsewhere.  The whole
+// initial state, with the DFTs, the series logarithm and the split divergence:
+// SU(3) 512 x 64^2, sigma_L = 4, 7.5 -> 1.8 ms, SU(2) 1024 x 128^2 13.5 -> 2.2 ms.
 // U1, the buffer the first step writes, only needs the absent z links of the
 // last slice (all of it on a slab, whose halo slices are not stepped).
 constexpr int kTileX = 16, kTileY = 8;
@@ -226,7 +229,7 @@ constexpr int kTileX = 16, kTileY = 8;
 template <int NC, typename R>
 __global__ void __launch_bounds__(kTileX * kTileY) k_init_links(
     const double* phi, const double* lam, const typename Group<NC, double>::M* full,
-    const typename Group<NC, double>::M* tail, typename V2T<R>::T* U0, typename V2T<R>::T* U1,
+    const typename V2T<R>::T* tail, typename V2T<R>::T* U0, typename V2T<R>::T* U1,
     typename V2T<R>::T* Uprev, R* E, Geom g, double dt, int* flag, int S, int whole) {
   typedef Group<NC, double> G;
   typedef typename G::M M;
@@ -244,7 +247,7 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_init_links(
   const bool copy1 = !whole || iz == g.nz - 1;
   const int N = lam[0 * g.nz + iz] != 0.0 || lam[2 * g.nz + iz] != 0.0 ? 0 : 1;
   const double l0 = lam[N * g.nz + iz], l1 = lam[(2 + N) * g.nz + iz];
-  const bool moving = l0 != l1;
+  const bool moving = l0 != l1 || (l0 != 0.0 && l0 != 1.0);
   if (moving) {
     for (int q = threadIdx.x; q < 2 * PN; q += kTileX * kTileY) {
       const int tm = q / PN, p = q - tm * PN;
@@ -255,37 +258,37 @@ __global__ void __launch_bounds__(kTileX * kTileY) k_init_links(
     __syncthreads();
   }
   if (!inside) return;
-  const M one = G::ident();
+  typedef LinkAlg<NC, R> L;  // links in their stored form
 #pragma unroll 1
   for (int i = 0; i < 2; ++i) {
-    M u0 = one, u1 = one;
-    double h[NA];
-#pragma unroll
-    for (int a = 0; a < NA; ++a) h[a] = 0.0;
     if (moving) {
       const int p = ly * PX + lx, pn = p + (i == 0 ? 1 : PX);
-      u0 = G::d_mul(v[p], v[pn]);
-      u1 = G::d_mul(v[PN + p], v[PN + pn]);
-      if (!same<NC>(u0, u1) && !group_log<NC>(G::mul_d(u0, u1), h)) atomicOr(flag, 1);
-    } else if (l0 != 0.0) {
-      u0 = l0 == 1.0 ? tail[(N * 2 + i) * g.nxy + t]
-                     : G::d_mul(wilson_dag<NC>(phi, N, g.nxy, t, l0, S),
-                                wilson_dag<NC>(phi, N, g.nxy,
-                                               i == 0 ? t - ix + (ix + 1) % g.nx
-                                                      : (int64_t)((iy + 1) % g.ny) * g.nx + ix, l0, S));
-      u1 = u0;
-    }
+      const M u0 = G::d_mul(v[p], v[pn]), u1 = G::d_mul(v[PN + p], v[PN + pn]);
+      double h[NA];
 #pragma unroll
-    for (int a = 0; a < NA; ++a) E[(int64_t)(i * NA + a) * g.V + s] = (R)(h[a] / dt);
-    IO::template store<double>(U0, i, g.V, s, u0);
-    if (copy1) IO::template store<double>(U1, i, g.V, s, u0);
-    if (Uprev) IO::template store<double>(Uprev, i, g.V, s, u1);
+      for (int a = 0; a < NA; ++a) h[a] = 0.0;
+      if (!same<NC>(u0, u1) && !group_log<NC>(G::mul_d(u0, u1), h)) atomicOr(flag, 1);
+#pragma unroll
+      for (int a = 0; a < NA; ++a) E[(int64_t)(i * NA + a) * g.V + s] = (R)(h[a] / dt);
+      IO::template store<double>(U0, i, g.V, s, u0);
+      if (copy1) IO::template store<double>(U1, i, g.V, s, u0);
+      if (Uprev) IO::template store<double>(Uprev, i, g.V, s, u1);
+    } else {
+      typename L::M u = L::ident();
+      if (l0 != 0.0) u = IO::template load<R>(tail, 2 * N + i, g.nxy, t);
+#pragma unroll
+      for (int a = 0; a < NA; ++a) E[(int64_t)(i * NA + a) * g.V + s] = (R)0;
+      IO::template store<R>(U0, i, g.V, s, u);
+      if (copy1) IO::template store<R>(U1, i, g.V, s, u);
+      if (Uprev) IO::template store<R>(Uprev, i, g.V, s, u);
+    }
   }
 #pragma unroll
   for (int a = 0; a < NA; ++a) E[(int64_t)(2 * NA + a) * g.V + s] = (R)0;
-  IO::template store<double>(U0, 2, g.V, s, one);
-  if (copy1) IO::template store<double>(U1, 2, g.V, s, one);
-  if (Uprev) IO::template store<double>(Uprev, 2, g.V, s, one);
+  const typename L::M one = L::ident();
+  IO::template store<R>(U0, 2, g.V, s, one);
+  if (copy1) IO::template store<R>(U1, 2, g.V, s, one);
+  if (Uprev) IO::template store<R>(Uprev, 2, g.V, s, one);
 }
 
 // rho(x) = sum_i [E_i(x) - U_i^dag(x-i) E_i(x-i) U_i(x-i)] / a_i^2 of the
@@ -311,15 +314,20 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
     for (int c = 0; c < NA; ++c) dv[c] = 0.0;
     for (int i = 0; i < 3; ++i) {
       const double w = i == 2 ? ia2z : ia2t;
-      for (int c = 0; c < NA; ++c) dv[c] += w * (double)E[(int64_t)(i * NA + c) * g.V + s];
-      if (i == 2 && iz == 0) continue;
-      double q[NA];
-      bool nz = false;
+      R e[NA], em[NA];
+      bool here = false, below = false;
       for (int c = 0; c < NA; ++c) {
-        q[c] = (double)E[(int64_t)(i * NA + c) * g.V + n.m[i]];
-        nz = nz || q[c] != 0.0;
+        e[c] = E[(int64_t)(i * NA + c) * g.V + s];
+        em[c] = i == 2 && iz == 0 ? R(0) : E[(int64_t)(i * NA + c) * g.V + n.m[i]];
+        here = here || e[c] != R(0);
+        below = below || em[c] != R(0);
       }
-      if (!nz) continue;  // the transported field is zero (E vanishes off the nuclei)
+      // E vanishes off the nuclei: no FP64 work there
+      if (here)
+        for (int c = 0; c < NA; ++c) dv[c] += w * (double)e[c];
+      if (!below) continue;
+      double q[NA];
+      for (int c = 0; c < NA; ++c) q[c] = (double)em[c];
       typename G::M um = LinkIO<NC, R>::template load<double>(U, i, g.V, n.m[i]);
       G::adj_dag(um, q);
       for (int c = 0; c < NA; ++c) dv[c] -= w * q[c];
@@ -376,7 +384,8 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
   double* smax = (double*)ctx_alloc(c, sizeof(double) * p.nz);
   typedef typename Group<NC, double>::M MD;
   MD* full = (MD*)ctx_alloc(c, sizeof(MD) * 2 * nxy);
-  MD* tail = (MD*)ctx_alloc(c, sizeof(MD) * 4 * nxy);
+  typedef typename V2T<R>::T V2;
+  V2* tail = (V2*)ctx_alloc(c, sizeof(V2) * 4 * (size_t)(link_elems(NC, nxy) / 3));
   if (!rho || !w0 || !w1 || !lam || !rho3 || !smax || !full || !tail) return set_error(GLASMA_ERR_OOM, "init scratch allocation failed");
   if (rho_host) {
     st = cuda_check(cudaMemcpyAsync(rho, rho_host, sizeof(double) * F * nxy, cudaMemcpyHostToDevice, c->stream),
@@ -396,7 +405,7 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
   cudaMemsetAsync(c->dflag, 0, sizeof(int) * 8, c->stream);
   cudaMemsetAsync(smax, 0, sizeof(double) * p.nz, c->stream);
   k_wilson_full<NC><<<grid_for(2 * nxy, 64), 64, 0, c->stream>>>(rho, full, nxy, S);
-  k_tail_links<NC><<<grid_for(4 * nxy, 64), 64, 0, c->stream>>>(full, tail, c->g);
+  k_tail_links<NC, R><<<grid_for(4 * nxy, 64), 64, 0, c->stream>>>(full, tail, c->g);
   const unsigned tiles = (unsigned)(((p.nx + kTileX - 1) / kTileX) * ((p.ny + kTileY - 1) / kTileY));
   k_init_links<NC, R><<<dim3(tiles, (unsigned)p.nz), kTileX * kTileY, 0, c->stream>>>(
       rho, lam, full, tail, (typename V2T<R>::T*)c->U[0], (typename V2T<R>::T*)c->U[1],
