@@ -136,7 +136,7 @@ static int check_params(const glasma_params* p) {
 // for the one-site staple kernel, bitwise the same result), else the staple
 // kernel (0.469 ms, against 0.521 for the plaquette kernel and 0.572 for
 // site pairs, whose 168 registers leave too few warps to hide latency); in
-// FP32 SU(2) one thread per site on large lattices (0.79 against 1.10 ms for
+// FP32 SU(2) one thread per site on large lattices (0.59 against 1.10 ms for
 // the staple kernel and 1.39 for site pairs per 1024 x 128^2 step), the staple
 // kernel on small ones.
 bool use_plaq_kernel(const glasma_ctx* c) {
@@ -156,7 +156,7 @@ bool use_pair_kernel(const glasma_ctx* c) {
 // One thread per site from 2^17 sites of the whole lattice on (a slab decides as
 // the lattice does): below that, three times fewer threads than links no longer
 // fill the GPU (200 x 30 x 20, 0.0129 against 0.0125 ms per step; 768 x 64^2,
-// 0.158 against 0.209).
+// 0.120 against 0.209).
 bool use_site_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_AUTO && c->rs == 4 && c->p.nc == 2 &&
          (long long)c->nz_glob * c->g.nxy >= (1 << 17);

@@ -15,8 +15,11 @@
 //   the plaquettes at x - e_x and x - e_y give the four values that are left.
 // That is 17 link loads for three links; exponential and unit norm are short
 // series.  Measured against the staple kernel, ms per step: SU(2) 1024 x 128^2
-// 1.10 -> 0.79, 768 x 64^2 0.209 -> 0.158, 200 x 30 x 20 0.0125 -> 0.0129 (there
+// 1.10 -> 0.59, 768 x 64^2 0.209 -> 0.120, 200 x 30 x 20 0.0125 -> 0.0129 (there
 // the staple kernel stays).
+// The fields are loaded at the start of a slice (loaded where they are used,
+// behind the stores of the link before, they cost a memory latency per link:
+// 0.79 -> 0.61 ms), and the lines of the next slice are brought to L2 (0.59).
 //
 // Links are stored as deviations from 1 (link_alg.cuh): quaternions (w, x, y,
 // z) of alpha = 1 + w + i z, beta = y + i x, one 16-byte word each.  Every
@@ -25,6 +28,9 @@
 #include "step_link.cuh"
 
 namespace glasma {
+
+// Bring the line of p from device memory to L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 constexpr int kSiteThreads = 256;  // consecutive transverse sites of a block
 constexpr int kSiteBlocks = 3;     // blocks per SM
@@ -106,9 +112,14 @@ __device__ __forceinline__ Dev4 dev_evolve(Vec3 e, float dt, Dev4 u) {
 }
 
 // E_i += dt F (+ dt J, given) and the new link of direction i at site s.
-__device__ __forceinline__ void site_update(const StepArgs<float>& a, int i, int64_t s, Vec3 F, Vec3 dj, Dev4 u) {
+__device__ __forceinline__ Vec3 site_field(const StepArgs<float>& a, int i, int64_t s) {
+  const float* e = a.E + (int64_t)(3 * i) * a.g.V + s;
+  return Vec3{e[0], e[a.g.V], e[2 * a.g.V]};
+}
+__device__ __forceinline__ void site_update(const StepArgs<float>& a, int i, int64_t s, Vec3 F, Vec3 E, Vec3 dj,
+                                            Dev4 u) {
   float* e = a.E + (int64_t)(3 * i) * a.g.V + s;
-  const Vec3 v{fma(a.dt, F.x, e[0]) + dj.x, fma(a.dt, F.y, e[a.g.V]) + dj.y, fma(a.dt, F.z, e[2 * a.g.V]) + dj.z};
+  const Vec3 v{fma(a.dt, F.x, E.x) + dj.x, fma(a.dt, F.y, E.y) + dj.y, fma(a.dt, F.z, E.z) + dj.z};
   e[0] = v.x;
   e[a.g.V] = v.y;
   e[2 * a.g.V] = v.z;
@@ -169,6 +180,19 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
     const int64_t s = (int64_t)z * g.nxy + t;
     Dev4 uz{0.f, 0.f, 0.f, 0.f}, nux = ux, nuy = uy;
     Vec3 Fx{0.f, 0.f, 0.f}, Fy = Fx, Fz = Fx, nx_{0.f, 0.f, 0.f}, ny_ = nx_;
+    if (z + 2 < g.nz) {
+      prefetch_l2(Ux + 2 * g.nxy + t);
+      prefetch_l2(Uy + 2 * g.nxy + t);
+      prefetch_l2(Uz + g.nxy + t);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) prefetch_l2(a.E + (int64_t)c * g.V + s + g.nxy);
+    }
+    Vec3 Ex{0.f, 0.f, 0.f}, Ey = Ex, Ez = Ex;
+    if (now) {
+      Ex = site_field(a, 0, s);
+      Ey = site_field(a, 1, s);
+      Ez = site_field(a, 2, s);
+    }
     if (up) {
       uz = dev_load(Uz + t);
       nux = dev_load(Ux + g.nxy + t);
@@ -218,9 +242,9 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
                vec_ab(dev_mul(uz, dev_dag(dev_load(Uy + g.nxy + tym))), dev_mul(dev_dag(dev_load(Uz + tym)), vy)));
       }
       const Vec3 zero{0.f, 0.f, 0.f};
-      site_update(a, 0, s, Fx, zero, ux);
-      site_update(a, 1, s, Fy, zero, uy);
-      if (up) site_update(a, 2, s, Fz, a.hop ? site_hop(a, z, t, uz) : zero, uz);
+      site_update(a, 0, s, Fx, Ex, zero, ux);
+      site_update(a, 1, s, Fy, Ey, zero, uy);
+      if (up) site_update(a, 2, s, Fz, Ez, a.hop ? site_hop(a, z, t, uz) : zero, uz);
     }
     cx = nx_;
     cy = ny_;
