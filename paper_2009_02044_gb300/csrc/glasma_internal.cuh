@@ -91,6 +91,37 @@ GL_HD bool hop_at(long long n, long long p, long long q) {
   return hop_count(n + 1, p, q) > hop_count(n, p, q);
 }
 
+// Launch a kernel that begins with follow(): it may be set up, and its first
+// blocks placed, while the kernel before it in the stream runs out.  Small
+// lattices spend their time between launches (us per step: SU(2) FP32 100 x 9 x 7
+// 6.3 -> 3.8, 200 x 30 x 20 12.6 -> 10.6; SU(3) FP32 131 x 45 x 48 73.0 -> 70.3).  Not
+// for kernels that the FP64 pipe bounds: blocks placed early crowd on the SMs
+// that had room first, and the pipes of the others idle (SU(2) 128 x 16^2, two
+// passes, 37 -> 49).
+template <typename... P, typename... A>
+int launch_following(const char* what, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cuda_check(cudaLaunchKernelEx(&cfg, k, (P)args...), what);
+}
+#ifdef __CUDACC__
+// Wait until the kernels before this one are complete and their writes can be
+// seen (nothing of theirs is read or overwritten before), then let the next be
+// set up.  Without launch_following the wait is over at once.
+__device__ __forceinline__ void follow() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // kernel launchers
 int launch_step_leapfrog(glasma_ctx* c, bool hop);
 // plaquette-centric leapfrog step (k_step_plaq.cu): zlen z slices per block

@@ -249,6 +249,7 @@ constexpr int kImplZ = 16;
 // compile time: the offset costs the 80-register sweep 12 B of spills).
 template <int NC, typename R, bool SLAB>
 __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_prep(ImplArgs<R> a) {
+  follow();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * a.zlen;
 #pragma unroll 1
@@ -294,6 +295,7 @@ __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t
 // Ework already holds E(t_{n-1/2}) + dt J + dt (F_1(U_n) + F_2(U_{n-1})).
 template <int NC, typename R, bool SLAB>
 __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_iter(ImplArgs<R> a) {
+  follow();
   typedef LinkAlg<NC, R> G;
   typedef typename G::M M;
   constexpr int NA = G::NA;
@@ -431,11 +433,8 @@ static int implicit_prepare(glasma_ctx* c, bool hop) {
   st = cuda_check(cudaMemsetAsync(c->conv, 0, sizeof(double) * 2 * (a.maxit + 1), c->stream), "conv clear");
   if (st) return st;
   a.Xn = (V2*)c->U[1 - c->cur];
-  if (c->lo > 0)
-    k_implicit_prep<NC, R, true><<<impl_grid(c), bs, 0, c->stream>>>(a);
-  else
-    k_implicit_prep<NC, R, false><<<impl_grid(c), bs, 0, c->stream>>>(a);
-  st = cuda_check(cudaGetLastError(), "k_implicit_prep launch");
+  st = launch_following("k_implicit_prep launch", c->lo > 0 ? k_implicit_prep<NC, R, true> : k_implicit_prep<NC, R, false>,
+                        impl_grid(c), bs, 0, c->stream, a);
   if (st || c->lo == 0) return st;
   k_implicit_prep_halo<NC, R><<<(unsigned)((c->g.nxy + 63) / 64), 64, 0, c->stream>>>(a);
   return cuda_check(cudaGetLastError(), "k_implicit_prep_halo launch");
@@ -454,11 +453,9 @@ static int implicit_launch_sweep(glasma_ctx* c, bool hop, int k, bool check) {
   set_relaxation<R>(c, k, a);
   a.X = (const V2*)(k % 2 == 0 ? xa : xb);
   a.Xn = (V2*)(k % 2 == 0 ? xb : xa);
-  if (c->lo > 0)
-    k_implicit_iter<NC, R, true><<<impl_grid(c), dim3(64, 3), 0, c->stream>>>(a);
-  else
-    k_implicit_iter<NC, R, false><<<impl_grid(c), dim3(64, 3), 0, c->stream>>>(a);
-  int st = cuda_check(cudaGetLastError(), "k_implicit_iter launch");
+  int st = launch_following("k_implicit_iter launch",
+                            c->lo > 0 ? k_implicit_iter<NC, R, true> : k_implicit_iter<NC, R, false>, impl_grid(c),
+                            dim3(64, 3), 0, c->stream, a);
   if (st || c->lo == 0) return st;
   k_implicit_iter_halo<NC, R><<<(unsigned)((c->g.nxy + 63) / 64), 64, 0, c->stream>>>(a);
   return cuda_check(cudaGetLastError(), "k_implicit_iter_halo launch");

@@ -264,6 +264,7 @@ template <> struct TmnOcc<2, float> { static constexpr int blocks = 4; };
 // 512 x 64^2 FP64 15.2 -> 10.8 ms.
 template <int NC, typename R>
 __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(TmnArgs<R> a) {
+  follow();
   typedef LinkAlg<NC, R> G;
   typedef LinkIO<NC, R> IO;
   typedef typename G::M M;
@@ -381,6 +382,7 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
 // tab[iz] = (sum over the split blocks of slice iz, in block order) / nxy;
 // a slice that met a non-finite value gets a NaN energy density.
 __global__ void k_tmunu_fold(const double* part, int split, int nz, double inv, double* tab) {
+  follow();
   const int iz = blockIdx.x * blockDim.x + threadIdx.x;
   if (iz >= nz) return;
   double v[5] = {0, 0, 0, 0, 0};
@@ -429,12 +431,11 @@ static int tmunu_t(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab) {
   a.split = (int)split;
   a.part = c->tpart;
   double* tab = dev_tab ? dev_tab : c->tab;
-  k_tmunu<NC, R><<<dim3((unsigned)c->g.nz, (unsigned)split), kRedThreads, 0, c->stream>>>(a);
-  int st = cuda_check(cudaGetLastError(), "k_tmunu launch");
+  int st = launch_following("k_tmunu launch", k_tmunu<NC, R>, dim3((unsigned)c->g.nz, (unsigned)split), kRedThreads, 0,
+                            c->stream, a);
   if (st) return st;
-  k_tmunu_fold<<<(c->g.nz + 127) / 128, 128, 0, c->stream>>>(c->tpart, (int)split, c->g.nz, 1.0 / (double)c->g.nxy,
-                                                              tab);
-  st = cuda_check(cudaGetLastError(), "k_tmunu_fold launch");
+  st = launch_following("k_tmunu_fold launch", k_tmunu_fold, (c->g.nz + 127) / 128, 128, 0, c->stream, c->tpart,
+                        (int)split, c->g.nz, 1.0 / (double)c->g.nxy, tab);
   if (st || !host_tab) return st;
   st = cuda_check(cudaMemcpyAsync(host_tab, c->tab, sizeof(double) * 4 * c->g.nz, cudaMemcpyDeviceToHost,
                                   c->stream),

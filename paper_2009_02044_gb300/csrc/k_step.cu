@@ -26,6 +26,7 @@ template <> struct StepOcc<double> {
 
 template <int NC, typename R>
 __global__ void __launch_bounds__(3 * StepOcc<R>::sites, StepOcc<R>::blocks) k_step_leapfrog(StepArgs<R> a) {
+  follow();
   step_link<NC, R>(a, (int)threadIdx.y, blockIdx.x * blockDim.x + threadIdx.x, (int)blockIdx.y + a.zlo);
 }
 
@@ -51,8 +52,8 @@ static int launch_t(glasma_ctx* c, bool hop) {
   a.zlo = c->lo;
   const int bs = StepOcc<R>::sites;
   const unsigned ntb = (unsigned)((c->g.nxy + bs - 1) / bs);
-  k_step_leapfrog<NC, R><<<dim3(ntb, (unsigned)(c->hi - c->lo)), dim3(bs, 3), 0, c->stream>>>(a);
-  return cuda_check(cudaGetLastError(), "k_step_leapfrog launch");
+  return launch_following("k_step_leapfrog launch", k_step_leapfrog<NC, R>, dim3(ntb, (unsigned)(c->hi - c->lo)),
+                          dim3(bs, 3), 0, c->stream, a);
 }
 
 // FP32 only: two sites per thread, (t, iz) and (t, iz + H) with

@@ -157,6 +157,7 @@ __device__ __forceinline__ Vec3 site_hop(const StepArgs<float>& a, int iz, uint3
 
 __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_site(StepArgs<float> a, int zlen,
                                                                                  int zhi) {
+  follow();
   const Geom& g = a.g;
   const uint32_t t = blockIdx.x * kSiteThreads + threadIdx.x;
   if (t >= (uint32_t)g.nxy) return;
@@ -278,9 +279,9 @@ int launch_step_site(glasma_ctx* c, bool hop) {
   int64_t zlen = tiles * nsl / (4 * (int64_t)c->sms * kSiteBlocks);
   if (zlen < 1) zlen = 1;
   if (zlen > 32) zlen = 32;
-  k_step_leapfrog_site<<<dim3((unsigned)tiles, (unsigned)((nsl + zlen - 1) / zlen)), kSiteThreads, 0, c->stream>>>(
-      a, (int)zlen, c->hi);
-  return cuda_check(cudaGetLastError(), "k_step_leapfrog_site launch");
+  return launch_following("k_step_leapfrog_site launch", k_step_leapfrog_site,
+                          dim3((unsigned)tiles, (unsigned)((nsl + zlen - 1) / zlen)), kSiteThreads, 0, c->stream, a,
+                          (int)zlen, c->hi);
 }
 
 }  // namespace glasma
