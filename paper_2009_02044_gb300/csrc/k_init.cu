@@ -324,10 +324,10 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
       }
       // E vanishes off the nuclei: no FP64 work there
       if (here)
-        for (int c = 0; c < NA; ++c) dv[c] += w * (double)e[c];
+        for (int c = 0; c < NA; ++c) dv[c] += w * widen<double>(e[c]);
       if (!below) continue;
       double q[NA];
-      for (int c = 0; c < NA; ++c) q[c] = (double)em[c];
+      for (int c = 0; c < NA; ++c) q[c] = widen<double>(em[c]);
       typename G::M um = LinkIO<NC, R>::template load<double>(U, i, g.V, n.m[i]);
       G::adj_dag(um, q);
       for (int c = 0; c < NA; ++c) dv[c] -= w * q[c];

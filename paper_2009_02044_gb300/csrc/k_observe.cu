@@ -59,11 +59,11 @@ __global__ void __launch_bounds__(kRedThreads) k_gauss(GaussArgs<R> a) {
     for (int i = 0; i < 3; ++i) {
       double q[NA];
 #pragma unroll
-      for (int c = 0; c < NA; ++c) gv[c] += a.ia2[i] * (double)a.E[(int64_t)(i * NA + c) * a.g.V + s];
+      for (int c = 0; c < NA; ++c) gv[c] += a.ia2[i] * widen<double>(a.E[(int64_t)(i * NA + c) * a.g.V + s]);
       if (i == 2 && n.iz == 0) continue;
       const int64_t sm = n.m[i];
 #pragma unroll
-      for (int c = 0; c < NA; ++c) q[c] = (double)a.E[(int64_t)(i * NA + c) * a.g.V + sm];
+      for (int c = 0; c < NA; ++c) q[c] = widen<double>(a.E[(int64_t)(i * NA + c) * a.g.V + sm]);
       typename G::M um = LinkIO<NC, R>::template load<double>(a.U, i, a.g.V, sm);
       G::adj_dag(um, q);
 #pragma unroll
@@ -76,10 +76,10 @@ __global__ void __launch_bounds__(kRedThreads) k_gauss(GaussArgs<R> a) {
     const int ka = n.iz - a.zA0, kb = n.iz - a.zB0;
     if (ka >= 0 && ka < a.WA)
 #pragma unroll
-      for (int c = 0; c < NA; ++c) rho[c] += (double)a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t];
+      for (int c = 0; c < NA; ++c) rho[c] += widen<double>(a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t]);
     if (kb >= 0 && kb < a.WB)
 #pragma unroll
-      for (int c = 0; c < NA; ++c) rho[c] += (double)a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t];
+      for (int c = 0; c < NA; ++c) rho[c] += widen<double>(a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t]);
 #pragma unroll
     for (int c = 0; c < NA; ++c) {
       double r = gv[c] - rho[c];
