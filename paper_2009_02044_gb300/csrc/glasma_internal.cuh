@@ -94,10 +94,7 @@ GL_HD bool hop_at(long long n, long long p, long long q) {
 // Launch a kernel that begins with follow(): it may be set up, and its first
 // blocks placed, while the kernel before it in the stream runs out.  Small
 // lattices spend their time between launches (us per step: SU(2) FP32 100 x 9 x 7
-// 6.3 -> 3.8, 200 x 30 x 20 12.6 -> 10.6; SU(3) FP32 131 x 45 x 48 73.0 -> 70.3).  Not
-// for kernels that the FP64 pipe bounds: blocks placed early crowd on the SMs
-// that had room first, and the pipes of the others idle (SU(2) 128 x 16^2, two
-// passes, 37 -> 49).
+// 6.3 -> 3.8, 200 x 30 x 20 12.6 -> 10.6; SU(3) FP32 131 x 45 x 48 73.0 -> 70.3).
 template <typename... P, typename... A>
 int launch_following(const char* what, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
@@ -120,6 +117,11 @@ __device__ __forceinline__ void follow() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// The same, the next kernel set up but not placed before this one is over: for
+// kernels that the FP64 pipe bounds.  Blocks placed early crowd on the SMs that
+// have room first, and the pipes of the others idle (SU(2) FP64 128 x 16^2, two
+// passes per step: 37 us by plain launches, 49 with follow, 32 with this).
+__device__ __forceinline__ void follow_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 
 // kernel launchers

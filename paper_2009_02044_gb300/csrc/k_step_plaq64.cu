@@ -20,9 +20,9 @@
 // warm-up slice in shared memory, no work is done twice, and threads of both
 // passes are numbered straight through the sites, so a small lattice spreads
 // over all SMs and a plane of any size fills its warps.
-// Measured, whole events in FP64 against the marching form: SU(2) 128 x 16^2,
-// 100 steps, 19.7 -> 4.56 ms; SU(3) 160 x 24^2, 40 steps, 61.6 -> 21.0 ms (both
-// with the series exponentials of su_n.cuh, which came with it).
+// Measured against the marching form, ms per step: SU(2) 128 x 16^2 0.191 -> 0.031, 512 x 64^2 2.45 -> 1.6; SU(3) 160 x 24^2 1.47 -> 0.449,
+// 512 x 64^2 12.3 -> 10.1 (with the series exponentials of su_n.cuh, which came
+// with it).
 //
 // The scratch holds a ring of slices (nine vectors per site).  A lattice whose
 // vectors pass kPartsBytes is stepped in chunks of slices; chunk k's parts
@@ -39,7 +39,7 @@ namespace glasma {
 // context steps with the staple kernel
 constexpr size_t kPartsBytes = (size_t)64 << 20;
 constexpr size_t kPartsMost = (size_t)512 << 20;
-constexpr int kPartsThreads = 128;
+constexpr int kPartsThreads = 64;  // 128 left a sixth of the SMs' FP64 pipes idle on 128 x 16^2
 
 // vectors per site: p0 of the planes xy, xz, yz, then their pAB, then pBA
 enum { kP0 = 0, kPAB = 3, kPBA = 6, kPartVecs = 9 };
@@ -84,7 +84,8 @@ struct PlaqCorners<2> {
 };
 
 template <int NC>
-__global__ void __launch_bounds__(kPartsThreads, 2) k_step_plaq_parts(PartsArgs a) {
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs a) {
+  follow_last();
   typedef Group<NC, double> G;
   typedef LinkIO<NC, double> IO;
   typedef typename G::M M;
@@ -125,7 +126,8 @@ struct PartLinksArgs {
 };
 
 template <int NC>
-__global__ void __launch_bounds__(kPartsThreads, 2) k_step_plaq_links(PartLinksArgs pa) {
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links(PartLinksArgs pa) {
+  follow_last();
   constexpr int NA = Group<NC, double>::NA;
   const uint32_t idx = blockIdx.x * kPartsThreads + threadIdx.x;
   if (idx >= pa.sites) return;
@@ -208,11 +210,15 @@ static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
     p.zfirst = z0 == c->lo && z0 > 0 ? z0 - 1 : z0;
     p.sites = (uint32_t)((z1 - p.zfirst) * c->g.nxy);
     l.sites = (uint32_t)((z1 - z0) * c->g.nxy);
-    k_step_plaq_parts<NC><<<dim3((p.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream>>>(p);
-    k_step_plaq_links<NC><<<dim3((l.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream>>>(l);
+    int st = launch_following("k_step_plaq_parts launch", k_step_plaq_parts<NC>,
+                              dim3((p.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream, p);
+    if (!st)
+      st = launch_following("k_step_plaq_links launch", k_step_plaq_links<NC>,
+                            dim3((l.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream, l);
+    if (st) return st;
     *launches += 2;
   }
-  return cuda_check(cudaGetLastError(), "k_step_plaq_parts / _links launch");
+  return GLASMA_OK;
 }
 
 // zlen: slices per chunk (0: as many as the scratch holds)
