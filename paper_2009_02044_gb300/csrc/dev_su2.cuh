@@ -1,0 +1,60 @@
+// FP32 SU(2) links as quaternions of their deviation from 1 (link_alg.cuh):
+// (w, x, y, z) of alpha = 1 + w + i z, beta = y + i x, one 16-byte word each.
+// Every product is (1+a)(1+b) - 1 = b + a (1+b), so rounding stays of the size
+// of the deviations.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace glasma {
+
+struct Dev4 {  // a link, less 1
+  float w, x, y, z;
+};
+
+__device__ __forceinline__ Dev4 dev_load(const float4* p) {
+  const float4 v = __ldg(p);  // (alpha.re - 1, alpha.im, beta.re, beta.im)
+  return Dev4{v.x, v.w, v.z, v.y};
+}
+__device__ __forceinline__ Dev4 dev_dag(Dev4 a) { return Dev4{a.w, -a.x, -a.y, -a.z}; }
+// (w + i a.s)(v + i b.s) = (w v - a.b) + i (w b + v a - a x b).s
+__device__ __forceinline__ Dev4 dev_mul(Dev4 a, Dev4 b) {
+  const float v = 1.f + b.w;
+  return Dev4{fma(a.w, v, fma(-a.x, b.x, fma(-a.y, b.y, fma(-a.z, b.z, b.w)))),
+              fma(a.w, b.x, fma(v, a.x, fma(-a.y, b.z, fma(a.z, b.y, b.x)))),
+              fma(a.w, b.y, fma(v, a.y, fma(-a.z, b.x, fma(a.x, b.z, b.y)))),
+              fma(a.w, b.z, fma(v, a.z, fma(-a.x, b.y, fma(a.y, b.x, b.z))))};
+}
+
+struct Vec3 {
+  float x, y, z;
+};
+__device__ __forceinline__ Vec3 cross3(Vec3 a, Vec3 b) {
+  return Vec3{fma(a.y, b.z, -(a.z * b.y)), fma(a.z, b.x, -(a.x * b.z)), fma(a.x, b.y, -(a.y * b.x))};
+}
+__device__ __forceinline__ void add3(Vec3& f, float w, Vec3 v) {
+  f.x = fma(w, v.x, f.x);
+  f.y = fma(w, v.y, f.y);
+  f.z = fma(w, v.z, f.z);
+}
+// the part of vec AB and vec BA that is the same, a (1 + B.w) + b (1 + A.w)
+__device__ __forceinline__ Vec3 sym3(Dev4 A, Dev4 B) {
+  return Vec3{fma(A.w, B.x, fma(B.w, A.x, A.x + B.x)), fma(A.w, B.y, fma(B.w, A.y, A.y + B.y)),
+              fma(A.w, B.z, fma(B.w, A.z, A.z + B.z))};
+}
+__device__ __forceinline__ Vec3 vec3(Dev4 a) { return Vec3{a.x, a.y, a.z}; }
+// vec AB = sym - a x b
+__device__ __forceinline__ Vec3 vec_ab(Dev4 A, Dev4 B) {
+  const Vec3 s = sym3(A, B), c = cross3(vec3(A), vec3(B));
+  return Vec3{s.x - c.x, s.y - c.y, s.z - c.z};
+}
+// v <- U v U^+, operation for operation Group<2>::rotate: a slab's halo charge
+// hops there (k_slab_halo_hop), and its owner's here
+__device__ __forceinline__ Vec3 turn3(Dev4 u, Vec3 v) {
+  const Vec3 c = cross3(vec3(u), v);
+  const float w = 1.f + u.w;
+  return Vec3{fma(2.f, fma(u.y, c.z, fma(-u.z, c.y, -(w * c.x))), v.x),
+              fma(2.f, fma(u.z, c.x, fma(-u.x, c.z, -(w * c.y))), v.y),
+              fma(2.f, fma(u.x, c.y, fma(-u.y, c.x, -(w * c.z))), v.z)};
+}
+
+}  // namespace glasma

@@ -20,11 +20,7 @@
 // The fields are loaded at the start of a slice (loaded where they are used,
 // behind the stores of the link before, they cost a memory latency per link:
 // 0.79 -> 0.61 ms), and the lines of the next slice are brought to L2 (0.59).
-//
-// Links are stored as deviations from 1 (link_alg.cuh): quaternions (w, x, y,
-// z) of alpha = 1 + w + i z, beta = y + i x, one 16-byte word each.  Every
-// product is (1+a)(1+b) - 1 = b + a (1+b), so rounding stays of the size of
-// the deviations.
+#include "dev_su2.cuh"
 #include "step_link.cuh"
 
 namespace glasma {
@@ -34,53 +30,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 
 constexpr int kSiteThreads = 256;  // consecutive transverse sites of a block
 constexpr int kSiteBlocks = 3;     // blocks per SM
-
-struct Dev4 {  // a link, less 1
-  float w, x, y, z;
-};
-
-__device__ __forceinline__ Dev4 dev_load(const float4* p) {
-  const float4 v = __ldg(p);  // (alpha.re - 1, alpha.im, beta.re, beta.im)
-  return Dev4{v.x, v.w, v.z, v.y};
-}
-__device__ __forceinline__ Dev4 dev_dag(Dev4 a) { return Dev4{a.w, -a.x, -a.y, -a.z}; }
-// (w + i a.s)(v + i b.s) = (w v - a.b) + i (w b + v a - a x b).s
-__device__ __forceinline__ Dev4 dev_mul(Dev4 a, Dev4 b) {
-  const float v = 1.f + b.w;
-  return Dev4{fma(a.w, v, fma(-a.x, b.x, fma(-a.y, b.y, fma(-a.z, b.z, b.w)))),
-              fma(a.w, b.x, fma(v, a.x, fma(-a.y, b.z, fma(a.z, b.y, b.x)))),
-              fma(a.w, b.y, fma(v, a.y, fma(-a.z, b.x, fma(a.x, b.z, b.y)))),
-              fma(a.w, b.z, fma(v, a.z, fma(-a.x, b.y, fma(a.y, b.x, b.z))))};
-}
-
-struct Vec3 {
-  float x, y, z;
-};
-__device__ __forceinline__ Vec3 cross3(Vec3 a, Vec3 b) {
-  return Vec3{fma(a.y, b.z, -(a.z * b.y)), fma(a.z, b.x, -(a.x * b.z)), fma(a.x, b.y, -(a.y * b.x))};
-}
-__device__ __forceinline__ void add3(Vec3& f, float w, Vec3 v) {
-  f.x = fma(w, v.x, f.x);
-  f.y = fma(w, v.y, f.y);
-  f.z = fma(w, v.z, f.z);
-}
-// the part of vec AB and vec BA that is the same, a (1 + B.w) + b (1 + A.w)
-__device__ __forceinline__ Vec3 sym3(Dev4 A, Dev4 B) {
-  return Vec3{fma(A.w, B.x, fma(B.w, A.x, A.x + B.x)), fma(A.w, B.y, fma(B.w, A.y, A.y + B.y)),
-              fma(A.w, B.z, fma(B.w, A.z, A.z + B.z))};
-}
-__device__ __forceinline__ Vec3 vec3(Dev4 a) { return Vec3{a.x, a.y, a.z}; }
-// vec AB = sym - a x b
-__device__ __forceinline__ Vec3 vec_ab(Dev4 A, Dev4 B) {
-  const Vec3 s = sym3(A, B), c = cross3(vec3(A), vec3(B));
-  return Vec3{s.x - c.x, s.y - c.y, s.z - c.z};
-}
-// v <- U v U^+ (Group<2>::rotate)
-__device__ __forceinline__ Vec3 turn3(Dev4 u, Vec3 v) {
-  const Vec3 n = vec3(u), c = cross3(n, v), d = cross3(n, c);
-  const float w = 1.f + u.w;
-  return Vec3{fma(2.f, fma(-w, c.x, d.x), v.x), fma(2.f, fma(-w, c.y, d.y), v.y), fma(2.f, fma(-w, c.z, d.z), v.z)};
-}
 
 // exp(i dt e.sigma/2) u, of unit norm: cos(th) - 1 and sin(th) / th by their
 // series in th^2 <= 1/4 (remainders below 2e-11).

@@ -1,0 +1,107 @@
+"""The kernels that a context takes by its sizes and types, each at the edges
+of its range and against the general path: the FP64 step in two passes (its
+ring of slices wrapping, rows longer than a block, planes whose scratch holds
+two slices), the FP32 SU(2) step with one thread per site (from 2^17 sites
+on), T^{mu nu} of SU(2), and the FP32 -> FP64 conversion of the observables."""
+import numpy as np
+import pytest
+
+import glasma_inputs as gi
+from oracle import glasma_oracle as O
+from test_gpu_slab import _compare, _run
+from test_gpu_step_kernels import G, TOL64, _ctx, _random_state, rel  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def _step_both(G, st, precision, steps, tol):
+    out = []
+    for kernel in ("staple", "auto"):
+        h = _ctx(G, st, precision)
+        G.glasma_set_step_kernel(h, kernel)
+        G.glasma_step(h, steps)
+        out.append(G.glasma_get_fields(h)[:4])
+        G.glasma_free(h)
+    errs = [rel(b, a) for a, b in zip(*out)]
+    assert all(e <= tol for e in errs), errs
+
+
+@pytest.mark.parametrize("nc,shape", [
+    (2, (40, 96, 96)), (3, (20, 96, 96)),   # 64 MB hold 32 and 12 slices: the ring wraps
+    (2, (7, 3, 400)), (3, (6, 1, 513)),     # rows that the marching kernel does not take
+    (3, (5, 256, 256)),                     # two slices of scratch, one per chunk
+    (2, (9, 9, 7)), (3, (5, 1, 1))])        # a last block of 55, and of 5, threads
+def test_fp64_two_passes_match_the_staple_form(G, nc, shape):
+    """Two orders of the same FP64 sums over three steps: the FP64 target."""
+    _step_both(G, _random_state(nc, *shape, seed=sum(shape) + nc), "fp64", 3, TOL64)
+
+
+@pytest.mark.parametrize("shape", [
+    (32, 64, 64), (140, 31, 31), (131, 1, 1001), (4099, 32, 1), (9, 121, 121)])
+def test_su2_fp32_site_kernel_matches_the_staple_form(G, shape):
+    """2^17 sites and a little more, with planes that end within a warp and
+    planes of one row or column.  Each form stays within 1.5e-6 of the FP64
+    step after three steps (the bound of the FP32 random-state test), so two
+    of them within 3e-6 of one another."""
+    _step_both(G, _random_state(2, *shape, seed=sum(shape)), "fp32", 3, 3e-6)
+
+
+@pytest.mark.parametrize("nranks", [2, 3])
+def test_su2_fp32_site_kernel_on_slabs(G, nranks):
+    """The rule counts the whole lattice's sites, so slabs below 2^17 sites of
+    a lattice above it take the same kernel: bitwise the whole lattice."""
+    cfg = dict(gi.small_config(2, nz=47, nx=53, ny=54, sigma_l=2.0), precision="fp32")
+    whole, ranks, T = _run(G, cfg, nranks, 44, "auto")
+    _compare(G, cfg, whole, ranks, T)
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", TOL64), ("fp32", 1e-5)])
+@pytest.mark.parametrize("shape", [
+    (6, 1, 1), (6, 1, 2), (7, 2, 1), (9, 17, 15), (6, 33, 67), (5, 3, 400)])
+def test_su2_tmunu_matches_oracle(G, shape, precision, tol):
+    """Slices below, at and above a block's 256 sites, and planes of one row
+    or column.  FP32: each entry is a mean of products of at most eight
+    rounded factors of O(1), 8 * 6e-8 absolute, against means of O(0.1)."""
+    st = _random_state(2, *shape, seed=sum(shape))
+    h = _ctx(G, st, precision)
+    G.glasma_step(h, 1)
+    tab, H = G.glasma_tmunu(h)
+    rtab, rH = O.tmunu(O.step(st, 1))
+    assert rel(tab, rtab) <= tol and abs(H - rH) <= tol * abs(rH)
+
+
+@pytest.mark.parametrize("angle", [1e-4, 0.7, 3.0, 25.0])
+@pytest.mark.parametrize("nc", [2, 3])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_link_update_at_any_angle(G, nc, angle, precision):
+    """exp(-i dt E) by a short series for small |dt E| and by the closed form
+    beyond, up to several turns.  FP32: E carries 6e-8 relative, so a link
+    turns by the angle with an error of 6e-8 * angle, beside the rounding of
+    the product; E itself, set by a force of O(1), is far below the angle's."""
+    st = _random_state(nc, 7, 5, 9, seed=17)
+    st.E *= angle / (st.p.dt * np.max(np.abs(st.E)))
+    ref = O.step(st, 2)
+    for kernel in ("auto", "staple"):
+        h = _ctx(G, st, precision)
+        G.glasma_set_step_kernel(h, kernel)
+        G.glasma_step(h, 2)
+        U, E = G.glasma_get_fields(h)[:2]
+        tol = TOL64 if precision == "fp64" else 1.5e-6 * (1 + angle)
+        assert rel(U, ref.U) <= tol and rel(E, ref.E) <= tol, kernel
+        G.glasma_free(h)
+
+
+@pytest.mark.parametrize("scale", [1.5e-45, 3e-40, 1.2e-38, 1.0, 1e30])
+def test_fp32_fields_are_widened_exactly(G, scale):
+    """The Gauss residual of FP32 fields on unit links is an FP64 sum of their
+    exact values, denormals among them."""
+    st = _random_state(2, 6, 5, 7, seed=3)
+    st.U[:] = np.eye(2)
+    rng = np.random.default_rng(5)
+    st.E = (scale * rng.integers(-7, 8, st.E.shape)).astype(np.float32).astype(np.float64)
+    st.E[2][st.p.nz - 1] = 0.0
+    st.QA[:] = 0.0
+    st.QB[:] = 0.0
+    g = G.glasma_gauss_residual(_ctx(G, st, "fp32"))
+    ref = O.gauss_residual(st)
+    assert abs(g[0] - ref[0]) <= 1e-14 * ref[0]
