@@ -2,20 +2,22 @@
 // (Sec. 3, Eq. gauss) and the per-slice energy-momentum tensor (Sec. 4).
 // Reductions are deterministic: fixed grid, fixed-order tree in shared
 // memory, fixed-order final pass over the block partials.
+#include "dev_su2.cuh"
 #include "glasma_internal.cuh"
 
 namespace glasma {
 
 constexpr int kRedThreads = 256;
+constexpr int kSu2Threads = 128;  // k_tmunu_su2
 
 // In-block tree reduction of NV doubles per thread; op 0 = sum, 1 = max.
-template <int NV>
-__device__ void block_reduce(double (*sh)[kRedThreads], double* v, const int* op) {
+template <int NV, int T>
+__device__ void block_reduce(double (*sh)[T], double* v, const int* op) {
   const int t = threadIdx.x;
 #pragma unroll
   for (int k = 0; k < NV; ++k) sh[k][t] = v[k];
   __syncthreads();
-  for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+  for (int w = T / 2; w > 0; w >>= 1) {
     if (t < w) {
 #pragma unroll
       for (int k = 0; k < NV; ++k)
@@ -191,6 +193,7 @@ struct TmnArgs {
   int hop;
   int zA0, WA, zB0, WB;
   int split;     // blocks per z slice
+  uint32_t per;  // consecutive sites of a block, a multiple of its threads
   double* part;  // [nz][split][5] block sums of eps, p_L, p_T, S_L, non-finite count
 };
 
@@ -244,18 +247,41 @@ struct SiteSum<float> {
   __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
 
+// The block's sums of E_x^2 + E_y^2, E_z^2, b_xy, b_xz + b_yz (without the
+// spacings) and E B as its row of partial sums.
+template <typename R, int T>
+__device__ __forceinline__ void tmunu_write(const TmnArgs<R>& a, double (*sh)[T], const SiteSum<R>& et,
+                                            const SiteSum<R>& ez, const SiteSum<R>& bl, const SiteSum<R>& bt,
+                                            const SiteSum<R>& sl) {
+  double v[5] = {et.get(), ez.get(), bl.get(), bt.get(), sl.get()};
+  const int op[5] = {0, 0, 0, 0, 0};
+  block_reduce<5>(sh, v, op);
+  if (threadIdx.x == 0) {
+    // eps, p_L, p_T, S_L and whether a value was not finite (the directions x
+    // and y have the same spacing)
+    const double e_t = 0.5 * v[0] * a.hinv2[0], e_z = 0.5 * v[1] * a.hinv2[2];
+    const double b_l = v[2] * a.binv[0], b_t = v[3] * a.binv[1];
+    const double p_t = e_z + b_l;
+    double* out = a.part + ((int64_t)blockIdx.x * a.split + blockIdx.y) * 5;
+    out[0] = e_t + e_z + b_l + b_t;
+    out[1] = e_t + b_t - p_t;
+    out[2] = p_t;
+    out[3] = v[4] * a.slc[0];
+    out[4] = isfinite(out[0]) && isfinite(out[3]) ? 0.0 : 1.0;
+  }
+}
+
 // Blocks per SM.  SU(3) FP32: 2 at 128 registers (16 warps; load latency is
 // what is left).
 template <int NC, typename R> struct TmnOcc { static constexpr int blocks = 1; };
 template <> struct TmnOcc<3, float> { static constexpr int blocks = 2; };
-template <> struct TmnOcc<2, float> { static constexpr int blocks = 4; };
 
 // Per-site arithmetic in the state's precision R (FP32 plaquette products in
 // the deviation form; the per-site sums of squares and of E B products in R,
 // all of positive terms except the Poynting sum), every accumulation over sites
-// as SiteSum, in FP64 between threads.  Block (iz, p) takes the sites
-// t = p*256 + threadIdx.x + k*split*256 of slice iz; k_tmunu_fold adds the
-// split block sums of a slice in a fixed order.
+// as SiteSum, in FP64 between threads.  Block (iz, p) takes `per` consecutive
+// sites of slice iz, 256 at a time (neighbouring rows meet in L1); k_tmunu_fold
+// adds the split block sums of a slice in a fixed order.
 // The plaquettes based at a site serve three ends at once: their energy, the
 // field B, and the forward half of the force on both their links; only the
 // backward staples are formed for the force alone.  That is 23 link products
@@ -274,7 +300,8 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
   const int iz = blockIdx.x;
   // sums of E_x^2 + E_y^2, E_z^2, b_xy, b_xz + b_yz (without the spacings), E B
   SiteSum<R> et, ez, bl, bt, sl;
-  for (uint32_t t = blockIdx.y * blockDim.x + threadIdx.x; t < (uint32_t)g.nxy; t += a.split * blockDim.x) {
+  for (uint32_t t = blockIdx.y * a.per + threadIdx.x, end = min((blockIdx.y + 1) * a.per, (uint32_t)g.nxy); t < end;
+       t += kRedThreads) {
     const SiteNbr n = site_nbr_tz(g, t, iz);
     const int64_t s = n.s;
     // plaquettes based here: b_ij = ||U_i(x) U_j(x+i) - U_j(x) U_i(x+j)||_F^2
@@ -361,22 +388,120 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
       }
     }
   }
-  double v[5] = {et.get(), ez.get(), bl.get(), bt.get(), sl.get()};
-  const int op[5] = {0, 0, 0, 0, 0};
-  block_reduce<5>(sh, v, op);
-  if (threadIdx.x == 0) {
-    // eps, p_L, p_T, S_L and whether a value was not finite (the directions x
-    // and y have the same spacing)
-    const double e_t = 0.5 * v[0] * a.hinv2[0], e_z = 0.5 * v[1] * a.hinv2[2];
-    const double b_l = v[2] * a.binv[0], b_t = v[3] * a.binv[1];
-    const double p_t = e_z + b_l;
-    double* out = a.part + ((int64_t)iz * a.split + blockIdx.y) * 5;
-    out[0] = e_t + e_z + b_l + b_t;
-    out[1] = e_t + b_t - p_t;
-    out[2] = p_t;
-    out[3] = v[4] * a.slc[0];
-    out[4] = isfinite(out[0]) && isfinite(out[3]) ? 0.0 : 1.0;
+  tmunu_write(a, sh, et, ez, bl, bt, sl);
+}
+
+// The same for FP32 SU(2) in the quaternion form of k_step_su2.cu: the six
+// backward staples are values vec AB, vec BA of the plaquettes at x - e_x, x -
+// e_y and x - e_z (46 multiply-adds each, where the general form takes two
+// products and a projection), and the fields are loaded before anything else.
+// Load latency and the waves of blocks bound it: 8 blocks of 128 threads per SM
+// at 64 registers (120 B of spills) take, on SU(2) 1024 x 128^2, 768 x 64^2 and
+// 131 x 45 x 48, 0.61, 0.137 and 0.022 ms (general form 0.94, 0.227 and 0.027);
+// 6 blocks at 80 registers 0.69, 0.159 and 0.021, blocks of 256 at 64 registers
+// 0.63, 0.176 and 0.026.
+__global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) {
+  follow();
+  __shared__ double sh[5][kSu2Threads];
+  const Geom& g = a.g;
+  const int iz = blockIdx.x;
+  const bool up = iz < g.nz - 1, down = iz > 0;
+  const uint32_t nx = (uint32_t)g.nx, ny = (uint32_t)g.ny;
+  const float4* Ux = reinterpret_cast<const float4*>(a.U) + (int64_t)iz * g.nxy;
+  const float4 *Uy = Ux + g.V, *Uz = Uy + g.V;
+  const float wt = a.w[0], wz = a.w[2];
+  SiteSum<float> et, ez, bl, bt, sl;
+  auto dist2 = [](Dev4 A, Dev4 B) {  // ||A - B||_F^2
+    const float w = A.w - B.w, x = A.x - B.x, y = A.y - B.y, z = A.z - B.z;
+    return 2.f * fma(w, w, fma(x, x, fma(y, y, z * z)));
+  };
+  for (uint32_t t = blockIdx.y * a.per + threadIdx.x, end = min((blockIdx.y + 1) * a.per, (uint32_t)g.nxy); t < end;
+       t += kSu2Threads) {
+    const uint32_t iy = t / nx, ix = t - iy * nx;
+    const uint32_t xp = ix + 1 == nx ? 0 : ix + 1, xm = ix == 0 ? nx - 1 : ix - 1;
+    const uint32_t yp = (iy + 1 == ny ? 0 : iy + 1) * nx, ym = (iy == 0 ? ny - 1 : iy - 1) * nx, y0 = iy * nx;
+    const uint32_t txp = y0 + xp, txm = y0 + xm, typ = yp + ix, tym = ym + ix, txmyp = yp + xm, txpym = ym + xp;
+    const int64_t s = (int64_t)iz * g.nxy + t;
+    Vec3 E[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float* e = a.E + (int64_t)(3 * i) * g.V + s;
+      E[i] = Vec3{e[0], e[g.V], e[2 * g.V]};
+    }
+    const Dev4 ux = dev_load(Ux + t), uy = dev_load(Uy + t);
+    Dev4 uz{0.f, 0.f, 0.f, 0.f};
+    Vec3 F[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, pxz{0.f, 0.f, 0.f}, pyz = pxz;
+    {
+      const Dev4 A = dev_mul(ux, dev_load(Uy + txp)), B = dev_mul(uy, dev_load(Ux + typ));
+      bl.add(dist2(A, B));
+      const Vec3 p = vec_ab(A, dev_dag(B));
+      add3(F[0], -wt, p);
+      add3(F[1], wt, p);
+    }
+    if (up) {
+      uz = dev_load(Uz + t);
+      Dev4 A = dev_mul(ux, dev_load(Uz + txp)), B = dev_mul(uz, dev_load(Ux + g.nxy + t));
+      bt.add(dist2(A, B));
+      pxz = vec_ab(A, dev_dag(B));
+      A = dev_mul(uy, dev_load(Uz + typ));
+      B = dev_mul(uz, dev_load(Uy + g.nxy + t));
+      bt.add(dist2(A, B));
+      pyz = vec_ab(A, dev_dag(B));
+      add3(F[0], -wz, pxz);
+      add3(F[1], -wz, pyz);
+      add3(F[2], wt, pxz);
+      add3(F[2], wt, pyz);
+    }
+    {
+      const Dev4 vx = dev_load(Ux + txm);
+      add3(F[1], -wt, vec_ab(dev_mul(uy, dev_dag(dev_load(Ux + txmyp))), dev_mul(dev_dag(dev_load(Uy + txm)), vx)));
+      if (up)
+        add3(F[2], -wt,
+             vec_ab(dev_mul(uz, dev_dag(dev_load(Ux + g.nxy + txm))), dev_mul(dev_dag(dev_load(Uz + txm)), vx)));
+    }
+    {
+      const Dev4 vy = dev_load(Uy + tym);
+      add3(F[0], wt, vec_ab(dev_mul(dev_dag(vy), dev_load(Ux + tym)), dev_mul(dev_load(Uy + txpym), dev_dag(ux))));
+      if (up)
+        add3(F[2], -wt,
+             vec_ab(dev_mul(uz, dev_dag(dev_load(Uy + g.nxy + tym))), dev_mul(dev_dag(dev_load(Uz + tym)), vy)));
+    }
+    if (down) {  // vec BA of the planes xz and yz of the slice below
+      const Dev4 vz = dev_dag(dev_load(Uz - g.nxy + t));
+      add3(F[0], wz, vec_ab(dev_mul(vz, dev_load(Ux - g.nxy + t)), dev_mul(dev_load(Uz - g.nxy + txp), dev_dag(ux))));
+      add3(F[1], wz, vec_ab(dev_mul(vz, dev_load(Uy - g.nxy + t)), dev_mul(dev_load(Uz - g.nxy + typ), dev_dag(uy))));
+    }
+    Vec3 dj{0.f, 0.f, 0.f};
+    if (a.hop && up) {
+      const int kb = iz - a.zB0, ka = iz + 1 - a.zA0;
+      if (kb >= 0 && kb < a.WB) {
+        const float* q = a.QB + (int64_t)kb * g.nxy + t;
+        const int64_t S = (int64_t)a.WB * g.nxy;
+        add3(dj, -a.az2, Vec3{q[0], q[S], q[2 * S]});
+      }
+      if (ka >= 0 && ka < a.WA) {
+        const float* q = a.QA + (int64_t)ka * g.nxy + t;
+        const int64_t S = (int64_t)a.WA * g.nxy;
+        add3(dj, a.az2, turn3(uz, Vec3{q[0], q[S], q[2 * S]}));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      Vec3 n = E[i];
+      add3(n, a.dt, F[i]);
+      if (i == 2) n = Vec3{n.x + dj.x, n.y + dj.y, n.z + dj.z};
+      const float sq = fma(E[i].x, E[i].x, fma(E[i].y, E[i].y, E[i].z * E[i].z)) +
+                       fma(n.x, n.x, fma(n.y, n.y, n.z * n.z));
+      if (i == 2) {
+        if (up) ez.add(sq);  // no z link on the last slice
+      } else {
+        const Vec3 p = i == 0 ? pxz : pyz;
+        et.add(sq);
+        sl.add(fma(E[i].x + n.x, p.x, fma(E[i].y + n.y, p.y, (E[i].z + n.z) * p.z)));
+      }
+    }
   }
+  tmunu_write(a, sh, et, ez, bl, bt, sl);
 }
 
 // tab[iz] = (sum over the split blocks of slice iz, in block order) / nxy;
@@ -392,6 +517,15 @@ __global__ void k_tmunu_fold(const double* part, int split, int nz, double inv, 
 #pragma unroll
   for (int k = 0; k < 4; ++k) tab[iz * 4 + k] = v[k] * inv;
   if (v[4] != 0.0) tab[iz * 4 + 0] = __longlong_as_double(0x7ff8000000000000LL);  // NaN marks it
+}
+
+template <int NC, typename R>
+static int launch_tmunu_kernel(const TmnArgs<R>& a, dim3 grid, cudaStream_t s) {
+  return launch_following("k_tmunu launch", k_tmunu<NC, R>, grid, kRedThreads, 0, s, a);
+}
+template <>
+int launch_tmunu_kernel<2, float>(const TmnArgs<float>& a, dim3 grid, cudaStream_t s) {
+  return launch_following("k_tmunu_su2 launch", k_tmunu_su2, grid, kSu2Threads, 0, s, a);
 }
 
 template <int NC, typename R>
@@ -424,15 +558,18 @@ static int tmunu_t(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab) {
   // threads): the split, and with it the order of each slice's sums, depends
   // on the transverse plane alone, not on the number of slices or the device,
   // so a z slab's rows equal the whole lattice's bit for bit
-  const int64_t per_slice = (c->g.nxy + kRedThreads - 1) / kRedThreads;
+  const int threads = NC == 2 && sizeof(R) == 4 ? kSu2Threads : kRedThreads;
+  const int64_t per_slice = (c->g.nxy + threads - 1) / threads;
   int64_t split = kTmunuSplit;
   if (split > per_slice) split = per_slice;
   if (split < 1) split = 1;
+  const int64_t chunks = (per_slice + split - 1) / split;  // of a block; the last may have fewer
+  split = (per_slice + chunks - 1) / chunks;
+  a.per = (uint32_t)(chunks * threads);
   a.split = (int)split;
   a.part = c->tpart;
   double* tab = dev_tab ? dev_tab : c->tab;
-  int st = launch_following("k_tmunu launch", k_tmunu<NC, R>, dim3((unsigned)c->g.nz, (unsigned)split), kRedThreads, 0,
-                            c->stream, a);
+  int st = launch_tmunu_kernel<NC>(a, dim3((unsigned)c->g.nz, (unsigned)split), c->stream);
   if (st) return st;
   st = launch_following("k_tmunu_fold launch", k_tmunu_fold, (c->g.nz + 127) / 128, 128, 0, c->stream, c->tpart,
                         (int)split, c->g.nz, 1.0 / (double)c->g.nxy, tab);
