@@ -2,7 +2,7 @@
 // (Sec. 3, Eqs. lattice_1, plaquette, lattice_2, continuity).
 //
 // GB300 does two FP64 multiply-adds per SM and clock, so the FP64 step is
-// bound by their number, and device memory has time to spare (SU(3): some 2400
+// bound by their number, and device memory has time to spare (SU(3): some 2300
 // multiply-adds against 1.9 KB per site, 4.5 us against 0.3 us per 1000 sites).
 // Hence every plaquette is formed once, by a thread of its own, and what it
 // contributes to its four links goes through a scratch array:
@@ -14,15 +14,16 @@
 //                      directions of -+ w p0 and +- w pAB or pBA of the
 //                      plaquette below, then update_link.
 // Two products, two projections and one transport of an algebra vector are
-// 534 multiply-adds per SU(3) plaquette (594 with p0 from a third product)
-// and 68 per SU(2) plaquette, whose pAB and pBA differ in a cross product's
-// sign only.  Against a block that marches through z with a halo row and a
+// 510 multiply-adds per SU(3) plaquette (594 with p0 from a third product; 534,
+// and 0.449 and 10.1 ms per step in the list below, with all rows of A and B by
+// their sums) and 68 per SU(2) plaquette, whose pAB and pBA differ in a cross
+// product's sign only.  Against a block that marches through z with a halo row and a
 // warm-up slice in shared memory, no work is done twice, and threads of both
 // passes are numbered straight through the sites, so a small lattice spreads
 // over all SMs and a plane of any size fills its warps.
 // Measured against the marching form, ms per step: SU(2) 128 x 16^2 0.191 ->
-// 0.031, 512 x 64^2 2.45 -> 1.6; SU(3) 160 x 24^2 1.47 -> 0.449, 512 x 64^2 12.3 ->
-// 10.1 (with the series exponentials of su_n.cuh, which came with it).
+// 0.031, 512 x 64^2 2.45 -> 1.6; SU(3) 160 x 24^2 1.47 -> 0.438, 512 x 64^2 12.3 ->
+// 9.7 (with the series exponentials of su_n.cuh, which came with it).
 //
 // The scratch holds a ring of slices (nine vectors per site).  A lattice whose
 // vectors pass kPartsBytes is stepped in chunks of slices; chunk k's parts
@@ -59,6 +60,43 @@ struct PlaqCorners;
 template <>
 struct PlaqCorners<3> {
   typedef Group<3, double> G;
+  typedef G::M M;
+  // A product of links is a link: conj(row 0 x row 1) is its third row.
+  __device__ __forceinline__ static void third_row(M& t) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+      const cplx<double> a1 = t.m[k1], a2 = t.m[k2], b1 = t.m[3 + k1], b2 = t.m[3 + k2];
+      const cplx<double> c = fma_c(cplx<double>{-a2.re, -a2.im}, b1, a1 * b2);
+      t.m[6 + k] = cj(c);
+    }
+  }
+  __device__ __forceinline__ static M mul_d(const M& x, const M& y) {
+    M t;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        cplx<double> acc = mulc(x.m[3 * i], y.m[3 * j]);
+        acc = fma_cj(x.m[3 * i + 1], y.m[3 * j + 1], acc);
+        t.m[3 * i + j] = fma_cj(x.m[3 * i + 2], y.m[3 * j + 2], acc);
+      }
+    third_row(t);
+    return t;
+  }
+  __device__ __forceinline__ static M d_mul(const M& x, const M& y) {
+    M t;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        cplx<double> acc = mulc(y.m[j], x.m[i]);
+        acc = fma_cj(y.m[3 + j], x.m[3 + i], acc);
+        t.m[3 * i + j] = fma_cj(y.m[6 + j], x.m[6 + i], acc);
+      }
+    third_row(t);
+    return t;
+  }
   __device__ __forceinline__ static void both(const G::M& A, const G::M& B, double* ab, double* ba) {
     G::proj_mul(A, B, ab);
     G::proj_mul(B, A, ba);
@@ -68,6 +106,9 @@ struct PlaqCorners<3> {
 template <>
 struct PlaqCorners<2> {
   typedef Group<2, double> G;
+  typedef G::M M;
+  __device__ __forceinline__ static M mul_d(const M& x, const M& y) { return G::mul_d(x, y); }
+  __device__ __forceinline__ static M d_mul(const M& x, const M& y) { return G::d_mul(x, y); }
   // A = p + i a.sigma, B = q + i b.sigma: AB and BA have the vector parts
   // p b + q a -+ a x b
   __device__ __forceinline__ static void both(const G::M& A, const G::M& B, double* ab, double* ba) {
@@ -102,9 +143,9 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs 
   const int64_t S = (int64_t)a.ring * nxy;
   double* out = a.part + (int64_t)(z % a.ring) * nxy + t;
   const M ua = IO::template load<double>(a.U, da, g.V, n.s);
-  const M A = G::mul_d(IO::template load<double>(a.U, db, g.V, n.p[da]),
-                       IO::template load<double>(a.U, da, g.V, n.p[db]));
-  const M B = G::d_mul(IO::template load<double>(a.U, db, g.V, n.s), ua);
+  const M A = PlaqCorners<NC>::mul_d(IO::template load<double>(a.U, db, g.V, n.p[da]),
+                                     IO::template load<double>(a.U, da, g.V, n.p[db]));
+  const M B = PlaqCorners<NC>::d_mul(IO::template load<double>(a.U, db, g.V, n.s), ua);
   double ab[NA], ba[NA];
   PlaqCorners<NC>::both(A, B, ab, ba);
 #pragma unroll
