@@ -133,6 +133,8 @@ bool plaq_fits(const glasma_ctx* c);
 // (k_step_plaq64.cu): its ring's slices (0: none) and bytes
 int parts_ring(const glasma_ctx* c);
 size_t parts_bytes(const glasma_ctx* c);
+// first pass over the slices [z0, z1), with the plaquette norms
+int launch_parts_norms(glasma_ctx* c, int z0, int z1);
 int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches);
 // the step kernel glasma_step launches for this context: plaquette (FP64 in
 // two passes), staple on site pairs (FP32), staged staple (FP32 SU(3)) or

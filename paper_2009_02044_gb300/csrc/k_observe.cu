@@ -4,6 +4,7 @@
 // memory, fixed-order final pass over the block partials.
 #include "dev_su2.cuh"
 #include "glasma_internal.cuh"
+#include "plaq_parts.cuh"
 
 namespace glasma {
 
@@ -252,7 +253,7 @@ struct SiteSum<float> {
 template <typename R, int T>
 __device__ __forceinline__ void tmunu_write(const TmnArgs<R>& a, double (*sh)[T], const SiteSum<R>& et,
                                             const SiteSum<R>& ez, const SiteSum<R>& bl, const SiteSum<R>& bt,
-                                            const SiteSum<R>& sl) {
+                                            const SiteSum<R>& sl, int iz) {
   double v[5] = {et.get(), ez.get(), bl.get(), bt.get(), sl.get()};
   const int op[5] = {0, 0, 0, 0, 0};
   block_reduce<5>(sh, v, op);
@@ -262,7 +263,7 @@ __device__ __forceinline__ void tmunu_write(const TmnArgs<R>& a, double (*sh)[T]
     const double e_t = 0.5 * v[0] * a.hinv2[0], e_z = 0.5 * v[1] * a.hinv2[2];
     const double b_l = v[2] * a.binv[0], b_t = v[3] * a.binv[1];
     const double p_t = e_z + b_l;
-    double* out = a.part + ((int64_t)blockIdx.x * a.split + blockIdx.y) * 5;
+    double* out = a.part + ((int64_t)iz * a.split + blockIdx.y) * 5;
     out[0] = e_t + e_z + b_l + b_t;
     out[1] = e_t + b_t - p_t;
     out[2] = p_t;
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
       }
     }
   }
-  tmunu_write(a, sh, et, ez, bl, bt, sl);
+  tmunu_write(a, sh, et, ez, bl, bt, sl, iz);
 }
 
 // The same for FP32 SU(2) in the quaternion form of k_step_su2.cu: the six
@@ -501,7 +502,72 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
       }
     }
   }
-  tmunu_write(a, sh, et, ez, bl, bt, sl);
+  tmunu_write(a, sh, et, ez, bl, bt, sl, iz);
+}
+
+// FP64 where the context has the step's scratch: the plaquettes and the forces
+// come from the step's first pass (k_step_plaq64.cu), which forms each
+// plaquette once where k_tmunu forms 23 link products per site, and this pass
+// adds E_{n+1/2} and the sums.  The FP64 pipe bounds both: SU(3) 160 x 24^2 0.607 ->
+// 0.354 ms, 90 x 7 x 11 0.109 -> 0.055, 512 x 64^2 10.8 -> 7.8; SU(2) 128 x 16^2
+// 0.049 -> 0.035, 512 x 64^2 2.33 -> 1.55.
+template <int NC>
+__global__ void __launch_bounds__(kRedThreads) k_tmunu_parts(TmnArgs<double> a, const double* vecs, int ring, int z0) {
+  follow();
+  typedef Group<NC, double> G;
+  constexpr int NA = G::NA;
+  __shared__ double sh[5][kRedThreads];
+  const Geom& g = a.g;
+  const int iz = z0 + (int)blockIdx.x;
+  const bool up = iz < g.nz - 1;
+  const int64_t S = (int64_t)ring * g.nxy, here = (int64_t)(iz % ring) * g.nxy;
+  SiteSum<double> et, ez, bl, bt, sl;
+  for (uint32_t t = blockIdx.y * a.per + threadIdx.x, end = min((blockIdx.y + 1) * a.per, (uint32_t)g.nxy); t < end;
+       t += kRedThreads) {
+    const SiteNbr n = site_nbr_tz(g, t, iz);
+    const double* norm = vecs + (int64_t)kPartVecs * NA * S + here + t;
+    bl.add(norm[0]);
+    if (up) bt.add(norm[S] + norm[2 * S]);
+#pragma unroll 1
+    for (int i = 0; i < (up ? 3 : 2); ++i) {
+      double F[NA], eo[NA], en[NA];
+      part_force<NA>(vecs, g, ring, n, t, iz, i, a.w, F);
+#pragma unroll
+      for (int c = 0; c < NA; ++c) {
+        eo[c] = a.E[(int64_t)(i * NA + c) * g.V + n.s];
+        en[c] = fma(a.dt, F[c], eo[c]);
+      }
+      if (i == 2 && a.hop) {
+        const int kb = iz - a.zB0, ka = iz + 1 - a.zA0;
+        if (kb >= 0 && kb < a.WB)
+#pragma unroll
+          for (int c = 0; c < NA; ++c) en[c] -= a.az2 * a.QB[((int64_t)c * a.WB + kb) * g.nxy + t];
+        if (ka >= 0 && ka < a.WA) {
+          double q[NA];
+#pragma unroll
+          for (int c = 0; c < NA; ++c) q[c] = a.QA[((int64_t)c * a.WA + ka) * g.nxy + t];
+          G::adj(LinkIO<NC, double>::template load<double>(a.U, 2, g.V, n.s), q);
+#pragma unroll
+          for (int c = 0; c < NA; ++c) en[c] += a.az2 * q[c];
+        }
+      }
+      double acc = 0.0, dot = 0.0;
+#pragma unroll
+      for (int c = 0; c < NA; ++c) acc = fma(eo[c], eo[c], fma(en[c], en[c], acc));
+      if (i == 2) {
+        ez.add(acc);
+        continue;
+      }
+      et.add(acc);
+      if (up) {  // S_L: (E_x, the plane xz) and (E_y, the plane yz), as in k_tmunu
+        const double* p = vecs + (int64_t)(kP0 + 1 + i) * NA * S + here + t;
+#pragma unroll
+        for (int c = 0; c < NA; ++c) dot = fma(eo[c] + en[c], p[c * S], dot);
+        sl.add(dot);
+      }
+    }
+  }
+  tmunu_write(a, sh, et, ez, bl, bt, sl, iz);
 }
 
 // tab[iz] = (sum over the split blocks of slice iz, in block order) / nxy;
@@ -520,12 +586,27 @@ __global__ void k_tmunu_fold(const double* part, int split, int nz, double inv, 
 }
 
 template <int NC, typename R>
-static int launch_tmunu_kernel(const TmnArgs<R>& a, dim3 grid, cudaStream_t s) {
-  return launch_following("k_tmunu launch", k_tmunu<NC, R>, grid, kRedThreads, 0, s, a);
-}
-template <>
-int launch_tmunu_kernel<2, float>(const TmnArgs<float>& a, dim3 grid, cudaStream_t s) {
-  return launch_following("k_tmunu_su2 launch", k_tmunu_su2, grid, kSu2Threads, 0, s, a);
+static int launch_tmunu_kernel(glasma_ctx* c, const TmnArgs<R>& a) {
+  const dim3 grid((unsigned)c->g.nz, (unsigned)a.split);
+  if constexpr (sizeof(R) == 4 && NC == 2) {
+    return launch_following("k_tmunu_su2 launch", k_tmunu_su2, grid, kSu2Threads, 0, c->stream, a);
+  } else {
+    if constexpr (sizeof(R) == 8) {
+      if (c->part) {
+        const int ring = parts_ring(c);
+        for (int z0 = 0; z0 < c->g.nz; z0 += ring - 1) {
+          const int z1 = min(z0 + ring - 1, c->g.nz);
+          int st = launch_parts_norms(c, z0, z1);
+          if (!st)
+            st = launch_following("k_tmunu_parts launch", k_tmunu_parts<NC>, dim3((unsigned)(z1 - z0), grid.y),
+                                  kRedThreads, 0, c->stream, a, (const double*)c->part, ring, z0);
+          if (st) return st;
+        }
+        return GLASMA_OK;
+      }
+    }
+    return launch_following("k_tmunu launch", k_tmunu<NC, R>, grid, kRedThreads, 0, c->stream, a);
+  }
 }
 
 template <int NC, typename R>
@@ -569,7 +650,7 @@ static int tmunu_t(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab) {
   a.split = (int)split;
   a.part = c->tpart;
   double* tab = dev_tab ? dev_tab : c->tab;
-  int st = launch_tmunu_kernel<NC>(a, dim3((unsigned)c->g.nz, (unsigned)split), c->stream);
+  int st = launch_tmunu_kernel<NC, R>(c, a);
   if (st) return st;
   st = launch_following("k_tmunu_fold launch", k_tmunu_fold, (c->g.nz + 127) / 128, 128, 0, c->stream, c->tpart,
                         (int)split, c->g.nz, 1.0 / (double)c->g.nxy, tab);

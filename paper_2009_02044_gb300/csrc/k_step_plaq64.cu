@@ -31,6 +31,7 @@
 // nor any other, as the ring has one slice more than a chunk.  Every value is
 // formed by the same instructions whatever the chunk, so results do not
 // depend on it.
+#include "plaq_parts.cuh"
 #include "step_link.cuh"
 
 namespace glasma {
@@ -41,9 +42,6 @@ namespace glasma {
 constexpr size_t kPartsBytes = (size_t)64 << 20;
 constexpr size_t kPartsMost = (size_t)512 << 20;
 constexpr int kPartsThreads = 64;  // 128 left a sixth of the SMs' FP64 pipes idle on 128 x 16^2
-
-// vectors per site: p0 of the planes xy, xz, yz, then their pAB, then pBA
-enum { kP0 = 0, kPAB = 3, kPBA = 6, kPartVecs = 9 };
 
 struct PartsArgs {
   const double2* U;
@@ -124,7 +122,8 @@ struct PlaqCorners<2> {
   }
 };
 
-template <int NC>
+// NORM: also ||A - B^dag||_F^2 = 2 (N - Re tr of the loop), for T^{mu nu}.
+template <int NC, bool NORM>
 __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs a) {
   follow_last();
   typedef Group<NC, double> G;
@@ -146,6 +145,7 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs 
   const M A = PlaqCorners<NC>::mul_d(IO::template load<double>(a.U, db, g.V, n.p[da]),
                                      IO::template load<double>(a.U, da, g.V, n.p[db]));
   const M B = PlaqCorners<NC>::d_mul(IO::template load<double>(a.U, db, g.V, n.s), ua);
+  if (NORM) out[(kPartVecs * NA + pl) * S] = G::fro2_diff(A, G::dag(B));
   double ab[NA], ba[NA];
   PlaqCorners<NC>::both(A, B, ab, ba);
 #pragma unroll
@@ -178,34 +178,15 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links(PartLinksA
   const int z = pa.z0 + (int)dz, i = (int)blockIdx.y;
   if (i == 2 && z == g.nz - 1) return;  // no z link on the last slice
   const SiteNbr n = site_nbr_tz(g, t, z);
-  const int64_t S = (int64_t)pa.ring * nxy, here = (int64_t)(z % pa.ring) * nxy;
   double F[NA];
-#pragma unroll
-  for (int c = 0; c < NA; ++c) F[c] = 0.0;
-#pragma unroll 1
-  for (int j = 0; j < 3; ++j) {
-    if (j == i) continue;
-    const int pl = i + j - 1;
-    const double w = a.w[j], sgn = i < j ? -w : w;
-    if (j != 2 || z < g.nz - 1) {
-      const double* p = pa.part + (int64_t)(kP0 + pl) * NA * S + here + t;
-#pragma unroll
-      for (int c = 0; c < NA; ++c) F[c] = fma(sgn, p[c * S], F[c]);
-    }
-    if (j != 2 || z > 0) {
-      const int64_t at = j == 2 ? (int64_t)((z - 1) % pa.ring) * nxy + t : here + (n.m[j] - (n.s - t));
-      const double* p = pa.part + (int64_t)((i < j ? kPBA : kPAB) + pl) * NA * S + at;
-#pragma unroll
-      for (int c = 0; c < NA; ++c) F[c] = fma(-sgn, p[c * S], F[c]);
-    }
-  }
+  part_force<NA>(pa.part, g, pa.ring, n, t, z, i, a.w, F);
   update_link<NC, double>(a, i, t, z, n.s, F);
 }
 
 // Slices of the ring a context's scratch has, 0 if it takes none.
 int parts_ring(const glasma_ctx* c) {
   if (c->rs != 8 || c->p.scheme != GLASMA_LEAPFROG) return 0;
-  const size_t slice = sizeof(double) * kPartVecs * (size_t)c->na * (size_t)c->g.nxy;
+  const size_t slice = sizeof(double) * (size_t)part_doubles(c->na) * (size_t)c->g.nxy;
   if (2 * slice > kPartsMost) return 0;
   size_t r = kPartsBytes / slice;
   if (r < 2) r = 2;
@@ -214,18 +195,34 @@ int parts_ring(const glasma_ctx* c) {
 }
 
 size_t parts_bytes(const glasma_ctx* c) {
-  return sizeof(double) * kPartVecs * (size_t)c->na * (size_t)c->g.nxy * (size_t)parts_ring(c);
+  return sizeof(double) * (size_t)part_doubles(c->na) * (size_t)c->g.nxy * (size_t)parts_ring(c);
 }
 
-template <int NC>
-static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
+// The parts of the slices [z0, z1), of z0 - 1 as well with `below`; at most
+// ring - 1 slices.
+template <int NC, bool NORM>
+static int launch_parts_pass(glasma_ctx* c, int z0, int z1, bool below) {
   PartsArgs p;
   p.U = (const double2*)c->U[c->cur];
   p.part = c->part;
   p.g = c->g;
+  p.ring = parts_ring(c);
+  p.z0 = z0;
+  p.zfirst = below ? z0 - 1 : z0;
+  p.sites = (uint32_t)((z1 - p.zfirst) * c->g.nxy);
+  return launch_following("k_step_plaq_parts launch", k_step_plaq_parts<NC, NORM>,
+                          dim3((p.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream, p);
+}
+
+int launch_parts_norms(glasma_ctx* c, int z0, int z1) {
+  return c->p.nc == 2 ? launch_parts_pass<2, true>(c, z0, z1, false) : launch_parts_pass<3, true>(c, z0, z1, false);
+}
+
+template <int NC>
+static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
   PartLinksArgs l;
   StepArgs<double>& a = l.s;
-  a.U = p.U;
+  a.U = (const double2*)c->U[c->cur];
   a.Un = (double2*)c->U[1 - c->cur];
   a.E = (double*)c->E;
   a.QA = (double*)c->QA;
@@ -243,16 +240,13 @@ static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
   a.WB = c->WB;
   a.zlo = c->lo;
   l.part = c->part;
-  p.ring = l.ring = parts_ring(c);
-  if (zlen <= 0 || zlen > p.ring - 1) zlen = p.ring - 1;
+  l.ring = parts_ring(c);
+  if (zlen <= 0 || zlen > l.ring - 1) zlen = l.ring - 1;
   for (int z0 = c->lo; z0 < c->hi; z0 += zlen) {
     const int z1 = z0 + zlen < c->hi ? z0 + zlen : c->hi;
-    p.z0 = l.z0 = z0;
-    p.zfirst = z0 == c->lo && z0 > 0 ? z0 - 1 : z0;
-    p.sites = (uint32_t)((z1 - p.zfirst) * c->g.nxy);
+    l.z0 = z0;
     l.sites = (uint32_t)((z1 - z0) * c->g.nxy);
-    int st = launch_following("k_step_plaq_parts launch", k_step_plaq_parts<NC>,
-                              dim3((p.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream, p);
+    int st = launch_parts_pass<NC, false>(c, z0, z1, z0 == c->lo && z0 > 0);
     if (!st)
       st = launch_following("k_step_plaq_links launch", k_step_plaq_links<NC>,
                             dim3((l.sites + kPartsThreads - 1) / kPartsThreads, 3), kPartsThreads, 0, c->stream, l);
