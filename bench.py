@@ -110,15 +110,18 @@ def step_kernel_hash():
     csrc = os.path.join(ROOT, "paper_2009_02044_gb300", "csrc")
     for f in ("k_step.cu", "step_link.cuh", "link_alg.cuh", "lattice.cuh",
               "su_n.cuh", "step_pair.cuh", "pair.cuh", "k_step_plaq.cu",
-              "k_step_staged.cu"):
+              "k_step_plaq64.cu", "plaq_parts.cuh", "k_step_su2.cu",
+              "dev_su2.cuh", "k_step_staged.cu"):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def step_kernel_name(nc, precision, kernel, nx=64):
-    """The CUDA kernel glasma_step launches for this choice (the library's
-    automatic choice: plaquette kernel in FP64; in FP32 the staged staple
-    kernel for SU(3) rows of 64 sites, else the one-site staple kernel)."""
+    """The CUDA kernel glasma_step launches for this choice, or the first part
+    of its name (the library's automatic choice: in FP64 the two passes
+    k_step_plaq_parts and k_step_plaq_links; in FP32 the staged staple kernel
+    for SU(3) rows of 64 sites, k_step_leapfrog_site for SU(2) lattices from
+    2^17 sites on, else the one-link staple kernel k_step_leapfrog)."""
     if kernel == "auto":
         kernel = ("plaquette" if precision == "fp64" else
                   "staple_staged" if (nc == 3 and nx == 64) else "staple")
@@ -379,6 +382,8 @@ def run_ours(args, cfg):
     # the "improved" field)
     per_launch_ms = ms / launches
     alg = V * bytes_per_site(nc, rs) + (hops / K) * qbytes
+    if cfg.get("scheme", "leapfrog") == "leapfrog":
+        alg *= K / launches     # the FP64 step is two launches or more
     peak, peak_kind = load_peaks()
     achieved = alg / (per_launch_ms * 1e-3) / 1e9
     kname = step_kernel_name(nc, args.precision, args.kernel, cfg["nx"])

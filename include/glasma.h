@@ -364,9 +364,14 @@ GLASMA_API int glasma_slab_unpack(glasma_ctx* c, int dir, const void* dev_buf);
  *                              z; each plaquette is formed once and its
  *                              projection, transported to each of its
  *                              corners, goes to the four links it bounds
- *                              (blocks of up to 320 threads);
+ *                              (blocks of up to 320 threads).  FP64 state
+ *                              is stepped in two passes instead, one thread
+ *                              per plaquette and then one per link, through
+ *                              a scratch of the context (at most 64 MB, or
+ *                              two slices of it up to 512 MB);
  *   GLASMA_KERNEL_PLAQUETTE_256  the same with blocks of up to 256 threads
- *                              (more registers per thread);
+ *                              (more registers per thread; FP64 state:
+ *                              the two passes);
  *   GLASMA_KERNEL_STAPLE_PAIRS the staple kernel on two sites per thread,
  *                              (x, y, z) and (x, y, z + ceil(nz/2)), in the
  *                              two lanes of the packed FP32 instructions
@@ -384,21 +389,25 @@ GLASMA_API int glasma_slab_unpack(glasma_ctx* c, int dir, const void* dev_buf);
  *                              reported as TIMEOUT by the next call that
  *                              returns host values;
  *   GLASMA_KERNEL_AUTO         the default, from GB300 timings: for FP64
- *                              state the plaquette kernel where a transverse
- *                              row fits one block (nx <= 320; its 24% fewer
- *                              FMAs win where the FP64 pipe bounds the
- *                              step), else the staple kernel; for FP32 the
- *                              staged staple kernel where it applies with
- *                              nx = 64 (SU(3), whole lattices), else the
- *                              staple kernel. */
+ *                              state the two passes of the plaquette form
+ *                              for rows of any length (fewer FMAs where the
+ *                              FP64 pipe bounds the step), the staple kernel
+ *                              where two slices of their scratch pass
+ *                              512 MB; for FP32 SU(2) lattices from 2^17
+ *                              sites on (a slab: of its whole lattice) one
+ *                              thread per site in the plaquette form; for
+ *                              FP32 SU(3) the staged staple kernel where it
+ *                              applies with nx = 64 (whole lattices); else
+ *                              the staple kernel. */
 enum { GLASMA_KERNEL_AUTO = 0, GLASMA_KERNEL_STAPLE = 1, GLASMA_KERNEL_PLAQUETTE = 2,
        GLASMA_KERNEL_PLAQUETTE_256 = 3, GLASMA_KERNEL_STAPLE_PAIRS = 4, GLASMA_KERNEL_STAPLE_STAGED = 5 };
 
 /*
  * Choose the leapfrog step kernel of a context and, for the plaquette
  * kernel, the number of z slices each block marches through (zlen; 0 =
- * automatic, about eight blocks per resident block slot).  Results of the
- * two kernels agree to rounding (their sums run in different orders); the
+ * automatic, about eight blocks per resident block slot), or in FP64 the
+ * slices of one pair of passes (0, or more than the scratch holds: as many
+ * as it holds).  Results of the two kernels agree to rounding (their sums run in different orders); the
  * choice never changes the state's layout, so it may change between steps.
  * Errors: INVALID_ARG (unknown kernel, zlen outside [0, nz], a plaquette
  * kernel asked for on a lattice whose transverse rows do not fit one
