@@ -131,17 +131,15 @@ __device__ void force_implicit(const ImplArgs<R>& a, const SiteNbr& n, int i, R*
       const typename V2T<R>::T* Bj = slot_buf(a, m, zplane, j);
       typename G::Sum S = G::zero_sum();
       if (fwd) {
-        M T = G::mul_d(LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi),
-                       LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, pj));
-        T = G::mul_d(T, LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, n.s));
-        G::sum_add(S, R(1), T);
+        G::sum_add(S, R(1), G::staple_fwd(LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi),
+                                          LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, pj),
+                                          LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, n.s)));
       }
       if (bwd) {
         // x + e_i - e_j (the wraps of x and y are independent)
-        M T = G::mul(LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, mj),
-                     LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi + mj - n.s));
-        T = G::d_mul(T, LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, mj));
-        G::sum_add(S, R(1), T);
+        G::sum_add(S, R(1), G::staple_bwd(LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, mj),
+                                          LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi + mj - n.s),
+                                          LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, mj)));
       }
       R pr[NA];
       G::proj_mul_sum(LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, n.s), S, pr);

@@ -348,9 +348,9 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
       for (int j = 0; j < 3; ++j) {
         if (j == i || (j == 2 && iz == 0)) continue;
         const int64_t mj = n.m[j];
-        M T = G::mul(IO::template load<R>(a.U, i, g.V, mj), IO::template load<R>(a.U, j, g.V, n.p[i] + mj - s));
-        T = G::d_mul(T, IO::template load<R>(a.U, j, g.V, mj));
-        G::sum_add(S, a.w[j], T);
+        G::sum_add(S, a.w[j], G::staple_bwd(IO::template load<R>(a.U, i, g.V, mj),
+                                            IO::template load<R>(a.U, j, g.V, n.p[i] + mj - s),
+                                            IO::template load<R>(a.U, j, g.V, mj)));
       }
       R q[NA];
       G::proj_mul_sum(IO::template load<R>(a.U, i, g.V, s), S, q);

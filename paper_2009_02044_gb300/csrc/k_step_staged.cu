@@ -243,15 +243,13 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
         nb(j, +1, qj, rj, cj_);
         nb(j, -1, qn, rn, cn);
         if (fwd) {
-          M T = G::mul_d(st_load<RB>(sm, qi, j, ri, ci), st_load<RB>(sm, qj, i, rj, cj_));
-          T = G::mul_d(T, st_load<RB>(sm, q0, j, rr0, ix));
-          G::sum_add(S, wj, T);
+          G::sum_add(S, wj, G::staple_fwd(st_load<RB>(sm, qi, j, ri, ci), st_load<RB>(sm, qj, i, rj, cj_),
+                                          st_load<RB>(sm, q0, j, rr0, ix)));
         }
         if (bwd) {
           const int qd = i == 2 ? qp : qn, rd = rn + ri - rr0, cd = i == 0 ? ci : cn;
-          M T = G::mul(st_load<RB>(sm, qn, i, rn, cn), st_load<RB>(sm, qd, j, rd, cd));
-          T = G::d_mul(T, st_load<RB>(sm, qn, j, rn, cn));
-          G::sum_add(S, wj, T);
+          G::sum_add(S, wj, G::staple_bwd(st_load<RB>(sm, qn, i, rn, cn), st_load<RB>(sm, qd, j, rd, cd),
+                                          st_load<RB>(sm, qn, j, rn, cn)));
         }
       }
       float pr[8], F[8];

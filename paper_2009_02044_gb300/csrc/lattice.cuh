@@ -211,17 +211,17 @@ GL_HD void link_force_staple(const typename V2T<Rs>::T* U, const Geom& g, const 
     const bool bwd = (j != 2) || (n.iz >= 1);
     const int64_t pj = n.p[j], mj = n.m[j];
     if (fwd) {
-      M T = G::mul_d(LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi),
-                     LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, pj));
-      T = G::mul_d(T, LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, n.s));
+      const M T = G::staple_fwd(LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi),
+                                LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, pj),
+                                LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, n.s));
       G::sum_add(S, wj, T);
     }
     if (bwd) {
       // x + e_i - e_j: the periodic wraps of x and y depend only on ix and
       // iy and z has no wrap, so the two offsets add
-      M T = G::mul(LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, mj),
-                   LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi + mj - n.s));
-      T = G::d_mul(T, LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, mj));
+      const M T = G::staple_bwd(LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, mj),
+                                LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi + mj - n.s),
+                                LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, mj));
       G::sum_add(S, wj, T);
     }
   }
