@@ -561,10 +561,19 @@ struct LinkAlgDev2 {
     proj_mul_sum(x, s, o);
   }
   // exp(i c v.sigma/2) - 1 = (cos th - 1 + i sin th n3, sin th (n2 + i n1)),
-  // cos th - 1 = -2 sin^2(th/2)
+  // cos th - 1 = -2 sin^2(th/2); by series where th allows, as in reunit (the
+  // staple step has few other instructions: 200 x 30 x 20 0.0105 -> 0.0098 ms)
   GL_HD static M expi(const R* v, R c) {
     const R n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
     if (all_zero_s(n2)) return G::zero();
+    const R x = R(0.25f) * c * c * n2;  // th^2: Taylor series up to 1/4 (remainders below 2e-11)
+    if (all_abs_lt_s(x, 0.25f)) {
+      const R co = x * fma(x, fma(x, fma(x, fma(x, R(-1.f / 3628800.f), R(1.f / 40320.f)), R(-1.f / 720.f)),
+                                  R(1.f / 24.f)), R(-0.5f));
+      const R f = R(0.5f) * c * fma(x, fma(x, fma(x, fma(x, R(1.f / 362880.f), R(-1.f / 5040.f)), R(1.f / 120.f)),
+                                           R(-1.f / 6.f)), R(1.f));
+      return M{{co, f * v[2]}, {f * v[1], f * v[0]}};
+    }
     const R nrm = gl_sqrt(n2);
     R sh, ch;
     gl_sincos(0.25f * c * nrm, &sh, &ch);  // half of th = c |v| / 2
@@ -575,7 +584,14 @@ struct LinkAlgDev2 {
   }
   GL_HD static M reunit(const M& x) {
     const R eps = 2.f * x.a.re + x.a.re * x.a.re + x.a.im * x.a.im + x.b.re * x.b.re + x.b.im * x.b.im;
-    const R r = gl_sqrt(R(1.f) + eps), g = lane_div_s(-eps, r * (R(1.f) + r)), f = R(1.f) + g;
+    R g;  // 1 / sqrt(1 + eps) - 1
+    if (all_abs_lt_s(eps, 1e-3f)) {
+      g = eps * fma(eps, fma(eps, R(-0.3125f), R(0.375f)), R(-0.5f));
+    } else {
+      const R r = gl_sqrt(R(1.f) + eps);
+      g = lane_div_s(-eps, r * (R(1.f) + r));
+    }
+    const R f = R(1.f) + g;
     return M{{g + f * x.a.re, f * x.a.im}, f * x.b};
   }
   GL_HD static void adj(const M& u, R* q) { G::adj(full(u), q); }
