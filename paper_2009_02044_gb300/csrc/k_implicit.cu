@@ -165,13 +165,16 @@ __global__ void __launch_bounds__(192) k_implicit_prev(ImplArgs<R> a) {
   R e[NA];
 #pragma unroll
   for (int c = 0; c < NA; ++c) e[c] = a.E[(int64_t)(i * NA + c) * a.g.V + s];
-  const typename G::M u = G::evolve_series(e, -a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s));
+  const typename G::M u = G::evolve(e, -a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s));
   LinkIO<NC, R>::template store<R>(a.Uout, i, a.g.V, s, u);
 }
 
 // Blocks per SM of the prepare and sweep kernels.  FP32: 4 blocks of 192
 // threads (80 registers; the load latency of the staples wants the warps
-// more than the spilled registers cost).  FP64 needs the registers of one
+// more than the spilled registers cost; 3 blocks 3.19 against 3.08 ms per step of
+// SU(3) 512 x 64^2).  The exponential is the step's: a Taylor-Horner series of
+// four matrix products, which fitted the registers before the staples formed
+// two rows, took 3.23 against 3.12.  FP64 needs the registers of one
 // block per SM instead of spilling.
 template <typename R> struct ImplOcc { static constexpr int blocks = 4; };
 template <> struct ImplOcc<double> { static constexpr int blocks = 1; };
@@ -224,7 +227,7 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
       for (int c = 0; c < NA; ++c) ew[c] += dj[c];
     }
     // X^(0) = exp(i dt E(t_{n-1/2})) U_n
-    LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, G::evolve_series(e, a.dt, Ui));
+    LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, G::evolve(e, a.dt, Ui));
   }
   R F[NA];
   force_implicit<NC, R>(a, site_nbr_tz(a.g, t, iz), i, F, 1, 3);
@@ -286,7 +289,7 @@ __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t
     a.E[idx] = e[c];
   }
   LinkIO<NC, R>::template store<R>(
-      a.Xn, i, a.g.V, s, G::evolve_series(e, a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s)));
+      a.Xn, i, a.g.V, s, G::evolve(e, a.dt, LinkIO<NC, R>::template load<R>(a.Un, i, a.g.V, s)));
 }
 
 // One fixed-point sweep: E = Ework + dt F_0(X), Xn = exp(i dt E) U_n, where

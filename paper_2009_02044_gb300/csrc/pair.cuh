@@ -42,7 +42,6 @@ __device__ __forceinline__ bool all_abs_lt(float a, float b) { return fabsf(a) <
 
 // per-lane functions without a packed form
 __device__ __forceinline__ f2 lane_sqrt(f2 a) { return f2(sqrtf(a.v.x), sqrtf(a.v.y)); }
-__device__ __forceinline__ f2 lane_abs(f2 a) { return f2(fabsf(a.v.x), fabsf(a.v.y)); }
 __device__ __forceinline__ f2 lane_div(f2 a, f2 b) { return f2(a.v.x / b.v.x, a.v.y / b.v.y); }
 __device__ __forceinline__ f2 lane_sincos_s(f2 a, f2* c) {
   float s0, c0, s1, c1;
