@@ -16,8 +16,19 @@ __device__ __forceinline__ Dev4 dev_load(const float4* p) {
   return Dev4{v.x, v.w, v.z, v.y};
 }
 __device__ __forceinline__ Dev4 dev_dag(Dev4 a) { return Dev4{a.w, -a.x, -a.y, -a.z}; }
-// (w + i a.s)(v + i b.s) = (w v - a.b) + i (w b + v a - a x b).s
+// (w + i a.s)(v + i b.s) = (w v - a.b) + i (w b + v a - a x b).s, the products
+// of two deviations first, so that each entry rounds twice at their own size;
+// rounding four times (dev_mulq, for T^{mu nu}, whose squares are averaged)
+// the step took 0.596 for 0.603 ms on 1024 x 128^2, with 1.4 times the error of E
+// and 1.3 times that of U
 __device__ __forceinline__ Dev4 dev_mul(Dev4 a, Dev4 b) {
+  const float v = 1.f + b.w, u = 1.f + a.w;
+  return Dev4{fma(a.w, v, fma(-a.x, b.x, fma(-a.y, b.y, -a.z * b.z))) + b.w,
+              fma(u, b.x, fma(v, a.x, fma(-a.y, b.z, a.z * b.y))),
+              fma(u, b.y, fma(v, a.y, fma(-a.z, b.x, a.x * b.z))),
+              fma(u, b.z, fma(v, a.z, fma(-a.x, b.y, a.y * b.x)))};
+}
+__device__ __forceinline__ Dev4 dev_mulq(Dev4 a, Dev4 b) {
   const float v = 1.f + b.w;
   return Dev4{fma(a.w, v, fma(-a.x, b.x, fma(-a.y, b.y, fma(-a.z, b.z, b.w)))),
               fma(a.w, b.x, fma(v, a.x, fma(-a.y, b.z, fma(a.z, b.y, b.x)))),

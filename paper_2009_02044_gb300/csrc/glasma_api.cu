@@ -136,7 +136,7 @@ static int check_params(const glasma_params* p) {
 // for the one-site staple kernel, bitwise the same result), else the staple
 // kernel (0.469 ms, against 0.521 for the plaquette kernel and 0.572 for
 // site pairs, whose 168 registers leave too few warps to hide latency); in
-// FP32 SU(2) one thread per site on large lattices (0.59 against 1.10 ms for
+// FP32 SU(2) one thread per site on large lattices (0.60 against 1.10 ms for
 // the staple kernel and 1.39 for site pairs per 1024 x 128^2 step), the staple
 // kernel on small ones.
 bool use_plaq_kernel(const glasma_ctx* c) {

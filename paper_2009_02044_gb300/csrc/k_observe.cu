@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
     Dev4 uz{0.f, 0.f, 0.f, 0.f};
     Vec3 F[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, pxz{0.f, 0.f, 0.f}, pyz = pxz;
     {
-      const Dev4 A = dev_mul(ux, dev_load(Uy + txp)), B = dev_mul(uy, dev_load(Ux + typ));
+      const Dev4 A = dev_mulq(ux, dev_load(Uy + txp)), B = dev_mulq(uy, dev_load(Ux + typ));
       bl.add(dist2(A, B));
       const Vec3 p = vec_ab(A, dev_dag(B));
       add3(F[0], -wt, p);
@@ -441,11 +441,11 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
     }
     if (up) {
       uz = dev_load(Uz + t);
-      Dev4 A = dev_mul(ux, dev_load(Uz + txp)), B = dev_mul(uz, dev_load(Ux + g.nxy + t));
+      Dev4 A = dev_mulq(ux, dev_load(Uz + txp)), B = dev_mulq(uz, dev_load(Ux + g.nxy + t));
       bt.add(dist2(A, B));
       pxz = vec_ab(A, dev_dag(B));
-      A = dev_mul(uy, dev_load(Uz + typ));
-      B = dev_mul(uz, dev_load(Uy + g.nxy + t));
+      A = dev_mulq(uy, dev_load(Uz + typ));
+      B = dev_mulq(uz, dev_load(Uy + g.nxy + t));
       bt.add(dist2(A, B));
       pyz = vec_ab(A, dev_dag(B));
       add3(F[0], -wz, pxz);
@@ -455,22 +455,22 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
     }
     {
       const Dev4 vx = dev_load(Ux + txm);
-      add3(F[1], -wt, vec_ab(dev_mul(uy, dev_dag(dev_load(Ux + txmyp))), dev_mul(dev_dag(dev_load(Uy + txm)), vx)));
+      add3(F[1], -wt, vec_ab(dev_mulq(uy, dev_dag(dev_load(Ux + txmyp))), dev_mulq(dev_dag(dev_load(Uy + txm)), vx)));
       if (up)
         add3(F[2], -wt,
-             vec_ab(dev_mul(uz, dev_dag(dev_load(Ux + g.nxy + txm))), dev_mul(dev_dag(dev_load(Uz + txm)), vx)));
+             vec_ab(dev_mulq(uz, dev_dag(dev_load(Ux + g.nxy + txm))), dev_mulq(dev_dag(dev_load(Uz + txm)), vx)));
     }
     {
       const Dev4 vy = dev_load(Uy + tym);
-      add3(F[0], wt, vec_ab(dev_mul(dev_dag(vy), dev_load(Ux + tym)), dev_mul(dev_load(Uy + txpym), dev_dag(ux))));
+      add3(F[0], wt, vec_ab(dev_mulq(dev_dag(vy), dev_load(Ux + tym)), dev_mulq(dev_load(Uy + txpym), dev_dag(ux))));
       if (up)
         add3(F[2], -wt,
-             vec_ab(dev_mul(uz, dev_dag(dev_load(Uy + g.nxy + tym))), dev_mul(dev_dag(dev_load(Uz + tym)), vy)));
+             vec_ab(dev_mulq(uz, dev_dag(dev_load(Uy + g.nxy + tym))), dev_mulq(dev_dag(dev_load(Uz + tym)), vy)));
     }
     if (down) {  // vec BA of the planes xz and yz of the slice below
       const Dev4 vz = dev_dag(dev_load(Uz - g.nxy + t));
-      add3(F[0], wz, vec_ab(dev_mul(vz, dev_load(Ux - g.nxy + t)), dev_mul(dev_load(Uz - g.nxy + txp), dev_dag(ux))));
-      add3(F[1], wz, vec_ab(dev_mul(vz, dev_load(Uy - g.nxy + t)), dev_mul(dev_load(Uz - g.nxy + typ), dev_dag(uy))));
+      add3(F[0], wz, vec_ab(dev_mulq(vz, dev_load(Ux - g.nxy + t)), dev_mulq(dev_load(Uz - g.nxy + txp), dev_dag(ux))));
+      add3(F[1], wz, vec_ab(dev_mulq(vz, dev_load(Uy - g.nxy + t)), dev_mulq(dev_load(Uz - g.nxy + typ), dev_dag(uy))));
     }
     Vec3 dj{0.f, 0.f, 0.f};
     if (a.hop && up) {

@@ -15,8 +15,8 @@ GL_HD constexpr int part_doubles(int na) { return kPartVecs * na + 3; }
 
 // Force on link i of site t of slice z from the scratch.
 template <int NA>
-__device__ __forceinline__ void part_force(const double* part, const Geom& g, int ring, const SiteNbr& n, uint32_t t, int z,
-                                           int i, const double* w, double* F) {
+__device__ __forceinline__ void part_force(const double* part, const Geom& g, int ring, const SiteNbr& n, uint32_t t,
+                                           int z, int i, const double* w, double* F) {
   const int64_t S = (int64_t)ring * g.nxy, here = (int64_t)(z % ring) * g.nxy;
 #pragma unroll
   for (int c = 0; c < NA; ++c) F[c] = 0.0;
