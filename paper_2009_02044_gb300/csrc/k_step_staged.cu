@@ -94,10 +94,7 @@ struct StagedGeo {
       (size_t)kStSlots * SLOTB * sizeof(float2) + (2 * kStSlots + 1) * sizeof(unsigned long long);
 };
 
-template <int RB>
-__device__ __forceinline__ LinkAlg<3, float>::M st_load(const float2* sm, int q, int d, int rr, int ix) {
-  typedef StagedGeo<RB> SG;
-  const float2* p = sm + (q * 3 + d) * SG::DIRB + (rr * RB + (ix >> 5)) * 288 + (ix & 31);
+__device__ __forceinline__ LinkAlg<3, float>::M st_load(const float2* p) {
   LinkAlg<3, float>::M m;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -203,6 +200,14 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
   const int iy = iy0 + r;
   const bool inner = iy < g.ny;
   const uint32_t t = (uint32_t)(inner ? iy : 0) * NX + ix;
+  // The thread's site in a slot's image of one direction, and the steps to its
+  // neighbours: the same for every slice, so a link's address is one addition
+  // (formed anew for every link it was 120 instructions of an update: 512 x 64^2
+  // 0.423 -> 0.398 ms per step).
+  auto col = [](int x) { return (x >> 5) * 288 + (x & 31); };
+  const float2* const own = sm + (r + 1) * RB * 288 + col(ix);
+  const int xp = col(ix + 1 == NX ? 0 : ix + 1) - col(ix), xm = col(ix == 0 ? NX - 1 : ix - 1) - col(ix);
+  constexpr int yp = RB * 288;
   auto wait_full = [&](int zs) -> bool {
     return mbar_wait(&full[zs & (kStSlots - 1)], (unsigned)(((zs - lo_load) >> 2) & 1), sa.wait);
   };
@@ -215,45 +220,30 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
       break;
     }
     if (inner && !(i == 2 && z == g.nz - 1)) {
-      const int q0 = z & 3, qm = (z - 1) & 3, qp = (z + 1) & 3;
-      const int rr0 = r + 1;
-      const int xp = ix + 1 == NX ? 0 : ix + 1, xm = ix == 0 ? NX - 1 : ix - 1;
+      // a step in z is one to a neighbouring slot
+      const int slot = (z & 3) * SG::SLOTB;
+      const int zp = ((z + 1) & 3) * SG::SLOTB - slot, zm = ((z - 1) & 3) * SG::SLOTB - slot;
       const int64_t s = (int64_t)z * g.nxy + t;
       float E0[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) E0[c] = a.E[(int64_t)(i * 8 + c) * g.V + s];
-      auto nb = [&](int d, int sgn, int& q, int& rr, int& cx) {
-        q = q0;
-        rr = rr0;
-        cx = ix;
-        if (d == 0) cx = sgn > 0 ? xp : xm;
-        else if (d == 1) rr = rr0 + sgn;
-        else q = sgn > 0 ? qp : qm;
-      };
       G::Sum S = G::zero_sum();
       const float wt = a.w[0], wz = a.w[2];
+      const float2* const here = own + slot;
+      const float2* const hi = here + i * SG::DIRB;
+      const int pi = i == 0 ? xp : i == 1 ? yp : zp;
 #pragma unroll 1
-      for (int j = 0; j < 3; ++j) {
-        if (j == i) continue;
+      for (int k = 0; k < 2; ++k) {
+        const int j = k == 0 ? (i == 0 ? 1 : 0) : (i == 2 ? 1 : 2);
         const float wj = j == 2 ? wz : wt;
-        const bool fwd = (j != 2) || (z <= g.nz - 2);
-        const bool bwd = (j != 2) || (z >= 1);
-        int qi, ri, ci, qj, rj, cj_, qn, rn, cn;
-        nb(i, +1, qi, ri, ci);
-        nb(j, +1, qj, rj, cj_);
-        nb(j, -1, qn, rn, cn);
-        if (fwd) {
-          G::sum_add(S, wj, G::staple_fwd(st_load<RB>(sm, qi, j, ri, ci), st_load<RB>(sm, qj, i, rj, cj_),
-                                          st_load<RB>(sm, q0, j, rr0, ix)));
-        }
-        if (bwd) {
-          const int qd = i == 2 ? qp : qn, rd = rn + ri - rr0, cd = i == 0 ? ci : cn;
-          G::sum_add(S, wj, G::staple_bwd(st_load<RB>(sm, qn, i, rn, cn), st_load<RB>(sm, qd, j, rd, cd),
-                                          st_load<RB>(sm, qn, j, rn, cn)));
-        }
+        const int pj = j == 0 ? xp : j == 1 ? yp : zp, mj = j == 0 ? xm : j == 1 ? -yp : zm;
+        const float2* const hj = here + j * SG::DIRB;
+        if (j != 2 || z <= g.nz - 2) G::sum_add(S, wj, G::staple_fwd(st_load(hj + pi), st_load(hi + pj), st_load(hj)));
+        if (j != 2 || z >= 1)
+          G::sum_add(S, wj, G::staple_bwd(st_load(hi + mj), st_load(hj + pi + mj), st_load(hj + mj)));
       }
       float pr[8], F[8];
-      const M Ui = st_load<RB>(sm, q0, i, rr0, ix);
+      const M Ui = st_load(hi);
       G::proj_mul_sum(Ui, S, pr);
 #pragma unroll
       for (int c = 0; c < 8; ++c) F[c] = -pr[c];
