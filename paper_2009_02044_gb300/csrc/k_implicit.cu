@@ -116,14 +116,14 @@ __device__ void force_implicit(const ImplArgs<R>& a, const SiteNbr& n, int i, R*
   constexpr int NA = G::NA;
 #pragma unroll
   for (int c = 0; c < NA; ++c) F[c] = R(0);
-  const int64_t pi = n.p[i];
+  const int64_t pi = nbr_p(n, i);
 #pragma unroll 1
   for (int j = 0; j < 3; ++j) {
     if (j == i) continue;
     const bool zplane = (i == 2) || (j == 2);
     const bool fwd = (j != 2) || (n.iz <= a.g.nz - 2);
     const bool bwd = (j != 2) || (n.iz >= 1);
-    const int64_t pj = n.p[j], mj = n.m[j];
+    const int64_t pj = nbr_p(n, j), mj = nbr_m(n, j);
     const R wj = j == 2 ? a.w[2] : a.w[0];
 #pragma unroll 1
     for (int m = m_begin; m < m_end; ++m) {

@@ -347,9 +347,9 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
 #pragma unroll 1
       for (int j = 0; j < 3; ++j) {
         if (j == i || (j == 2 && iz == 0)) continue;
-        const int64_t mj = n.m[j];
+        const int64_t mj = nbr_m(n, j);
         G::sum_add(S, a.w[j], G::staple_bwd(IO::template load<R>(a.U, i, g.V, mj),
-                                            IO::template load<R>(a.U, j, g.V, n.p[i] + mj - s),
+                                            IO::template load<R>(a.U, j, g.V, nbr_p(n, i) + mj - s),
                                             IO::template load<R>(a.U, j, g.V, mj)));
       }
       R q[NA];

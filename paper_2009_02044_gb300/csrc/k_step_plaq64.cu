@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs 
   const int64_t S = (int64_t)a.ring * nxy;
   double* out = a.part + (int64_t)(z % a.ring) * nxy + t;
   const M ua = IO::template load<double>(a.U, da, g.V, n.s);
-  const M A = PlaqCorners<NC>::mul_d(IO::template load<double>(a.U, db, g.V, n.p[da]),
-                                     IO::template load<double>(a.U, da, g.V, n.p[db]));
+  const M A = PlaqCorners<NC>::mul_d(IO::template load<double>(a.U, db, g.V, nbr_p(n, da)),
+                                     IO::template load<double>(a.U, da, g.V, nbr_p(n, db)));
   const M B = PlaqCorners<NC>::d_mul(IO::template load<double>(a.U, db, g.V, n.s), ua);
   if (NORM) out[(kPartVecs * NA + pl) * S] = G::fro2_diff(A, G::dag(B));
   double ab[NA], ba[NA];

@@ -148,6 +148,13 @@ struct SiteNbr {
   int64_t m[3];  // x - e_d
 };
 
+// n.p[d], n.m[d] for a direction known at run time: selects, where an index
+// would put the arrays in local memory.  Improved scheme, SU(2) 160 x 32^2
+// 0.130 -> 0.123 ms per step, SU(3) 512 x 64^2 3.12 -> 3.09; T^{mu nu} 0.440 -> 0.427
+// (the staple step, with its own arrays, gained nothing)
+GL_HD int64_t nbr_p(const SiteNbr& n, int d) { return d == 0 ? n.p[0] : d == 1 ? n.p[1] : n.p[2]; }
+GL_HD int64_t nbr_m(const SiteNbr& n, int d) { return d == 0 ? n.m[0] : d == 1 ? n.m[1] : n.m[2]; }
+
 GL_HD SiteNbr site_nbr(const Geom& g, int64_t s) {
   SiteNbr n;
   n.s = s;

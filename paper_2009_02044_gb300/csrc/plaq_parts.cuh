@@ -31,7 +31,7 @@ __device__ __forceinline__ void part_force(const double* part, const Geom& g, in
       for (int c = 0; c < NA; ++c) F[c] = fma(sgn, p[c * S], F[c]);
     }
     if (j != 2 || z > 0) {
-      const int64_t at = j == 2 ? (int64_t)((z - 1) % ring) * g.nxy + t : here + (n.m[j] - (n.s - t));
+      const int64_t at = j == 2 ? (int64_t)((z - 1) % ring) * g.nxy + t : here + (nbr_m(n, j) - (n.s - t));
       const double* p = part + (int64_t)((i < j ? kPBA : kPAB) + pl) * NA * S + at;
 #pragma unroll
       for (int c = 0; c < NA; ++c) F[c] = fma(-sgn, p[c * S], F[c]);
