@@ -208,6 +208,9 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
   const float2* const own = sm + (r + 1) * RB * 288 + col(ix);
   const int xp = col(ix + 1 == NX ? 0 : ix + 1) - col(ix), xm = col(ix == 0 ? NX - 1 : ix - 1) - col(ix);
   constexpr int yp = RB * 288;
+  // its field and new link on slice z
+  float* E = a.E + (int64_t)(i * 8) * g.V + (int64_t)z0 * g.nxy + t;
+  float2* Un = a.Un + link_index(3, i, 0, g.V, (int64_t)z0 * g.nxy + t);
   auto wait_full = [&](int zs) -> bool {
     return mbar_wait(&full[zs & (kStSlots - 1)], (unsigned)(((zs - lo_load) >> 2) & 1), sa.wait);
   };
@@ -223,10 +226,9 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
       // a step in z is one to a neighbouring slot
       const int slot = (z & 3) * SG::SLOTB;
       const int zp = ((z + 1) & 3) * SG::SLOTB - slot, zm = ((z - 1) & 3) * SG::SLOTB - slot;
-      const int64_t s = (int64_t)z * g.nxy + t;
       float E0[8];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) E0[c] = a.E[(int64_t)(i * 8 + c) * g.V + s];
+      for (int c = 0; c < 8; ++c) E0[c] = E[c * g.V];
       G::Sum S = G::zero_sum();
       const float wt = a.w[0], wz = a.w[2];
       const float2* const here = own + slot;
@@ -247,8 +249,10 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
       G::proj_mul_sum(Ui, S, pr);
 #pragma unroll
       for (int c = 0; c < 8; ++c) F[c] = -pr[c];
-      update_link_ue<3, float>(a, i, t, z, s, F, Ui, E0);
+      update_link_ue<3, float>(a, i, t, z, E, Un, F, Ui, E0);
     }
+    E += g.nxy;
+    Un += 9 * g.nxy;  // whole link blocks
     // iteration z is the last to read slice z - 1
     if (z - 1 >= lo_load) mbar_arrive(&empty[(z - 1) & (kStSlots - 1)]);
   }

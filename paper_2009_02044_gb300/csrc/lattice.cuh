@@ -94,11 +94,14 @@ struct LinkIO<2, R> {
   }
   template <typename Rc>
   GL_HD static void store(typename V2T<R>::T* U, int d, int64_t V, int64_t s, const typename Group<2, Rc>::M& m) {
+    put<Rc>(U + link_index(2, d, 0, V, s), m);
+  }
+  template <typename Rc>
+  GL_HD static void put(typename V2T<R>::T* p, const typename Group<2, Rc>::M& m) {
     typename V2T<R>::T a, b;
     const Rc one = DeltaConv<R, Rc>::to_full ? Rc(1) : Rc(0);
     a.x = R(m.a.re - one); a.y = R(m.a.im);
     b.x = R(m.b.re); b.y = R(m.b.im);
-    typename V2T<R>::T* p = U + link_index(2, d, 0, V, s);
     if (sizeof(R) == 4) {
       *reinterpret_cast<float4*>(p) = make_float4(float(a.x), float(a.y), float(b.x), float(b.y));
     } else {
@@ -128,8 +131,11 @@ struct LinkIO<3, R> {
   }
   template <typename Rc>
   GL_HD static void store(typename V2T<R>::T* U, int d, int64_t V, int64_t s, const typename Group<3, Rc>::M& m) {
+    put<Rc>(U + link_index(3, d, 0, V, s), m);
+  }
+  template <typename Rc>
+  GL_HD static void put(typename V2T<R>::T* p, const typename Group<3, Rc>::M& m) {
     const Rc one = DeltaConv<R, Rc>::to_full ? Rc(1) : Rc(0);
-    typename V2T<R>::T* p = U + link_index(3, d, 0, V, s);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       typename V2T<R>::T v;

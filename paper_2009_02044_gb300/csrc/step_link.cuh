@@ -34,10 +34,12 @@ struct StepArgs {
 // Shared by the staple kernel below, the plaquette kernel (k_step_plaq.cu)
 // and the staged kernel (k_step_staged.cu), so all apply the same update
 // arithmetic.  update_link_ue takes the link U_i(x) and the field
-// E_i(t_{n-1/2}) already loaded (Ui, E0); update_link loads them.
+// E_i(t_{n-1/2}) already loaded (Ui, E0), and where
+// their new values go; update_link loads them.
 template <int NC, typename R>
-__device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint32_t t, int iz, int64_t s,
-                                               const R* F, const typename LinkAlg<NC, R>::M& Ui, const R* E0) {
+__device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint32_t t, int iz, R* E,
+                                               typename V2T<R>::T* Un, const R* F,
+                                               const typename LinkAlg<NC, R>::M& Ui, const R* E0) {
   typedef LinkAlg<NC, R> G;
   typedef typename G::M M;
   constexpr int NA = G::NA;
@@ -75,8 +77,8 @@ __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint
     for (int c = 0; c < NA; ++c) e[c] += dj[c];
   }
 #pragma unroll
-  for (int c = 0; c < NA; ++c) a.E[(int64_t)(i * NA + c) * a.g.V + s] = e[c];
-  LinkIO<NC, R>::template store<R>(a.Un, i, a.g.V, s, G::evolve(e, a.dt, Ui));
+  for (int c = 0; c < NA; ++c) E[c * a.g.V] = e[c];
+  LinkIO<NC, R>::template put<R>(Un, G::evolve(e, a.dt, Ui));
 }
 
 template <int NC, typename R>
@@ -84,10 +86,11 @@ __device__ __forceinline__ void update_link(const StepArgs<R>& a, int i, uint32_
                                             const R* F) {
   constexpr int NA = LinkAlg<NC, R>::NA;
   const typename LinkAlg<NC, R>::M Ui = LinkIO<NC, R>::template load<R>(a.U, i, a.g.V, s);
+  R* const E = a.E + (int64_t)(i * NA) * a.g.V + s;
   R E0[NA];
 #pragma unroll
-  for (int c = 0; c < NA; ++c) E0[c] = a.E[(int64_t)(i * NA + c) * a.g.V + s];
-  update_link_ue<NC, R>(a, i, t, iz, s, F, Ui, E0);
+  for (int c = 0; c < NA; ++c) E0[c] = E[c * a.g.V];
+  update_link_ue<NC, R>(a, i, t, iz, E, a.Un + link_index(NC, i, 0, a.g.V, s), F, Ui, E0);
 }
 
 // Link i of the site with transverse index t on slice iz, its force from
