@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
     mbar_fence_init();
   }
   __syncthreads();
+  follow();
   if (tid >= SG::CONSUMERS) {
     // ---- producer ----
     if (tid != SG::CONSUMERS) return;
@@ -202,8 +203,8 @@ __global__ void __launch_bounds__(StagedGeo<RB>::THREADS, 1) k_step_staged(Stage
   const uint32_t t = (uint32_t)(inner ? iy : 0) * NX + ix;
   // The thread's site in a slot's image of one direction, and the steps to its
   // neighbours: the same for every slice, so a link's address is one addition
-  // (formed anew for every link it was 120 instructions of an update: 512 x 64^2
-  // 0.423 -> 0.398 ms per step).
+  // (formed anew for every link and field, addresses were 225 integer instructions
+  // of 1825 per update, now 128 of 1699: 512 x 64^2 0.423 -> 0.390 ms per step).
   auto col = [](int x) { return (x >> 5) * 288 + (x & 31); };
   const float2* const own = sm + (r + 1) * RB * 288 + col(ix);
   const int xp = col(ix + 1 == NX ? 0 : ix + 1) - col(ix), xm = col(ix == 0 ? NX - 1 : ix - 1) - col(ix);
@@ -312,9 +313,9 @@ static int launch_staged_t(glasma_ctx* c, bool hop) {
   if (chunks > nsl) chunks = nsl;
   sa.zlen = (nsl + chunks - 1) / chunks;
   chunks = (nsl + sa.zlen - 1) / sa.zlen;
-  k_step_staged<RB><<<dim3((unsigned)tiles, (unsigned)chunks), SG::THREADS, SG::smem, c->stream>>>(sa);
   c->staged_launched = true;
-  return cuda_check(cudaGetLastError(), "k_step_staged launch");
+  return launch_following("k_step_staged launch", k_step_staged<RB>, dim3((unsigned)tiles, (unsigned)chunks),
+                          SG::THREADS, SG::smem, c->stream, sa);
 }
 
 int launch_step_staged(glasma_ctx* c, bool hop) {
