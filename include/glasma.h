@@ -545,8 +545,9 @@ GLASMA_API int glasma_adjoint_energy(const glasma_params* p, const double* rho_h
  * Batched ensemble (the event averages of Sec. 2 and Sec. 4): several
  * independent leapfrog events, possibly of different nz, ny, nx, advanced
  * together.  Each event's result is bitwise the one glasma_step gives it
- * alone (the same per-link arithmetic).  Execution modes:
- *   GLASMA_BATCH_GRAPH (default): per time step, one kernel launch per
+ * alone with the same step kernel (graph and persistent: the staple kernel;
+ * per-event: the context's own).  Execution modes:
+ *   GLASMA_BATCH_GRAPH: per time step, one kernel launch per
  *     geometry class (the events of equal nz, ny, nx together); the
  *     launches of one call are captured on a private stream into one CUDA
  *     graph, launched on the events' stream.  The call does not
@@ -559,8 +560,12 @@ GLASMA_API int glasma_adjoint_energy(const glasma_params* p, const double* rho_h
  *     checkpoint).  The call synchronises the stream to read the barrier's
  *     status after each launch.
  *   GLASMA_BATCH_PER_EVENT: the single-event step kernel of every event and
- *     step captured into one graph (best for events that fill the GPU on
- *     their own).  The call does not synchronise.
+ *     step, launched in turn (best for events that fill the GPU on their
+ *     own).  The call does not synchronise.
+ *   The default, until glasma_batch_set_shape or glasma_batch_tune, is the
+ *   graph with blocks of 32 sites, or the per-event mode where every event's
+ *   own step kernel is the two-pass FP64 kernel or the one-thread-per-site
+ *   FP32 SU(2) kernel (fewer operations than the graph's staple form).
  *
  * glasma_batch_create: ctxs[0..n-1], 1 <= n <= 64, distinct contexts that
  *   share nc, precision, dt, a_t, a_z, the device and the stream, all with

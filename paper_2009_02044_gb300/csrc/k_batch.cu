@@ -287,8 +287,8 @@ static int launch_persistent(PersistArgs<R>& a, int bx, int extra_arrivals, cuda
 
 struct glasma_batch {
   std::vector<glasma_ctx*> ev;
-  int bx = 64;                       // transverse sites per block
-  int mode = GLASMA_BATCH_GRAPH;
+  int bx = 32;                       // transverse sites per block
+  int mode = -1;                     // set by the caller or the tuner; -1: default_mode
   int device = 0;
   cudaStream_t stream = nullptr;     // the events' stream
   cudaStream_t capture = nullptr;    // private stream the graph is captured on
@@ -537,10 +537,23 @@ GLASMA_API int glasma_batch_create(glasma_ctx* const* ctxs, int n, glasma_batch*
   return GLASMA_OK;
 }
 
+// Where every event's own step kernel does less arithmetic than the staple form
+// of the graph's kernel, that is worth more than filling the GPU with one launch
+// for a class, whatever the events' sizes (ms per step: 24 events, FP64 SU(3) 256 x
+// {32, 48, 64}^2 105 -> 70 and 128 x {16, 24, 33}^2 14.1 -> 9.4; 12 events of 160 x
+// {8, 11}^2 1.36 -> 0.94, SU(2) 0.26 -> 0.19; FP32 SU(2) 256 x {32, 48, 64}^2 0.98 ->
+// 0.78).  With the staple form in both, the graph is faster (FP32 SU(3), the same
+// lattices, 3.26 against 3.47, 0.46 against 0.55, 0.056 against 0.109).
+static int default_mode(const glasma_batch* b) {
+  for (const glasma_ctx* c : b->ev)
+    if (!use_parts_kernel(c) && !use_site_kernel(c)) return GLASMA_BATCH_GRAPH;
+  return GLASMA_BATCH_PER_EVENT;
+}
+
 GLASMA_API int glasma_batch_step(glasma_batch* b, int n_steps) {
   if (!b || n_steps < 0) return set_error(GLASMA_ERR_INVALID_ARG, "bad batch or n_steps");
   cudaSetDevice(b->device);
-  return batch_dispatch(b, n_steps, b->mode, b->bx);
+  return batch_dispatch(b, n_steps, b->mode < 0 ? default_mode(b) : b->mode, b->bx);
 }
 
 GLASMA_API int glasma_batch_set_shape(glasma_batch* b, int mode, int block_sites) {

@@ -2,7 +2,8 @@
 of its range and against the general path: the FP64 step in two passes (its
 ring of slices wrapping, rows longer than a block, planes whose scratch holds
 two slices), the FP32 SU(2) step with one thread per site (from 2^17 sites
-on), T^{mu nu} of SU(2), and the FP32 -> FP64 conversion of the observables."""
+on), T^{mu nu} of SU(2), the FP32 -> FP64 conversion of the observables, and the
+kernels of a batch."""
 import numpy as np
 import pytest
 
@@ -105,3 +106,26 @@ def test_fp32_fields_are_widened_exactly(G, scale):
     g = G.glasma_gauss_residual(_ctx(G, st, "fp32"))
     ref = O.gauss_residual(st)
     assert abs(g[0] - ref[0]) <= 1e-14 * ref[0]
+
+
+@pytest.mark.parametrize("nc,precision,sizes,kernel", [
+    (2, "fp64", [(48, 12, 10), (40, 16, 16)], "auto"),
+    (3, "fp64", [(48, 12, 10), (56, 9, 5)], "auto"),
+    (2, "fp32", [(40, 64, 64), (34, 64, 64)], "auto"),
+    (2, "fp32", [(40, 64, 64), (40, 16, 16)], "staple"),
+    (3, "fp32", [(48, 12, 10), (40, 64, 16)], "staple")])
+def test_default_batch_takes_the_cheaper_kernel(G, nc, precision, sizes, kernel):
+    """The events' own kernels where all of them do less arithmetic than the
+    staple form, else the graph's staple form: bitwise the single steps."""
+    cfgs = [dict(gi.small_config(nc, nz=nz, nx=nx, ny=ny, sigma_l=1.0, seed=60 + k),
+                 precision=precision) for k, (nz, nx, ny) in enumerate(sizes)]
+    batched = [G.glasma_init_mv(c, None) for c in cfgs]
+    b = G.glasma_batch_create(batched)
+    G.glasma_batch_step(b, 9)
+    for c, h in zip(cfgs, batched):
+        one = G.glasma_init_mv(c, None)
+        G.glasma_set_step_kernel(one, kernel)
+        G.glasma_step(one, 9)
+        for x, y in zip(G.glasma_get_fields(one)[:4], G.glasma_get_fields(h)[:4]):
+            assert np.array_equal(x, y)
+    b.close()
