@@ -131,12 +131,12 @@ static int check_params(const glasma_params* p) {
 // The automatic choice, from CUDA-event timings on GB300: in FP64 the
 // two-pass plaquette form on every lattice whose scratch was allocated (the
 // fewest multiply-adds, and the FP64 pipe bounds the step; figures in
-// k_step_plaq64.cu); in FP32 SU(3) with rows
-// of 64 sites the staged staple kernel (0.446-0.449 ms against 0.472-0.475
-// for the one-site staple kernel, bitwise the same result), else the staple
-// kernel (0.469 ms, against 0.521 for the plaquette kernel and 0.572 for
-// site pairs, whose 168 registers leave too few warps to hide latency); in
-// FP32 SU(2) one thread per site on large lattices (0.60 against 1.10 ms for
+// k_step_plaq64.cu); in FP32 SU(3) with rows of 64 sites the staged staple
+// kernel (0.388 ms per 512 x 64^2 step against 0.432 for the staple kernel,
+// bitwise the same result; with rows of 32 sites 0.125 against 0.111 per
+// 512 x 32^2 step), else the staple kernel (with full triple products 0.469 ms,
+// against 0.521 for the plaquette kernel and 0.572 for site pairs, whose 168
+// registers leave too few warps to hide latency); in FP32 SU(2) one thread per site on large lattices (0.60 against 1.10 ms for
 // the staple kernel and 1.39 for site pairs per 1024 x 128^2 step), the staple
 // kernel on small ones.
 bool use_plaq_kernel(const glasma_ctx* c) {
@@ -155,8 +155,9 @@ bool use_pair_kernel(const glasma_ctx* c) {
 
 // One thread per site from 2^17 sites of the whole lattice on (a slab decides as
 // the lattice does): below that, three times fewer threads than links no longer
-// fill the GPU (200 x 30 x 20, 0.0129 against 0.0125 ms per step; 768 x 64^2,
-// 0.120 against 0.209).
+// fill the GPU (ns per site and step: the staple kernel 0.082 on 200 x 30 x 20, this
+// one 0.079 on 140 x 31^2, 0.060 on 131 x 45 x 48 and 0.038 on 768 x 64^2, where
+// the staple kernel took 0.066).
 bool use_site_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_AUTO && c->rs == 4 && c->p.nc == 2 &&
          (long long)c->nz_glob * c->g.nxy >= (1 << 17);
