@@ -11,9 +11,26 @@ struct Dev4 {  // a link, less 1
   float w, x, y, z;
 };
 
-__device__ __forceinline__ Dev4 dev_load(const float4* p) {
-  const float4 v = __ldg(p);  // (alpha.re - 1, alpha.im, beta.re, beta.im)
+// Loads for kernels that begin with follow(), which are placed while the step
+// before them still writes the links: no read-only loads, those are for data that
+// nothing writes in the kernel's lifetime.
+__device__ __forceinline__ Dev4 dev_of(float4 v) {  // (alpha.re - 1, alpha.im, beta.re, beta.im)
   return Dev4{v.x, v.w, v.z, v.y};
+}
+__device__ __forceinline__ Dev4 dev_load(const float4* p) { return dev_of(*p); }
+// The same for a kernel that writes no link of the array it reads: the load need
+// not keep its place among the kernel's stores, as dev_load does (1024 x 128^2
+// 0.601 for 0.593 ms per step).  links_of, on whose result every address depends,
+// keeps it behind follow()'s wait.
+__device__ __forceinline__ const float4* links_of(const float2* U) {
+  const float4* p = reinterpret_cast<const float4*>(U);
+  asm volatile("" : "+l"(p));
+  return p;
+}
+__device__ __forceinline__ Dev4 dev_load_free(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return dev_of(v);
 }
 __device__ __forceinline__ Dev4 dev_dag(Dev4 a) { return Dev4{a.w, -a.x, -a.y, -a.z}; }
 // (w + i a.s)(v + i b.s) = (w v - a.b) + i (w b + v a - a x b).s, the products

@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
   // next slice, by the same instructions, so that results do not depend on
   // where the blocks' ranges begin.
   int z = z0 > 0 ? z0 - 1 : 0;
-  const float4* Ux = reinterpret_cast<const float4*>(a.U) + (int64_t)z * g.nxy;
-  Dev4 ux = dev_load(Ux + t), uy = dev_load(Ux + g.V + t);
+  const float4* Ux = links_of(a.U) + (int64_t)z * g.nxy;
+  Dev4 ux = dev_load_free(Ux + t), uy = dev_load_free(Ux + g.V + t);
   Vec3 cx{0.f, 0.f, 0.f}, cy{0.f, 0.f, 0.f};  // vec BA of the planes xz, yz of the slice below
 #pragma unroll 1
   for (; z < z1; ++z, Ux += g.nxy) {
@@ -144,12 +144,12 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
       Ez = site_field(a, 2, s);
     }
     if (up) {
-      uz = dev_load(Uz + t);
-      nux = dev_load(Ux + g.nxy + t);
-      nuy = dev_load(Uy + g.nxy + t);
+      uz = dev_load_free(Uz + t);
+      nux = dev_load_free(Ux + g.nxy + t);
+      nuy = dev_load_free(Uy + g.nxy + t);
       // planes xz and yz based here: A = U_z(x+a) U_a^dag(x+z), B = U_z^dag U_a
       {
-        const Dev4 A = dev_mul(dev_load(Uz + txp), dev_dag(nux)), B = dev_mul(dev_dag(uz), ux);
+        const Dev4 A = dev_mul(dev_load_free(Uz + txp), dev_dag(nux)), B = dev_mul(dev_dag(uz), ux);
         const Vec3 m = sym3(A, B), c = cross3(vec3(A), vec3(B));
         nx_ = Vec3{m.x + c.x, m.y + c.y, m.z + c.z};
         const Vec3 p = turn3(ux, Vec3{m.x - c.x, m.y - c.y, m.z - c.z});
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
         add3(Fz, wt, p);
       }
       {
-        const Dev4 A = dev_mul(dev_load(Uz + typ), dev_dag(nuy)), B = dev_mul(dev_dag(uz), uy);
+        const Dev4 A = dev_mul(dev_load_free(Uz + typ), dev_dag(nuy)), B = dev_mul(dev_dag(uz), uy);
         const Vec3 m = sym3(A, B), c = cross3(vec3(A), vec3(B));
         ny_ = Vec3{m.x + c.x, m.y + c.y, m.z + c.z};
         const Vec3 p = turn3(uy, Vec3{m.x - c.x, m.y - c.y, m.z - c.z});
@@ -170,26 +170,26 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
       add3(Fy, wz, cy);
       // plane xy based here: Im tr t (U_x U_y(x+x)) (U_y U_x(x+y))^dag
       {
-        const Dev4 A = dev_mul(ux, dev_load(Uy + txp)), B = dev_mul(uy, dev_load(Ux + typ));
+        const Dev4 A = dev_mul(ux, dev_load_free(Uy + txp)), B = dev_mul(uy, dev_load_free(Ux + typ));
         const Vec3 p = vec_ab(A, dev_dag(B));
         add3(Fx, -wt, p);
         add3(Fy, wt, p);
       }
       // plaquettes at x - e_x: vec AB of the planes xy (link y) and xz (link z)
       {
-        const Dev4 vx = dev_load(Ux + txm);
-        add3(Fy, -wt, vec_ab(dev_mul(uy, dev_dag(dev_load(Ux + txmyp))), dev_mul(dev_dag(dev_load(Uy + txm)), vx)));
+        const Dev4 vx = dev_load_free(Ux + txm);
+        add3(Fy, -wt, vec_ab(dev_mul(uy, dev_dag(dev_load_free(Ux + txmyp))), dev_mul(dev_dag(dev_load_free(Uy + txm)), vx)));
         if (up)
           add3(Fz, -wt,
-               vec_ab(dev_mul(uz, dev_dag(dev_load(Ux + g.nxy + txm))), dev_mul(dev_dag(dev_load(Uz + txm)), vx)));
+               vec_ab(dev_mul(uz, dev_dag(dev_load_free(Ux + g.nxy + txm))), dev_mul(dev_dag(dev_load_free(Uz + txm)), vx)));
       }
       // plaquettes at x - e_y: vec BA of the plane xy (link x), vec AB of yz (link z)
       {
-        const Dev4 vy = dev_load(Uy + tym);
-        add3(Fx, wt, vec_ab(dev_mul(dev_dag(vy), dev_load(Ux + tym)), dev_mul(dev_load(Uy + txpym), dev_dag(ux))));
+        const Dev4 vy = dev_load_free(Uy + tym);
+        add3(Fx, wt, vec_ab(dev_mul(dev_dag(vy), dev_load_free(Ux + tym)), dev_mul(dev_load_free(Uy + txpym), dev_dag(ux))));
         if (up)
           add3(Fz, -wt,
-               vec_ab(dev_mul(uz, dev_dag(dev_load(Uy + g.nxy + tym))), dev_mul(dev_dag(dev_load(Uz + tym)), vy)));
+               vec_ab(dev_mul(uz, dev_dag(dev_load_free(Uy + g.nxy + tym))), dev_mul(dev_dag(dev_load_free(Uz + tym)), vy)));
       }
       const Vec3 zero{0.f, 0.f, 0.f};
       site_update(a, 0, s, Fx, Ex, zero, ux);
