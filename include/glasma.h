@@ -15,7 +15,11 @@
  *
  * Memory: a context owns every device buffer it uses.  It allocates them at
  * glasma_init_mv through the optional allocator (or cudaMallocAsync on the
- * given stream) and releases them in glasma_free.  All host pointers passed
+ * given stream) and releases them in glasma_free.  An FP64 leapfrog context
+ * holds a scratch for its step beside the state: up to 64 MB (where that holds
+ * the whole lattice's 600 (SU(3)) or 240 bytes (SU(2)) per site, no more), and
+ * two slices of it on larger planes.  Where that much is refused, half of it is
+ * asked for, down to two slices; results do not depend on it.  All host pointers passed
  * in are owned by the caller and only read or written during the call.
  *
  * Streams: a context is bound to one CUDA stream and one device.  Calls that
@@ -367,8 +371,9 @@ GLASMA_API int glasma_slab_unpack(glasma_ctx* c, int dir, const void* dev_buf);
  *                              (blocks of up to 320 threads).  FP64 state
  *                              is stepped in two passes instead, one thread
  *                              per plaquette and then one per link, through
- *                              a scratch of the context (at most 64 MB, or
- *                              two slices of it up to 512 MB);
+ *                              a scratch of the context (see Memory above;
+ *                              the limit on rows holds there too, though
+ *                              AUTO takes rows of any length);
  *   GLASMA_KERNEL_PLAQUETTE_256  the same with blocks of up to 256 threads
  *                              (more registers per thread; FP64 state:
  *                              the two passes);
@@ -391,9 +396,8 @@ GLASMA_API int glasma_slab_unpack(glasma_ctx* c, int dir, const void* dev_buf);
  *   GLASMA_KERNEL_AUTO         the default, from GB300 timings: for FP64
  *                              state the two passes of the plaquette form
  *                              for rows of any length (fewer FMAs where the
- *                              FP64 pipe bounds the step), the staple kernel
- *                              where two slices of their scratch pass
- *                              512 MB; for FP32 SU(2) lattices from 2^17
+ *                              FP64 pipe bounds the step); for FP32 SU(2)
+ *                              lattices from 2^17
  *                              sites on (a slab: of its whole lattice) one
  *                              thread per site in the plaquette form; for
  *                              FP32 SU(3) the staged staple kernel where it

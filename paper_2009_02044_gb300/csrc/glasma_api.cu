@@ -129,9 +129,8 @@ static int check_params(const glasma_params* p) {
 }
 
 // The automatic choice, from CUDA-event timings on GB300: in FP64 the
-// two-pass plaquette form on every lattice whose scratch was allocated (the
-// fewest multiply-adds, and the FP64 pipe bounds the step; figures in
-// k_step_plaq64.cu); in FP32 SU(3) with rows of 64 sites the staged staple
+// two-pass plaquette form (the fewest multiply-adds, and the FP64 pipe bounds
+// the step; figures in k_step_plaq64.cu); in FP32 SU(3) with rows of 64 sites the staged staple
 // kernel (0.388 ms per 512 x 64^2 step against 0.432 for the staple kernel,
 // bitwise the same result; with rows of 32 sites 0.125 against 0.111 per
 // 512 x 32^2 step), else the staple kernel (with full triple products 0.469 ms,
@@ -292,10 +291,9 @@ static int create_ctx(const glasma_params* p, const double* rho_host, void* stre
       return st;
     }
   }
-  // scratch of the FP64 step: without it (too large a plane, or no memory
-  // left) the context steps with the staple kernel
-  if (parts_ring(c) > 0) c->part = (double*)ctx_alloc(c, parts_bytes(c));
   st = run_init(c, rho_host);
+  // after the initial state, whose scratch is free again
+  if (!st) st = parts_alloc(c);
   if (st) {
     std::string keep = g_last_error;
     glasma_free(c);

@@ -45,6 +45,7 @@ struct glasma_ctx {
   int step_zlen = 0;          // z slices per block of the plaquette kernel (0 = automatic)
   bool plaq_ready = false;    // the plaquette kernel's attributes are set on this device
   double* part = nullptr;     // FP64 leapfrog: plaquette contributions (k_step_plaq64.cu)
+  int ring = 0;               // slices of it
   // staged step kernel (k_step_staged.cu): spin budget of one wait on its
   // copies (SM cycles), the timeout test's stall, and whether it has run
   // since its status word (dflag[1]) was last read
@@ -130,9 +131,8 @@ int launch_step_leapfrog(glasma_ctx* c, bool hop);
 int launch_step_plaq(glasma_ctx* c, bool hop, int zlen);
 bool plaq_fits(const glasma_ctx* c);
 // the same form in FP64, in two passes through a scratch array
-// (k_step_plaq64.cu): its ring's slices (0: none) and bytes
-int parts_ring(const glasma_ctx* c);
-size_t parts_bytes(const glasma_ctx* c);
+// (k_step_plaq64.cu), which parts_alloc allocates where the context uses it
+int parts_alloc(glasma_ctx* c);
 // first pass over the slices [z0, z1), with the plaquette norms
 int launch_parts_norms(glasma_ctx* c, int z0, int z1);
 int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches);

@@ -593,7 +593,7 @@ static int launch_tmunu_kernel(glasma_ctx* c, const TmnArgs<R>& a) {
   } else {
     if constexpr (sizeof(R) == 8) {
       if (c->part) {
-        const int ring = parts_ring(c);
+        const int ring = c->ring;
         for (int z0 = 0; z0 < c->g.nz; z0 += ring - 1) {
           const int z1 = min(z0 + ring - 1, c->g.nz);
           int st = launch_parts_norms(c, z0, z1);

@@ -37,10 +37,8 @@
 namespace glasma {
 
 // the scratch aims at this size (it then stays in the L2 cache between the
-// two passes); a ring of two slices may take kPartsMost, above which the
-// context steps with the staple kernel
+// two passes) and holds two slices at least
 constexpr size_t kPartsBytes = (size_t)64 << 20;
-constexpr size_t kPartsMost = (size_t)512 << 20;
 constexpr int kPartsThreads = 64;  // 128 left a sixth of the SMs' FP64 pipes idle on 128 x 16^2
 
 struct PartsArgs {
@@ -183,19 +181,25 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links(PartLinksA
   update_link<NC, double>(a, i, t, z, n.s, F);
 }
 
-// Slices of the ring a context's scratch has, 0 if it takes none.
-int parts_ring(const glasma_ctx* c) {
-  if (c->rs != 8 || c->p.scheme != GLASMA_LEAPFROG) return 0;
+// The scratch of an FP64 leapfrog context.  Where the allocator refuses it, half
+// the slices are tried, down to two: results do not depend on the ring, where
+// stepping with another kernel would change their rounding (and on one rank of
+// several, the slabs).  Two slices are a part 1.2 / nz (SU(3)) or 2.9 / nz (SU(2))
+// of the links and fields, less than the initial state's scratch, which is free by
+// then, on lattices of 20 slices.
+int parts_alloc(glasma_ctx* c) {
+  if (c->rs != 8 || c->p.scheme != GLASMA_LEAPFROG) return GLASMA_OK;
   const size_t slice = sizeof(double) * (size_t)part_doubles(c->na) * (size_t)c->g.nxy;
-  if (2 * slice > kPartsMost) return 0;
+  const size_t whole = (size_t)(c->hi - c->lo) + 1;
   size_t r = kPartsBytes / slice;
+  if (r > whole) r = whole;
   if (r < 2) r = 2;
-  if (r > (size_t)(c->hi - c->lo) + 1) r = (size_t)(c->hi - c->lo) + 1;
-  return (int)r;
-}
-
-size_t parts_bytes(const glasma_ctx* c) {
-  return sizeof(double) * (size_t)part_doubles(c->na) * (size_t)c->g.nxy * (size_t)parts_ring(c);
+  while (!(c->part = (double*)ctx_alloc(c, slice * r))) {
+    if (r == 2) return set_error(GLASMA_ERR_OOM, "step scratch allocation failed");
+    r = r / 2 > 2 ? r / 2 : 2;
+  }
+  c->ring = (int)r;
+  return GLASMA_OK;
 }
 
 // The parts of the slices [z0, z1), of z0 - 1 as well with `below`; at most
@@ -206,7 +210,7 @@ static int launch_parts_pass(glasma_ctx* c, int z0, int z1, bool below) {
   p.U = (const double2*)c->U[c->cur];
   p.part = c->part;
   p.g = c->g;
-  p.ring = parts_ring(c);
+  p.ring = c->ring;
   p.z0 = z0;
   p.zfirst = below ? z0 - 1 : z0;
   p.sites = (uint32_t)((z1 - p.zfirst) * c->g.nxy);
@@ -240,7 +244,7 @@ static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
   a.WB = c->WB;
   a.zlo = c->lo;
   l.part = c->part;
-  l.ring = parts_ring(c);
+  l.ring = c->ring;
   if (zlen <= 0 || zlen > l.ring - 1) zlen = l.ring - 1;
   for (int z0 = c->lo; z0 < c->hi; z0 += zlen) {
     const int z1 = z0 + zlen < c->hi ? z0 + zlen : c->hi;
