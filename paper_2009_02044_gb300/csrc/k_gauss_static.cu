@@ -1,6 +1,7 @@
 // Gauss-law residual over caller-owned device fields that allocates no
 // device memory: its scratch is a fixed array in this file (see
 // glasma_gauss_residual_static in glasma.h).
+#include "divergence.cuh"
 #include "glasma_internal.cuh"
 
 namespace glasma {
@@ -60,23 +61,9 @@ __global__ void __launch_bounds__(kStaticThreads) k_gauss_static_slices(StaticGa
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int t = threadIdx.x; t < a.g.nxy; t += blockDim.x) {
     const int64_t s = (int64_t)iz * a.g.nxy + t;
-    SiteNbr n = site_nbr(a.g, s);
+    const SiteNbr n = site_nbr(a.g, s);
     double gv[NA];
-#pragma unroll
-    for (int c = 0; c < NA; ++c) gv[c] = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-#pragma unroll
-      for (int c = 0; c < NA; ++c) gv[c] += a.ia2[i] * (double)E[(int64_t)(i * NA + c) * a.g.V + s];
-      if (i == 2 && iz == 0) continue;
-      double q[NA];
-#pragma unroll
-      for (int c = 0; c < NA; ++c) q[c] = (double)E[(int64_t)(i * NA + c) * a.g.V + n.m[i]];
-      typename G::M um = LinkIO<NC, R>::template load<double>(U, i, a.g.V, n.m[i]);
-      G::adj_dag(um, q);
-#pragma unroll
-      for (int c = 0; c < NA; ++c) gv[c] -= a.ia2[i] * q[c];
-    }
+    divergence_at<NC, R>(U, E, a.g, n, a.ia2, gv);
     const int ka = iz - a.zA0, kb = iz - a.zB0;
 #pragma unroll
     for (int c = 0; c < NA; ++c) {

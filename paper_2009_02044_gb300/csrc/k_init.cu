@@ -329,7 +329,8 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
       double q[NA];
       for (int c = 0; c < NA; ++c) q[c] = widen<double>(em[c]);
       typename G::M um = LinkIO<NC, R>::template load<double>(U, i, g.V, n.m[i]);
-      G::adj_dag(um, q);
+      // the links of an FP32 state are unitary to their rounding only
+      G::template adj_dag<sizeof(R) == 4>(um, q);
       for (int c = 0; c < NA; ++c) dv[c] -= w * q[c];
     }
     for (int c = 0; c < NA; ++c) {

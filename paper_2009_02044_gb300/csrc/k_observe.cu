@@ -3,6 +3,7 @@
 // Reductions are deterministic: fixed grid, fixed-order tree in shared
 // memory, fixed-order final pass over the block partials.
 #include "dev_su2.cuh"
+#include "divergence.cuh"
 #include "glasma_internal.cuh"
 #include "plaq_parts.cuh"
 
@@ -46,53 +47,46 @@ struct GaussArgs {
   double* part;    // [gridDim][4]
 };
 
+// The FP64 pipe bounds it (SU(3): some 475 of its operations per site; 160 x 64^2
+// FP32 0.651 ms, 0.700 with the general transport but its sums formed link by
+// link and the maximum by FP64 comparisons).  More registers than this leave
+// too few warps for the loads (0.674 at 250).
 template <int NC, typename R>
-__global__ void __launch_bounds__(kRedThreads) k_gauss(GaussArgs<R> a) {
+__global__ void __launch_bounds__(kRedThreads, NC == 2 ? 3 : 2) k_gauss(GaussArgs<R> a) {
   typedef Group<NC, double> G;
   constexpr int NA = G::NA;
   __shared__ double sh[4][kRedThreads];
-  double gmax = 0, gsum2 = 0, rmax = 0, bad = 0;
+  unsigned long long gmax = 0;  // bits of the largest |G|
+  double gsum2 = 0, rmax = 0, bad = 0;
   for (int64_t s = a.s0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.s1;
        s += (int64_t)gridDim.x * blockDim.x) {
-    SiteNbr n = site_nbr(a.g, s);
+    const SiteNbr n = site_nbr(a.g, s);
     double gv[NA];
-#pragma unroll
-    for (int c = 0; c < NA; ++c) gv[c] = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      double q[NA];
-#pragma unroll
-      for (int c = 0; c < NA; ++c) gv[c] += a.ia2[i] * widen<double>(a.E[(int64_t)(i * NA + c) * a.g.V + s]);
-      if (i == 2 && n.iz == 0) continue;
-      const int64_t sm = n.m[i];
-#pragma unroll
-      for (int c = 0; c < NA; ++c) q[c] = widen<double>(a.E[(int64_t)(i * NA + c) * a.g.V + sm]);
-      typename G::M um = LinkIO<NC, R>::template load<double>(a.U, i, a.g.V, sm);
-      G::adj_dag(um, q);
-#pragma unroll
-      for (int c = 0; c < NA; ++c) gv[c] -= a.ia2[i] * q[c];
-    }
-    const int64_t t = s % a.g.nxy;
-    double rho[NA];
-#pragma unroll
-    for (int c = 0; c < NA; ++c) rho[c] = 0.0;
+    divergence_at<NC, R>(a.U, a.E, a.g, n, a.ia2, gv);
     const int ka = n.iz - a.zA0, kb = n.iz - a.zB0;
-    if (ka >= 0 && ka < a.WA)
+    const bool ina = ka >= 0 && ka < a.WA, inb = kb >= 0 && kb < a.WB;
+    if (ina || inb) {
+      const int64_t t = s % a.g.nxy;
 #pragma unroll
-      for (int c = 0; c < NA; ++c) rho[c] += widen<double>(a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t]);
-    if (kb >= 0 && kb < a.WB)
-#pragma unroll
-      for (int c = 0; c < NA; ++c) rho[c] += widen<double>(a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t]);
+      for (int c = 0; c < NA; ++c) {
+        double rho = 0.0;
+        if (ina) rho += widen<double>(a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t]);
+        if (inb) rho += widen<double>(a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t]);
+        gv[c] -= rho;
+        rmax = fmax(rmax, fabs(rho));
+      }
+    }
 #pragma unroll
     for (int c = 0; c < NA; ++c) {
-      double r = gv[c] - rho[c];
-      if (!isfinite(r)) bad += 1.0;
-      gmax = fmax(gmax, fabs(r));
-      gsum2 += r * r;
-      rmax = fmax(rmax, fabs(rho[c]));
+      // the bits of non-negative doubles order as they do: no FP64 comparison
+      const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(gv[c]));
+      const unsigned long long inf = 0x7ff0000000000000ULL;
+      if (b >= inf) bad += 1.0;
+      if (b <= inf && b > gmax) gmax = b;
+      gsum2 += gv[c] * gv[c];
     }
   }
-  double v[4] = {gmax, gsum2, rmax, bad};
+  double v[4] = {__longlong_as_double((long long)gmax), gsum2, rmax, bad};
   const int op[4] = {1, 0, 1, 0};
   block_reduce<4>(sh, v, op);
   if (threadIdx.x == 0)

@@ -142,21 +142,58 @@ struct Group<2, R> {
     const M e = expi_m1(v, c);
     return M{fma_c(e.a, u.a, fma_cj(-e.b, u.b, u.a)), fma_c(e.a, u.b, fma_cj(e.b, u.a, u.b))};
   }
-  // U = w + i (x, y, z).sigma with alpha = w + i z, beta = y + i x rotates
+  // U = w + i (x, y, z).sigma with alpha = w + i z, beta = y + i x turns
   // the algebra vector: with c = (x, y, z) x q,
-  // U q U^+ = q + 2 [(x, y, z) x c - w c], and U^+ q U has w -> -w: 18
-  // multiply-adds, where the two matrix products take 32.
-  GL_HD static void rotate(R w, const M& u, R* q) {
+  // U q U^+ = |U|^2 q + 2 [(x, y, z) x c - w c], and U^+ q U has w -> -w.
+  // half_turn adds the bracket to h: 15 multiply-adds.
+  GL_HD static void half_turn(R w, const M& u, const R* q, R* h) {
     const R x = u.b.im, y = u.b.re, z = u.a.im;
     const R c0 = fma(y, q[2], -(z * q[1])), c1 = fma(z, q[0], -(x * q[2])), c2 = fma(x, q[1], -(y * q[0]));
-    q[0] = fma(R(2), fma(y, c2, fma(-z, c1, -(w * c0))), q[0]);
-    q[1] = fma(R(2), fma(z, c0, fma(-x, c2, -(w * c1))), q[1]);
-    q[2] = fma(R(2), fma(x, c1, fma(-y, c0, -(w * c2))), q[2]);
+    h[0] = fma(y, c2, fma(-z, c1, fma(-w, c0, h[0])));
+    h[1] = fma(z, c0, fma(-x, c2, fma(-w, c1, h[1])));
+    h[2] = fma(x, c1, fma(-y, c0, fma(-w, c2, h[2])));
   }
-  // q <- U^dagger q U
-  GL_HD static void adj_dag(const M& u, R* q) { rotate(-u.a.re, u, q); }
-  // q <- U q U^dagger
-  GL_HD static void adj(const M& u, R* q) { rotate(u.a.re, u, q); }
+  // for |U| = 1: 18 multiply-adds, where the two matrix products take 32
+  GL_HD static void rotate(R w, const M& u, R* q) {
+    R h[3] = {R(0), R(0), R(0)};
+    half_turn(w, u, q, h);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = fma(R(2), h[k], q[k]);
+  }
+  // A sum of algebra vectors n + 2 h, and what U q U^+ (DAG: U^+ q U) adds to
+  // it for any U: 22 multiply-adds
+  struct Acc {
+    R n[3], h[3];
+  };
+  GL_HD static Acc acc(const R* q) { return Acc{{q[0], q[1], q[2]}, {R(0), R(0), R(0)}}; }
+  template <bool DAG>
+  GL_HD static void conj_add(const M& u, const R* q, Acc& t) {
+    const R n = fma(u.a.re, u.a.re, fma(u.a.im, u.a.im, fma(u.b.re, u.b.re, u.b.im * u.b.im)));
+    half_turn(DAG ? -u.a.re : u.a.re, u, q, t.h);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t.n[k] = fma(n, q[k], t.n[k]);
+  }
+  GL_HD static void from_acc(const Acc& t, R* q) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = fma(R(2), t.h[k], t.n[k]);
+  }
+  template <bool DAG>
+  GL_HD static void conj_any(const M& u, R* q) {
+    Acc t{{R(0), R(0), R(0)}, {R(0), R(0), R(0)}};
+    conj_add<DAG>(u, q, t);
+    from_acc(t, q);
+  }
+  // q <- U^dagger q U and U q U^dagger for U in SU(2); ANY: for any U
+  template <bool ANY = false>
+  GL_HD static void adj_dag(const M& u, R* q) {
+    if (ANY) conj_any<true>(u, q);
+    else rotate(-u.a.re, u, q);
+  }
+  template <bool ANY = false>
+  GL_HD static void adj(const M& u, R* q) {
+    if (ANY) conj_any<false>(u, q);
+    else rotate(u.a.re, u, q);
+  }
   GL_HD static M reunit(const M& x) {
     R n2 = x.a.re * x.a.re + x.a.im * x.a.im + x.b.re * x.b.re + x.b.im * x.b.im;
     R f = R(1) / gl_sqrt(n2);
@@ -332,50 +369,90 @@ struct Group<3, R> {
     v[6] = h.m[7].im - h.m[5].im;
     v[7] = r3 * (h.m[0].re + h.m[4].re - R(2) * h.m[8].re);
   }
-  // q <- V q V^+ (V = U, or V = U^+ for DAG) through the hermitian matrix H
-  // of q: M = V H with H's real diagonal (10 multiply-adds per entry), then
-  // the upper triangle of the hermitian M V^+ (its trace is that of H, 0):
-  // 138 multiply-adds, where two full products take 216.
-  template <bool DAG>
-  GL_HD static void conj_alg(const M& u, R* q) {
-    const M h = herm(q);
-    cplx<R> m[9], v[9];
+  // The upper triangle of a sum of hermitian matrices 2 q^a t^a, whose entries
+  // off the diagonal are the components themselves, and what V q V^+ (V = U, or
+  // V = U^+ for DAG) adds to it: rows 0 and 1 of M = V H, H = 2 q^a t^a with a
+  // real diagonal (10 multiply-adds per entry), the triangle of M V^+ and its
+  // last diagonal entry as a quadratic form of V's third row (28): 136
+  // multiply-adds, where two full products take 216.  SU: V in SU(3), so that the
+  // trace stays that of H, 0 (t2 is left out): 108.  (The Gauss residual is held
+  // to its formula on any links: those of an FP32 state are unitary to their
+  // rounding only, and a residual is what differences leave.)
+  struct Acc {
+    cplx<R> t01, t02, t12;
+    R t0, t1, t2;
+  };
+  GL_HD static Acc acc(const R* q) {
+    const R r3 = R(0.57735026918962576451);  // 1/sqrt 3
+    return Acc{{q[0], -q[1]}, {q[3], -q[4]}, {q[5], -q[6]}, fma(r3, q[7], q[2]), fma(r3, q[7], -q[2]),
+               R(-2) * (r3 * q[7])};
+  }
+  template <bool DAG, bool SU = false>
+  GL_HD static void conj_add(const M& u, const R* q, Acc& t) {
+    const Acc H = acc(q);
+    const R hd[3] = {H.t0, H.t1, H.t2};
+    const cplx<R> h[3] = {H.t01, H.t02, H.t12};
+    cplx<R> v[9], m[6];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) v[3 * i + j] = DAG ? cj(u.m[3 * j + i]) : u.m[3 * i + j];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         const cplx<R> d = v[3 * i + j];
-        cplx<R> acc{h.m[4 * j].re * d.re, h.m[4 * j].re * d.im};
+        cplx<R> s{hd[j] * d.re, hd[j] * d.im};
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-          if (k != j) acc = fma_c(v[3 * i + k], h.m[3 * k + j], acc);
-        m[3 * i + j] = acc;
+        for (int k = 0; k < 3; ++k) {  // H_kj = conj(H_jk)
+          if (k < j) s = fma_c(v[3 * i + k], h[k + j - 1], s);
+          if (k > j) s = fma_cj(v[3 * i + k], h[k + j - 1], s);
+        }
+        m[3 * i + j] = s;
       }
-    cplx<R> t01{R(0), R(0)}, t02{R(0), R(0)}, t12{R(0), R(0)};
-    R t0 = R(0), t1 = R(0);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      t01 = fma_cj(m[k], v[3 + k], t01);
-      t02 = fma_cj(m[k], v[6 + k], t02);
-      t12 = fma_cj(m[3 + k], v[6 + k], t12);
-      t0 = fma(m[k].re, v[k].re, fma(m[k].im, v[k].im, t0));
-      t1 = fma(m[3 + k].re, v[3 + k].re, fma(m[3 + k].im, v[3 + k].im, t1));
+      t.t01 = fma_cj(m[k], v[3 + k], t.t01);
+      t.t02 = fma_cj(m[k], v[6 + k], t.t02);
+      t.t12 = fma_cj(m[3 + k], v[6 + k], t.t12);
+      t.t0 = fma(m[k].re, v[k].re, fma(m[k].im, v[k].im, t.t0));
+      t.t1 = fma(m[3 + k].re, v[3 + k].re, fma(m[3 + k].im, v[3 + k].im, t.t1));
     }
-    q[0] = R(2) * t01.re;
-    q[1] = R(-2) * t01.im;
-    q[2] = t0 - t1;
-    q[3] = R(2) * t02.re;
-    q[4] = R(-2) * t02.im;
-    q[5] = R(2) * t12.re;
-    q[6] = R(-2) * t12.im;
-    q[7] = R(1.73205080756887729353) * (t0 + t1);  // (t0 + t1 - 2 t2) / sqrt 3, t2 = -t0 - t1
+    if (SU) return;
+    R s = R(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const cplx<R> p = mulc(v[k == 2 ? 7 : 6], v[k == 0 ? 7 : 8]);  // of the pairs 01, 02, 12
+      s = fma(h[k].re, p.re, fma(-h[k].im, p.im, s));
+      t.t2 = fma(hd[k], fma(v[6 + k].re, v[6 + k].re, v[6 + k].im * v[6 + k].im), t.t2);
+    }
+    t.t2 = fma(R(2), s, t.t2);
   }
-  GL_HD static void adj_dag(const M& u, R* q) { conj_alg<true>(u, q); }
-  GL_HD static void adj(const M& u, R* q) { conj_alg<false>(u, q); }
+  template <bool SU = false>
+  GL_HD static void from_acc(const Acc& t, R* q) {
+    q[0] = t.t01.re;
+    q[1] = -t.t01.im;
+    q[2] = R(0.5) * (t.t0 - t.t1);
+    q[3] = t.t02.re;
+    q[4] = -t.t02.im;
+    q[5] = t.t12.re;
+    q[6] = -t.t12.im;
+    // (t0 + t1 - 2 t2) / (2 sqrt 3); SU: t2 = -t0 - t1
+    if (SU) q[7] = R(0.86602540378443864676) * (t.t0 + t.t1);
+    else q[7] = R(0.28867513459481288225) * fma(R(-2), t.t2, t.t0 + t.t1);
+  }
+  template <bool DAG, bool SU>
+  GL_HD static void conj_alg(const M& u, R* q) {
+    const cplx<R> z{R(0), R(0)};
+    Acc t{z, z, z, R(0), R(0), R(0)};
+    conj_add<DAG, SU>(u, q, t);
+    from_acc<SU>(t, q);
+  }
+  // q <- U^dagger q U and U q U^dagger for U in SU(3); ANY: for any U
+  template <bool ANY = false>
+  GL_HD static void adj_dag(const M& u, R* q) { conj_alg<true, !ANY>(u, q); }
+  template <bool ANY = false>
+  GL_HD static void adj(const M& u, R* q) { conj_alg<false, !ANY>(u, q); }
 
   // exp(i c v^a t^a) - 1 by Cayley-Hamilton for ||Q||_F <= 1/2, Q = c v^a t^a:
   // Q^3 = c1 Q + c0 with c1 = tr(Q^2)/2 and c0 = det Q, so every power is
