@@ -121,7 +121,7 @@ def step_kernel_name(nc, precision, kernel, nx=64):
     of its name (the library's automatic choice: in FP64 the two passes
     k_step_plaq_parts and k_step_plaq_links; in FP32 the staged staple kernel
     for SU(3) rows of 64 sites, k_step_leapfrog_site for SU(2) lattices from
-    2^17 sites on, else the one-link staple kernel k_step_leapfrog)."""
+    3 * 2^16 sites on, else the one-link staple kernel k_step_leapfrog)."""
     if kernel == "auto":
         kernel = ("plaquette" if precision == "fp64" else
                   "staple_staged" if (nc == 3 and nx == 64) else "staple")

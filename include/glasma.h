@@ -397,7 +397,7 @@ GLASMA_API int glasma_slab_unpack(glasma_ctx* c, int dir, const void* dev_buf);
  *                              state the two passes of the plaquette form
  *                              for rows of any length (fewer FMAs where the
  *                              FP64 pipe bounds the step); for FP32 SU(2)
- *                              lattices from 2^17
+ *                              lattices from 3 * 2^16
  *                              sites on (a slab: of its whole lattice) one
  *                              thread per site in the plaquette form; for
  *                              FP32 SU(3) the staged staple kernel where it

@@ -152,14 +152,16 @@ bool use_pair_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_STAPLE_PAIRS;
 }
 
-// One thread per site from 2^17 sites of the whole lattice on (a slab decides as
-// the lattice does): below that, three times fewer threads than links no longer
-// fill the GPU (ns per site and step: the staple kernel 0.082 on 200 x 30 x 20, this
-// one 0.079 on 140 x 31^2, 0.060 on 131 x 45 x 48 and 0.038 on 768 x 64^2, where
-// the staple kernel took 0.066).
+// One thread per site from 3 * 2^16 sites of the whole lattice on (a slab decides
+// as the lattice does).  Alone it is faster than the staple kernel from 2^17 sites on
+// (us per step, 32 x 64^2 9.7 against 10.2, 48 x 64^2 11.8 against 13.8, 768 x 64^2 119
+// against 199, 4099 x 32 x 1 9.3 against 9.9), but a batch steps an event by the kernel
+// the event takes alone, and there the staple form shares one launch (24 events: 32 x
+// 64^2 259 against 210, 40 x 64^2 293 against 260, 48 x 64^2 322 against 311, 64^3 406
+// against 414): the line is where the one gains what the other loses.
 bool use_site_kernel(const glasma_ctx* c) {
   return c->step_kernel == GLASMA_KERNEL_AUTO && c->rs == 4 && c->p.nc == 2 &&
-         (long long)c->nz_glob * c->g.nxy >= (1 << 17);
+         (long long)c->nz_glob * c->g.nxy >= 3 * (1 << 16);
 }
 
 bool use_staged_kernel(const glasma_ctx* c) {

@@ -28,7 +28,7 @@ namespace glasma {
 // Bring the line of p from device memory to L2.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-constexpr int kSiteThreads = 256;  // consecutive transverse sites of a block
+constexpr int kSiteThreads = 256;  // consecutive transverse sites of a block, at most
 constexpr int kSiteBlocks = 3;     // blocks per SM
 
 // exp(i dt e.sigma/2) u, of unit norm: cos(th) - 1 and sin(th) / th by their
@@ -104,11 +104,14 @@ __device__ __forceinline__ Vec3 site_hop(const StepArgs<float>& a, int iz, uint3
   return dj;
 }
 
-__global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_site(StepArgs<float> a, int zlen,
+// T threads per block (of 32, at 96 registers: 80 would spill 164 B and take 13.2
+// us on 4099 x 32 x 1)
+template <int T>
+__global__ void __launch_bounds__(T, T == 32 ? 20 : kSiteBlocks * kSiteThreads / T) k_step_leapfrog_site(StepArgs<float> a, int zlen,
                                                                                  int zhi) {
   follow();
   const Geom& g = a.g;
-  const uint32_t t = blockIdx.x * kSiteThreads + threadIdx.x;
+  const uint32_t t = blockIdx.x * T + threadIdx.x;
   if (t >= (uint32_t)g.nxy) return;
   const uint32_t nx = (uint32_t)g.nx, ny = (uint32_t)g.ny, iy = t / nx, ix = t - iy * nx;
   const uint32_t xp = ix + 1 == nx ? 0 : ix + 1, xm = ix == 0 ? nx - 1 : ix - 1;
@@ -203,6 +206,21 @@ __global__ void __launch_bounds__(kSiteThreads, kSiteBlocks) k_step_leapfrog_sit
   }
 }
 
+// Threads of a block, all on one slice: the most that leave at most a tenth more
+// of them without a site than the fewest do.  Planes of 32 sites ran one warp of
+// eight per block of 256 (us per step: 4099 x 32 x 1 14.6 -> 9.3, 65535 x 1 x 3 168 ->
+// 76, 2048 x 8^2 12.0 -> 9.2, 512 x 17^2 13.2 -> 11.2).
+// Threads numbered through several ranges of slices fill any block, but then a
+// slice is a thread's own number: 80 registers and spills, 1024 x 128^2 0.59 ->
+// 0.82 ms.
+static int site_threads(int64_t nxy) {
+  const int64_t least = (nxy + 31) / 32 * 32;
+  static_assert(kSiteThreads == 256, "launch_step_site lists the kernels");
+  for (int b = kSiteThreads; b > 32; b /= 2)
+    if (10 * ((nxy + b - 1) / b * b) <= 11 * least) return b;
+  return 32;
+}
+
 int launch_step_site(glasma_ctx* c, bool hop) {
   if (c->rs != 4 || c->p.nc != 2) return set_error(GLASMA_ERR_INTERNAL, "the site kernel is FP32 SU(2) only");
   StepArgs<float> a;
@@ -223,13 +241,18 @@ int launch_step_site(glasma_ctx* c, bool hop) {
   a.zB0 = c->zB0;
   a.WB = c->WB;
   a.zlo = c->lo;
+  const int threads = site_threads(c->g.nxy);
   // about four waves of blocks; a range of n slices enters n + 1
-  const int64_t tiles = (c->g.nxy + kSiteThreads - 1) / kSiteThreads, nsl = c->hi - c->lo;
-  int64_t zlen = tiles * nsl / (4 * (int64_t)c->sms * kSiteBlocks);
+  const int64_t tiles = (c->g.nxy + threads - 1) / threads, nsl = c->hi - c->lo;
+  int64_t zlen = tiles * threads * nsl / (4 * (int64_t)c->sms * kSiteBlocks * kSiteThreads);
   if (zlen < 1) zlen = 1;
   if (zlen > 32) zlen = 32;
-  return launch_following("k_step_leapfrog_site launch", k_step_leapfrog_site,
-                          dim3((unsigned)tiles, (unsigned)((nsl + zlen - 1) / zlen)), kSiteThreads, 0, c->stream, a,
+  auto kernel = threads == 256   ? k_step_leapfrog_site<256>
+                : threads == 128 ? k_step_leapfrog_site<128>
+                : threads == 64  ? k_step_leapfrog_site<64>
+                                 : k_step_leapfrog_site<32>;
+  return launch_following("k_step_leapfrog_site launch", kernel,
+                          dim3((unsigned)tiles, (unsigned)((nsl + zlen - 1) / zlen)), threads, 0, c->stream, a,
                           (int)zlen, c->hi);
 }
 

@@ -129,3 +129,61 @@ def test_default_batch_takes_the_cheaper_kernel(G, nc, precision, sizes, kernel)
         for x, y in zip(G.glasma_get_fields(one)[:4], G.glasma_get_fields(h)[:4]):
             assert np.array_equal(x, y)
     b.close()
+
+
+# from 3 * 2^16 sites of FP32 SU(2) on one thread steps a site: planes of whole
+# blocks, planes that end within a warp, planes of less than a block of 256, 64
+# or 32 threads, and the longest lattices
+SITE_SHAPES = [(48, 64, 64), (205, 31, 31), (197, 1, 1001), (6145, 32, 1), (14, 121, 121),
+               (681, 17, 17), (1366, 12, 12), (65535, 1, 4)]
+
+
+@pytest.mark.parametrize("shape", SITE_SHAPES)
+def test_su2_fp32_site_kernel_in_blocks_of_any_size(G, shape):
+    """Within 3e-6 of the staple form after three steps (each within 1.5e-6 of
+    the FP64 step), and no kernel of the staple's bits."""
+    st = _random_state(2, *shape, seed=sum(shape))
+    out = []
+    for kernel in ("staple", "auto"):
+        h = _ctx(G, st, "fp32")
+        G.glasma_set_step_kernel(h, kernel)
+        G.glasma_step(h, 3)
+        out.append(G.glasma_get_fields(h)[:4])
+        G.glasma_free(h)
+    assert all(rel(b, a) <= 3e-6 for a, b in zip(*out))
+    assert not np.array_equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("nranks", [2, 3])
+def test_su2_fp32_site_kernel_on_slabs_of_a_larger_lattice(G, nranks):
+    """Slabs below the kernel's sites of a lattice above them: bitwise the
+    whole lattice."""
+    cfg = dict(gi.small_config(2, nz=71, nx=53, ny=54, sigma_l=2.0), precision="fp32")
+    whole, ranks, T = _run(G, cfg, nranks, 44, "auto")
+    _compare(G, cfg, whole, ranks, T)
+
+
+@pytest.mark.parametrize("shape", [(65535, 1, 4), (6145, 32, 1), (4096, 8, 8), (768, 16, 17)])
+def test_su2_fp32_site_kernel_fills_its_blocks_on_small_planes(G, shape):
+    """The kernel that AUTO takes is no slower than the staple kernel where a
+    plane is a part of a block of 256 (it was by up to 1.5 times)."""
+    import torch
+    st = _random_state(2, *shape, seed=1)
+    st.QA[:] = 0.0
+    st.QB[:] = 0.0
+    best = {}
+    for kernel in ("staple", "auto"):
+        h = _ctx(G, st, "fp32")
+        G.glasma_set_step_kernel(h, kernel)
+        G.glasma_step(h, 100)
+        times = []
+        for _ in range(10):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            G.glasma_step(h, 200)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        best[kernel] = min(times)
+        G.glasma_free(h)
+    assert best["auto"] <= 1.1 * best["staple"], best
