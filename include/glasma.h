@@ -549,8 +549,12 @@ GLASMA_API int glasma_adjoint_energy(const glasma_params* p, const double* rho_h
  * Batched ensemble (the event averages of Sec. 2 and Sec. 4): several
  * independent leapfrog events, possibly of different nz, ny, nx, advanced
  * together.  Each event's result is bitwise the one glasma_step gives it
- * alone with the same step kernel (graph and persistent: the staple kernel;
- * per-event: the context's own).  Execution modes:
+ * alone, whatever its companions: by default and in the per-event mode for
+ * every event, in the graph and persistent modes for FP32 events but those
+ * set to GLASMA_KERNEL_PLAQUETTE or _STAPLE_PAIRS (these two modes run the
+ * staple kernel's arithmetic, FP64 events as with GLASMA_KERNEL_STAPLE; FP32
+ * SU(2) events whose own kernel is the one-thread-per-site kernel are launched
+ * on their own).  Execution modes:
  *   GLASMA_BATCH_GRAPH: per time step, one kernel launch per
  *     geometry class (the events of equal nz, ny, nx together); the
  *     launches of one call are captured on a private stream into one CUDA
@@ -565,11 +569,12 @@ GLASMA_API int glasma_adjoint_energy(const glasma_params* p, const double* rho_h
  *     status after each launch.
  *   GLASMA_BATCH_PER_EVENT: the single-event step kernel of every event and
  *     step, launched in turn (best for events that fill the GPU on their
- *     own).  The call does not synchronise.
+ *     own); small FP64 events of one geometry share the launches of their two
+ *     passes.  The call does not synchronise.
  *   The default, until glasma_batch_set_shape or glasma_batch_tune, is the
- *   graph with blocks of 32 sites, or the per-event mode where every event's
- *   own step kernel is the two-pass FP64 kernel or the one-thread-per-site
- *   FP32 SU(2) kernel (fewer operations than the graph's staple form).
+ *   graph with blocks of 32 sites for the events whose own kernel has the
+ *   staple kernel's bits (FP32 staple and staged), and the per-event mode for
+ *   the others.
  *
  * glasma_batch_create: ctxs[0..n-1], 1 <= n <= 64, distinct contexts that
  *   share nc, precision, dt, a_t, a_z, the device and the stream, all with
@@ -594,7 +599,9 @@ GLASMA_API int glasma_adjoint_energy(const glasma_params* p, const double* rho_h
  *   store it in *block_sites and *mode (either may be NULL).  The events'
  *   states are saved before and restored after each trial (temporary device
  *   copies of U, E and the charges, through each context's allocator), so
- *   the call leaves every event as it found it.  Synchronises the stream.
+ *   the call leaves every event as it found it.  For FP64 events the choice
+ *   decides between two forms that differ in rounding (the staple kernel and
+ *   the context's own).  Synchronises the stream.
  *   Errors: INVALID_ARG, OOM, PARTICLE_EXIT (steps + 1 trial steps would
  *   move a charge off a lattice), TIMEOUT, CUDA.
  * glasma_batch_set_barrier: spin budget of one grid-barrier wait in SM clock

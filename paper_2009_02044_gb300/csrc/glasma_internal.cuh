@@ -136,6 +136,9 @@ int parts_alloc(glasma_ctx* c);
 // first pass over the slices [z0, z1), with the plaquette norms
 int launch_parts_norms(glasma_ctx* c, int z0, int z1);
 int launch_step_parts(glasma_ctx* c, bool hop, int zlen, int* launches);
+constexpr int kMaxBatch = 64;  // events per batch: their kernel parameters stay under the 32 KB limit
+int parts_group_size(const glasma_ctx* c);
+int launch_parts_group(glasma_ctx* const* c, int n, const bool* hop, int* launches);
 // the step kernel glasma_step launches for this context: plaquette (FP64 in
 // two passes), staple on site pairs (FP32), staged staple (FP32 SU(3)) or
 // staple

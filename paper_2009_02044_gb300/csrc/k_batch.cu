@@ -21,7 +21,6 @@
 
 namespace glasma {
 
-constexpr int kMaxBatch = 64;  // events per batch: their kernel parameters stay under the 32 KB limit
 constexpr int kPersistSteps = 64;  // steps per persistent launch (one hop bit each)
 
 // Graph mode's kernel: the events of one geometry class (equal nx, ny, nz)
@@ -288,7 +287,7 @@ static int launch_persistent(PersistArgs<R>& a, int bx, int extra_arrivals, cuda
 struct glasma_batch {
   std::vector<glasma_ctx*> ev;
   int bx = 32;                       // transverse sites per block
-  int mode = -1;                     // set by the caller or the tuner; -1: default_mode
+  int mode = -1;                     // set by the caller or the tuner; -1: the default (own_kernel)
   int device = 0;
   cudaStream_t stream = nullptr;     // the events' stream
   cudaStream_t capture = nullptr;    // private stream the graph is captured on
@@ -300,12 +299,14 @@ struct glasma_batch {
 
 using namespace glasma;
 
+typedef std::vector<glasma_ctx*> Events;
+
 // Host copy of the per-event bookkeeping that a batched call advances.
 struct EventCursor {
   std::vector<int> cur, zA0, zB0;
   std::vector<long long> n;
-  explicit EventCursor(const glasma_batch* b) {
-    for (const glasma_ctx* c : b->ev) {
+  explicit EventCursor(const Events& ev) {
+    for (const glasma_ctx* c : ev) {
       cur.push_back(c->cur);
       zA0.push_back(c->zA0);
       zB0.push_back(c->zB0);
@@ -313,18 +314,18 @@ struct EventCursor {
     }
   }
   // true if no charge of any event leaves its lattice in the next step
-  bool next_step_fits(const glasma_batch* b) const {
-    for (size_t e = 0; e < b->ev.size(); ++e) {
-      const glasma_ctx* c = b->ev[e];
+  bool next_step_fits(const Events& ev) const {
+    for (size_t e = 0; e < ev.size(); ++e) {
+      const glasma_ctx* c = ev[e];
       if (!hop_at(n[e], c->hop_p, c->hop_q)) continue;
       if (c->WB > 0 && zB0[e] + c->WB - 1 >= c->g.nz - 1) return false;
       if (c->WA > 0 && zA0[e] <= 0) return false;
     }
     return true;
   }
-  void advance(const glasma_batch* b) {
-    for (size_t e = 0; e < b->ev.size(); ++e) {
-      const glasma_ctx* c = b->ev[e];
+  void advance(const Events& ev) {
+    for (size_t e = 0; e < ev.size(); ++e) {
+      const glasma_ctx* c = ev[e];
       if (hop_at(n[e], c->hop_p, c->hop_q)) {
         zB0[e] += 1;
         zA0[e] -= 1;
@@ -333,24 +334,22 @@ struct EventCursor {
       n[e] += 1;
     }
   }
-  void store(glasma_batch* b, int launches) const {
-    for (size_t e = 0; e < b->ev.size(); ++e) {
-      glasma_ctx* c = b->ev[e];
+  void store(const Events& ev) const {
+    for (size_t e = 0; e < ev.size(); ++e) {
+      glasma_ctx* c = ev[e];
       c->cur = cur[e];
       c->zA0 = zA0[e];
       c->zB0 = zB0[e];
       c->n = n[e];
-      c->last_launches = launches;
     }
-    b->last_launches = launches;
   }
 };
 
 // Number of the next n_steps steps that every event can take.
 static int steps_allowed(const glasma_batch* b, int n_steps) {
-  EventCursor cs(b);
+  EventCursor cs(b->ev);
   int k = 0;
-  for (; k < n_steps && cs.next_step_fits(b); ++k) cs.advance(b);
+  for (; k < n_steps && cs.next_step_fits(b->ev); ++k) cs.advance(b->ev);
   return k;
 }
 
@@ -358,19 +357,18 @@ static int steps_allowed(const glasma_batch* b, int n_steps) {
 // geometry class on the private stream, launch the graph on the events'
 // stream, advance the bookkeeping.
 template <int NC, typename R>
-static int graph_run(glasma_batch* b, int steps, int bx) {
-  if (steps == 0) return GLASMA_OK;
-  EventCursor cs(b);
-  const std::vector<std::vector<int>> groups = geometry_groups(b->ev);
+static int graph_run(glasma_batch* b, const Events& ev, int steps, int bx, int* launches) {
+  EventCursor cs(ev);
+  const std::vector<std::vector<int>> groups = geometry_groups(ev);
   int st = cuda_check(cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal), "batch capture begin");
   if (st) return st;
   for (int k = 0; k < steps && !st; ++k) {
     for (size_t q = 0; q < groups.size() && !st; ++q) {
       GroupArgs<R> args;
-      plan_group<R>(b->ev, groups[q], cs.cur, cs.n, cs.zA0, cs.zB0, args);
+      plan_group<R>(ev, groups[q], cs.cur, cs.n, cs.zA0, cs.zB0, args);
       st = launch_group<NC, R>(args, (int)groups[q].size(), bx, b->capture);
     }
-    cs.advance(b);
+    cs.advance(ev);
   }
   cudaGraph_t graph = nullptr;
   const int st_end = cuda_check(cudaStreamEndCapture(b->capture, &graph), "batch capture end");
@@ -384,17 +382,18 @@ static int graph_run(glasma_batch* b, int steps, int bx) {
   if (exec) cudaGraphExecDestroy(exec);  // freed once the launch completes
   cudaGraphDestroy(graph);
   if (st) return st;
-  cs.store(b, steps * (int)groups.size());
+  cs.store(ev);
+  *launches += steps * (int)groups.size();
   return GLASMA_OK;
 }
 
 // Persistent mode: one cooperative launch for all `steps` steps; reads the
 // barrier's error word back (synchronises the stream).
 template <int NC, typename R>
-static int persistent_launch_run(glasma_batch* b, int steps, int bx) {
-  const glasma_params& p = b->ev[0]->p;
+static int persistent_launch_run(glasma_batch* b, const Events& ev, int steps, int bx) {
+  const glasma_params& p = ev[0]->p;
   PersistArgs<R> a;
-  a.n = (int)b->ev.size();
+  a.n = (int)ev.size();
   a.steps = steps;
   a.dt = (R)p.dt;
   a.w[0] = (R)(2.0 / (p.a_t * p.a_t));
@@ -405,8 +404,8 @@ static int persistent_launch_run(glasma_batch* b, int steps, int bx) {
   a.bar = b->bar;
   a.err = (int*)(b->bar + 1);
   uint32_t block0 = 0;
-  for (size_t e = 0; e < b->ev.size(); ++e) {
-    glasma_ctx* c = b->ev[e];
+  for (size_t e = 0; e < ev.size(); ++e) {
+    glasma_ctx* c = ev[e];
     PersistEvent<R>& d = a.ev[e];
     d.U[0] = (typename V2T<R>::T*)c->U[c->cur];
     d.U[1] = (typename V2T<R>::T*)c->U[1 - c->cur];
@@ -435,59 +434,94 @@ static int persistent_launch_run(glasma_batch* b, int steps, int bx) {
   if (herr)
     return set_error(GLASMA_ERR_TIMEOUT,
                      "a grid barrier wait of the persistent step ran out; the events' states are undefined");
-  EventCursor cs(b);
-  for (int k = 0; k < steps; ++k) cs.advance(b);
-  cs.store(b, 1);
+  EventCursor cs(ev);
+  for (int k = 0; k < steps; ++k) cs.advance(ev);
+  cs.store(ev);
   return GLASMA_OK;
 }
 
 template <int NC, typename R>
-static int persistent_run(glasma_batch* b, int steps, int bx) {
-  int launches = 0;
+static int persistent_run(glasma_batch* b, const Events& ev, int steps, int bx, int* launches) {
   for (int done = 0; done < steps; done += kPersistSteps) {
     const int n = steps - done < kPersistSteps ? steps - done : kPersistSteps;
-    const int st = persistent_launch_run<NC, R>(b, n, bx);
+    const int st = persistent_launch_run<NC, R>(b, ev, n, bx);
     if (st) return st;
-    ++launches;
+    *launches += 1;
   }
-  for (glasma_ctx* c : b->ev) c->last_launches = launches;
-  b->last_launches = launches;
   return GLASMA_OK;
 }
 
-// Per-event mode: the single-event step kernel of every event and step
-// (the kernel glasma_step would use for that context), launched step by step
-// on the batch's stream; no batched kernel, for events that fill the GPU on
-// their own.  Their launches queue far ahead of the GPU, so a graph saves
-// nothing here, while capturing and instantiating one per call (steps x
-// events nodes) cost 10 % of the ensemble's step time.
-static int per_event_run(glasma_batch* b, int steps) {
-  if (steps == 0) return GLASMA_OK;
-  const size_t ne = b->ev.size();
-  EventCursor cs(b);
-  int st = GLASMA_OK, launches = 0;
-  for (int k = 0; k < steps && !st; ++k) {
-    for (size_t e = 0; e < ne && !st; ++e) {
-      glasma_ctx* c = b->ev[e];
-      c->cur = cs.cur[e];
-      c->zA0 = cs.zA0[e];
-      c->zB0 = cs.zB0[e];
-      st = launch_step_chosen(c, hop_at(cs.n[e], c->hop_p, c->hop_q), &launches);
+// Every event by the step kernel glasma_step would use for it, launched step
+// by step on the batch's stream: for events that fill the GPU on their own.
+// Those of the two FP64 passes that do not share their launches with others of
+// their geometry.  The launches queue far ahead of the GPU, so a graph saves
+// nothing here, while capturing and instantiating one per call (steps x events
+// nodes) cost 10 % of the ensemble's step time.
+static int own_run(const Events& ev, int steps, int* launches) {
+  std::vector<std::vector<int>> groups;  // events that share their launches
+  for (const std::vector<int>& same : geometry_groups(ev)) {
+    int open = -1;
+    for (int e : same) {
+      const int size = use_parts_kernel(ev[e]) ? parts_group_size(ev[e]) : 1;
+      if (size > 1 && open >= 0 && (int)groups[open].size() < size) {
+        groups[open].push_back(e);
+        continue;
+      }
+      groups.push_back({e});
+      if (size > 1) open = (int)groups.size() - 1;
     }
-    cs.advance(b);
   }
-  if (st) return st;
-  cs.store(b, launches);
-  return GLASMA_OK;
+  EventCursor cs(ev);
+  int st = GLASMA_OK;
+  for (int k = 0; k < steps && !st; ++k) {
+    cs.store(ev);  // a step's launches read the contexts
+    for (size_t q = 0; q < groups.size() && !st; ++q) {
+      glasma_ctx* c[kMaxBatch];
+      bool hop[kMaxBatch];
+      int n = 0;
+      for (int e : groups[q]) {
+        c[n] = ev[e];
+        hop[n++] = hop_at(cs.n[e], ev[e]->hop_p, ev[e]->hop_q);
+      }
+      st = n > 1 ? launch_parts_group(c, n, hop, launches) : launch_step_chosen(c[0], hop[0], launches);
+    }
+    cs.advance(ev);
+  }
+  if (!st) cs.store(ev);
+  return st;
+}
+
+// Whether an event is stepped by its own kernel.  By default every event whose
+// kernel rounds otherwise than the staple form is, so that its result is
+// glasma_step's whatever its companions; that kernel also does less arithmetic,
+// which is worth more than filling the GPU with one launch for a class (ms per
+// step: 24 events, FP64 SU(3) 256 x {32, 48, 64}^2 105 -> 70 and 128 x {16, 24, 33}^2
+// 14.1 -> 9.4; 12 events of 160 x {8, 11}^2 1.36 -> 0.94, SU(2) 0.26 -> 0.19; FP32 SU(2)
+// 256 x {32, 48, 64}^2 0.98 -> 0.78).  With the staple form in both, the graph is
+// faster (FP32 SU(3), the same lattices, 3.26 against 3.47, 0.46 against 0.55,
+// 0.056 against 0.109).  In the graph and persistent modes FP64 events take the
+// staple form; FP32 events keep their own bits there too.
+static bool own_kernel(const glasma_ctx* c, int mode) {
+  if (mode == GLASMA_BATCH_PER_EVENT || use_site_kernel(c)) return true;
+  return mode < 0 && (use_parts_kernel(c) || use_plaq_kernel(c) || use_pair_kernel(c));
 }
 
 template <int NC, typename R>
 static int batch_run(glasma_batch* b, int n_steps, int mode, int bx) {
   const int allowed = steps_allowed(b, n_steps);
-  const int st = mode == GLASMA_BATCH_PERSISTENT ? persistent_run<NC, R>(b, allowed, bx)
-                 : mode == GLASMA_BATCH_PER_EVENT ? per_event_run(b, allowed)
-                                                  : graph_run<NC, R>(b, allowed, bx);
-  if (st) return st;
+  Events own, rest;
+  for (glasma_ctx* c : b->ev) (own_kernel(c, mode) ? own : rest).push_back(c);
+  int st = GLASMA_OK, launches = 0;
+  if (allowed > 0) {
+    // the persistent mode may run out of its wait: before any other event moves
+    if (!rest.empty())
+      st = mode == GLASMA_BATCH_PERSISTENT ? persistent_run<NC, R>(b, rest, allowed, bx, &launches)
+                                           : graph_run<NC, R>(b, rest, allowed, bx, &launches);
+    if (!st && !own.empty()) st = own_run(own, allowed, &launches);
+    if (st) return st;
+    for (glasma_ctx* c : b->ev) c->last_launches = launches;
+    b->last_launches = launches;
+  }
   if (allowed < n_steps)
     return set_error(GLASMA_ERR_PARTICLE_EXIT, "a charge of a batched event would leave its lattice");
   return GLASMA_OK;
@@ -537,23 +571,10 @@ GLASMA_API int glasma_batch_create(glasma_ctx* const* ctxs, int n, glasma_batch*
   return GLASMA_OK;
 }
 
-// Where every event's own step kernel does less arithmetic than the staple form
-// of the graph's kernel, that is worth more than filling the GPU with one launch
-// for a class, whatever the events' sizes (ms per step: 24 events, FP64 SU(3) 256 x
-// {32, 48, 64}^2 105 -> 70 and 128 x {16, 24, 33}^2 14.1 -> 9.4; 12 events of 160 x
-// {8, 11}^2 1.36 -> 0.94, SU(2) 0.26 -> 0.19; FP32 SU(2) 256 x {32, 48, 64}^2 0.98 ->
-// 0.78).  With the staple form in both, the graph is faster (FP32 SU(3), the same
-// lattices, 3.26 against 3.47, 0.46 against 0.55, 0.056 against 0.109).
-static int default_mode(const glasma_batch* b) {
-  for (const glasma_ctx* c : b->ev)
-    if (!use_parts_kernel(c) && !use_site_kernel(c)) return GLASMA_BATCH_GRAPH;
-  return GLASMA_BATCH_PER_EVENT;
-}
-
 GLASMA_API int glasma_batch_step(glasma_batch* b, int n_steps) {
   if (!b || n_steps < 0) return set_error(GLASMA_ERR_INVALID_ARG, "bad batch or n_steps");
   cudaSetDevice(b->device);
-  return batch_dispatch(b, n_steps, b->mode < 0 ? default_mode(b) : b->mode, b->bx);
+  return batch_dispatch(b, n_steps, b->mode, b->bx);
 }
 
 GLASMA_API int glasma_batch_set_shape(glasma_batch* b, int mode, int block_sites) {

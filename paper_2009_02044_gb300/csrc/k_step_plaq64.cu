@@ -120,19 +120,18 @@ struct PlaqCorners<2> {
   }
 };
 
-// NORM: also ||A - B^dag||_F^2 = 2 (N - Re tr of the loop), for T^{mu nu}.
+// Plane pl of site idx of the launch.  NORM: also ||A - B^dag||_F^2 =
+// 2 (N - Re tr of the loop), for T^{mu nu}.
 template <int NC, bool NORM>
-__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs a) {
-  follow_last();
+__device__ __forceinline__ void parts_of(const PartsArgs& a, uint32_t idx, int pl) {
   typedef Group<NC, double> G;
   typedef LinkIO<NC, double> IO;
   typedef typename G::M M;
   constexpr int NA = G::NA;
-  const uint32_t idx = blockIdx.x * kPartsThreads + threadIdx.x;
   if (idx >= a.sites) return;
   const Geom& g = a.g;
   const uint32_t nxy = (uint32_t)g.nxy, dz = idx / nxy, t = idx - dz * nxy;
-  const int z = a.zfirst + (int)dz, pl = (int)blockIdx.y;
+  const int z = a.zfirst + (int)dz;
   const bool below = z < a.z0;  // only what reaches the slice above is wanted
   if (pl == 0 ? below : z >= g.nz - 1) return;
   const int da = pl == 2 ? 1 : 0, db = pl == 0 ? 1 : 2;
@@ -156,6 +155,12 @@ __global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs 
   for (int c = 0; c < NA; ++c) out[((kP0 + pl) * NA + c) * S] = ab[c];
 }
 
+template <int NC, bool NORM>
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts(PartsArgs a) {
+  follow_last();
+  parts_of<NC, NORM>(a, blockIdx.x * kPartsThreads + threadIdx.x, (int)blockIdx.y);
+}
+
 struct PartLinksArgs {
   StepArgs<double> s;
   const double* part;
@@ -164,21 +169,73 @@ struct PartLinksArgs {
   uint32_t sites;
 };
 
+// Link i of site idx of the launch.
 template <int NC>
-__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links(PartLinksArgs pa) {
-  follow_last();
+__device__ __forceinline__ void links_of_parts(const PartLinksArgs& pa, uint32_t idx, int i) {
   constexpr int NA = Group<NC, double>::NA;
-  const uint32_t idx = blockIdx.x * kPartsThreads + threadIdx.x;
   if (idx >= pa.sites) return;
   const StepArgs<double>& a = pa.s;
   const Geom& g = a.g;
   const uint32_t nxy = (uint32_t)g.nxy, dz = idx / nxy, t = idx - dz * nxy;
-  const int z = pa.z0 + (int)dz, i = (int)blockIdx.y;
+  const int z = pa.z0 + (int)dz;
   if (i == 2 && z == g.nz - 1) return;  // no z link on the last slice
   const SiteNbr n = site_nbr_tz(g, t, z);
   double F[NA];
   part_force<NA>(pa.part, g, pa.ring, n, t, z, i, a.w, F);
   update_link<NC, double>(a, i, t, z, n.s, F);
+}
+
+template <int NC>
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links(PartLinksArgs pa) {
+  follow_last();
+  links_of_parts<NC>(pa, blockIdx.x * kPartsThreads + threadIdx.x, (int)blockIdx.y);
+}
+
+// The two passes of several events of one geometry, whole lattices in their
+// scratch, blockIdx.z the event: events that do not fill the GPU cost a launch
+// each otherwise (us per step, 64 events, SU(2) 40 x 4^2 618 -> 44, SU(3) 3250 -> 310;
+// the graph's staple form 124 and 786).
+struct PartsEvent {
+  void* U[2];  // this step's links and the next step's
+  double *part, *E, *QA, *QB;
+  int zA0, WA, zB0, WB, hop;
+};
+struct PartsGroup {
+  PartLinksArgs l;
+  PartsEvent ev[kMaxBatch];
+};
+
+template <int NC>
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_parts_group(const __grid_constant__ PartsGroup b) {
+  follow_last();
+  const PartsEvent& e = b.ev[blockIdx.z];
+  PartsArgs a;
+  a.U = (const double2*)e.U[0];
+  a.part = e.part;
+  a.g = b.l.s.g;
+  a.zfirst = a.z0 = 0;
+  a.ring = b.l.ring;
+  a.sites = b.l.sites;
+  parts_of<NC, false>(a, blockIdx.x * kPartsThreads + threadIdx.x, (int)blockIdx.y);
+}
+
+template <int NC>
+__global__ void __launch_bounds__(kPartsThreads, 4) k_step_plaq_links_group(const __grid_constant__ PartsGroup b) {
+  follow_last();
+  const PartsEvent& e = b.ev[blockIdx.z];
+  PartLinksArgs l = b.l;
+  l.part = e.part;
+  l.s.U = (const double2*)e.U[0];
+  l.s.Un = (double2*)e.U[1];
+  l.s.E = e.E;
+  l.s.QA = e.QA;
+  l.s.QB = e.QB;
+  l.s.hop = e.hop;
+  l.s.zA0 = e.zA0;
+  l.s.WA = e.WA;
+  l.s.zB0 = e.zB0;
+  l.s.WB = e.WB;
+  links_of_parts<NC>(l, blockIdx.x * kPartsThreads + threadIdx.x, (int)blockIdx.y);
 }
 
 // The scratch of an FP64 leapfrog context.  Where the allocator refuses it, half
@@ -222,9 +279,7 @@ int launch_parts_norms(glasma_ctx* c, int z0, int z1) {
   return c->p.nc == 2 ? launch_parts_pass<2, true>(c, z0, z1, false) : launch_parts_pass<3, true>(c, z0, z1, false);
 }
 
-template <int NC>
-static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
-  PartLinksArgs l;
+static void links_args(const glasma_ctx* c, bool hop, PartLinksArgs& l) {
   StepArgs<double>& a = l.s;
   a.U = (const double2*)c->U[c->cur];
   a.Un = (double2*)c->U[1 - c->cur];
@@ -245,6 +300,12 @@ static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
   a.zlo = c->lo;
   l.part = c->part;
   l.ring = c->ring;
+}
+
+template <int NC>
+static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
+  PartLinksArgs l;
+  links_args(c, hop, l);
   if (zlen <= 0 || zlen > l.ring - 1) zlen = l.ring - 1;
   for (int z0 = c->lo; z0 < c->hi; z0 += zlen) {
     const int z1 = z0 + zlen < c->hi ? z0 + zlen : c->hi;
@@ -258,6 +319,51 @@ static int launch_parts_t(glasma_ctx* c, bool hop, int zlen, int* launches) {
     *launches += 2;
   }
   return GLASMA_OK;
+}
+
+// Events of the context's geometry that share its launches: as many as keep
+// their scratches in the L2 cache together, 1 where one event's ring is shorter
+// than its lattice.
+int parts_group_size(const glasma_ctx* c) {
+  if (c->slab || c->ring != c->g.nz + 1 || c->step_zlen != 0) return 1;
+  const size_t n = kPartsBytes / (sizeof(double) * (size_t)part_doubles(c->na) * (size_t)c->g.nxy * (size_t)c->ring);
+  return n < 1 ? 1 : n > (size_t)kMaxBatch ? kMaxBatch : (int)n;
+}
+
+template <int NC>
+static int launch_group_t(glasma_ctx* const* c, int n, const bool* hop, int* launches) {
+  PartsGroup b;
+  links_args(c[0], false, b.l);
+  b.l.z0 = 0;
+  b.l.sites = (uint32_t)c[0]->g.V;
+  for (int k = 0; k < n; ++k) {
+    PartsEvent& e = b.ev[k];
+    e.U[0] = c[k]->U[c[k]->cur];
+    e.U[1] = c[k]->U[1 - c[k]->cur];
+    e.part = c[k]->part;
+    e.E = (double*)c[k]->E;
+    e.QA = (double*)c[k]->QA;
+    e.QB = (double*)c[k]->QB;
+    e.zA0 = c[k]->zA0;
+    e.WA = c[k]->WA;
+    e.zB0 = c[k]->zB0;
+    e.WB = c[k]->WB;
+    e.hop = hop[k] ? 1 : 0;
+  }
+  const dim3 grid((b.l.sites + kPartsThreads - 1) / kPartsThreads, 3, (unsigned)n);
+  int st = launch_following("k_step_plaq_parts_group launch", k_step_plaq_parts_group<NC>, grid, kPartsThreads, 0,
+                            c[0]->stream, b);
+  if (!st)
+    st = launch_following("k_step_plaq_links_group launch", k_step_plaq_links_group<NC>, grid, kPartsThreads, 0,
+                          c[0]->stream, b);
+  *launches += 2;
+  return st;
+}
+
+// One step of n events of equal geometry and stream, n at most parts_group_size
+// of each
+int launch_parts_group(glasma_ctx* const* c, int n, const bool* hop, int* launches) {
+  return c[0]->p.nc == 2 ? launch_group_t<2>(c, n, hop, launches) : launch_group_t<3>(c, n, hop, launches);
 }
 
 // zlen: slices per chunk (0: as many as the scratch holds)

@@ -200,3 +200,75 @@ def test_persistent_call_longer_than_one_launch(G):
         G.glasma_step(h, 150)
     for h1, h2 in zip(single, batched):
         _same(G, h1, h2)
+
+
+def _batch_cfgs(nc, precision, sizes):
+    return [dict(gi.small_config(nc, nz=nz, nx=nx, ny=ny, sigma_l=1.0, seed=60 + k),
+                 precision=precision) for k, (nz, nx, ny) in enumerate(sizes)]
+
+
+@pytest.mark.parametrize("mode", [None, "graph", "persistent", "per_event", "tuned"])
+def test_fp32_events_keep_their_bits_in_any_company_and_mode(G, mode):
+    """FP32 SU(2) events below and from 3 * 2^16 sites on, whose own step kernels
+    round differently, in one batch: each event is what glasma_step makes of
+    it, whatever its companions, the mode or the tuner's choice."""
+    cfgs = _batch_cfgs(2, "fp32", [(48, 64, 64), (40, 16, 16), (51, 64, 64)])
+    single = [G.glasma_init_mv(c, None) for c in cfgs]
+    batched = [G.glasma_init_mv(c, None) for c in cfgs]
+    b = G.glasma_batch_create(batched)
+    if mode == "tuned":
+        G.glasma_batch_tune(b, 2)
+    elif mode:
+        G.glasma_batch_set_shape(b, mode, 64)
+    G.glasma_batch_step(b, 3)
+    G.glasma_batch_step(b, 6)
+    for h in single:
+        G.glasma_step(h, 9)
+    for h1, h2 in zip(single, batched):
+        _same(G, h1, h2)
+    b.close()
+
+
+@pytest.mark.parametrize("nc", [2, 3])
+def test_fp64_events_keep_their_bits_in_any_company(G, nc):
+    """By default an FP64 event is stepped in its two passes beside one that
+    was set to the staple kernel, and that one by the staple kernel."""
+    cfgs = _batch_cfgs(nc, "fp64", [(48, 12, 10), (40, 16, 16), (48, 12, 10)])
+    single = [G.glasma_init_mv(c, None) for c in cfgs]
+    batched = [G.glasma_init_mv(c, None) for c in cfgs]
+    for h in (single[0], batched[0]):
+        G.glasma_set_step_kernel(h, "staple")
+    b = G.glasma_batch_create(batched)
+    G.glasma_batch_step(b, 9)
+    for h in single:
+        G.glasma_step(h, 9)
+    for h1, h2 in zip(single, batched):
+        _same(G, h1, h2)
+    b.close()
+
+
+@pytest.mark.parametrize("nc", [2, 3])
+def test_small_fp64_events_share_launches(G, nc):
+    """24 events of two geometries, at different steps of the hop schedule,
+    take two launches per geometry and step and are bitwise the single
+    steps; an event with chunks of its own keeps its own launches."""
+    sizes = [(48, 5, 4), (40, 8, 7)]
+    cfgs = _batch_cfgs(nc, "fp64", [sizes[k % 2] for k in range(24)])
+    single = [G.glasma_init_mv(c, None) for c in cfgs]
+    batched = [G.glasma_init_mv(c, None) for c in cfgs]
+    for k, (h1, h2) in enumerate(zip(single, batched)):
+        G.glasma_step(h1, k % 3)
+        G.glasma_step(h2, k % 3)
+    b = G.glasma_batch_create(batched)
+    G.glasma_batch_step(b, 1)
+    assert G.glasma_get_info(batched[0]).kernel_launches == 4
+    G.glasma_set_step_kernel(batched[5], "auto", 9)   # 40 slices: 5 pairs of passes
+    G.glasma_batch_step(b, 1)
+    assert G.glasma_get_info(batched[0]).kernel_launches == 14
+    G.glasma_set_step_kernel(batched[5], "auto", 0)
+    G.glasma_batch_step(b, 7)
+    for h in single:
+        G.glasma_step(h, 9)
+    for h1, h2 in zip(single, batched):
+        _same(G, h1, h2)
+    b.close()
