@@ -301,7 +301,7 @@ constexpr int kDivSplit = 8;
 
 template <int NC, typename R>
 __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U, const R* E, Geom g, double ia2t,
-                                                    double ia2z, double* rho3, double* slice_max) {
+                                                    double* rho3, double* slice_max) {
   typedef Group<NC, double> G;
   constexpr int NA = G::NA;
   __shared__ double sh[256];
@@ -312,26 +312,25 @@ __global__ void __launch_bounds__(256) k_divergence(const typename V2T<R>::T* U,
     const SiteNbr n = site_nbr_tz(g, t, iz);
     double dv[NA];
     for (int c = 0; c < NA; ++c) dv[c] = 0.0;
-    for (int i = 0; i < 3; ++i) {
-      const double w = i == 2 ? ia2z : ia2t;
+    for (int i = 0; i < 2; ++i) {  // E_z = 0
       R e[NA], em[NA];
       bool here = false, below = false;
       for (int c = 0; c < NA; ++c) {
         e[c] = E[(int64_t)(i * NA + c) * g.V + s];
-        em[c] = i == 2 && iz == 0 ? R(0) : E[(int64_t)(i * NA + c) * g.V + n.m[i]];
+        em[c] = E[(int64_t)(i * NA + c) * g.V + n.m[i]];
         here = here || e[c] != R(0);
         below = below || em[c] != R(0);
       }
       // E vanishes off the nuclei: no FP64 work there
       if (here)
-        for (int c = 0; c < NA; ++c) dv[c] += w * widen<double>(e[c]);
+        for (int c = 0; c < NA; ++c) dv[c] += ia2t * widen<double>(e[c]);
       if (!below) continue;
       double q[NA];
       for (int c = 0; c < NA; ++c) q[c] = widen<double>(em[c]);
       typename G::M um = LinkIO<NC, R>::template load<double>(U, i, g.V, n.m[i]);
       // the links of an FP32 state are unitary to their rounding only
       G::template adj_dag<sizeof(R) == 4>(um, q);
-      for (int c = 0; c < NA; ++c) dv[c] -= w * q[c];
+      for (int c = 0; c < NA; ++c) dv[c] -= ia2t * q[c];
     }
     for (int c = 0; c < NA; ++c) {
       rho3[(int64_t)c * g.V + s] = dv[c];
@@ -413,7 +412,7 @@ static int init_t(glasma_ctx* c, const double* rho_host) {
       (typename V2T<R>::T*)c->Uprev, (R*)c->E, c->g, p.dt, c->dflag, S, c->slab ? 0 : 1);
   const int64_t per_slice = (nxy + 255) / 256;
   k_divergence<NC, R><<<dim3(p.nz, (unsigned)(per_slice < kDivSplit ? per_slice : kDivSplit)), 256, 0, c->stream>>>(
-      (const typename V2T<R>::T*)c->U[0], (const R*)c->E, c->g, 1.0 / (p.a_t * p.a_t), 1.0 / (p.a_z * p.a_z), rho3,
+      (const typename V2T<R>::T*)c->U[0], (const R*)c->E, c->g, 1.0 / (p.a_t * p.a_t), rho3,
       smax);
   st = cuda_check(cudaGetLastError(), "init kernels");
   if (st) return st;
