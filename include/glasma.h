@@ -267,7 +267,12 @@ GLASMA_API int glasma_get_fields(glasma_ctx* c, double* U, double* E, double* QA
  * the last slice must be the identity and E_z there zero.  The charge
  * windows are rebuilt from the nonzero slices of QA and QB.  U_prev (the
  * links at t_{n-1}, used by the implicit scheme) may be NULL, in which case
- * exp(-i dt E) U is used.  Errors: INVALID_ARG, OOM, CUDA.
+ * exp(-i dt E) U is used.
+ * Links are meant to be in SU(nc) (SU(2) keeps the first row).  Those that are
+ * not, by more than 1e-10 (FP64) or 4e-6 (FP32) in orthonormality or determinant,
+ * are multiplied as they are, by the staple kernel whatever kernel was chosen:
+ * FP32 state until a step has re-unitarised them, FP64 state for good.  The same
+ * holds for glasma_set_state.  Errors: INVALID_ARG, OOM, CUDA.
  */
 GLASMA_API int glasma_set_fields(glasma_ctx* c, const double* U, const double* E, const double* QA,
                       const double* QB, const double* U_prev, long long step_n);

@@ -145,7 +145,9 @@ bool use_plaq_kernel(const glasma_ctx* c) {
 }
 
 // both plaquette choices name this form in FP64
-bool use_parts_kernel(const glasma_ctx* c) { return c->part && c->step_kernel != GLASMA_KERNEL_STAPLE; }
+bool use_parts_kernel(const glasma_ctx* c) {
+  return c->part && c->step_kernel != GLASMA_KERNEL_STAPLE && !c->links_off;
+}
 
 bool use_pair_kernel(const glasma_ctx* c) {
   if (c->rs != 4 || c->slab) return false;  // the pairs span the whole z range
@@ -170,6 +172,10 @@ bool use_staged_kernel(const glasma_ctx* c) {
 }
 
 int launch_step_chosen(glasma_ctx* c, bool hop, int* launches) {
+  if (c->links_off) {  // the staple form multiplies links as they are
+    *launches += 1;
+    return launch_step_leapfrog(c, hop);
+  }
   if (use_parts_kernel(c)) return launch_step_parts(c, hop, c->step_zlen, launches);
   *launches += 1;
   if (use_plaq_kernel(c)) return launch_step_plaq(c, hop, c->step_zlen);
@@ -364,6 +370,7 @@ int glasma_step(glasma_ctx* c, int n_steps) {
       c->zA0 -= 1;
     }
     c->n += 1;
+    step_taken(c);
     if (st) {
       c->last_launches = launches;
       return st;
@@ -427,6 +434,7 @@ int glasma_implicit_end(glasma_ctx* c) {
     c->zA0 -= 1;
   }
   c->n += 1;
+  step_taken(c);
   c->last_iters = c->impl_k;
   c->last_launches = c->impl_k + 1;
   c->impl_active = false;
@@ -670,6 +678,18 @@ static void support(const glasma_ctx* c, const double* Q, int* lo, int* W) {
   }
 }
 
+// After the links (and those of t_{n-1}, where the context holds valid ones) were
+// replaced: are they on the group?
+static int check_links(glasma_ctx* c) {
+  bool now = false, prev = false;
+  int st = links_off_group(c, c->U[c->cur], &now);
+  if (!st && c->Uprev && c->uprev_valid) st = links_off_group(c, c->Uprev, &prev);
+  if (st) return st;
+  // FP32 steps put the new links on the group; U(t_n) is used as U(t_{n-1}) once more
+  c->links_off = !now && !prev ? 0 : c->rs == 8 ? -1 : now && c->Uprev ? 2 : 1;
+  return GLASMA_OK;
+}
+
 int glasma_set_fields(glasma_ctx* c, const double* U, const double* E, const double* QA, const double* QB,
                       const double* U_prev, long long step_n) {
   if (!c || !U || !E || step_n < 0) return set_error(GLASMA_ERR_INVALID_ARG, "bad context, U, E or step_n");
@@ -745,7 +765,7 @@ int glasma_set_fields(glasma_ctx* c, const double* U, const double* E, const dou
     }
   }
   c->n = step_n;
-  return GLASMA_OK;
+  return check_links(c);
 }
 
 // ---------------------------------------------------------------------------
@@ -897,7 +917,7 @@ int glasma_set_state(glasma_ctx* c, const void* host_buf, size_t bytes) {
   c->zA0 = h.zA0;
   c->zB0 = h.zB0;
   c->n = h.n;
-  return cuda_check(cudaStreamSynchronize(c->stream), "state sync");
+  return check_links(c);  // synchronises
 }
 
 int glasma_set_step_kernel(glasma_ctx* c, int kernel, int zlen) {

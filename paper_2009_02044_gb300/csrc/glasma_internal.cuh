@@ -24,6 +24,10 @@ struct glasma_ctx {
   int cur = 0;                // U[cur] holds U(t_n)
   void* Uprev = nullptr;      // U(t_{n-1}), implicit scheme only
   void* Uit = nullptr;        // implicit scheme: second iterate buffer of U(t_{n+1})
+  // links that the caller set off the group (check_links): the kernels that take
+  // them for members of SU(N) are left to others for this many steps (FP32, whose
+  // steps put them back on it) or for good (-1)
+  int links_off = 0;
   bool uprev_valid = false;   // Uprev holds U(t_{n-1})
   void* E = nullptr;          // E(t_{n-1/2})
   void* Ework = nullptr;      // implicit scheme: E(t_{n-1/2}) + current, fixed during iteration
@@ -92,6 +96,10 @@ GL_HD bool hop_at(long long n, long long p, long long q) {
   return hop_count(n + 1, p, q) > hop_count(n, p, q);
 }
 
+inline void step_taken(glasma_ctx* c) {
+  if (c->links_off > 0) --c->links_off;
+}
+
 // Launch a kernel that begins with follow(): it may be set up, and its first
 // blocks placed, while the kernel before it in the stream runs out.  Small
 // lattices spend their time between launches (us per step: SU(2) FP32 100 x 9 x 7
@@ -126,6 +134,9 @@ __device__ __forceinline__ void follow_last() { asm volatile("griddepcontrol.wai
 #endif
 
 // kernel launchers
+// whether a link of U (in the context's layout) is off the group by more than
+// an evolution's rounding, or not finite (synchronises)
+int links_off_group(glasma_ctx* c, const void* U, bool* off);
 int launch_step_leapfrog(glasma_ctx* c, bool hop);
 // plaquette-centric leapfrog step (k_step_plaq.cu): zlen z slices per block
 int launch_step_plaq(glasma_ctx* c, bool hop, int zlen);

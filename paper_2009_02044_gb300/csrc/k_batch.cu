@@ -484,6 +484,7 @@ static int own_run(const Events& ev, int steps, int* launches) {
         hop[n++] = hop_at(cs.n[e], ev[e]->hop_p, ev[e]->hop_q);
       }
       st = n > 1 ? launch_parts_group(c, n, hop, launches) : launch_step_chosen(c[0], hop[0], launches);
+      for (int e = 0; e < n && !st; ++e) step_taken(c[e]);
     }
     cs.advance(ev);
   }
@@ -502,7 +503,7 @@ static int own_run(const Events& ev, int steps, int* launches) {
 // 0.056 against 0.109).  In the graph and persistent modes FP64 events take the
 // staple form; FP32 events keep their own bits there too.
 static bool own_kernel(const glasma_ctx* c, int mode) {
-  if (mode == GLASMA_BATCH_PER_EVENT || use_site_kernel(c)) return true;
+  if (mode == GLASMA_BATCH_PER_EVENT || use_site_kernel(c) || c->links_off) return true;
   return mode < 0 && (use_parts_kernel(c) || use_plaq_kernel(c) || use_pair_kernel(c));
 }
 
@@ -605,7 +606,7 @@ GLASMA_API int glasma_batch_tune(glasma_batch* b, int steps, int* block_sites, i
   struct Snap {
     void* buf[4] = {nullptr, nullptr, nullptr, nullptr};
     size_t bytes[4] = {0, 0, 0, 0};
-    int cur = 0, zA0 = 0, zB0 = 0;
+    int cur = 0, zA0 = 0, zB0 = 0, links_off = 0;
     long long n = 0;
   };
   std::vector<Snap> snap(ne);
@@ -624,6 +625,7 @@ GLASMA_API int glasma_batch_tune(glasma_batch* b, int steps, int* block_sites, i
     s.zA0 = c->zA0;
     s.zB0 = c->zB0;
     s.n = c->n;
+    s.links_off = c->links_off;
     for (int k = 0; k < 4 && !st; ++k) {
       if (!s.bytes[k]) continue;
       s.buf[k] = ctx_alloc(c, s.bytes[k]);
@@ -640,6 +642,7 @@ GLASMA_API int glasma_batch_tune(glasma_batch* b, int steps, int* block_sites, i
       c->zA0 = s.zA0;
       c->zB0 = s.zB0;
       c->n = s.n;
+      c->links_off = s.links_off;
       for (int k = 0; k < 4 && !r; ++k)
         if (s.bytes[k])
           r = cuda_check(cudaMemcpyAsync(live(c, k), s.buf[k], s.bytes[k], cudaMemcpyDeviceToDevice, b->stream), "restore");

@@ -109,7 +109,7 @@ __device__ __forceinline__ const typename V2T<R>::T* slot_buf(const ImplArgs<R>&
 // Time-averaged force on link i at x from the time slots m_begin..m_end-1
 // (0: the iterate of t_{n+1}, 1: t_n, 2: t_{n-1}); the force is linear in
 // the slot terms, so the fixed slots 1 and 2 are summed once per step.
-template <int NC, typename R>
+template <int NC, typename R, bool ANY>
 __device__ void force_implicit(const ImplArgs<R>& a, const SiteNbr& n, int i, R* F, int m_begin, int m_end) {
   typedef LinkAlg<NC, R> G;
   typedef typename G::M M;
@@ -131,13 +131,13 @@ __device__ void force_implicit(const ImplArgs<R>& a, const SiteNbr& n, int i, R*
       const typename V2T<R>::T* Bj = slot_buf(a, m, zplane, j);
       typename G::Sum S = G::zero_sum();
       if (fwd) {
-        G::sum_add(S, R(1), G::staple_fwd(LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi),
+        G::sum_add(S, R(1), G::template staple_fwd<ANY>(LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi),
                                           LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, pj),
                                           LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, n.s)));
       }
       if (bwd) {
         // x + e_i - e_j (the wraps of x and y are independent)
-        G::sum_add(S, R(1), G::staple_bwd(LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, mj),
+        G::sum_add(S, R(1), G::template staple_bwd<ANY>(LinkIO<NC, R>::template load<R>(Bi, i, a.g.V, mj),
                                           LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, pi + mj - n.s),
                                           LinkIO<NC, R>::template load<R>(Bj, j, a.g.V, mj)));
       }
@@ -182,7 +182,7 @@ template <> struct ImplOcc<double> { static constexpr int blocks = 1; };
 // Hop (charges committed, current into Ework), the first iterate and the
 // force of the two fixed time slots.  The first iterate is written before
 // the staples, so U_n(x) and E(t_{n-1/2}) are not live across them.
-template <int NC, typename R>
+template <int NC, typename R, bool ANY = false>
 __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t t, int iz) {
   typedef LinkAlg<NC, R> G;
   typedef typename G::M M;
@@ -207,7 +207,7 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
         for (int c = 0; c < NA; ++c) q[c] = a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t];
 #pragma unroll
         for (int c = 0; c < NA; ++c) dj[c] -= a.az2 * q[c];
-        G::adj_dag(Ui, q);
+        G::template adj_dag<ANY>(Ui, q);
 #pragma unroll
         for (int c = 0; c < NA; ++c) a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t] = q[c];
       }
@@ -216,7 +216,7 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
         R q[NA];
 #pragma unroll
         for (int c = 0; c < NA; ++c) q[c] = a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t];
-        G::adj(Ui, q);
+        G::template adj<ANY>(Ui, q);
 #pragma unroll
         for (int c = 0; c < NA; ++c) {
           dj[c] += a.az2 * q[c];
@@ -230,7 +230,7 @@ __device__ __forceinline__ void prep_link(const ImplArgs<R>& a, int i, uint32_t 
     LinkIO<NC, R>::template store<R>(a.Xn, i, a.g.V, s, G::evolve(e, a.dt, Ui));
   }
   R F[NA];
-  force_implicit<NC, R>(a, site_nbr_tz(a.g, t, iz), i, F, 1, 3);
+  force_implicit<NC, R, ANY>(a, site_nbr_tz(a.g, t, iz), i, F, 1, 3);
 #pragma unroll
   for (int c = 0; c < NA; ++c) a.Ework[(int64_t)(i * NA + c) * a.g.V + s] = ew[c] + a.dt * F[c];
 }
@@ -248,13 +248,14 @@ constexpr int kImplZ = 16;
 
 // SLAB: the owned slices start at zlo (a whole lattice's at 0, fixed at
 // compile time: the offset costs the 80-register sweep 12 B of spills).
-template <int NC, typename R, bool SLAB>
+// ANY: for links off the group (whole lattices).
+template <int NC, typename R, bool SLAB, bool ANY = false>
 __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_prep(ImplArgs<R> a) {
   follow();
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   const int z0 = (SLAB ? a.zlo : 0) + (int)blockIdx.y * a.zlen;
 #pragma unroll 1
-  for (int k = 0; k < a.zlen && z0 + k < a.zhi; ++k) prep_link<NC, R>(a, (int)threadIdx.y, t, z0 + k);
+  for (int k = 0; k < a.zlen && z0 + k < a.zhi; ++k) prep_link<NC, R, ANY>(a, (int)threadIdx.y, t, z0 + k);
 }
 
 // The z links of a slab's lower halo slice (zlo - 1), as its owner prepares
@@ -267,7 +268,7 @@ __global__ void __launch_bounds__(64) k_implicit_prep_halo(ImplArgs<R> a) {
 // Link i at (t, iz) in one sweep: G = Ework + dt F_0(X), E <- (1 - omega) E
 // + omega G (omega = 1: E = G exactly), Xn = exp(i dt E) U_n; the largest
 // change and the largest E component go to dmax, emax.
-template <int NC, typename R>
+template <int NC, typename R, bool ANY = false>
 __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t t, int iz, R& dmax, R& emax) {
   typedef LinkAlg<NC, R> G;
   typedef typename G::M M;
@@ -275,7 +276,7 @@ __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t
   const SiteNbr n = site_nbr_tz(a.g, t, iz);
   const int64_t s = n.s;
   R F[NA];
-  force_implicit<NC, R>(a, n, i, F, 0, 1);
+  force_implicit<NC, R, ANY>(a, n, i, F, 0, 1);
   R e[NA];
 #pragma unroll
   for (int c = 0; c < NA; ++c) {
@@ -294,7 +295,7 @@ __device__ __forceinline__ void sweep_link(const ImplArgs<R>& a, int i, uint32_t
 
 // One fixed-point sweep: E = Ework + dt F_0(X), Xn = exp(i dt E) U_n, where
 // Ework already holds E(t_{n-1/2}) + dt J + dt (F_1(U_n) + F_2(U_{n-1})).
-template <int NC, typename R, bool SLAB>
+template <int NC, typename R, bool SLAB, bool ANY = false>
 __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_iter(ImplArgs<R> a) {
   follow();
   typedef LinkAlg<NC, R> G;
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(192, ImplOcc<R>::blocks) k_implicit_iter(ImplA
   for (int kz = 0; kz < a.zlen && z0 + kz < a.zhi; ++kz) {
     const int iz = z0 + kz;
     if (t >= (uint32_t)a.g.nxy || (i == 2 && iz == a.g.nz - 1)) continue;
-    sweep_link<NC, R>(a, i, t, iz, dmax, emax);
+    sweep_link<NC, R, ANY>(a, i, t, iz, dmax, emax);
   }
   // block max: warp shuffles, then one value per warp
 #pragma unroll
@@ -434,7 +435,9 @@ static int implicit_prepare(glasma_ctx* c, bool hop) {
   st = cuda_check(cudaMemsetAsync(c->conv, 0, sizeof(double) * 2 * (a.maxit + 1), c->stream), "conv clear");
   if (st) return st;
   a.Xn = (V2*)c->U[1 - c->cur];
-  st = launch_following("k_implicit_prep launch", c->lo > 0 ? k_implicit_prep<NC, R, true> : k_implicit_prep<NC, R, false>,
+  st = launch_following("k_implicit_prep launch", c->lo > 0       ? k_implicit_prep<NC, R, true>
+                        : c->links_off ? k_implicit_prep<NC, R, false, true>
+                                       : k_implicit_prep<NC, R, false>,
                         impl_grid(c), bs, 0, c->stream, a);
   if (st || c->lo == 0) return st;
   k_implicit_prep_halo<NC, R><<<(unsigned)((c->g.nxy + 63) / 64), 64, 0, c->stream>>>(a);
@@ -455,7 +458,10 @@ static int implicit_launch_sweep(glasma_ctx* c, bool hop, int k, bool check) {
   a.X = (const V2*)(k % 2 == 0 ? xa : xb);
   a.Xn = (V2*)(k % 2 == 0 ? xb : xa);
   int st = launch_following("k_implicit_iter launch",
-                            c->lo > 0 ? k_implicit_iter<NC, R, true> : k_implicit_iter<NC, R, false>, impl_grid(c),
+                            c->lo > 0      ? k_implicit_iter<NC, R, true>
+                            : c->links_off ? k_implicit_iter<NC, R, false, true>
+                                           : k_implicit_iter<NC, R, false>,
+                            impl_grid(c),
                             dim3(64, 3), 0, c->stream, a);
   if (st || c->lo == 0) return st;
   k_implicit_iter_halo<NC, R><<<(unsigned)((c->g.nxy + 63) / 64), 64, 0, c->stream>>>(a);

@@ -167,6 +167,65 @@ int launch_gauss(glasma_ctx* c, double* out3) {
 }
 
 // ---------------------------------------------------------------------------
+// Are the links on the group?  An FP64 evolution leaves it by some 1e-16 per
+// step, an FP32 link by the rounding of its entries (1e-7).
+// ---------------------------------------------------------------------------
+template <int NC, typename R>
+__global__ void __launch_bounds__(kRedThreads) k_links_off(const typename V2T<R>::T* U, int64_t V, double tol, int* off) {
+  typedef Group<NC, double> G;
+  double dev = 0.0;
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < V; s += (int64_t)gridDim.x * blockDim.x) {
+    const typename G::M u = LinkIO<NC, R>::template load<double>(U, (int)blockIdx.y, V, s);
+    double d;
+    if constexpr (NC == 2) {
+      d = fabs(fma(u.a.re, u.a.re, fma(u.a.im, u.a.im, fma(u.b.re, u.b.re, fma(u.b.im, u.b.im, -1.0)))));
+    } else {
+      // rows 0 and 1 orthonormal, row 2 their cross product's conjugate
+      cplx<double> p = mulc(u.m[0], u.m[3]);
+      p = fma_cj(u.m[1], u.m[4], p);
+      p = fma_cj(u.m[2], u.m[5], p);
+      d = fabs(p.re) + fabs(p.im);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        double n = -1.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n = fma(u.m[3 * r + k].re, u.m[3 * r + k].re, fma(u.m[3 * r + k].im, u.m[3 * r + k].im, n));
+        d += fabs(n);
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int a = (k + 1) % 3, b = (k + 2) % 3;
+        const cplx<double> x = u.m[a] * u.m[3 + b] - u.m[b] * u.m[3 + a] - cj(u.m[6 + k]);
+        d += fabs(x.re) + fabs(x.im);
+      }
+    }
+    if (!(d <= dev)) dev = d;  // a NaN stays
+    if (!(dev <= tol)) break;
+  }
+  if (!(dev <= tol)) atomicOr(off, 1);
+}
+
+template <int NC, typename R>
+static int links_off_t(glasma_ctx* c, const void* U, bool* off) {
+  int* flag = c->dflag + 2;
+  int st = cuda_check(cudaMemsetAsync(flag, 0, sizeof(int), c->stream), "link check");
+  if (st) return st;
+  k_links_off<NC, R><<<dim3(4 * c->sms, 3), kRedThreads, 0, c->stream>>>((const typename V2T<R>::T*)U, c->g.V,
+                                                                        sizeof(R) == 8 ? 1e-10 : 4e-6, flag);
+  st = cuda_check(cudaGetLastError(), "k_links_off launch");
+  int h = 0;
+  if (!st) st = cuda_check(cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "link check");
+  if (!st) st = cuda_check(cudaStreamSynchronize(c->stream), "link check");
+  *off = h != 0;
+  return st;
+}
+
+int links_off_group(glasma_ctx* c, const void* U, bool* off) {
+  if (c->p.nc == 2) return c->rs == 8 ? links_off_t<2, double>(c, U, off) : links_off_t<2, float>(c, U, off);
+  return c->rs == 8 ? links_off_t<3, double>(c, U, off) : links_off_t<3, float>(c, U, off);
+}
+
+// ---------------------------------------------------------------------------
 // T^{mu nu} per z slice
 // ---------------------------------------------------------------------------
 template <typename R>
@@ -283,7 +342,8 @@ template <> struct TmnOcc<3, float> { static constexpr int blocks = 2; };
 // per site where forward staples by themselves made 35.  Per sample: SU(3)
 // 512 x 64^2 FP32 0.797 -> 0.449 ms, SU(2) 1024 x 128^2 FP32 1.78 -> 0.936 ms, SU(3)
 // 512 x 64^2 FP64 15.2 -> 10.8 ms.
-template <int NC, typename R>
+// ANY: for links off the group.
+template <int NC, typename R, bool ANY>
 __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(TmnArgs<R> a) {
   follow();
   typedef LinkAlg<NC, R> G;
@@ -342,7 +402,7 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
       for (int j = 0; j < 3; ++j) {
         if (j == i || (j == 2 && iz == 0)) continue;
         const int64_t mj = nbr_m(n, j);
-        G::sum_add(S, a.w[j], G::staple_bwd(IO::template load<R>(a.U, i, g.V, mj),
+        G::sum_add(S, a.w[j], G::template staple_bwd<ANY>(IO::template load<R>(a.U, i, g.V, mj),
                                             IO::template load<R>(a.U, j, g.V, nbr_p(n, i) + mj - s),
                                             IO::template load<R>(a.U, j, g.V, mj)));
       }
@@ -363,7 +423,7 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
         if (ka >= 0 && ka < a.WA) {
 #pragma unroll
           for (int c = 0; c < NA; ++c) q[c] = a.QA[((int64_t)c * a.WA + ka) * g.nxy + t];
-          G::adj(IO::template load<R>(a.U, 2, g.V, s), q);
+          G::template adj<ANY>(IO::template load<R>(a.U, 2, g.V, s), q);
 #pragma unroll
           for (int c = 0; c < NA; ++c) en[c] += a.az2 * q[c];
         }
@@ -582,6 +642,8 @@ __global__ void k_tmunu_fold(const double* part, int split, int nz, double inv, 
 template <int NC, typename R>
 static int launch_tmunu_kernel(glasma_ctx* c, const TmnArgs<R>& a) {
   const dim3 grid((unsigned)c->g.nz, (unsigned)a.split);
+  if (c->links_off)
+    return launch_following("k_tmunu launch", k_tmunu<NC, R, true>, grid, kRedThreads, 0, c->stream, a);
   if constexpr (sizeof(R) == 4 && NC == 2) {
     return launch_following("k_tmunu_su2 launch", k_tmunu_su2, grid, kSu2Threads, 0, c->stream, a);
   } else {
@@ -599,7 +661,7 @@ static int launch_tmunu_kernel(glasma_ctx* c, const TmnArgs<R>& a) {
         return GLASMA_OK;
       }
     }
-    return launch_following("k_tmunu launch", k_tmunu<NC, R>, grid, kRedThreads, 0, c->stream, a);
+    return launch_following("k_tmunu launch", k_tmunu<NC, R, false>, grid, kRedThreads, 0, c->stream, a);
   }
 }
 
@@ -633,7 +695,7 @@ static int tmunu_t(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab) {
   // threads): the split, and with it the order of each slice's sums, depends
   // on the transverse plane alone, not on the number of slices or the device,
   // so a z slab's rows equal the whole lattice's bit for bit
-  const int threads = NC == 2 && sizeof(R) == 4 ? kSu2Threads : kRedThreads;
+  const int threads = NC == 2 && sizeof(R) == 4 && !c->links_off ? kSu2Threads : kRedThreads;
   const int64_t per_slice = (c->g.nxy + threads - 1) / threads;
   int64_t split = kTmunuSplit;
   if (split > per_slice) split = per_slice;

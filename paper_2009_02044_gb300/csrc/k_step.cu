@@ -24,10 +24,11 @@ template <> struct StepOcc<double> {
   static constexpr int sites = 64;
 };
 
-template <int NC, typename R>
+// ANY: for links off the group
+template <int NC, typename R, bool ANY>
 __global__ void __launch_bounds__(3 * StepOcc<R>::sites, StepOcc<R>::blocks) k_step_leapfrog(StepArgs<R> a) {
   follow();
-  step_link<NC, R>(a, (int)threadIdx.y, blockIdx.x * blockDim.x + threadIdx.x, (int)blockIdx.y + a.zlo);
+  step_link<NC, R, ANY>(a, (int)threadIdx.y, blockIdx.x * blockDim.x + threadIdx.x, (int)blockIdx.y + a.zlo);
 }
 
 template <int NC, typename R>
@@ -52,7 +53,8 @@ static int launch_t(glasma_ctx* c, bool hop) {
   a.zlo = c->lo;
   const int bs = StepOcc<R>::sites;
   const unsigned ntb = (unsigned)((c->g.nxy + bs - 1) / bs);
-  return launch_following("k_step_leapfrog launch", k_step_leapfrog<NC, R>, dim3(ntb, (unsigned)(c->hi - c->lo)),
+  return launch_following("k_step_leapfrog launch",
+                          c->links_off ? k_step_leapfrog<NC, R, true> : k_step_leapfrog<NC, R, false>, dim3(ntb, (unsigned)(c->hi - c->lo)),
                           dim3(bs, 3), 0, c->stream, a);
 }
 

@@ -207,7 +207,8 @@ GL_HD SiteNbr site_nbr_tz(const Geom& g, uint32_t t, int iz) {
 //                + U_j^dag(x+i-j) U_i^dag(x-j) U_j(x-j)],
 // since Im tr t^a (U_i S) is linear in S.  Only the anti-hermitian part of
 // the last product is formed.
-template <int NC, typename Rs, typename Rc>
+// ANY: for links off the group.
+template <int NC, typename Rs, typename Rc, bool ANY = false>
 GL_HD void link_force_staple(const typename V2T<Rs>::T* U, const Geom& g, const SiteNbr& n, int i, const Rc* w,
                              Rc* F) {
   typedef LinkAlg<NC, Rc> G;
@@ -224,7 +225,7 @@ GL_HD void link_force_staple(const typename V2T<Rs>::T* U, const Geom& g, const 
     const bool bwd = (j != 2) || (n.iz >= 1);
     const int64_t pj = n.p[j], mj = n.m[j];
     if (fwd) {
-      const M T = G::staple_fwd(LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi),
+      const M T = G::template staple_fwd<ANY>(LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi),
                                 LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, pj),
                                 LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, n.s));
       G::sum_add(S, wj, T);
@@ -232,7 +233,7 @@ GL_HD void link_force_staple(const typename V2T<Rs>::T* U, const Geom& g, const 
     if (bwd) {
       // x + e_i - e_j: the periodic wraps of x and y depend only on ix and
       // iy and z has no wrap, so the two offsets add
-      const M T = G::staple_bwd(LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, mj),
+      const M T = G::template staple_bwd<ANY>(LinkIO<NC, Rs>::template load<Rc>(U, i, g.V, mj),
                                 LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, pi + mj - n.s),
                                 LinkIO<NC, Rs>::template load<Rc>(U, j, g.V, mj));
       G::sum_add(S, wj, T);

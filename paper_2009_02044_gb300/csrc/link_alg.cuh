@@ -19,6 +19,8 @@
 //   evolve(v, c, u)                                 exp(i c v^a t^a) u,
 //                                                   re-unitarised in FP32
 //   reunit, adj (U q U^+), adj_dag (U^+ q U)
+// Links are members of SU(N); staple_fwd, staple_bwd, adj and adj_dag with ANY
+// true take them as any matrices (SU(2): real quaternions).
 //
 // The FP32 forms are templates over the lane type T: float (one site per
 // thread) or f2 (pair.cuh: two sites per thread in the lanes of the packed
@@ -71,7 +73,9 @@ struct LinkAlg<NC, double> : Group<NC, double> {
   GL_HD static M evolve(const double* v, double c, const M& u) { return G::evolve(v, c, u); }
   GL_HD static Sum zero_sum() { return G::zero(); }
   GL_HD static void sum_add(Sum& s, double w, const M& t) { G::scale_add(s, w, t); }
+  template <bool ANY = false>
   GL_HD static M staple_fwd(const M& x, const M& y, const M& z) { return G::mul_d(G::mul_d(x, y), z); }
+  template <bool ANY = false>
   GL_HD static M staple_bwd(const M& x, const M& y, const M& z) { return G::d_mul(G::mul(x, y), z); }
   GL_HD static void proj_mul_sum(const M& u, const Sum& s, double* out) { G::proj_mul(u, s, out); }
   GL_HD static void proj_prod(const M& x, const M& y, double* out) { G::proj_mul(x, y, out); }
@@ -207,7 +211,9 @@ struct LinkAlgDev3 {
     d.re = fma(a[r1].re, b2, fma(-a[r1].im, b[r2].im, fma(a[r2].im, b[r1].im, -a[r2].re * b[r1].re)) + b[r2].re);
     d.im = fma(-a[r1].im, b2, fma(-a1, b[r2].im, fma(a[r2].im, b[r1].re, a[r2].re * b[r1].im)));
   }
+  template <bool ANY = false>
   GL_HD static M staple_fwd(const M& x, const M& y, const M& z) {
+    if (ANY) return mul_d(mul_d(x, y), z);
     M p, t;
     dev_row_d<0>(x, y, p);
     dev_row_d<1>(x, y, p);
@@ -216,7 +222,9 @@ struct LinkAlgDev3 {
     third_row<2>(t);
     return t;
   }
+  template <bool ANY = false>
   GL_HD static M staple_bwd(const M& x, const M& y, const M& z) {
+    if (ANY) return d_mul(mul(x, y), z);
     M p, t;
     dev_col<1>(x, y, p);
     dev_col<2>(x, y, p);
@@ -442,8 +450,8 @@ struct LinkAlgDev3 {
 
   // Adjoint transport of an algebra vector (not a small difference: the full
   // link is used).
-  GL_HD static void adj(const M& u, R* q) { G::adj(full(u), q); }
-  GL_HD static void adj_dag(const M& u, R* q) { G::adj_dag(full(u), q); }
+  template <bool ANY = false> GL_HD static void adj(const M& u, R* q) { G::template adj<ANY>(full(u), q); }
+  template <bool ANY = false> GL_HD static void adj_dag(const M& u, R* q) { G::template adj_dag<ANY>(full(u), q); }
   // the re-unitarised exp(i c v^a t^a) u
   GL_HD static M evolve(const R* v, R c, const M& u) { return reunit(mul(expi(v, c), u)); }
 };
@@ -471,7 +479,9 @@ struct LinkAlgDev2 {
   }
   GL_HD static M mul_d(const M& x, const M& y) { return mul(x, dag(y)); }
   GL_HD static M d_mul(const M& x, const M& y) { return mul(dag(x), y); }
+  template <bool ANY = false>
   GL_HD static M staple_fwd(const M& x, const M& y, const M& z) { return mul_d(mul_d(x, y), z); }
+  template <bool ANY = false>
   GL_HD static M staple_bwd(const M& x, const M& y, const M& z) { return d_mul(mul(x, y), z); }
 
   struct Sum {
@@ -538,8 +548,8 @@ struct LinkAlgDev2 {
     const R f = R(1.f) + g;
     return M{{g + f * x.a.re, f * x.a.im}, f * x.b};
   }
-  GL_HD static void adj(const M& u, R* q) { G::adj(full(u), q); }
-  GL_HD static void adj_dag(const M& u, R* q) { G::adj_dag(full(u), q); }
+  template <bool ANY = false> GL_HD static void adj(const M& u, R* q) { G::template adj<ANY>(full(u), q); }
+  template <bool ANY = false> GL_HD static void adj_dag(const M& u, R* q) { G::template adj_dag<ANY>(full(u), q); }
   // the re-unitarised exp(i c v^a t^a) u
   GL_HD static M evolve(const R* v, R c, const M& u) { return reunit(mul(expi(v, c), u)); }
 };

@@ -36,7 +36,7 @@ struct StepArgs {
 // arithmetic.  update_link_ue takes the link U_i(x) and the field
 // E_i(t_{n-1/2}) already loaded (Ui, E0), and where
 // their new values go; update_link loads them.
-template <int NC, typename R>
+template <int NC, typename R, bool ANY = false>
 __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint32_t t, int iz, R* E,
                                                typename V2T<R>::T* Un, const R* F,
                                                const typename LinkAlg<NC, R>::M& Ui, const R* E0) {
@@ -57,7 +57,7 @@ __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint
       for (int c = 0; c < NA; ++c) q[c] = a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t];
 #pragma unroll
       for (int c = 0; c < NA; ++c) dj[c] -= a.az2 * q[c];
-      G::adj_dag(Ui, q);
+      G::template adj_dag<ANY>(Ui, q);
 #pragma unroll
       for (int c = 0; c < NA; ++c) a.QB[((int64_t)c * a.WB + kb) * a.g.nxy + t] = q[c];
     }
@@ -66,7 +66,7 @@ __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint
       R q[NA];
 #pragma unroll
       for (int c = 0; c < NA; ++c) q[c] = a.QA[((int64_t)c * a.WA + ka) * a.g.nxy + t];
-      G::adj(Ui, q);
+      G::template adj<ANY>(Ui, q);
 #pragma unroll
       for (int c = 0; c < NA; ++c) {
         dj[c] += a.az2 * q[c];
@@ -81,7 +81,7 @@ __device__ __forceinline__ void update_link_ue(const StepArgs<R>& a, int i, uint
   LinkIO<NC, R>::template put<R>(Un, G::evolve(e, a.dt, Ui));
 }
 
-template <int NC, typename R>
+template <int NC, typename R, bool ANY = false>
 __device__ __forceinline__ void update_link(const StepArgs<R>& a, int i, uint32_t t, int iz, int64_t s,
                                             const R* F) {
   constexpr int NA = LinkAlg<NC, R>::NA;
@@ -90,21 +90,21 @@ __device__ __forceinline__ void update_link(const StepArgs<R>& a, int i, uint32_
   R E0[NA];
 #pragma unroll
   for (int c = 0; c < NA; ++c) E0[c] = E[c * a.g.V];
-  update_link_ue<NC, R>(a, i, t, iz, E, a.Un + link_index(NC, i, 0, a.g.V, s), F, Ui, E0);
+  update_link_ue<NC, R, ANY>(a, i, t, iz, E, a.Un + link_index(NC, i, 0, a.g.V, s), F, Ui, E0);
 }
 
 // Link i of the site with transverse index t on slice iz, its force from
 // the four staples (link_force_staple); the z link of the last slice does
 // not exist.
-template <int NC, typename R>
+template <int NC, typename R, bool ANY = false>
 __device__ __forceinline__ void step_link(const StepArgs<R>& a, int i, uint32_t t, int iz) {
   constexpr int NA = LinkAlg<NC, R>::NA;
   if (t >= (uint32_t)a.g.nxy) return;
   if (i == 2 && iz == a.g.nz - 1) return;  // no z link on the last slice
   const SiteNbr n = site_nbr_tz(a.g, t, iz);
   R F[NA];
-  link_force_staple<NC, R, R>(a.U, a.g, n, i, a.w, F);
-  update_link<NC, R>(a, i, t, iz, n.s, F);
+  link_force_staple<NC, R, R, ANY>(a.U, a.g, n, i, a.w, F);
+  update_link<NC, R, ANY>(a, i, t, iz, n.s, F);
 }
 
 }  // namespace glasma
