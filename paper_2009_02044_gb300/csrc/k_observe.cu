@@ -279,26 +279,18 @@ struct Fro2<2, R> {
   }
 };
 
-// Sum of a thread's per-site values: FP64, or for an FP32 state the unevaluated
-// sum hi + lo of two floats (Knuth's two-sum: the rounding error of every
-// addition is exact and goes to lo, so the sum is good to 2^-48), which keeps
-// the conversions and additions of every site off the narrow FP64 pipe.
-template <typename R> struct SiteSum;
-template <>
-struct SiteSum<double> {
+// FP64 sum of a thread's per-site values.  Those of an FP32 state are widened on
+// the integer pipe (add) or by the conversion instruction of the FP64 pipe
+// (add_cvt), whichever has time to spare: SU(3) 512 x 64^2 0.419 ms per sample by
+// add alone; SU(2) 1024 x 128^2 0.660 by add alone, 0.665 by conversions alone,
+// 0.631 with both (two floats, whose sum is good to 2^-48 and overflows where a
+// double does not, 0.424 and 0.614).
+template <typename R>
+struct SiteSum {
   double s = 0.0;
-  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ void add(R x) { s += widen<double>(x); }
+  __device__ __forceinline__ void add_cvt(R x) { s += (double)x; }
   __device__ __forceinline__ double get() const { return s; }
-};
-template <>
-struct SiteSum<float> {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
-    hi = t;
-  }
-  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
 
 // The block's sums of E_x^2 + E_y^2, E_z^2, b_xy, b_xz + b_yz (without the
@@ -333,7 +325,7 @@ template <> struct TmnOcc<3, float> { static constexpr int blocks = 2; };
 // Per-site arithmetic in the state's precision R (FP32 plaquette products in
 // the deviation form; the per-site sums of squares and of E B products in R,
 // all of positive terms except the Poynting sum), every accumulation over sites
-// as SiteSum, in FP64 between threads.  Block (iz, p) takes `per` consecutive
+// in FP64.  Block (iz, p) takes `per` consecutive
 // sites of slice iz, 256 at a time (neighbouring rows meet in L1); k_tmunu_fold
 // adds the split block sums of a slice in a fixed order.
 // The plaquettes based at a site serve three ends at once: their energy, the
@@ -452,7 +444,7 @@ __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(Tm
 // products and a projection), and the fields are loaded before anything else.
 // Load latency and the waves of blocks bound it: 8 blocks of 128 threads per SM
 // at 64 registers (120 B of spills) take, on SU(2) 1024 x 128^2, 768 x 64^2 and
-// 131 x 45 x 48, 0.61, 0.137 and 0.022 ms (general form 0.94, 0.227 and 0.027);
+// 131 x 45 x 48, 0.63, 0.139 and 0.021 ms (general form 0.94, 0.227 and 0.027);
 // 6 blocks at 80 registers 0.69, 0.159 and 0.021, blocks of 256 at 64 registers
 // 0.63, 0.176 and 0.026.
 __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) {
@@ -488,7 +480,7 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
     Vec3 F[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, pxz{0.f, 0.f, 0.f}, pyz = pxz;
     {
       const Dev4 A = dev_mulq(ux, dev_load(Uy + txp)), B = dev_mulq(uy, dev_load(Ux + typ));
-      bl.add(dist2(A, B));
+      bl.add_cvt(dist2(A, B));
       const Vec3 p = vec_ab(A, dev_dag(B));
       add3(F[0], -wt, p);
       add3(F[1], wt, p);
@@ -496,11 +488,11 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
     if (up) {
       uz = dev_load(Uz + t);
       Dev4 A = dev_mulq(ux, dev_load(Uz + txp)), B = dev_mulq(uz, dev_load(Ux + g.nxy + t));
-      bt.add(dist2(A, B));
+      bt.add_cvt(dist2(A, B));
       pxz = vec_ab(A, dev_dag(B));
       A = dev_mulq(uy, dev_load(Uz + typ));
       B = dev_mulq(uz, dev_load(Uy + g.nxy + t));
-      bt.add(dist2(A, B));
+      bt.add_cvt(dist2(A, B));
       pyz = vec_ab(A, dev_dag(B));
       add3(F[0], -wz, pxz);
       add3(F[1], -wz, pyz);
@@ -548,7 +540,7 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
       const float sq = fma(E[i].x, E[i].x, fma(E[i].y, E[i].y, E[i].z * E[i].z)) +
                        fma(n.x, n.x, fma(n.y, n.y, n.z * n.z));
       if (i == 2) {
-        if (up) ez.add(sq);  // no z link on the last slice
+        if (up) ez.add_cvt(sq);  // no z link on the last slice
       } else {
         const Vec3 p = i == 0 ? pxz : pyz;
         et.add(sq);

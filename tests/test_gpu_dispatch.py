@@ -187,3 +187,20 @@ def test_su2_fp32_site_kernel_fills_its_blocks_on_small_planes(G, shape):
         best[kernel] = min(times)
         G.glasma_free(h)
     assert best["auto"] <= 1.1 * best["staple"], best
+
+
+@pytest.mark.parametrize("nc,field", [(2, 3e18), (3, 3e18)])
+def test_fp32_table_sums_beyond_the_range_of_fp32(G, nc, field):
+    """T^{mu nu} adds up sites in FP64: squares of 1e38, of which an FP32 sum
+    holds three, in slices of 4096 sites.  Products of two rounded factors,
+    summed in FP64: 4 * 6e-8 of the entry."""
+    st = _random_state(nc, 6, 64, 64, seed=1)
+    st.U[:] = np.eye(nc)
+    st.E[:] = field
+    st.E[2][st.p.nz - 1] = 0.0
+    st.QA[:] = 0.0
+    st.QB[:] = 0.0
+    tab, H = G.glasma_tmunu(_ctx(G, st, "fp32"))
+    ref, rH = O.tmunu(st)
+    assert np.max(np.abs(tab - ref)) <= 2.4e-7 * np.max(ref)
+    assert abs(H - rH) <= 2.4e-7 * rH
