@@ -227,3 +227,38 @@ def test_su3_fp32_error_of_two_steps(G, kernel, shape):
     G.glasma_step(h, 2)
     E, ref = G.glasma_get_fields(h)[1], O.step(st, 2).E
     assert np.linalg.norm(E - ref) <= 2.484e-7 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("angle", [1e-4, 0.7, 3.0, 25.0])
+@pytest.mark.parametrize("nc,shape", [(2, (48, 64, 64)), (3, (9, 6, 64)), (3, (9, 6, 32))])
+def test_link_update_at_any_angle_by_the_large_lattice_kernels(G, nc, shape, angle):
+    """As test_link_update_at_any_angle, where AUTO is the one-thread-per-site
+    kernel (its own exponential) and the staged kernel (rows of 64; of 32 it is
+    asked for)."""
+    st = _random_state(nc, *shape, seed=23)
+    st.E *= angle / (st.p.dt * np.max(np.abs(st.E)))
+    ref = O.step(st, 2)
+    h = _ctx(G, st, "fp32")
+    if shape[2] == 32:
+        G.glasma_set_step_kernel(h, "staple_staged")
+    G.glasma_step(h, 2)
+    U, E = G.glasma_get_fields(h)[:2]
+    tol = 1.5e-6 * (1 + angle)
+    assert rel(U, ref.U) <= tol and rel(E, ref.E) <= tol
+
+
+# 64 MB hold 32 (SU(2)) and 12 (SU(3)) slices of 96^2, and two of 256^2
+@pytest.mark.parametrize("nc,shape", [(2, (40, 96, 96)), (3, (26, 96, 96)), (3, (5, 256, 256)), (2, (9, 384, 384))])
+def test_fp64_table_across_the_ring_of_the_two_passes(G, nc, shape):
+    """eps, p_L, p_T and S_L of every slice from a scratch that holds a part of
+    the lattice: the FP64 target."""
+    st = _random_state(nc, *shape, seed=sum(shape))
+    ref, rH = O.tmunu(st)
+    h = _ctx(G, st, "fp64")
+    tab, H = G.glasma_tmunu(h)
+    assert np.all(np.abs(tab - ref) <= TOL64 * np.max(np.abs(ref), axis=0))
+    assert abs(H - rH) <= TOL64 * rH
+    G.glasma_step(h, 1)
+    ref, rH = O.tmunu(O.step(st, 1))
+    tab, H = G.glasma_tmunu(h)
+    assert np.all(np.abs(tab - ref) <= TOL64 * np.max(np.abs(ref), axis=0))
