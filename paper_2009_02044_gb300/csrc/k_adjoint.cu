@@ -212,7 +212,7 @@ int adjoint_run(glasma_ctx* c, const double* rho_host, int n_steps, double half_
                 rs * 3 * (size_t)c->WB * g.nxy};
   Scratch sc(c);
   const int ncp = n_steps > 0 ? (n_steps + K - 1) / K : 0;
-  std::vector<StateRef> ck(ncp);
+  std::vector<StateRef> ck(ncp > 1 ? ncp - 1 : 0);  // the last segment begins in seg[0]
   for (auto& r : ck) r = alloc_state(sc, c);
   const int seg_len = n_steps > 0 ? (K < n_steps ? K : n_steps) : 0;
   std::vector<StateRef> seg(seg_len + 1);

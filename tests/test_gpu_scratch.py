@@ -81,3 +81,13 @@ def test_planes_of_any_size_take_the_two_passes(G):
     assert launches["plaquette"] == launches["auto"] >= 2 and launches["staple"] == 1
     assert np.array_equal(tabs["plaquette"], tabs["auto"])
     assert np.max(np.abs(tabs["auto"] - tabs["staple"])) <= 1e-11 * np.max(np.abs(tabs["staple"]))
+
+
+def test_gradient_holds_a_checkpoint_per_recomputed_segment(G, monkeypatch):
+    """Seven steps in segments of three: buffers of the links' size are the
+    context's two, the checkpoints of the first two segments, four states of a
+    segment, the final state and the links' adjoints."""
+    cfg = dict(gi.small_config(2, nz=48, nx=5, ny=7, sigma_l=2.0))
+    sizes = _allocator(G, monkeypatch, lambda k, n: False)
+    G.glasma_adjoint_energy(cfg, None, 7, 4.0, checkpoint_every=3)
+    assert sizes.count(96 * 48 * 5 * 7) == 2 + 2 + 4 + 1 + 1
