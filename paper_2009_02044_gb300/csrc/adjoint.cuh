@@ -33,12 +33,8 @@ struct Q4 {
 };
 
 GL_HD Q4 q_zero() { return Q4{0.0, 0.0, 0.0, 0.0}; }
-GL_HD Q4 q_one() { return Q4{1.0, 0.0, 0.0, 0.0}; }
 GL_HD Q4 q_pure(const double* v) { return Q4{0.0, v[0], v[1], v[2]}; }
 GL_HD Q4 q_dag(const Q4& a) { return Q4{a.w, -a.x, -a.y, -a.z}; }
-GL_HD Q4 q_add(const Q4& a, const Q4& b) { return Q4{a.w + b.w, a.x + b.x, a.y + b.y, a.z + b.z}; }
-GL_HD Q4 q_sub(const Q4& a, const Q4& b) { return Q4{a.w - b.w, a.x - b.x, a.y - b.y, a.z - b.z}; }
-GL_HD Q4 q_scale(const Q4& a, double s) { return Q4{s * a.w, s * a.x, s * a.y, s * a.z}; }
 GL_HD void q_acc(Q4& acc, const Q4& a) {
   acc.w += a.w;
   acc.x += a.x;

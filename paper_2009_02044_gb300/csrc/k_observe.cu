@@ -238,12 +238,11 @@ struct TmnArgs {
   R dt;
   R w[3];
   R az2;
-  double a[3];
   // products of reciprocals of the spacings, formed on the host (an FP64
   // division is a long sequence on GB300's narrow FP64 pipe):
-  double binv[3];   // 1 / (a_i a_j)^2 of the planes xy, xz, yz
-  double hinv2[3];  // 1 / (2 a_i^2)
-  double slc[2];    // Poynting weights 1 / (a_x^2 a_z), 1 / (a_y^2 a_z)
+  double binv[2];   // 1 / (a_i a_j)^2 of the plane xy and of xz and yz
+  double hinv2[2];  // 1 / (2 a_i^2) of x and y, and of z
+  double slc;       // Poynting weight 1 / (a_t^2 a_z)
   int hop;
   int zA0, WA, zB0, WB;
   int split;     // blocks per z slice
@@ -305,14 +304,14 @@ __device__ __forceinline__ void tmunu_write(const TmnArgs<R>& a, double (*sh)[T]
   if (threadIdx.x == 0) {
     // eps, p_L, p_T, S_L and whether a value was not finite (the directions x
     // and y have the same spacing)
-    const double e_t = 0.5 * v[0] * a.hinv2[0], e_z = 0.5 * v[1] * a.hinv2[2];
+    const double e_t = 0.5 * v[0] * a.hinv2[0], e_z = 0.5 * v[1] * a.hinv2[1];
     const double b_l = v[2] * a.binv[0], b_t = v[3] * a.binv[1];
     const double p_t = e_z + b_l;
     double* out = a.part + ((int64_t)iz * a.split + blockIdx.y) * 5;
     out[0] = e_t + e_z + b_l + b_t;
     out[1] = e_t + b_t - p_t;
     out[2] = p_t;
-    out[3] = v[4] * a.slc[0];
+    out[3] = v[4] * a.slc;
     out[4] = isfinite(out[0]) && isfinite(out[3]) ? 0.0 : 1.0;
   }
 }
@@ -670,14 +669,12 @@ static int tmunu_t(glasma_ctx* c, bool hop, double* host_tab, double* dev_tab) {
   a.w[1] = a.w[0];
   a.w[2] = (R)(2.0 / (c->p.a_z * c->p.a_z));
   a.az2 = (R)(c->p.a_z * c->p.a_z);
-  a.a[0] = a.a[1] = c->p.a_t;
-  a.a[2] = c->p.a_z;
-  a.binv[0] = 1.0 / (a.a[0] * a.a[1] * a.a[0] * a.a[1]);
-  a.binv[1] = 1.0 / (a.a[0] * a.a[2] * a.a[0] * a.a[2]);
-  a.binv[2] = 1.0 / (a.a[1] * a.a[2] * a.a[1] * a.a[2]);
-  for (int i = 0; i < 3; ++i) a.hinv2[i] = 0.5 / (a.a[i] * a.a[i]);
-  a.slc[0] = 1.0 / (a.a[0] * a.a[0] * a.a[2]);
-  a.slc[1] = 1.0 / (a.a[1] * a.a[1] * a.a[2]);
+  const double at = c->p.a_t, az = c->p.a_z;
+  a.binv[0] = 1.0 / (at * at * at * at);
+  a.binv[1] = 1.0 / (at * az * at * az);
+  a.hinv2[0] = 0.5 / (at * at);
+  a.hinv2[1] = 0.5 / (az * az);
+  a.slc = 1.0 / (at * at * az);
   a.hop = hop ? 1 : 0;
   a.zA0 = c->zA0;
   a.WA = c->WA;

@@ -40,9 +40,8 @@
 
 namespace glasma {
 
-template <typename R>
 struct PlaqArgs {
-  StepArgs<R> s;
+  StepArgs<float> s;
   int rows;      // interior rows per block (== ny: the block holds the plane)
   int halo;      // 1 if the block has a -y halo row
   int zlen;      // slices per block
@@ -55,42 +54,42 @@ struct PlaqArgs {
 // force partials (read by the thread itself)
 enum { kCxY = 0, kCxZ = 1, kCyX = 2, kCyZ = 3, kCzX = 4, kCzY = 5, kF = 6, kVecs = 9 };
 
-template <int NC, typename R>
+template <int NC>
 struct PlaqWork {
-  typedef LinkAlg<NC, R> G;
+  typedef LinkAlg<NC, float> G;
   typedef typename G::M M;
   static constexpr int NA = G::NA;
 
   // The two partial products of the plaquette in plane (a, b) based at s:
   // A = U_b(x+a) U_a^dag(x+b), B = U_b^dag(x) U_a(x).
-  __device__ __forceinline__ static void partials(const typename V2T<R>::T* U, const Geom& g, int a, int b,
+  __device__ __forceinline__ static void partials(const float2* U, const Geom& g, int a, int b,
                                                   int64_t s, int64_t sa, int64_t sb, M& A, M& B) {
-    A = G::mul_d(LinkIO<NC, R>::template load<R>(U, b, g.V, sa), LinkIO<NC, R>::template load<R>(U, a, g.V, sb));
-    B = G::d_mul(LinkIO<NC, R>::template load<R>(U, b, g.V, s), LinkIO<NC, R>::template load<R>(U, a, g.V, s));
+    A = G::mul_d(LinkIO<NC, float>::template load<float>(U, b, g.V, sa), LinkIO<NC, float>::template load<float>(U, a, g.V, sb));
+    B = G::d_mul(LinkIO<NC, float>::template load<float>(U, b, g.V, s), LinkIO<NC, float>::template load<float>(U, a, g.V, s));
   }
   // p0 = proj(U_a(x) A U_b^dag(x))
-  __device__ __forceinline__ static void corner0(const typename V2T<R>::T* U, const Geom& g, int a, int b,
-                                                 int64_t s, const M& A, R* p0) {
-    const M C = G::mul(LinkIO<NC, R>::template load<R>(U, a, g.V, s), A);
-    G::proj_prod_d(C, LinkIO<NC, R>::template load<R>(U, b, g.V, s), p0);
+  __device__ __forceinline__ static void corner0(const float2* U, const Geom& g, int a, int b,
+                                                 int64_t s, const M& A, float* p0) {
+    const M C = G::mul(LinkIO<NC, float>::template load<float>(U, a, g.V, s), A);
+    G::proj_prod_d(C, LinkIO<NC, float>::template load<float>(U, b, g.V, s), p0);
   }
 };
 
 // Block shapes: V = 0 up to 320 threads (96 registers at 2 FP32 blocks per
 // SM), V = 1 up to 256 threads (128 registers).
-template <typename R, int V> struct PlaqOcc {
+template <int V> struct PlaqOcc {
   static constexpr int threads = V == 0 ? 320 : 256, blocks = 2;
 };
 
-template <int NC, typename R, int V>
-__global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks) k_step_plaq(PlaqArgs<R> pa) {
-  typedef PlaqWork<NC, R> W;
+template <int NC, int V>
+__global__ void __launch_bounds__(PlaqOcc<V>::threads, PlaqOcc<V>::blocks) k_step_plaq(PlaqArgs pa) {
+  typedef PlaqWork<NC> W;
   typedef typename W::M M;
   constexpr int NA = W::NA;
-  const StepArgs<R>& a = pa.s;
+  const StepArgs<float>& a = pa.s;
   const Geom& g = a.g;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* sm = (R*)smem_raw;
+  float* sm = (float*)smem_raw;
   const int nx = g.nx, ny = g.ny;
   const int trows = pa.rows + pa.halo;      // thread rows of the block
   const int TS = trows * nx;                // shared-memory slots per vector
@@ -111,14 +110,14 @@ __global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks)
   // shared slots of the -x and -y neighbours
   const int slot_mx = ix == 0 ? l + nx - 1 : l - 1;
   const int slot_my = pa.halo ? l - nx : (r == 0 ? l + (ny - 1) * nx : l - nx);
-  const R wt = a.w[0], wz = a.w[2];
+  const float wt = a.w[0], wz = a.w[2];
 
   const int z0 = a.zlo + blockIdx.y * pa.zlen;
   const int z1 = min(z0 + pa.zlen, pa.zhi);
-  R* cz = sm;
+  float* cz = sm;
   if (inner && z0 == 0) {
 #pragma unroll
-    for (int c = 0; c < NA; ++c) cz[(kCzX * NA + c) * TS + l] = cz[(kCzY * NA + c) * TS + l] = R(0);
+    for (int c = 0; c < NA; ++c) cz[(kCzX * NA + c) * TS + l] = cz[(kCzY * NA + c) * TS + l] = float(0);
   }
 
   // A chunk that starts above slice 0 first runs a warm-up iteration on the
@@ -128,7 +127,7 @@ __global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks)
   // chunks (or the slabs of a split lattice) begin.
   for (int iz = z0 > 0 ? z0 - 1 : z0; iz < z1; ++iz) {
     const bool warm = iz < z0;
-    R* buf = sm;
+    float* buf = sm;
     const int64_t s = (int64_t)iz * g.nxy + t;
     const int64_t sxp = s - t + txp, syp = s - t + typ;
     const bool zlink = iz < g.nz - 1;
@@ -138,7 +137,7 @@ __global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks)
       for (int c = 0; c < NA; ++c) {
         buf[((kF + 0) * NA + c) * TS + l] = cz[(kCzX * NA + c) * TS + l];
         buf[((kF + 1) * NA + c) * TS + l] = cz[(kCzY * NA + c) * TS + l];
-        buf[((kF + 2) * NA + c) * TS + l] = R(0);
+        buf[((kF + 2) * NA + c) * TS + l] = float(0);
       }
     }
     // planes (x, y), (x, z), (y, z); the last slice has only (x, y), the
@@ -154,27 +153,27 @@ __global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks)
       const bool need_ba = inner || (!warm && hrow && pl == 0);
       if (!(need_ab || need_ba)) continue;
       const int64_t sa = pa_ == 0 ? sxp : syp, sb = pb == 1 ? syp : s + g.nxy;
-      const R wa = wt, wb = pb == 2 ? wz : wt;  // w_a, w_b = 2 / a^2 of the plane's directions
+      const float wa = wt, wb = pb == 2 ? wz : wt;  // w_a, w_b = 2 / a^2 of the plane's directions
       // shared vector of pAB (to link b of x+a) and of pBA (to link a of x+b)
       const int vab = pl == 0 ? kCxY : (pl == 1 ? kCxZ : kCyZ);
       const int vba = pl == 0 ? kCyX : (pl == 1 ? kCzX : kCzY);
       M A, B;
-      R p[NA];
+      float p[NA];
       W::partials(a.U, g, pa_, pb, s, sa, sb, A, B);
       if (need_ab) {
-        LinkAlg<NC, R>::proj_prod(A, B, p);
+        LinkAlg<NC, float>::proj_prod(A, B, p);
 #pragma unroll
         for (int c = 0; c < NA; ++c) buf[(vab * NA + c) * TS + l] = -wa * p[c];
       }
       if (need_ba) {
-        LinkAlg<NC, R>::proj_prod(B, A, p);
+        LinkAlg<NC, float>::proj_prod(B, A, p);
 #pragma unroll
         for (int c = 0; c < NA; ++c) buf[(vba * NA + c) * TS + l] = wb * p[c];
       }
       if (inner && !warm) {
         W::corner0(a.U, g, pa_, pb, s, A, p);
-        R* fa = buf + (kF + pa_) * NA * TS + l;
-        R* fb = buf + (kF + pb) * NA * TS + l;
+        float* fa = buf + (kF + pa_) * NA * TS + l;
+        float* fb = buf + (kF + pb) * NA * TS + l;
 #pragma unroll
         for (int c = 0; c < NA; ++c) {
           fa[c * TS] -= wb * p[c];
@@ -202,10 +201,10 @@ __global__ void __launch_bounds__(PlaqOcc<R, V>::threads, PlaqOcc<R, V>::blocks)
       const int nl = zlink ? 3 : 2;
 #pragma unroll 1
       for (int i = 0; i < nl; ++i) {
-        R F[NA];
+        float F[NA];
 #pragma unroll
         for (int c = 0; c < NA; ++c) F[c] = buf[((kF + i) * NA + c) * TS + l];
-        update_link<NC, R>(a, i, t, iz, s, F);
+        update_link<NC, float>(a, i, t, iz, s, F);
       }
     }
   }
@@ -236,21 +235,21 @@ static bool plaq_shape(int nx, int ny, int tmax, int* rows, int* halo) {
   return true;
 }
 
-template <int NC, typename R, int V>
+template <int NC, int V>
 static int launch_plaq_t(glasma_ctx* c, bool hop, int zlen) {
-  PlaqArgs<R> pa;
-  StepArgs<R>& a = pa.s;
-  a.U = (const typename V2T<R>::T*)c->U[c->cur];
-  a.Un = (typename V2T<R>::T*)c->U[1 - c->cur];
-  a.E = (R*)c->E;
-  a.QA = (R*)c->QA;
-  a.QB = (R*)c->QB;
+  PlaqArgs pa;
+  StepArgs<float>& a = pa.s;
+  a.U = (const float2*)c->U[c->cur];
+  a.Un = (float2*)c->U[1 - c->cur];
+  a.E = (float*)c->E;
+  a.QA = (float*)c->QA;
+  a.QB = (float*)c->QB;
   a.g = c->g;
-  a.dt = (R)c->p.dt;
-  a.w[0] = (R)(2.0 / (c->p.a_t * c->p.a_t));
+  a.dt = (float)c->p.dt;
+  a.w[0] = (float)(2.0 / (c->p.a_t * c->p.a_t));
   a.w[1] = a.w[0];
-  a.w[2] = (R)(2.0 / (c->p.a_z * c->p.a_z));
-  a.az2 = (R)(c->p.a_z * c->p.a_z);
+  a.w[2] = (float)(2.0 / (c->p.a_z * c->p.a_z));
+  a.az2 = (float)(c->p.a_z * c->p.a_z);
   a.hop = hop ? 1 : 0;
   a.zA0 = c->zA0;
   a.WA = c->WA;
@@ -258,12 +257,12 @@ static int launch_plaq_t(glasma_ctx* c, bool hop, int zlen) {
   a.WB = c->WB;
   a.zlo = c->lo;
   pa.zhi = c->hi;
-  constexpr int T = PlaqOcc<R, V>::threads;
+  constexpr int T = PlaqOcc<V>::threads;
   if (!plaq_shape(c->g.nx, c->g.ny, T, &pa.rows, &pa.halo))
     return set_error(GLASMA_ERR_INTERNAL, "plaquette kernel: transverse rows too long");
   pa.zlen = zlen;
   const int TS = (pa.rows + pa.halo) * c->g.nx;
-  const size_t smem = (size_t)kVecs * LinkAlg<NC, R>::NA * TS * sizeof(R);
+  const size_t smem = (size_t)kVecs * LinkAlg<NC, float>::NA * TS * sizeof(float);
   if (!c->plaq_ready) {
     int st = plaq_prepare(c);
     if (st) return st;
@@ -271,7 +270,7 @@ static int launch_plaq_t(glasma_ctx* c, bool hop, int zlen) {
   const unsigned tiles = (unsigned)((c->g.ny + pa.rows - 1) / pa.rows);
   const unsigned chunks = (unsigned)((c->hi - c->lo + zlen - 1) / zlen);
   const unsigned threads = (unsigned)((TS + 31) / 32 * 32);
-  k_step_plaq<NC, R, V><<<dim3(tiles, chunks), threads, smem, c->stream>>>(pa);
+  k_step_plaq<NC, V><<<dim3(tiles, chunks), threads, smem, c->stream>>>(pa);
   return cuda_check(cudaGetLastError(), "k_step_plaq launch");
 }
 
@@ -280,23 +279,23 @@ static int plaq_variant(const glasma_ctx* c) { return c->step_kernel == GLASMA_K
 
 // The dynamic shared-memory limit is a per-device function attribute: set
 // it for every instance this context may launch, on the context's device.
-template <int NC, typename R>
+template <int NC>
 static int plaq_attrs() {
-  int st = cuda_check(cudaFuncSetAttribute(k_step_plaq<NC, R, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(kVecs * LinkAlg<NC, R>::NA * PlaqOcc<R, 0>::threads * sizeof(R))),
+  int st = cuda_check(cudaFuncSetAttribute(k_step_plaq<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(kVecs * LinkAlg<NC, float>::NA * PlaqOcc<0>::threads * sizeof(float))),
                       "k_step_plaq attributes");
   if (st) return st;
-  return cuda_check(cudaFuncSetAttribute(k_step_plaq<NC, R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(kVecs * LinkAlg<NC, R>::NA * PlaqOcc<R, 1>::threads * sizeof(R))),
+  return cuda_check(cudaFuncSetAttribute(k_step_plaq<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kVecs * LinkAlg<NC, float>::NA * PlaqOcc<1>::threads * sizeof(float))),
                     "k_step_plaq attributes");
 }
 
 int plaq_prepare(glasma_ctx* c) {
   int st;
   if (c->p.nc == 2)
-    st = plaq_attrs<2, float>();
+    st = plaq_attrs<2>();
   else
-    st = plaq_attrs<3, float>();
+    st = plaq_attrs<3>();
   if (!st) c->plaq_ready = true;
   return st;
 }
@@ -324,8 +323,8 @@ int launch_step_plaq(glasma_ctx* c, bool hop, int zlen) {
   if (zlen <= 0) zlen = plaq_default_zlen(c);
   const int v = plaq_variant(c);
   if (c->rs != 4) return set_error(GLASMA_ERR_INTERNAL, "the marching plaquette kernel is FP32 only");
-  if (c->p.nc == 2) return v ? launch_plaq_t<2, float, 1>(c, hop, zlen) : launch_plaq_t<2, float, 0>(c, hop, zlen);
-  return v ? launch_plaq_t<3, float, 1>(c, hop, zlen) : launch_plaq_t<3, float, 0>(c, hop, zlen);
+  if (c->p.nc == 2) return v ? launch_plaq_t<2, 1>(c, hop, zlen) : launch_plaq_t<2, 0>(c, hop, zlen);
+  return v ? launch_plaq_t<3, 1>(c, hop, zlen) : launch_plaq_t<3, 0>(c, hop, zlen);
 }
 
 }  // namespace glasma

@@ -315,7 +315,7 @@ struct LinkAlgDev3 {
   // every power is Q^n = al_n + be_n Q + ga_n Q^2 with
   //   al_{n+1} = c0 ga_n,  be_{n+1} = al_n + c1 ga_n,  ga_{n+1} = be_n.
   // exp(iQ) - 1 = sum_{n>=1} (i^n/n!) Q^n = f0 + f1 Q + f2 Q^2, summed to
-  // n = 9: the remainder is below ||Q||^10/10! < 3e-10 ||Q|| for
+  // n = 9: the remainder is below ||Q||^10/10! < 6e-10 ||Q|| for
   // ||Q||_F <= 1/2.  f0 collects only terms of order ||Q||^3 and up, so
   // nothing of size 1 is formed.  Larger ||Q|| is halved s times first and
   // the result doubled exactly, e_{2h} = 2 e_h + e_h^2.
@@ -537,7 +537,7 @@ struct LinkAlgDev2 {
   GL_HD static M expi(const R* v, R c) {
     const R n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
     if (all_zero_s(n2)) return G::zero();
-    const R x = R(0.25f) * c * c * n2;  // th^2: Taylor series up to 1/4 (remainders below 2e-11)
+    const R x = R(0.25f) * c * c * n2;  // th^2: Taylor series up to 1/4 (remainders below 2.5e-11)
     if (all_abs_lt_s(x, 0.25f)) {
       const R co = x * fma(x, fma(x, fma(x, fma(x, R(-1.f / 3628800.f), R(1.f / 40320.f)), R(-1.f / 720.f)),
                                   R(1.f / 24.f)), R(-0.5f));

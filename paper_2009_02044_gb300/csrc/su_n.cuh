@@ -519,7 +519,7 @@ struct Group<3, R> {
   }
 
   // exp(i c v^a t^a) - 1.  ||Q||_F <= 1/16 (a time step's links, dt E ~ 0.05)
-  // takes 9 terms (remainder below 4e-19 ||Q||), ||Q||_F <= 1/2 takes 15
+  // takes 9 terms (remainder below 4.1e-18 ||Q||), ||Q||_F <= 1/2 takes 15
   // (below 2e-18 ||Q||), about 170 and 200 multiply-adds; larger arguments
   // take the eigenvalue form below, whose inverse cosine, square roots,
   // divisions and four sine and cosine pairs are some 600 operations of the
