@@ -318,8 +318,9 @@ GLASMA_API int glasma_get_info(const glasma_ctx* c, glasma_info* info);
  *   glasma_init_mv, every rank passing the same p and charges).  Its local
  *   lattice is the slab plus a halo slice below (if z0 > 0) and above (if
  *   z1 < nz); the initial state of every owned and halo slice equals the
- *   whole lattice's bit for bit.  The leapfrog step kernel is the staple or
- *   plaquette kernel (never the site-paired one); the improved scheme runs
+ *   whole lattice's bit for bit.  The leapfrog step kernel is the staple, the
+ *   plaquette or (FP32 SU(2), by the whole lattice's sites) the one-thread-per-
+ *   site kernel (never the site-paired or staged one); the improved scheme runs
  *   sweep by sweep (glasma_implicit_begin below).  Errors: INVALID_ARG (as
  *   glasma_init_mv; z0 < 0, z1 > nz, z1 <= z0), OOM, CUDA.
  * glasma_slab_info: owned global slices [*z0, *z1), local slices, and the

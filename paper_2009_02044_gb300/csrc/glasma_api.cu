@@ -130,14 +130,15 @@ static int check_params(const glasma_params* p) {
 
 // The automatic choice, from CUDA-event timings on GB300: in FP64 the
 // two-pass plaquette form (the fewest multiply-adds, and the FP64 pipe bounds
-// the step; figures in k_step_plaq64.cu); in FP32 SU(3) with rows of 64 sites the staged staple
-// kernel (0.388 ms per 512 x 64^2 step against 0.432 for the staple kernel,
-// bitwise the same result; with rows of 32 sites 0.125 against 0.111 per
-// 512 x 32^2 step), else the staple kernel (with full triple products 0.469 ms,
-// against 0.521 for the plaquette kernel and 0.572 for site pairs, whose 168
-// registers leave too few warps to hide latency); in FP32 SU(2) one thread per site on large lattices (0.60 against 1.10 ms for
-// the staple kernel and 1.39 for site pairs per 1024 x 128^2 step), the staple
-// kernel on small ones.
+// the step; figures in k_step_plaq64.cu); in FP32 SU(3) with rows of 64 sites
+// the staged staple kernel (0.388 ms per 512 x 64^2 step against 0.437 for the
+// staple kernel, bitwise the same result; with rows of 32 sites 0.125 against
+// 0.111 per 512 x 32^2 step), else the staple kernel (with full triple products
+// 0.469 ms, against 0.521 for the plaquette kernel and 0.572 for site pairs,
+// whose 168 registers leave too few warps to hide latency); in FP32 SU(2) one
+// thread per site on large lattices (0.59 against 1.01 ms for the staple kernel
+// and 1.39 for site pairs per 1024 x 128^2 step), the staple kernel on small
+// ones.
 bool use_plaq_kernel(const glasma_ctx* c) {
   if (c->rs == 8) return false;
   if (c->step_kernel == GLASMA_KERNEL_PLAQUETTE || c->step_kernel == GLASMA_KERNEL_PLAQUETTE_256) return plaq_fits(c);

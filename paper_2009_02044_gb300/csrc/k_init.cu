@@ -221,7 +221,7 @@ __global__ void k_tail_links(const typename Group<NC, double>::M* full, typename
 // shared memory (2.4 exponentials per site instead of the 6 that a thread by
 // itself takes): FP64-pipe bound there, bound by the stores elsewhere.  The whole
 // initial state, with the DFTs, the series logarithm and the split divergence:
-// SU(3) 512 x 64^2, sigma_L = 4, 7.5 -> 1.8 ms, SU(2) 1024 x 128^2 13.5 -> 2.2 ms.
+// SU(3) 512 x 64^2, sigma_L = 4, 7.5 -> 1.6 ms, SU(2) 1024 x 128^2 13.5 -> 1.7 ms.
 // U1, the buffer the first step writes, only needs the absent z links of the
 // last slice (all of it on a slab, whose halo slices are not stepped).
 constexpr int kTileX = 16, kTileY = 8;

@@ -331,8 +331,8 @@ template <> struct TmnOcc<3, float> { static constexpr int blocks = 2; };
 // field B, and the forward half of the force on both their links; only the
 // backward staples are formed for the force alone.  That is 23 link products
 // per site where forward staples by themselves made 35.  Per sample: SU(3)
-// 512 x 64^2 FP32 0.797 -> 0.449 ms, SU(2) 1024 x 128^2 FP32 1.78 -> 0.936 ms, SU(3)
-// 512 x 64^2 FP64 15.2 -> 10.8 ms.
+// 512 x 64^2 FP32 0.797 -> 0.449 ms (0.42 with staples of two rows and FP64 sums),
+// FP64 15.2 -> 10.8 ms.
 // ANY: for links off the group.
 template <int NC, typename R, bool ANY>
 __global__ void __launch_bounds__(kRedThreads, TmnOcc<NC, R>::blocks) k_tmunu(TmnArgs<R> a) {
@@ -554,8 +554,8 @@ __global__ void __launch_bounds__(kSu2Threads, 8) k_tmunu_su2(TmnArgs<float> a) 
 // come from the step's first pass (k_step_plaq64.cu), which forms each
 // plaquette once where k_tmunu forms 23 link products per site, and this pass
 // adds E_{n+1/2} and the sums.  The FP64 pipe bounds both: SU(3) 160 x 24^2 0.607 ->
-// 0.354 ms, 90 x 7 x 11 0.109 -> 0.055, 512 x 64^2 10.8 -> 7.8; SU(2) 128 x 16^2
-// 0.049 -> 0.035, 512 x 64^2 2.33 -> 1.55.
+// 0.347 ms, 90 x 7 x 11 0.109 -> 0.055, 512 x 64^2 10.8 -> 7.7; SU(2) 128 x 16^2
+// 0.049 -> 0.035, 512 x 64^2 2.33 -> 1.50.
 template <int NC>
 __global__ void __launch_bounds__(kRedThreads) k_tmunu_parts(TmnArgs<double> a, const double* vecs, int ring, int z0) {
   follow();

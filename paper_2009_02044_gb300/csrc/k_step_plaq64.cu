@@ -22,8 +22,8 @@
 // passes are numbered straight through the sites, so a small lattice spreads
 // over all SMs and a plane of any size fills its warps.
 // Measured against the marching form, ms per step: SU(2) 128 x 16^2 0.191 ->
-// 0.031, 512 x 64^2 2.45 -> 1.6; SU(3) 160 x 24^2 1.47 -> 0.438, 512 x 64^2 12.3 ->
-// 9.7 (with the series exponentials of su_n.cuh, which came with it).
+// 0.031, 512 x 64^2 2.45 -> 1.6; SU(3) 160 x 24^2 1.47 -> 0.431, 512 x 64^2 12.3 ->
+// 9.5 (with the series exponentials of su_n.cuh, which came with it).
 //
 // The scratch holds a ring of slices (nine vectors per site).  A lattice whose
 // vectors pass kPartsBytes is stepped in chunks of slices; chunk k's parts

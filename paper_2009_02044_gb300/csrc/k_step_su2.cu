@@ -15,8 +15,8 @@
 //   the plaquettes at x - e_x and x - e_y give the four values that are left.
 // That is 17 link loads for three links; exponential and unit norm are short
 // series.  Measured against the staple kernel, ms per step: SU(2) 1024 x 128^2
-// 1.10 -> 0.60, 768 x 64^2 0.209 -> 0.120, 200 x 30 x 20 0.0125 -> 0.0129 (there
-// the staple kernel stays).
+// 1.01 -> 0.59, 768 x 64^2 0.192 -> 0.117, 48 x 64^2 0.0138 -> 0.0118 (below that the
+// staple kernel stays, glasma_api.cu).
 // The fields are loaded at the start of a slice (loaded where they are used,
 // behind the stores of the link before, they cost a memory latency per link:
 // 0.79 -> 0.61 ms), and the lines of the next slice are brought to L2 (0.60).
