@@ -679,6 +679,9 @@ static void support(const glasma_ctx* c, const double* Q, int* lo, int* W) {
   }
 }
 
+// Until the new links are checked (a call may fail in between): as if off
+static int links_unknown(const glasma_ctx* c) { return c->rs == 8 ? -1 : 2; }
+
 // After the links (and those of t_{n-1}, where the context holds valid ones) were
 // replaced: are they on the group?
 static int check_links(glasma_ctx* c) {
@@ -711,6 +714,7 @@ int glasma_set_fields(glasma_ctx* c, const double* U, const double* E, const dou
       if (E[((size_t)2 * V + s) * na + a] != 0.0)
         return set_error(GLASMA_ERR_INVALID_ARG, "E_z on the last slice must be zero");
   }
+  c->links_off = links_unknown(c);
   int st = upload_links(c, c->U[0], U);
   if (st) return st;
   st = upload_links(c, c->U[1], U);
@@ -896,6 +900,7 @@ int glasma_set_state(glasma_ctx* c, const void* host_buf, size_t bytes) {
     c->QB_cap = (size_t)h.WB;
   }
   if (!c->QA || !c->QB) return set_error(GLASMA_ERR_OOM, "charge window allocation failed");
+  c->links_off = links_unknown(c);
   c->cur = 0;
   void* dst[5] = {c->U[0], c->E, c->QA, c->QB, c->Uprev};
   off = sizeof(h);
